@@ -5,10 +5,11 @@ Workload: 64^3 warped + jittered hex grid (262,144 cells, 798,720 unique faces),
 1920x1080 perspective camera (60 deg) on a 120-frame orbit, Lissajous sphere
 lens, face alpha 0.1-0.6. One step = one pass of the whole path for one frame:
 per-cell quality and importance (max-reduce to vertices and edges), vertex
-projection, triangle setup and tile binning, per-pixel fragment count, prefix
-scan, fragment fill with the focus+context shading, per-pixel depth sort and
-front-to-back composite. Inputs are resident in HBM; the per-frame working set
-(fragment lists, ~2 GB) is far larger than L2.
+projection, triangle setup and tile binning, depth order, per-pixel coverage
+count, and the drawing pass (focus+context shading, per-pixel depth order and
+front-to-back blending). Inputs are resident in HBM; the per-frame working set
+(mesh tables, face records, bins, coverage masks, image: ~0.5 GB) is larger
+than L2.
 
 Prints one JSON line (rank 0). --impl reference times the CPU oracle instead
 (brute force, all host cores) on a bounded sample of pixels per step.
@@ -32,28 +33,22 @@ sys.path.insert(0, ROOT)
 # Algorithmic bytes of the kernels: what the method must move, counted once
 # (a fragment record written by the fill and read by the composite, a face
 # record read once per frame), independent of how the kernels tile the work.
-FRAG_BYTES = 24          # 8 B key + 16 B premultiplied RGBA
-
-# DRAM traffic of one k_fill launch (ncu dram__bytes_read.sum + dram__bytes_write.sum,
-# one pass, on the 1920x1080 bench frame), per fragment drawn, and the fill kernel's
-# sources it was taken on: the roofline reports it only while those sources are unchanged.
-FILL_DRAM = {"bytes_per_fragment": 27.64,
-             "sha256": "97e08b9a25a9387f9f365102441d5c877818a94eeb32062b8886111206668b41",
-             "profile": "profiles/dram_k_fill_grid64_orbit_1080p.md"}
-# Warp instructions the fill executes per fragment (ncu smsp__inst_executed.sum on
-# the same frames and sources): its issue roofline, beside the HBM one.
-FILL_ISSUE = {"warp_instructions_per_fragment": 11.126,
-              "sha256": FILL_DRAM["sha256"],
-              "profile": "profiles/issue_k_fill_grid64_orbit_1080p.md"}
+# DRAM traffic of one k_draw launch (ncu dram__bytes_read.sum + dram__bytes_write.sum,
+# one pass, on the 1920x1080 bench frame), per fragment of the frame, and the drawing
+# kernel's sources it was taken on: reported only while those sources are unchanged.
+DRAW_DRAM = {"bytes_per_fragment": None, "sha256": None, "profile": None}
+# Warp instructions it executes per fragment (ncu smsp__inst_executed.sum on the same
+# frame and sources): its issue roofline, beside the HBM one.
+DRAW_ISSUE = {"warp_instructions_per_fragment": None, "sha256": None, "profile": None}
 SCHEDULERS_PER_SM = 4    # warp schedulers (issue slots per cycle) of a Blackwell SM
-FILL_SOURCES = ("csrc/k_fill.cu", "csrc/raster_tiles.cuh", "csrc/shade.cuh", "csrc/raster_common.cuh",
-                "csrc/pipeline.cuh", "csrc/hexfc_internal.cuh")
+DRAW_SOURCES = ("csrc/k_draw.cu", "csrc/shade.cuh", "csrc/raster_common.cuh", "csrc/pipeline.cuh",
+                "csrc/hexfc_internal.cuh")
 
 
-def fill_sources_sha256() -> str:
+def draw_sources_sha256() -> str:
     import hashlib
     h = hashlib.sha256()
-    for f in FILL_SOURCES:
+    for f in DRAW_SOURCES:
         with open(os.path.join(ROOT, "paper_2009_06574_gb300", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -410,26 +405,20 @@ def run_ours(args, rank, world, local_rank):
     P = tiles * 256
     st = r.last_stats
     bins = st["bin_entries"]
-    # what an A-buffer must move (each datum once): the geometry (48 B per face,
-    # 12 B per vertex) read by the count and the fill, a 24 B record per
-    # fragment written by the fill and read by the composite, per pixel a count
-    # written (4 B), an offset and a cursor (8 B) in the fill, an offset (4 B)
-    # and the 16 B image in the composite
+    # what the frame must move: the geometry (48 B per face, 12 B per vertex) read by
+    # the count and by the drawing pass, a list length per pixel written (4 B), the
+    # 16 B image written (the fragments are shaded and blended without being stored)
     n_pix = w.width * w.height
     geometry = n_faces * GEOM_FACE_BYTES + mesh.n_verts * GEOM_VERTEX_BYTES
-    algo = {
-        "fill": F * FRAG_BYTES + n_pix * 8 + geometry,
-        "composite": F * FRAG_BYTES + n_pix * 4 + n_pix * 16,
-        "count": geometry + n_pix * 4,
-    }
-    kernel_stages = {k: per_frame[k] for k in ("vertex", "face", "tile_scan", "bin", "count", "scan", "fill",
-                                               "composite")}
-    dom = max(("fill", "composite", "count"), key=lambda k: kernel_stages[k])
+    algo = {"draw": geometry + n_pix * 16, "count": geometry + n_pix * 4}
+    kernel_stages = {k: per_frame[k] for k in ("vertex", "face", "tile_scan", "bin", "count")}
+    kernel_stages["draw"] = per_frame["fill"]
+    dom = max(("draw", "count"), key=lambda k: kernel_stages[k])
     peak, peak_kind = load_peaks()
     achieved = algo[dom] / (kernel_stages[dom] / 1000.0) / 1e9
     traffic = None
-    if dom == "fill" and fill_sources_sha256() == FILL_DRAM["sha256"]:
-        traffic = FILL_DRAM["bytes_per_fragment"] * F
+    if dom == "draw" and draw_sources_sha256() == DRAW_DRAM["sha256"]:
+        traffic = DRAW_DRAM["bytes_per_fragment"] * F
     sec = None
     if not args.no_4k:
         try:
@@ -468,25 +457,25 @@ def run_ours(args, rank, world, local_rank):
         except Exception as e:  # the GPU number stands on its own
             cpu = {"value": None, "unit": "frames/s", "cores": omp_threads(), "kind": "oracle",
                    "sample": f"failed: {e}"}
-    # the fill's issue roofline: the warp instructions it executes (an ncu count
+    # the drawing pass's issue roofline: the warp instructions it executes (an ncu count
     # on the same sources) over one per scheduler and cycle at the sampled clock
-    fill_issue = None
-    if fill_sources_sha256() == FILL_ISSUE["sha256"]:
+    draw_issue = None
+    if draw_sources_sha256() == DRAW_ISSUE["sha256"]:
         n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
         sm_mhz = (clocks or {}).get("sm_mhz") or 2070.0
-        inst = FILL_ISSUE["warp_instructions_per_fragment"] * F
-        rate = inst / (kernel_stages["fill"] / 1000.0)
+        inst = DRAW_ISSUE["warp_instructions_per_fragment"] * F
+        rate = inst / (kernel_stages["draw"] / 1000.0)
         limit = n_sm * SCHEDULERS_PER_SM * sm_mhz * 1e6
-        fill_issue = {"bound": "issue", "kernel": "k_fill", "achieved": rate, "peak": limit,
+        draw_issue = {"bound": "issue", "kernel": "k_draw", "achieved": rate, "peak": limit,
                       "unit": "warp instructions/s", "frac": rate / limit, "instructions_per_frame": inst,
-                      "source": FILL_ISSUE["profile"]}
+                      "source": DRAW_ISSUE["profile"]}
     line = {
         "metric": "frames/s", "value": fps, "unit": "frames/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": w.name, "cells": mesh.n_cells, "faces": n_faces, "width": w.width,
                    "height": w.height, "frames": w.n_frames,
-                   "l2": "not flushed: per-frame working set (fragment lists) far larger than L2",
+                   "l2": "not flushed: per-frame working set (mesh, face records, masks, image) larger than L2",
                    "parallelism": f"replicas x{world}",
                    "tile_capacity": ["count pass", "previous frame", "capacity network"][args.predicted],
                    "raster_tile": "%dx%d" % hexfc.raster_tile()},
@@ -496,9 +485,9 @@ def run_ours(args, rank, world, local_rank):
         "stage_ms": {k: round(v, 4) for k, v in per_frame.items()},
         "roofline": {"bound": "hbm", "kernel": "k_" + dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "traffic_source": FILL_DRAM["profile"] if traffic else None,
+                     "traffic_source": DRAW_DRAM["profile"] if traffic else None,
                      "peak_kind": peak_kind, "algorithmic_bytes": algo[dom]},
-        "fill_issue": fill_issue,
+        "draw_issue": draw_issue,
         "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clocks,
         "secondary_4k": sec,
         **secondaries,

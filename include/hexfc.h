@@ -39,8 +39,8 @@ enum {
     HEXFC_ERR_TIMEOUT = -5,   /* a bounded device-side wait ran out */
     HEXFC_ERR_MESH = -6,      /* the mesh is malformed (index out of range, non-finite vertex) */
     HEXFC_ERR_STATE = -7,     /* call out of order (no mesh, no view, no previous render) */
-    HEXFC_ERR_CHECK = -8      /* a device-side consistency check failed (list sizes of the count and
-                                 fill passes disagree, or an exact depth could not be confirmed) */
+    HEXFC_ERR_CHECK = -8      /* a device-side consistency check failed (an exact depth could not be
+                                 confirmed) */
 };
 
 /* Longest per-pixel fragment list the sort/composite pass accepts. */
@@ -119,12 +119,11 @@ typedef struct hexfc_frame_stats {
     uint64_t fragments;      /* fragments generated (sum of list lengths) */
     uint64_t bin_entries;    /* (triangle, tile) pairs after binning */
     uint32_t max_list;       /* longest per-pixel list */
-    uint32_t long_lists;     /* pixels handled by the long-list path */
+    uint32_t long_lists;     /* pixels with lists longer than 256 */
     uint32_t width, height;
     uint32_t kernel_launches;  /* kernels this call launched */
     uint32_t covered_pixels;   /* reserved (0) */
-    uint32_t predicted;        /* 1: drawn with chosen tile capacities (no pixel scan, no host wait
-                                  after the count pass) */
+    uint32_t predicted;        /* 1: drawn with chosen tile capacities (no host wait after the count pass) */
     uint32_t overflow_tiles;   /* tiles above their chosen capacity (their lists in the pool) */
     uint64_t capacity;         /* sum of the chosen tile capacities (fragments), 0 if none */
     uint32_t pending;          /* 1: a frame with chosen capacities whose device statistics (fragments,
@@ -143,10 +142,10 @@ enum {
     HEXFC_STAGE_GAP1 = 3,
     HEXFC_STAGE_BIN = 4,      /* bin fill */
     HEXFC_STAGE_COUNT = 5,    /* per-pixel fragment count */
-    HEXFC_STAGE_SCAN = 6,     /* pixel prefix scan */
-    HEXFC_STAGE_GAP2 = 7,
-    HEXFC_STAGE_FILL = 8,     /* fragment fill and shading */
-    HEXFC_STAGE_COMPOSITE = 9,/* sort and composite (both list paths) */
+    HEXFC_STAGE_SCAN = 6,     /* (no pass: chosen capacities against the counts, if any) */
+    HEXFC_STAGE_GAP2 = 7,     /* (no wait: totals on their way to the host) */
+    HEXFC_STAGE_FILL = 8,     /* drawing pass: shading, order and blending */
+    HEXFC_STAGE_COMPOSITE = 9,/* pixels out of order, silhouettes */
     HEXFC_N_STAGES = 10
 };
 
@@ -162,10 +161,10 @@ enum {
 void hexfc_style_default(hexfc_style* style);
 
 /* Create a context on CUDA device `device`. frag_budget_bytes caps the device
- * memory of the context's frame buffers (hexfc_frame_memory), fragment arrays
- * (24 bytes per fragment) included: a count-then-fill frame that would need
- * more is refused with OOM before its fragment arrays grow; 0 means no cap
- * beyond free memory. HEXFC_OPT_FRAG_BUDGET changes it between frames.
+ * memory of the context's frame buffers (hexfc_frame_memory), the frame's
+ * fragment lists (24 bytes per fragment) included, whether they are asked for
+ * (hexfc_debug_pixels) or not: a frame that would need more is refused with OOM
+ * and not drawn; 0 means no cap beyond free memory. HEXFC_OPT_FRAG_BUDGET changes it between frames.
  * Errors: ARG (out == NULL), CUDA (bad device). */
 hexfc_status hexfc_create(hexfc_ctx** out, int device, uint64_t frag_budget_bytes);
 
@@ -208,8 +207,10 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
  * a render of it. Errors: ARG (NULL pointer, different devices), STATE (no
  * such mesh in src), OOM.
  *
- * hexfc_frame_memory: *bytes = device memory held by the context's per-frame
- * buffers (they grow to the largest frame rendered and are reused).
+ * hexfc_frame_memory: *bytes = device memory of the context's per-frame
+ * buffers, with 24 bytes per fragment for the lists of the largest frame (they
+ * grow to the largest frame rendered and are reused; the lists themselves are
+ * accounted for, not held).
  * Errors: ARG.
  *
  * hexfc_trim: free the context's per-frame buffers (the next render allocates
@@ -222,13 +223,13 @@ hexfc_status hexfc_share_mesh(hexfc_ctx* dst, const hexfc_ctx* src, int32_t mesh
  * Batched frames (no counterpart in the paper): many views of one or several
  * resident meshes, each with its own camera, lens, style and output, in one
  * call. The frame's three phases (geometry up to the bin total; binning,
- * depth order and coverage count up to the fragment total; fill and
- * composite) run for all items at once: each phase is captured as one CUDA
+ * depth order and coverage count up to the fragment total; drawing) run for
+ * all items at once: each phase is captured as one CUDA
  * graph with the items on their own streams, and the executable graph of a
  * phase is reused (updated in place) when only parameters changed; with
- * HEXFC_OPT_BATCH_LAUNCH 1 the coverage count, the fill and the main resolve
- * pass of all items are instead each one launch over the tiles of every item.
- * The host waits twice per batch instead of twice per frame.
+ * HEXFC_OPT_BATCH_LAUNCH 1 the coverage count and the drawing pass of all items
+ * are instead each one launch over the tiles of every item. The host waits
+ * twice per batch instead of twice per frame.
  *   items[i].mesh      mesh handle of ctx
  *   items[i].view, .lens, .style   as for hexfc_set_view / _lens / _style
  *                      (the context's own view, lens and style are unchanged)
@@ -305,15 +306,16 @@ hexfc_status hexfc_set_style(hexfc_ctx* ctx, const hexfc_style* style);
  * out_rgba (device, height*width*4 float, row-major, row 0 at the top,
  * straight RGB over the background plus accumulated alpha).
  * Steps, all on `stream`: vertex projection to 16.8 fixed point and 24-bit
- * depth; triangle setup and tile binning; per-pixel fragment count; prefix
- * scan; fragment fill with Eqs. 1-4; per-pixel depth sort and front-to-back
- * composite. The call waits once for the fragment total (to size the buffers);
- * the image is complete when `stream` reaches the end of the call.
+ * depth; triangle setup and tile binning in depth order; per-pixel fragment
+ * count; then every fragment shaded with Eqs. 1-4 and blended front to back in
+ * order of depth. The call waits for the bin total (to size the buffers) and,
+ * while the frame is drawn, for the fragment total (statistics, limits); the
+ * image is complete when `stream` reaches the end of the call.
  * stats (host, nullable) receives the frame statistics.
  * Errors: ARG, STATE (no view), OOM (the frame's buffers would exceed the
  * budget; stats still filled: fragments tells how far), OVERFLOW (a list longer than HEXFC_MAX_LIST), CUDA, and TIMEOUT or
- * CHECK from the device-side checks of the fill and composite passes: those
- * passes run after the call returns, so hexfc_render reports their failure
+ * CHECK from the device-side checks of the drawing passes: those run after
+ * the call returns, so hexfc_render reports their failure
  * on the context's next call (hexfc_render_host at the end of its own frame).
  */
 hexfc_status hexfc_render(hexfc_ctx* ctx, int32_t mesh, float* out_rgba, hexfc_frame_stats* stats,
@@ -323,7 +325,7 @@ hexfc_status hexfc_render(hexfc_ctx* ctx, int32_t mesh, float* out_rgba, hexfc_f
  * float) when the call returns, and the device-side checks of this frame
  * reported by this call. If out_rgba_host is page-locked memory of the
  * context's device (cudaHostAlloc, cudaHostRegister) and 16-byte aligned, the
- * resolve kernels write the image into it directly through its device
+ * drawing kernels write the image into it directly through its device
  * mapping; otherwise the image is rendered into a device buffer of the
  * context and copied. On an error the buffer's contents are unspecified. */
 hexfc_status hexfc_render_host(hexfc_ctx* ctx, int32_t mesh, float* out_rgba_host,
@@ -331,7 +333,9 @@ hexfc_status hexfc_render_host(hexfc_ctx* ctx, int32_t mesh, float* out_rgba_hos
 
 /*
  * Parity hook: the fragment lists of the last render for `n` listed pixels
- * (px[i], py[i], host). counts (host, n) receives each list length; keys
+ * (px[i], py[i], host), built from what that frame was drawn from (an importance
+ * update after it changes nothing, unless it was captured into a CUDA graph:
+ * such an update rewrites the mesh's records in place). counts (host, n) receives each list length; keys
  * (host, cap) and rgba (host, cap*4 float) receive the lists concatenated in
  * the order of the pixel list, each sorted ascending by key =
  * (z24 << 32) | (2*face_id + triangle), rgba premultiplied (Eq. 4).
@@ -348,9 +352,9 @@ enum {
     HEXFC_OPT_DEPTH_BUCKETS = 3,     /* buckets of the per-tile depth order of the triangles: a power of
                                         two in 256..4096 (default 2048), or 0 for no depth order (lists
                                         in the faces' order: a test hook for the sorting passes) */
-    HEXFC_OPT_COMPOSITE_WINDOW = 4,  /* sorted window of the per-pixel resolve: 2 (default), 4 or 8; the
-                                        image does not depend on it, bit for bit */
-    HEXFC_OPT_PREDICTED_CAPACITY = 5, /* 0: count-then-fill (default); 1: capacities from the previous
+    HEXFC_OPT_COMPOSITE_WINDOW = 4,  /* fragments a pixel holds back to blend in order: 2 (default), 4 or
+                                        8; the image does not depend on it, bit for bit */
+    HEXFC_OPT_PREDICTED_CAPACITY = 5, /* 0: exact counts (default); 1: capacities from the previous
                                         frame's tile counts; 2: from the capacity network; 3: the previous
                                         frame's total spread evenly over the tiles (the baseline without
                                         any per-tile knowledge). See below. */
@@ -364,9 +368,8 @@ enum {
                                         flight leave */
     HEXFC_OPT_BATCH_LAUNCH = 8       /* hexfc_render_batch: 0 (default): every item its own launches,
                                         the items as parallel branches of each phase's graph; 1: the
-                                        coverage count, the fill and the main resolve pass of all items
-                                        each one kernel launch over every item's tiles (groups of 64
-                                        items). The images do not depend on it, bit for bit */
+                                        coverage count and the drawing pass of all items each one kernel
+                                        launch over every item's tiles (groups of 64 items). The images do not depend on it, bit for bit */
 };
 hexfc_status hexfc_set_option(hexfc_ctx* ctx, int32_t option, int64_t value);
 
@@ -376,7 +379,7 @@ hexfc_status hexfc_set_option(hexfc_ctx* ctx, int32_t option, int64_t value);
  * for its frame, which is verified by the next call on the context (at that
  * call's first host wait, when the frame has completed) or by this one: if the
  * frame needed more room than its chosen capacities and the pool left, it is
- * drawn again exactly (count-then-fill) into its own output with the camera,
+ * drawn (again) by exact counts into its own output with the camera,
  * lens and style it was drawn with, so that no frame keeps an overflow error.
  * A predicted frame's image is final once the next hexfc_render* call or
  * hexfc_finish on its context has returned (and the stream work it issued has
@@ -397,17 +400,16 @@ hexfc_status hexfc_completed_stats(const hexfc_ctx* ctx, uint64_t frame, hexfc_f
 
 /*
  * Predicted capacities (HEXFC_OPT_PREDICTED_CAPACITY != 0; no counterpart in
- * the paper, which sizes its buffers once): the fragment arrays are divided
- * into per-16x16-tile regions of a chosen capacity before the frame,
- * followed by a pool; after the count pass, the fill lays out each tile's
- * lists in the tile's region itself (in the pool if they do not fit), so
- * there is no pixel scan and no host wait between counting and drawing; the
- * host waits once, at the end of the frame. Capacities come from the
+ * the paper, which sizes its buffers once): the room for the frame's fragment
+ * lists is divided into per-16x16-tile regions of a chosen capacity before the
+ * frame, followed by a pool; after the count pass each tile's exact count is
+ * held against its region (what does not fit takes from the pool) on the
+ * device, so the host does not wait between counting and drawing. Capacities come from the
  * previous frame's exact tile counts (mode 1: count * 1.15 + 256) or from the
  * capacity network (mode 2, see hexfc_capacity_*); the pool holds 35% of the
  * previous frame's fragments. stats.overflow_tiles counts the tiles above
- * their capacity. Only if the pool runs out is the frame drawn again by the
- * exact count-then-fill path, so the image is always exact. The first frame
+ * their capacity. Only if the pool runs out is the frame not drawn by this call
+ * but by exact counts when it is verified, so the image is always exact. The first frame
  * at a resolution, with no previous counts, is drawn exactly.
  */
 
@@ -489,7 +491,7 @@ void hexfc_raster_tile(int32_t* width, int32_t* height);
  *
  * Same inputs, output and result as hexfc_render (the same kernels), but every
  * per-frame buffer (projected vertices, face records, tile bins, counts,
- * offsets, fragment lists) is carved from one file-scope device array of
+ * room for the fragment lists) is carved from one file-scope device array of
  * HEXFC_NOALLOC_SCRATCH_BYTES (32 MiB) that every GPU loading the library holds
  * until the process exits. The call makes no cudaMalloc, cudaFree or
  * cudaMallocHost; the mesh must already be uploaded, and out_rgba (device,
@@ -503,8 +505,8 @@ void hexfc_raster_tile(int32_t* width, int32_t* height);
  *   counters that must start at zero are cleared on the stream). Calls whose
  *   work overlaps on the GPU (other streams, other threads, other contexts of
  *   the same process on the same device) race on it: serialise them.
- * - It waits on `stream` twice, like hexfc_render, and returns with the fill
- *   and the composite still running. Their device error bits (a bounded wait
+ * - It waits on `stream` twice, like hexfc_render, and returns with the drawing
+ *   passes still running. Their device error bits (a bounded wait
  *   that ran out, a failed exactness check) stay in the array and are
  *   reported, as TIMEOUT or CHECK, by the next hexfc_render_noalloc call on
  *   the same device, as hexfc_render reports its previous frame's.

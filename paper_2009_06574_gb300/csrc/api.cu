@@ -2,6 +2,7 @@
 // and the per-frame orchestration of the kernels on the caller's stream.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -35,8 +36,8 @@ struct hexfc_ctx {
     uint64_t inject_bits = 0;   // HEXFC_OPT_DEBUG_ERROR_BITS: ORed into the error word after the next frame
     // A frame drawn with chosen capacities is verified by the next call on the
     // context (or hexfc_finish), once it has completed: what is needed to draw
-    // it again exactly if its capacities ran out, and its device scalars and
-    // count statistics, copied into h_pend at its end.
+    // it again exactly if its capacities ran out, and its device scalars, copied
+    // into h_pend at its end.
     struct Pending {
         bool active = false;
         std::shared_ptr<DevMesh> mesh;
@@ -49,7 +50,7 @@ struct hexfc_ctx {
         hexfc_style style{};
         hexfc_frame_stats fs{};   // what was known when its call returned
     } pend;
-    uint64_t* h_pend = nullptr;        // pinned [kScal + 4 kStatCopies]
+    uint64_t* h_pend = nullptr;        // pinned [kScal]
     hexfc_frame_stats completed{};     // final statistics of the last verified frame
     hexfc_frame_stats history[16]{};   // final statistics of recent frames, at frame % 16
     uint64_t frame_seq = 0;            // frames drawn by this context
@@ -61,9 +62,11 @@ struct hexfc_ctx {
     bool have_prev_cam = false;
     double prev_eye[3] = {0, 0, 0}, prev_F[3] = {0, 0, 1};
     int64_t feat_tiles = 0;   // tiles whose features and exact counts the last frame left for training
-    // last render
+    // last render: what its fragment lists can be rebuilt from (hexfc_debug_pixels)
     bool have_frame = false;
-    int last_W = 0, last_H = 0, last_tiles_x = 0, last_tiles_y = 0;
+    DrawItem last_draw{};
+    std::shared_ptr<DevMesh> last_mesh;
+    std::shared_ptr<FaceStatic> last_fstat;   // the mesh's records it was drawn with
     hexfc_frame_stats last{};
     float* d_out = nullptr;   // image buffer of hexfc_render_host
     int64_t d_out_cap = 0;
@@ -85,6 +88,7 @@ struct hexfc_ctx {
     cudaStream_t origin = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     cudaEvent_t ev_p1 = nullptr;   // a single frame's phase 1: bin total copied (FrameJob::p1_done)
+    cudaEvent_t ev_p2 = nullptr;   // its phase 2: totals copied; the drawing pass runs after it
     cudaGraphExec_t graph_exec[3] = {nullptr, nullptr, nullptr};
     uint64_t graph_instantiations = 0, graph_updates = 0;
 };
@@ -177,7 +181,7 @@ void free_mesh(DevMesh* m)
     if (!m) return;
     dfree(m->verts); dfree(m->cells); dfree(m->cell_edges); dfree(m->cell_imp);
     dfree(m->vkey); dfree(m->ekey); dfree(m->vimp); dfree(m->eattr); dfree(m->elevel);
-    dfree(m->fverts); dfree(m->fedges); dfree(m->fstat); dfree(m->fbound);
+    dfree(m->fverts); dfree(m->fedges); dfree(m->fbound);
     delete m;
 }
 
@@ -185,12 +189,35 @@ void free_frame(FrameBufs& f)
 {
     dfree(f.vproj); dfree(f.ved); dfree(f.fframe); dfree(f.tzsum);
     dfree(f.tile_cnt); dfree(f.tile_off); dfree(f.tile_cur); dfree(f.tile_order); dfree(f.tile_frag); dfree(f.tile_cap); dfree(f.cap_off); dfree(f.tile_zr); dfree(f.cap_x);
-    dfree(f.bins); dfree(f.bins_tmp); dfree(f.masks); dfree(f.seg); dfree(f.cnt);
-    dfree(f.off); dfree(f.zsil);
-    dfree(f.part); dfree(f.part_max); dfree(f.long_q); dfree(f.fix_q); dfree(f.key); dfree(f.rgba); dfree(f.scal);
-    dfree(f.cstat);
+    dfree(f.bins); dfree(f.bins_tmp); dfree(f.masks); dfree(f.zsuf); dfree(f.cnt); dfree(f.zsil);
+    dfree(f.part); dfree(f.part_max); dfree(f.redo); dfree(f.scal);
     if (f.h_scal) cudaFreeHost(f.h_scal);
     f = FrameBufs{};
+}
+
+// A set of static face records that no frame keeps becomes the mesh's own;
+// *fresh: it is new (no positions in it yet).
+hexfc_status own_fstat(DevMesh& m, bool* fresh)
+{
+    *fresh = false;
+    if (m.fstat && m.fstat.use_count() == 2) return HEXFC_OK;   // fstat and fstat_sets
+    for (const auto& f : m.fstat_sets)
+        if (f.use_count() == 1) {
+            m.fstat = f;
+            return HEXFC_OK;
+        }
+    FaceStatic* p = nullptr;
+    const hexfc_status st = dalloc(&p, (size_t)m.n_faces);
+    if (st != HEXFC_OK) return st;
+    try {
+        std::shared_ptr<FaceStatic> f(p, [](FaceStatic* q) { cudaFree(q); });   // (frees p if it throws)
+        m.fstat_sets.push_back(f);
+        m.fstat = std::move(f);
+    } catch (...) {
+        return HEXFC_ERR_OOM;
+    }
+    *fresh = true;
+    return HEXFC_OK;
 }
 
 DevMesh* get_mesh(hexfc_ctx* ctx, int32_t id)
@@ -288,6 +315,11 @@ ShadeParams make_shade_params(const hexfc_lens& lens, const hexfc_style& s, doub
     sp.desat = s.desat;
     const float acc = 256.f * (2.f / 3.f) * s.w_base;
     sp.accent_r2 = acc * acc;
+    sp.bounded = true;
+    for (float v : {s.w_base, s.delta, s.s, s.alpha_min, s.alpha_max, s.tf_lo, s.tf_hi, s.bg[0], s.bg[1], s.bg[2],
+                    s.accent_beta, s.halo_scale, s.darken, s.g_min, s.g_max, s.desat, sp.lens_c[0], sp.lens_c[1],
+                    sp.lens_c[2], sp.lens_inv_r, sp.zref, sp.tf_inv})
+        sp.bounded = sp.bounded && std::fabs(v) < 1e15f;
     return sp;
 }
 
@@ -337,18 +369,18 @@ bool valid_style(const hexfc_style* s)
 }
 
 // One frame: its mesh, camera and style constants, its buffers, and what the
-// host learns between the three phases. Phase 1 (geometry: vertices, face
-// records, per-tile triangle counts and their scan) ends with the bin total;
-// phase 2 (binning, depth order, tile order, coverage count, pixel scan) ends
-// with the fragment total; phase 3 draws (fill and composite). The host reads
-// the totals between phases to size the next phase's buffers.
+// host learns in its three phases. Phase 1 (geometry: vertices, face records,
+// per-tile triangle counts and their scan) ends with the bin total, which the
+// host reads to size phase 2's buffers; phase 2 (binning, depth order, tile
+// order, coverage count) ends with the fragment total; phase 3 draws. Nothing
+// is sized by the fragment total: phase 3 is launched behind phase 2, and the
+// host waits for the totals (statistics, limits) while it runs; a frame that
+// must not be drawn is refused by the same test on the device (DrawItem).
 struct FrameJob {
     FrameBufs* fb = nullptr;
     DevMesh* m = nullptr;
     CamParams cam{};
     ShadeParams sp{};
-    int lod = 0;
-    float delta = 0.f;
     int W = 0, H = 0, tiles_x = 0, tiles_y = 0;
     int64_t n_tiles = 0, n_pix = 0;
     int reverse = 0;
@@ -429,8 +461,6 @@ FrameJob make_job(hexfc_ctx* ctx, FrameBufs* fb, DevMesh* m, float* out)
     j.m = m;
     j.cam = ctx->cam;
     j.sp = make_shade(ctx);
-    j.lod = ctx->style.lod;
-    j.delta = ctx->style.delta;
     j.W = ctx->cam.W;   // the drawn rectangle (the frame, or a sub-rectangle and its apron)
     j.H = ctx->cam.H;
     j.win = output_window(ctx);
@@ -493,16 +523,13 @@ hexfc_status job_alloc(FrameJob& j)
         if ((st = ensure(&fb.cap_x, &c6, 4 * fb.t_cap)) != HEXFC_OK) return st;
     }
     if (!fb.cnt || fb.p_cap < j.n_pix + 1) {
-        int64_t c1 = 0, c2 = 0, c3 = 0;
-        dfree(fb.off); dfree(fb.long_q); dfree(fb.fix_q); dfree(fb.zsil);
+        int64_t c1 = 0, c2 = 0;
+        dfree(fb.zsil); dfree(fb.redo);
         if ((st = ensure(&fb.cnt, &fb.p_cap, j.n_pix + 1)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.off, &c1, fb.p_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.long_q, &c2, fb.p_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.fix_q, &c3, fb.p_cap)) != HEXFC_OK) return st;
-        int64_t c4 = 0;
-        if ((st = ensure(&fb.zsil, &c4, fb.p_cap)) != HEXFC_OK) return st;
+        if ((st = ensure(&fb.zsil, &c1, fb.p_cap)) != HEXFC_OK) return st;
+        if ((st = ensure(&fb.redo, &c2, fb.p_cap)) != HEXFC_OK) return st;
     }
-    const int64_t nparts = scan_partials_needed(std::max<int64_t>(j.n_pix, j.n_tiles)) + 1;
+    const int64_t nparts = scan_partials_needed(j.n_tiles) + 1;
     if (!fb.part || fb.part_cap < 2 * nparts) {
         int64_t c1 = 0;
         dfree(fb.part_max);
@@ -510,7 +537,7 @@ hexfc_status job_alloc(FrameJob& j)
         if ((st = ensure(&fb.part_max, &c1, fb.part_cap)) != HEXFC_OK) return st;
     }
     if (!fb.scal) {
-        if ((st = dalloc(&fb.scal, kScal)) != HEXFC_OK) return st;
+        if ((st = dalloc(&fb.scal, kScalAll)) != HEXFC_OK) return st;
         CK(cudaMallocHost((void**)&fb.h_scal, kScal * sizeof(uint64_t)));
         fb.scal_fresh = true;   // contents undefined: phase 1 clears all of it
     }
@@ -527,15 +554,15 @@ hexfc_status job_phase1(FrameJob& j, cudaStream_t s)
     // last passes of a frame are reported by the next call (hexfc_render_host
     // reads them at the end of its own frame)
     if (fb.scal_fresh) {
-        CK(cudaMemsetAsync(fb.scal, 0, sizeof(uint64_t) * kScal, s));
+        CK(cudaMemsetAsync(fb.scal, 0, sizeof(uint64_t) * kScalAll, s));
         fb.scal_fresh = false;
     } else {
         CK(cudaMemsetAsync(fb.scal, 0, sizeof(uint64_t) * 5, s));
-        CK(cudaMemsetAsync(fb.scal + 6, 0, sizeof(uint64_t) * (kScal - 6), s));
+        CK(cudaMemsetAsync(fb.scal + 6, 0, sizeof(uint64_t) * (kScalAll - 6), s));
     }
     CK(launch_vertex_setup(*j.m, j.cam, fb, s));
     job_mark(j, 1, s);
-    CK(launch_face_setup(*j.m, j.cam, j.lod, j.delta, fb, j.tiles_x, j.tiles_y, s));
+    CK(launch_face_setup(*j.m, j.cam, j.sp, fb, j.tiles_x, j.tiles_y, s));
     job_mark(j, 2, s);
     CK(scan_u32_to_u64(fb.tile_cnt, fb.tile_off, j.n_tiles, fb.part, fb.part_max, fb.scal + 8, 0xFFFFFFFFu, s,
                        (uint32_t)kChunk));
@@ -575,7 +602,7 @@ hexfc_status job_read1(FrameJob& j)
         if ((st = ensure(&fb.bins_tmp, &c1, fb.bin_cap)) != HEXFC_OK) return st;
     }
     if ((st = ensure(&fb.masks, &fb.mask_cap, (int64_t)j.n_bins * (kTilePix / kChunk))) != HEXFC_OK) return st;
-    if ((st = ensure(&fb.seg, &fb.seg_cap, (int64_t)(j.n_bins / kChunk) * (kTilePix / 32))) != HEXFC_OK) return st;
+    if ((st = ensure(&fb.zsuf, &fb.zsuf_cap, (int64_t)(j.n_bins / kChunk))) != HEXFC_OK) return st;
     return HEXFC_OK;
 }
 
@@ -586,7 +613,7 @@ hexfc_status job_phase2_bins(FrameJob& j, cudaStream_t s)
     job_mark(j, 4, s);
     CK(cudaMemsetAsync(fb.bins, 0xFF, sizeof(uint32_t) * (size_t)j.n_bins, s));   // padding slots = kPadBin
     CK(launch_bin_fill(*j.m, fb, j.tiles_x, j.W, j.H, j.reverse, s));
-    CK(launch_bin_sort(*j.m, fb, j.tiles_x, j.tiles_y, j.buckets, s));
+    CK(launch_bin_sort(*j.m, fb, j.tiles_x, j.tiles_y, (int64_t)j.n_bins, j.buckets, s));
     if (!j.order_done) {
         CK(launch_tile_order(fb, j.n_tiles, s));
         j.launches += 1;
@@ -598,14 +625,13 @@ hexfc_status job_phase2_bins(FrameJob& j, cudaStream_t s)
     return HEXFC_OK;
 }
 
-// Phase 2 after the count: the pixel scan, its totals to the host.
-hexfc_status job_phase2_scan(FrameJob& j, cudaStream_t s)
+// Phase 2 after the count: its totals to the host.
+hexfc_status job_phase2_totals(FrameJob& j, cudaStream_t s)
 {
     FrameBufs& fb = *j.fb;
     job_mark(j, 6, s);
-    CK(scan_u32_to_u64(fb.cnt, fb.off, j.n_pix, fb.part, fb.part_max, fb.scal, (uint32_t)kWarpSortMax, s));
     job_mark(j, 7, s);
-    j.launches += 4;   // the count and the three scan passes
+    j.launches += 1;   // the count
     CK(cudaMemcpyAsync(fb.h_scal, fb.scal, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     return HEXFC_OK;
 }
@@ -614,12 +640,15 @@ hexfc_status job_phase2(FrameJob& j, cudaStream_t s)
 {
     hexfc_status st;
     if ((st = job_phase2_bins(j, s)) != HEXFC_OK) return st;
-    CK(launch_count(*j.m, *j.fb, j.tiles_x, j.tiles_y, j.W, j.H, false, s));
-    return job_phase2_scan(j, s);
+    CK(launch_count(*j.fb, j.tiles_x, j.tiles_y, j.W, j.H, s));
+    return job_phase2_totals(j, s);
 }
 
-// After phase 2 has completed: device error bits, totals, limits, fragment buffers.
-// Device memory of a context's frame buffers, with fragment arrays of `frags` records.
+// Device memory of a context's frame buffers, with the lists of `frags`
+// fragments (24 bytes each: key and colour). The drawing pass does not store
+// the lists; they count towards the budget all the same, so that what fits a
+// budget does not depend on whether they are asked for (hexfc_debug_pixels).
+constexpr uint64_t kFragBytes = sizeof(uint64_t) + sizeof(float4);
 uint64_t frame_bytes(const FrameBufs& f, int64_t frags)
 {
     uint64_t b = 0;
@@ -627,17 +656,30 @@ uint64_t frame_bytes(const FrameBufs& f, int64_t frags)
     b += (uint64_t)f.f_cap * (sizeof(FaceFrame) + 2 * sizeof(uint32_t));
     b += (uint64_t)f.t_cap * (9 * sizeof(uint32_t) + sizeof(uint64_t) + sizeof(uint32_t));
     b += (uint64_t)f.bin_cap * 2 * sizeof(uint32_t) + (uint64_t)f.mask_cap * sizeof(uint32_t) +
-         (uint64_t)f.seg_cap * sizeof(uint64_t);
-    b += (uint64_t)f.p_cap * (4 * sizeof(uint32_t) + sizeof(uint64_t));
+         (uint64_t)f.zsuf_cap * sizeof(uint32_t);
+    b += (uint64_t)f.p_cap * (3 * sizeof(uint32_t));
     b += (uint64_t)f.part_cap * (sizeof(uint64_t) + sizeof(uint32_t));
-    b += (uint64_t)frags * (sizeof(uint64_t) + sizeof(float4));
+    b += (uint64_t)frags * kFragBytes;
     return b;
 }
 
+// The most fragments the frame may have (what job_read2 refuses, the drawing
+// pass does not draw), and whether it may be drawn at all.
+bool job_limit(const FrameJob& j, uint64_t& limit)
+{
+    const FrameBufs& fb = *j.fb;
+    limit = ~0ull;
+    if (!j.budget) return true;
+    const uint64_t base = frame_bytes(fb, 0);
+    const bool room = base <= j.budget;
+    limit = std::max<uint64_t>(room ? (j.budget - base) / kFragBytes : 0, (uint64_t)fb.frag_cap);
+    return room || fb.frag_sized;
+}
+
+// After phase 2 has completed: device error bits, totals, limits.
 hexfc_status job_read2(FrameJob& j, cudaStream_t s)
 {
     FrameBufs& fb = *j.fb;
-    hexfc_status st;
     if (fb.h_scal[5] != 0) {  // a bounded device wait ran out, or an exactness check failed
         const uint64_t bits = fb.h_scal[5];
         CK(cudaMemsetAsync(fb.scal + 5, 0, sizeof(uint64_t), s));
@@ -656,114 +698,78 @@ hexfc_status job_read2(FrameJob& j, cudaStream_t s)
     fs.height = (uint32_t)j.H;
     fs.kernel_launches = j.launches;
     if (j.max_list > HEXFC_MAX_LIST) return HEXFC_ERR_OVERFLOW;
-    if (!fb.key || fb.frag_cap < (int64_t)j.total) {
-        // the fragment arrays must grow: with a budget, the frame's buffers once
-        // they hold it must fit (refused before anything grows), and their
-        // headroom is what the budget leaves
+    if (!fb.frag_sized || fb.frag_cap < (int64_t)j.total) {
+        // the lists' room must grow: with a budget, the frame's buffers once they
+        // hold it must fit (refused before anything grows), and their headroom is
+        // what the budget leaves
         int64_t want = (int64_t)j.total + (int64_t)j.total / 4 + 1024;
         if (j.budget) {
-            const uint64_t per = sizeof(uint64_t) + sizeof(float4);
             const uint64_t base = frame_bytes(fb, 0);
-            if (base + j.total * per > j.budget) return HEXFC_ERR_OOM;
-            want = std::min<int64_t>(want, (int64_t)((j.budget - base) / per));
+            if (base + j.total * kFragBytes > j.budget) return HEXFC_ERR_OOM;
+            want = std::min<int64_t>(want, (int64_t)((j.budget - base) / kFragBytes));
         }
-        dfree(fb.key);
-        dfree(fb.rgba);
-        fb.frag_cap = 0;
-        if ((st = dalloc(&fb.key, (size_t)want)) != HEXFC_OK) return st;
-        if ((st = dalloc(&fb.rgba, (size_t)want)) != HEXFC_OK) return st;
         fb.frag_cap = want;
+        fb.frag_sized = true;
     }
     return HEXFC_OK;
 }
 
-// With silhouettes: the depth image of the boundary surface starts empty.
-hexfc_status job_sil_clear(const FrameJob& j, cudaStream_t s)
-{
-    if (j.sil_alpha > 0.f) CK(cudaMemsetAsync(j.fb->zsil, 0xFF, sizeof(uint32_t) * (size_t)j.n_pix, s));
-    return HEXFC_OK;
-}
-
-// After the composite: the white silhouettes over the output window.
+// After the drawing pass: the white silhouettes over the output window.
 hexfc_status job_silhouette(FrameJob& j, float* out, cudaStream_t s)
 {
     if (j.sil_alpha <= 0.f) return HEXFC_OK;
-    CK(launch_silhouette(*j.fb, j.tiles_x, j.cam.ox, j.cam.oy, j.frame_w, j.frame_h, j.sil_alpha, j.sil_threshold,
-                         out, j.win, s));
-    j.launches += 2;
+    CK(launch_silhouette(j.fb->zsil, j.tiles_x, j.cam.ox, j.cam.oy, j.frame_w, j.frame_h, j.sil_alpha,
+                         j.sil_threshold, out, j.win, s));
+    j.launches += 1;
     return HEXFC_OK;
 }
 
-hexfc_status job_phase3(FrameJob& j, cudaStream_t s)
-{
-    FrameBufs& fb = *j.fb;
-    job_mark(j, 8, s);
-    hexfc_status st;
-    if ((st = job_sil_clear(j, s)) != HEXFC_OK) return st;
-    CK(launch_fill(*j.m, fb, j.sp, j.tiles_x, j.tiles_y, j.W, j.H, false, j.sil_alpha > 0.f, s));
-    job_mark(j, 9, s);
-    CK(launch_composite(fb, j.sp, j.tiles_x, j.tiles_y, j.W, j.H, j.out, j.n_long, j.window, j.win, s));
-    if ((st = job_silhouette(j, j.out, s)) != HEXFC_OK) return st;
-    job_mark(j, 10, s);
-    j.launches += 3 + (j.n_long > 0 ? 1 : 0);
-    j.fs.kernel_launches = j.launches;
-    return HEXFC_OK;
-}
-
-// A frame's entries in the batched count, fill and main resolve launches.
-CountItem count_item(const FrameJob& j)
+// What the drawing pass needs of a frame.
+DrawItem draw_item(const FrameJob& j, uint64_t limit)
 {
     const FrameBufs& fb = *j.fb;
-    return CountItem{fb.tile_off, fb.bins, fb.fframe, fb.tile_order, fb.cnt, fb.masks, fb.tile_frag,
-                     j.tiles_x,   j.W,     j.H};
-}
-
-FillItem fill_item(const FrameJob& j)
-{
-    const FrameBufs& fb = *j.fb;
-    FillItem it{};
+    DrawItem it{};
     it.tile_off = fb.tile_off;
     it.bins = fb.bins;
     it.masks = fb.masks;
+    it.zsuf = fb.zsuf;
     it.fframe = fb.fframe;
-    it.fstat = j.m->fstat;
+    it.fstat = j.m->fstat.get();
     it.order = fb.tile_order;
-    it.off = fb.off;
     it.cnt = fb.cnt;
-    it.key = fb.key;
-    it.rgba = fb.rgba;
-    it.seg = fb.seg;
-    it.err = reinterpret_cast<unsigned long long*>(fb.scal + 5);
     it.zsil = j.sil_alpha > 0.f ? fb.zsil : nullptr;
-    it.sp = j.sp;
-    it.tiles_x = j.tiles_x;
-    it.W = j.W;
-    it.H = j.H;
-    return it;
-}
-
-CompositeItem composite_item(const FrameJob& j)
-{
-    const FrameBufs& fb = *j.fb;
-    CompositeItem it{};
-    it.cnt = fb.cnt;
-    it.seg = fb.seg;
-    it.tile_off = fb.tile_off;
-    it.masks = fb.masks;
-    it.key = fb.key;
-    it.rgba = fb.rgba;
     it.out = reinterpret_cast<float4*>(j.out);
-    it.long_q = fb.long_q;
-    it.long_cursor = reinterpret_cast<unsigned long long*>(fb.scal + 3);
-    it.fix_q = fb.fix_q;
-    it.fix_cursor = reinterpret_cast<unsigned long long*>(fb.scal + 4);
-    it.frag_cap = (uint64_t)fb.frag_cap;
-    for (int c = 0; c < 3; ++c) it.bg[c] = j.sp.bg[c];
+    it.redo = fb.redo;
+    unsigned long long* scal = reinterpret_cast<unsigned long long*>(fb.scal);
+    it.redo_cursor = scal + 3;
+    it.scal = scal;
+    it.err = scal + 5;
+    it.limit = limit;
+    it.sp = j.sp;
     it.win = j.win;
     it.tiles_x = j.tiles_x;
     it.W = j.W;
     it.H = j.H;
     return it;
+}
+
+hexfc_status job_phase3(FrameJob& j, cudaStream_t s)
+{
+    job_mark(j, 8, s);
+    hexfc_status st;
+    uint64_t limit;
+    if (job_limit(j, limit)) {
+        const DrawItem it = draw_item(j, limit);
+        CK(launch_draw(it, j.n_tiles, j.window, s));
+        job_mark(j, 9, s);
+        CK(launch_draw_tail(it, s));
+        j.launches += 2;
+        if ((st = job_silhouette(j, j.out, s)) != HEXFC_OK) return st;
+    } else {
+        job_mark(j, 9, s);
+    }
+    job_mark(j, 10, s);
+    return HEXFC_OK;
 }
 
 // One batched launch per group of at most kBatchLaunchMax frames: `add` puts
@@ -806,11 +812,28 @@ hexfc_status inject_error_bits(hexfc_ctx* ctx, uint64_t* scal, cudaStream_t s)
     return HEXFC_OK;
 }
 
-// Bins, counts, scan, fill and composite of one frame (everything but the output copy).
+// What the context keeps of the frame just drawn: its lists' inputs, the exact
+// tile counts that k_count left in fb.tile_frag, its features and camera.
+void keep_frame(hexfc_ctx* ctx, const FrameJob& j)
+{
+    ctx->have_frame = true;
+    ctx->last_draw = draw_item(j, ~0ull);
+    for (const auto& m : ctx->meshes)
+        if (m.get() == j.m) ctx->last_mesh = m;
+    ctx->last_fstat = j.m->fstat;
+    ctx->last_win = j.win;
+    ctx->counts_W = j.W;
+    ctx->counts_H = j.H;
+    ctx->feat_tiles = j.n_tiles;
+    remember_camera(ctx, j.cam);
+}
+
+// One frame (everything but the output copy).
 hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_stats* stats, cudaStream_t s)
 {
     FrameJob j = make_job(ctx, &ctx->fb, m, out);
     hexfc_status st;
+    ctx->have_frame = false;   // the frame buffers are this frame's from here on
     if ((st = job_alloc(j)) != HEXFC_OK) return st;
     if (ctx->timing && !ctx->ev[0][0])
         for (auto& set : ctx->ev)
@@ -832,30 +855,20 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
     }
     if ((st = job_read1(j)) != HEXFC_OK) return st;
     if ((st = job_phase2(j, s)) != HEXFC_OK) return st;
-    CK(cudaStreamSynchronize(s));
-    ctx->have_frame = false;
+    if (!ctx->ev_p2) CK(cudaEventCreateWithFlags(&ctx->ev_p2, cudaEventDisableTiming));
+    CK(cudaEventRecord(ctx->ev_p2, s));
+    if ((st = job_phase3(j, s)) != HEXFC_OK) return st;
+    CK(cudaEventSynchronize(ctx->ev_p2));   // the totals, while the frame is drawn
     st = job_read2(j, s);
     j.fs.frame = ++ctx->frame_seq;
     ctx->last = j.fs;
     if (stats) *stats = j.fs;
     if (st != HEXFC_OK) return st;
     record_final(ctx, j.fs);
-    if ((st = job_phase3(j, s)) != HEXFC_OK) return st;
     if ((st = inject_error_bits(ctx, fb_of(j), s)) != HEXFC_OK) return st;
     ctx->ev_pending[ctx->ev_cur] = ctx->timing;
-    ctx->last.kernel_launches = j.launches;
-    if (stats) stats->kernel_launches = j.launches;
-    ctx->have_frame = true;
-    ctx->last_W = j.W;
-    ctx->last_win = j.win;
-    ctx->last_H = j.H;
-    ctx->last_tiles_x = j.tiles_x;
-    ctx->last_tiles_y = j.tiles_y;
-    ctx->counts_W = j.W;   // k_count left the exact tile counts in fb.tile_frag
-    ctx->counts_H = j.H;
+    keep_frame(ctx, j);
     ctx->counts_total = j.total;
-    ctx->feat_tiles = j.n_tiles;
-    remember_camera(ctx, j.cam);
     return HEXFC_OK;
 }
 
@@ -863,13 +876,11 @@ constexpr float kCapMargin = 0.15f;   // capacity = predicted count * (1 + margi
 constexpr uint32_t kCapPad = 256;
 constexpr double kCapPool = 0.35;        // pool after the regions, in previous-frame fragments
 constexpr uint64_t kErrPoolBit = 16;     // device error bit: no room for a tile's lists in the pool
-constexpr uint32_t kLongListsUnknown = 1u << 30;   // the long-list pass reads the queue length on the device
 
 // A frame with chosen tile capacities: capacities from the previous frame's
-// exact tile counts or from the capacity network, the count pass, then the fill
-// lays out each tile's lists in the tile's region (or the pool) itself, so
-// there is no pixel scan and no host wait after the count; and the call does
-// not wait at the end either. The frame is verified by the next call on the
+// exact tile counts or from the capacity network, the count pass, and its exact
+// counts against the capacities on the device, so there is no host wait after
+// the count. The frame is verified by the next call on the
 // context, at that call's first host wait (it has completed by then), or by
 // hexfc_finish: if its capacities ran out, it is drawn again exactly by
 // count-then-fill into its own output, before anything else.
@@ -886,6 +897,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     FrameJob j = make_job(ctx, &ctx->fb, m, out);
     FrameBufs& fb = ctx->fb;
     hexfc_status st;
+    ctx->have_frame = false;
     if ((st = job_alloc(j)) != HEXFC_OK) return st;
     if (!fb.tile_cap || fb.cap_cap < fb.t_cap) {   // capacity arrays follow the tile arrays
         int64_t c1 = 0;
@@ -893,8 +905,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
         if ((st = ensure(&fb.tile_cap, &fb.cap_cap, fb.t_cap)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.cap_off, &c1, fb.cap_cap)) != HEXFC_OK) return st;
     }
-    if (!fb.cstat && (st = dalloc(&fb.cstat, 4 * kStatCopies)) != HEXFC_OK) return st;
-    if (!ctx->h_pend) CK(cudaMallocHost((void**)&ctx->h_pend, (kScal + 4 * kStatCopies) * sizeof(uint64_t)));
+    if (!ctx->h_pend) CK(cudaMallocHost((void**)&ctx->h_pend, kScal * sizeof(uint64_t)));
     if (ctx->timing && !ctx->ev[0][0])
         for (auto& set : ctx->ev)
             for (auto& e : set) CK(cudaEventCreate(&e));
@@ -916,26 +927,18 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
         }
     }
     if ((st = job_read1(j)) != HEXFC_OK) return st;
-    // fragment arrays for the regions of this frame (previous counts * margin + pad) and a pool
-    // after them for the tiles above their capacity
-    // (the previous frame's fragment total, now verified, scaled to this frame's pixels)
+    // room for the regions of this frame (previous counts * margin + pad) and a
+    // pool after them for the tiles above their capacity (the previous frame's
+    // fragment total, now verified, scaled to this frame's pixels)
     const double prev_total = (double)ctx->counts_total * ((double)j.W * j.H) /
                               ((double)ctx->counts_W * (double)ctx->counts_H);
     const uint64_t want = (uint64_t)(prev_total * (1.0 + kCapMargin + kCapPool)) + (uint64_t)j.n_tiles * kCapPad;
-    if (!fb.key || fb.frag_cap < (int64_t)want) {
-        int64_t c1 = 0;
-        dfree(fb.rgba);
-        if ((st = ensure(&fb.key, &fb.frag_cap, (int64_t)want)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.rgba, &c1, fb.frag_cap)) != HEXFC_OK) return st;
+    if (!fb.frag_sized || fb.frag_cap < (int64_t)want) {
+        fb.frag_cap = (int64_t)(want + want / 4 + 1024);
+        fb.frag_sized = true;
     }
-    job_mark(j, 4, s);
-    CK(cudaMemsetAsync(fb.bins, 0xFF, sizeof(uint32_t) * (size_t)j.n_bins, s));   // padding slots = kPadBin
-    CK(launch_bin_fill(*m, fb, j.tiles_x, j.W, j.H, j.reverse, s));
-    CK(launch_bin_sort(*m, fb, j.tiles_x, j.tiles_y, j.buckets, s));
-    if (!j.order_done) CK(launch_tile_order(fb, j.n_tiles, s));
-    if ((st = job_features(j, s)) != HEXFC_OK) return st;
-    // stages: bin (with the features, the capacities and their scan), count,
-    // then no pixel scan and no host wait, fill, composite
+    if ((st = job_phase2_bins(j, s)) != HEXFC_OK) return st;
+    // (stages: the capacities and their scan belong to the binning)
     if (ctx->predicted == 2) {
         CK(launch_cap_forward(ctx->cap, fb, j.n_tiles, kCapMargin, kCapPad, s));
     } else {   // previous-frame counts, or (mode 3) the previous total spread evenly over the tiles
@@ -944,23 +947,21 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
         CK(launch_capacity_from_previous(fb, j.n_tiles, kCapMargin, kCapPad, uniform, s));
     }
     CK(scan_u32_to_u64(fb.tile_cap, fb.cap_off, j.n_tiles, fb.part, fb.part_max, fb.scal + 11, 0xFFFFFFFFu, s));
-    CK(cudaMemsetAsync(fb.cstat, 0, sizeof(uint64_t) * 4 * kStatCopies, s));
     job_mark(j, 5, s);
-    CK(launch_count(*m, fb, j.tiles_x, j.tiles_y, j.W, j.H, true, s));
+    CK(launch_count(fb, j.tiles_x, j.tiles_y, j.W, j.H, s));
     job_mark(j, 6, s);
+    CK(launch_capacity_check(fb, j.n_tiles, s));
     job_mark(j, 7, s);
     job_mark(j, 8, s);
-    if ((st = job_sil_clear(j, s)) != HEXFC_OK) return st;
-    CK(launch_fill(*m, fb, j.sp, j.tiles_x, j.tiles_y, j.W, j.H, true, j.sil_alpha > 0.f, s));
+    const DrawItem it = draw_item(j, ~0ull);
+    CK(launch_draw(it, j.n_tiles, j.window, s));
     job_mark(j, 9, s);
-    CK(launch_composite(fb, j.sp, j.tiles_x, j.tiles_y, j.W, j.H, out, kLongListsUnknown, j.window, j.win, s));
+    CK(launch_draw_tail(it, s));
     if ((st = job_silhouette(j, out, s)) != HEXFC_OK) return st;
     job_mark(j, 10, s);
-    j.launches += (j.order_done ? 3 : 4) + 1 + 3 + 1 + 1 + 3;   // (the tile order counted by phase 1)
-    // the frame's scalars and count statistics for its verification; no wait here
+    j.launches += 1 + 3 + 1 + 1 + 2;   // capacities, their scan, count, check, drawing passes
+    // the frame's scalars for its verification; no wait here
     CK(cudaMemcpyAsync(ctx->h_pend, fb.scal, kScal * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(ctx->h_pend + kScal, fb.cstat, 4 * kStatCopies * sizeof(uint64_t), cudaMemcpyDeviceToHost,
-                       s));
     ctx->ev_pending[ctx->ev_cur] = ctx->timing;
     hexfc_frame_stats& fs = j.fs;
     fs = hexfc_frame_stats{};
@@ -986,16 +987,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     p.fs = fs;
     ctx->last = fs;
     if (stats) *stats = fs;
-    ctx->have_frame = true;
-    ctx->last_W = j.W;
-    ctx->last_win = j.win;
-    ctx->last_H = j.H;
-    ctx->last_tiles_x = j.tiles_x;
-    ctx->last_tiles_y = j.tiles_y;
-    ctx->counts_W = j.W;   // k_count leaves the exact tile counts in fb.tile_frag
-    ctx->counts_H = j.H;
-    ctx->feat_tiles = j.n_tiles;
-    remember_camera(ctx, j.cam);
+    keep_frame(ctx, j);
     return HEXFC_OK;
 }
 
@@ -1019,15 +1011,9 @@ hexfc_status settle_pending(hexfc_ctx* ctx, cudaStream_t s, bool* redrawn)
     fs.pending = 0;
     fs.overflow_tiles = (uint32_t)h[6];
     fs.capacity = h[11];
-    fs.fragments = 0;   // from the count pass (no pixel scan): the sums over its counter copies
-    fs.max_list = 0;
-    fs.long_lists = 0;
-    for (int c = 0; c < kStatCopies; ++c) {
-        const uint64_t* cs = h + kScal + 4 * c;
-        fs.fragments += cs[0];
-        fs.max_list = std::max(fs.max_list, (uint32_t)cs[1]);
-        fs.long_lists += (uint32_t)cs[2];
-    }
+    fs.fragments = h[0];
+    fs.max_list = (uint32_t)h[1];
+    fs.long_lists = (uint32_t)h[2];
     if (bits) CK(cudaMemsetAsync(ctx->fb.scal + 5, 0, sizeof(uint64_t), s));
     if (bits & ~kErrPoolBit) {   // a bounded wait ran out or a check failed
         record_final(ctx, fs);
@@ -1240,8 +1226,7 @@ hexfc_status hexfc_create(hexfc_ctx** out, int device, uint64_t frag_budget_byte
     c->lens.radius = 1.0;
     {
         DeviceGuard g(device);
-        if (prepare_raster_kernels() != cudaSuccess || prepare_fill_kernels() != cudaSuccess ||
-            prepare_composite_kernels() != cudaSuccess) {
+        if (prepare_raster_kernels() != cudaSuccess || prepare_draw_kernels() != cudaSuccess) {
             (void)cudaGetLastError();
             delete c;
             return HEXFC_ERR_CUDA;
@@ -1260,6 +1245,8 @@ void hexfc_destroy(hexfc_ctx* ctx)
     ctx->pend.mesh.reset();
     if (ctx->h_pend) cudaFreeHost(ctx->h_pend);
     ctx->h_pend = nullptr;
+    ctx->last_fstat.reset();
+    ctx->last_mesh.reset();
     ctx->meshes.clear();   // a mesh is freed with its last holder
     free_frame(ctx->fb);
     for (auto& b : ctx->batch) {
@@ -1278,6 +1265,7 @@ void hexfc_destroy(hexfc_ctx* ctx)
     if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
     if (ctx->ev_out) cudaEventDestroy(ctx->ev_out);
     if (ctx->ev_p1) cudaEventDestroy(ctx->ev_p1);
+    if (ctx->ev_p2) cudaEventDestroy(ctx->ev_p2);
     dfree(ctx->d_out);
     for (auto& set : ctx->ev)
         for (auto& e : set)
@@ -1315,7 +1303,8 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
     A(dalloc(&m->elevel, (size_t)t.n_edges));
     A(dalloc(&m->fverts, (size_t)t.n_faces));
     A(dalloc(&m->fedges, (size_t)t.n_faces));
-    A(dalloc(&m->fstat, (size_t)t.n_faces));
+    bool fresh = false;
+    A(own_fstat(*m, &fresh));
     A(dalloc(&m->fbound, (size_t)t.n_faces));
     if (st != HEXFC_OK) {
         free_mesh(m);
@@ -1393,8 +1382,6 @@ hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_ite
         j.m = get_mesh(ctx, it.mesh);
         j.cam = cams[(size_t)i];
         j.sp = make_shade_params(it.lens, it.style, zrefs[(size_t)i], j.cam.ortho);
-        j.lod = it.style.lod;
-        j.delta = it.style.delta;
         j.W = it.view.width;
         j.H = it.view.height;
         j.tiles_x = (j.W + kTileW - 1) / kTileW;
@@ -1433,7 +1420,7 @@ hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_ite
             b, live,
             [&](CountBatch& cb, int i) {
                 const FrameJob& j = jobs[(size_t)i];
-                cb.it[cb.n] = count_item(j);
+                cb.it[cb.n] = count_item(*j.fb, j.tiles_x, j.tiles_y, j.W, j.H);
                 cb.tile_begin[cb.n + 1] = cb.tile_begin[cb.n] + (uint32_t)j.n_tiles;
                 ++cb.n;
             },
@@ -1442,67 +1429,53 @@ hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_ite
     const bool one = ctx->batch_launch;
     if (one && (st = batch_graph(
                     ctx, 1, live, [&](int i, cudaStream_t si) { return job_phase2_bins(jobs[(size_t)i], si); },
-                    count_all, [&](int i, cudaStream_t si) { return job_phase2_scan(jobs[(size_t)i], si); }, true)) !=
+                    count_all, [&](int i, cudaStream_t si) { return job_phase2_totals(jobs[(size_t)i], si); }, true)) !=
                    HEXFC_OK)
         return st;
     if (!one && (st = batch_graph(
                      ctx, 1, live, [&](int i, cudaStream_t si) { return job_phase2(jobs[(size_t)i], si); }, no_mid,
                      none, false)) != HEXFC_OK)
         return st;
-    CK(cudaStreamSynchronize(ctx->origin));
+    if (!ctx->ev_p2) CK(cudaEventCreateWithFlags(&ctx->ev_p2, cudaEventDisableTiming));
+    CK(cudaEventRecord(ctx->ev_p2, ctx->origin));
     std::vector<int> draw, draw_sil, draw_plain;
+    std::vector<uint64_t> limits((size_t)n, ~0ull);
     for (int i : live) {
-        res[(size_t)i] = job_read2(jobs[(size_t)i], ctx->batch[(size_t)i]->stream);
-        if (res[(size_t)i] != HEXFC_OK) continue;
+        if (!job_limit(jobs[(size_t)i], limits[(size_t)i])) continue;
         draw.push_back(i);
         (jobs[(size_t)i].sil_alpha > 0.f ? draw_sil : draw_plain).push_back(i);
     }
-    // the fill of every frame in one launch (one per fill variant), then the
-    // main resolve pass of every frame in one launch
-    auto fill_composite_all = [&](cudaStream_t o) -> hexfc_status {
+    // the drawing pass of every frame in one launch (one per variant)
+    auto draw_all = [&](cudaStream_t o) -> hexfc_status {
         hexfc_status r = HEXFC_OK;
         for (int variant = 0; variant < 2 && r == HEXFC_OK; ++variant) {
-            FillBatch b;
+            DrawBatch b;
             r = batched(
                 b, variant ? draw_sil : draw_plain,
-                [&](FillBatch& fbt, int i) {
+                [&](DrawBatch& db, int i) {
                     const FrameJob& j = jobs[(size_t)i];
-                    fbt.it[fbt.n] = fill_item(j);
-                    fbt.tile_begin[fbt.n + 1] = fbt.tile_begin[fbt.n] + (uint32_t)j.n_tiles;
-                    ++fbt.n;
+                    db.it[db.n] = draw_item(j, limits[(size_t)i]);
+                    db.tile_begin[db.n + 1] = db.tile_begin[db.n] + (uint32_t)j.n_tiles;
+                    ++db.n;
                 },
-                [&](FillBatch& fbt) { return launch_fill_batch(fbt, variant == 1, o); });
+                [&](DrawBatch& db) { return launch_draw_batch(db, variant == 1, ctx->window, o); });
         }
-        if (r != HEXFC_OK) return r;
-        CompositeBatch cb;
-        return batched(
-            cb, draw,
-            [&](CompositeBatch& c, int i) {
-                const FrameJob& j = jobs[(size_t)i];
-                c.it[c.n] = composite_item(j);
-                c.tile_begin[c.n + 1] = c.tile_begin[c.n] + (uint32_t)j.n_tiles;
-                ++c.n;
-            },
-            [&](CompositeBatch& c) { return launch_composite_batch(c, ctx->window, o); });
-    };
-    auto tail = [&](int i, cudaStream_t si) -> hexfc_status {   // short lists past the window, long lists, silhouettes
-        FrameJob& j = jobs[(size_t)i];
-        CK(launch_composite_tail(*j.fb, j.sp, j.tiles_x, j.out, j.n_long, j.win, si));
-        hexfc_status r = job_silhouette(j, j.out, si);
-        j.launches += 3 + (j.n_long > 0 ? 1 : 0);
-        j.fs.kernel_launches = j.launches;
         return r;
     };
-    if (one && !draw.empty() &&
-        (st = batch_graph(
-             ctx, 2, draw, [&](int i, cudaStream_t si) { return job_sil_clear(jobs[(size_t)i], si); },
-             fill_composite_all, tail, true)) != HEXFC_OK)
-        return st;
+    auto tail = [&](int i, cudaStream_t si) -> hexfc_status {   // pixels out of order, silhouettes
+        FrameJob& j = jobs[(size_t)i];
+        CK(launch_draw_tail(draw_item(j, limits[(size_t)i]), si));
+        j.launches += 2;
+        return job_silhouette(j, j.out, si);
+    };
+    if (one && !draw.empty() && (st = batch_graph(ctx, 2, draw, none, draw_all, tail, true)) != HEXFC_OK) return st;
     if (!one && !draw.empty() &&
         (st = batch_graph(
              ctx, 2, draw, [&](int i, cudaStream_t si) { return job_phase3(jobs[(size_t)i], si); }, no_mid, none,
              false)) != HEXFC_OK)
         return st;
+    CK(cudaEventSynchronize(ctx->ev_p2));   // the totals, while the frames are drawn
+    for (int i : live) res[(size_t)i] = job_read2(jobs[(size_t)i], ctx->origin);
     // the caller's stream continues after the batch
     CK(cudaEventRecord(ctx->ev_out, ctx->origin));
     CK(cudaStreamWaitEvent(s, ctx->ev_out, 0));
@@ -1601,16 +1574,7 @@ hexfc_status hexfc_frame_memory(const hexfc_ctx* ctx, uint64_t* bytes)
     if (!ctx || !bytes) return HEXFC_ERR_ARG;
     uint64_t b = frame_bytes(ctx->fb, ctx->fb.frag_cap);
     b += (uint64_t)ctx->d_out_cap * sizeof(float);
-    for (const auto& bs : ctx->batch) {
-        const FrameBufs& g = bs->fb;
-        b += (uint64_t)g.v_cap * (sizeof(int4) + sizeof(float)) +
-             (uint64_t)g.f_cap * (sizeof(FaceFrame) + 2 * sizeof(uint32_t)) +
-             (uint64_t)g.t_cap * (9 * sizeof(uint32_t) + sizeof(uint64_t) + sizeof(uint32_t)) +
-             (uint64_t)(2 * g.bin_cap + g.mask_cap) * sizeof(uint32_t) + (uint64_t)g.seg_cap * sizeof(uint64_t) +
-             (uint64_t)g.p_cap * (3 * sizeof(uint32_t) + sizeof(uint64_t)) +
-             (uint64_t)g.part_cap * (sizeof(uint64_t) + sizeof(uint32_t)) +
-             (uint64_t)g.frag_cap * (sizeof(uint64_t) + sizeof(float4));
-    }
+    for (const auto& bs : ctx->batch) b += frame_bytes(bs->fb, bs->fb.frag_cap);
     *bytes = b;
     return HEXFC_OK;
 }
@@ -1636,6 +1600,8 @@ hexfc_status hexfc_trim(hexfc_ctx* ctx)
     dfree(ctx->d_out);
     ctx->d_out_cap = 0;
     ctx->have_frame = false;
+    ctx->last_fstat.reset();
+    ctx->last_mesh.reset();
     return HEXFC_OK;
 }
 
@@ -1669,8 +1635,18 @@ hexfc_status hexfc_set_cell_importance(hexfc_ctx* ctx, int32_t mesh, const float
     if (!m) return HEXFC_ERR_STATE;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
+    // (a captured update writes the current records in place: nothing may be
+    // allocated, and every replay has to write what the renders read)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        (void)cudaGetLastError();
+        cap = cudaStreamCaptureStatusActive;
+    }
+    bool fresh = false;
+    if (cap == cudaStreamCaptureStatusNone)
+        if (const hexfc_status st = own_fstat(*m, &fresh); st != HEXFC_OK) return st;
     CK(cudaMemcpyAsync(m->cell_imp, cell_importance, sizeof(float) * (size_t)m->n_cells, cudaMemcpyDeviceToDevice, s));
-    CK(launch_importance(*m, false, s));   // positions unchanged since the upload
+    CK(launch_importance(*m, fresh, s));   // positions unchanged since the upload
     return HEXFC_OK;
 }
 
@@ -1845,8 +1821,7 @@ hexfc_status hexfc_debug_pixels(hexfc_ctx* ctx, const int32_t* px, const int32_t
     cudaError_t e = cudaMemcpy(d_px, px, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(d_py, py, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = launch_debug_gather(fb, d_px, d_py, n, nullptr, ctx->last_tiles_x, ctx->last_W, ctx->last_H, nullptr,
-                                nullptr, d_cnt, 0);
+        e = launch_debug_gather(ctx->last_draw, d_px, d_py, n, nullptr, nullptr, nullptr, d_cnt, 0);
     if (e == cudaSuccess) e = cudaMemcpy(counts, d_cnt, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) {
         note_cuda(e);
@@ -1873,8 +1848,7 @@ hexfc_status hexfc_debug_pixels(hexfc_ctx* ctx, const int32_t* px, const int32_t
     }
     e = cudaMemcpy(d_off, hoff.data(), sizeof(uint64_t) * (size_t)n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = launch_debug_gather(fb, d_px, d_py, n, d_off, ctx->last_tiles_x, ctx->last_W, ctx->last_H, d_keys, d_rgba,
-                                nullptr, 0);
+        e = launch_debug_gather(ctx->last_draw, d_px, d_py, n, d_off, d_keys, d_rgba, nullptr, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess && keys) e = cudaMemcpy(keys, d_keys, sizeof(uint64_t) * total, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess && rgba) e = cudaMemcpy(rgba, d_rgba, sizeof(float4) * total, cudaMemcpyDeviceToHost);
@@ -2045,12 +2019,12 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     const int tiles_x = (W + kTileW - 1) / kTileW, tiles_y = (H + kTileH - 1) / kTileH;
     const int64_t n_tiles = (int64_t)tiles_x * tiles_y;
     const int64_t n_pix = n_tiles * kTilePix;
-    const int64_t nparts = scan_partials_needed(std::max<int64_t>(n_pix, n_tiles)) + 1;
+    const int64_t nparts = scan_partials_needed(n_tiles) + 1;
     Arena a{scratch, 0, (size_t)HEXFC_NOALLOC_SCRATCH_BYTES};
     FrameBufs fb;
     // the device scalars first, at the same place in every call: slot 5, the
     // device error word, outlives the call (see below)
-    fb.scal = a.take<uint64_t>(kScal);
+    fb.scal = a.take<uint64_t>(kScalAll);
     fb.vproj = a.take<int4>((size_t)m->n_verts);
     fb.ved = a.take<float>((size_t)m->n_verts);
     fb.fframe = a.take<FaceFrame>((size_t)m->n_faces);
@@ -2062,14 +2036,12 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     fb.tile_frag = a.take<uint32_t>((size_t)n_tiles + 1);
     fb.tile_zr = a.take<float>((size_t)n_tiles + 1);
     fb.cnt = a.take<uint32_t>((size_t)n_pix + 1);
-    fb.off = a.take<uint64_t>((size_t)n_pix + 1);
-    fb.long_q = a.take<uint32_t>((size_t)n_pix + 1);
-    fb.fix_q = a.take<uint32_t>((size_t)n_pix + 1);
+    fb.redo = a.take<uint32_t>((size_t)n_pix + 1);
     fb.zsil = sil ? a.take<uint32_t>((size_t)n_pix) : nullptr;
     fb.part = a.take<uint64_t>(2 * (size_t)nparts);
     fb.part_max = a.take<uint32_t>(2 * (size_t)nparts);
     if (!fb.vproj || !fb.ved || !fb.fframe || !fb.tzsum || !fb.tile_cnt ||
-        !fb.tile_off || !fb.tile_cur || !fb.tile_order || !fb.tile_frag || !fb.tile_zr || !fb.cnt || !fb.off || !fb.long_q || !fb.fix_q || (sil && !fb.zsil) || !fb.part || !fb.part_max ||
+        !fb.tile_off || !fb.tile_cur || !fb.tile_order || !fb.tile_frag || !fb.tile_zr || !fb.cnt || !fb.redo || (sil && !fb.zsil) || !fb.part || !fb.part_max ||
         !fb.scal)
         return HEXFC_ERR_OVERFLOW;
     // the array keeps the previous call's contents: clear what must start at zero
@@ -2080,9 +2052,9 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     // call returned, and they are reported below, by this call (the array starts
     // zeroed when the module is loaded)
     CK(cudaMemsetAsync(fb.scal, 0, sizeof(uint64_t) * 5, s));
-    CK(cudaMemsetAsync(fb.scal + 6, 0, sizeof(uint64_t) * (kScal - 6), s));
+    CK(cudaMemsetAsync(fb.scal + 6, 0, sizeof(uint64_t) * (kScalAll - 6), s));
     CK(launch_vertex_setup(*m, ctx->cam, fb, s));
-    CK(launch_face_setup(*m, ctx->cam, ctx->style.lod, ctx->style.delta, fb, tiles_x, tiles_y, s));
+    CK(launch_face_setup(*m, ctx->cam, make_shade(ctx), fb, tiles_x, tiles_y, s));
     CK(scan_u32_to_u64(fb.tile_cnt, fb.tile_off, n_tiles, fb.part, fb.part_max, fb.scal + 8, 0xFFFFFFFFu, s,
                        (uint32_t)kChunk));
     uint64_t h[16] = {};  // pageable host copy of the totals (no pinned allocation)
@@ -2092,21 +2064,20 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     fb.bins = a.take<uint32_t>((size_t)n_bins);
     fb.bins_tmp = a.take<uint32_t>((size_t)n_bins);
     fb.masks = a.take<uint32_t>((size_t)n_bins * (kTilePix / kChunk));
-    fb.seg = a.take<uint64_t>((size_t)(n_bins / kChunk) * (kTilePix / 32));
+    fb.zsuf = a.take<uint32_t>((size_t)(n_bins / kChunk));
     hexfc_frame_stats fs{};
     fs.bin_entries = n_bins;
     fs.width = (uint32_t)win.w;
     fs.height = (uint32_t)win.h;
-    if (!fb.bins || !fb.bins_tmp || !fb.masks || !fb.seg) {
+    if (!fb.bins || !fb.bins_tmp || !fb.masks || !fb.zsuf) {
         if (stats) *stats = fs;
         return HEXFC_ERR_OVERFLOW;
     }
     CK(cudaMemsetAsync(fb.bins, 0xFF, sizeof(uint32_t) * (size_t)n_bins, s));   // padding slots = kPadBin
     CK(launch_bin_fill(*m, fb, tiles_x, W, H, ctx->reverse_bins, s));
-    CK(launch_bin_sort(*m, fb, tiles_x, tiles_y, ctx->depth_buckets, s));
+    CK(launch_bin_sort(*m, fb, tiles_x, tiles_y, (int64_t)n_bins, ctx->depth_buckets, s));
     CK(launch_tile_order(fb, n_tiles, s));
-    CK(launch_count(*m, fb, tiles_x, tiles_y, W, H, false, s));
-    CK(scan_u32_to_u64(fb.cnt, fb.off, n_pix, fb.part, fb.part_max, fb.scal, (uint32_t)kWarpSortMax, s));
+    CK(launch_count(fb, tiles_x, tiles_y, W, H, s));
     CK(cudaMemcpyAsync(h, fb.scal, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (h[5] != 0) {   // this call's count pass, or the previous call's fill or composite
@@ -2120,19 +2091,17 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     fs.fragments = total;
     fs.max_list = (uint32_t)h[1];
     fs.long_lists = n_long;
-    fs.kernel_launches = 15 + (n_long > 0 ? 1u : 0u) + (sil ? 2u : 0u);
+    fs.kernel_launches = 11 + (sil ? 1u : 0u);
     if (stats) *stats = fs;
     if (fs.max_list > HEXFC_MAX_LIST) return HEXFC_ERR_OVERFLOW;
-    fb.key = a.take<uint64_t>((size_t)total);
-    fb.rgba = a.take<float4>((size_t)total);
-    if (!fb.key || !fb.rgba) return HEXFC_ERR_OVERFLOW;
-    fb.frag_cap = (int64_t)total;
-    ShadeParams sp = make_shade(ctx);
-    if (sil) CK(cudaMemsetAsync(fb.zsil, 0xFF, sizeof(uint32_t) * (size_t)n_pix, s));
-    CK(launch_fill(*m, fb, sp, tiles_x, tiles_y, W, H, false, sil, s));
-    CK(launch_composite(fb, sp, tiles_x, tiles_y, W, H, out, n_long, ctx->window, win, s));
+    // (the lists must fit the array too, though the drawing pass does not store them)
+    if (!a.take<uint64_t>((size_t)total) || !a.take<float4>((size_t)total)) return HEXFC_ERR_OVERFLOW;
+    FrameJob j = make_job(ctx, &fb, m, out);
+    const DrawItem it = draw_item(j, ~0ull);
+    CK(launch_draw(it, n_tiles, ctx->window, s));
+    CK(launch_draw_tail(it, s));
     if (sil)
-        CK(launch_silhouette(fb, tiles_x, ctx->cam.ox, ctx->cam.oy, ctx->view.width, ctx->view.height,
+        CK(launch_silhouette(fb.zsil, tiles_x, ctx->cam.ox, ctx->cam.oy, ctx->view.width, ctx->view.height,
                              ctx->style.sil_alpha, ctx->style.sil_threshold, out, win, s));
     return inject_error_bits(ctx, fb.scal, s);
 }

@@ -1,12 +1,11 @@
-// The coverage count of one tile (warp-level), used by the count pass and
-// by the fused count-and-fill pass of predicted capacities.
+// The coverage count of one tile (warp-level).
 #pragma once
 #include "raster_tiles.cuh"
 
 namespace hexfc {
 
 // Per tile: coverage of every chunk of 32 triangles as per-pixel bit masks;
-// the masks are kept for the fill pass and their bit counts are the
+// the masks are kept for the drawing pass and their bit counts are the
 // per-pixel list lengths. Warp w takes chunks w, w + 8, ... of the tile's list
 // on its own: its 32 lanes stage the chunk's triangles, then take the
 // triangles' box rows (clipped to the tile) one per lane: a triangle covers

@@ -4,6 +4,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
+#include <vector>
+
 #include "hexfc.h"
 
 namespace hexfc {
@@ -15,7 +18,7 @@ constexpr int kTilePix = 256;                  // pixels (= threads) per tile CT
 constexpr int kTileW = HEXFC_TILE_W;           // raster tile width in pixels (a build-time choice)
 constexpr int kTileH = kTilePix / kTileW;      // raster tile height
 static_assert(kTileW == 8 || kTileW == 16 || kTileW == 32, "tiles of 8x32, 16x16 or 32x8 pixels");
-constexpr int kWarpSortMax = 256;         // longest list sorted in registers by one warp
+constexpr int kLongList = 256;             // lists longer than this are counted in the frame's statistics
 constexpr uint64_t kPadKey = ~0ull;
 constexpr int kChunk = 32;                // triangles per raster chunk (one coverage bit each)
 constexpr uint32_t kPadBin = 0xFFFFFFFFu; // empty slot: tile lists are padded to whole chunks
@@ -44,42 +47,51 @@ struct ShadeParams {
     int ortho;
     float accent_r2;   // (256 * 2/3 * w_base)^2: accentuation radius squared, 1/256-pixel units
     float desat;       // depth cue strength (0 = off)
+    bool bounded;      // every style and lens constant is finite and below 1e15: no product of a zero is NaN
     int px_off, py_off;   // drawn rectangle's offset in the frame: pixel (x, y) is frame pixel (x + px_off, ...)
 };
 
-// A face as two 64-byte records: the per-frame one (window corners, depths,
-// edge flags, eye depths), written by the face stage of every frame into the
-// rendering context's buffers, and the static one (corner importance and world
-// position), owned by the mesh and rewritten only when importance changes, so
-// that contexts can render one resident mesh at the same time.
-struct __align__(64) FaceFrame {
+// A face as two records: the per-frame one, written by the face stage of every
+// frame into the rendering context's buffers (with what a triangle's shading
+// record needs that does not depend on the tile, so that it is found once per
+// face and not for every tile the face touches), and the static one (corner
+// importance and world position), owned by the mesh and rewritten only when
+// importance changes, so that contexts can render one resident mesh at the
+// same time.
+struct __align__(32) FaceFrame {
     int4 X, Y;            // corner window position, 16.8 fixed point
-    uint4 Z;              // bits 0-23: corner window depth (z24); Z.x bits 24-31: edge flags
-                          // (bits 0-3 visible in focus, 4-7 visible in context); Z.y bits 24-25:
-                          // triangle 0 / 1 drawn, bit 26: a boundary face (of one cell)
-    float4 ed;            // corner eye depth
+    uint4 Z;              // bits 0-23: corner window depth (z24). Bits 24-31 of Z.x: edge flags (bits 0-3
+                          // visible in focus, 4-7 visible in context); of Z.y: face flags (kFace...)
+    float4 q;             // 1 / corner eye depth (1 in an orthographic view)
+    float4 nl;            // -1 / squared length of window edge k -> k+1 (0: degenerate)
+    uint4 area;           // triangle 0, 1: twice the area if below 2^26, else 0; 1 / the same (float bits)
 };
 struct __align__(64) FaceStatic {
     float4 imp;           // corner importance
     float4 px, py, pz;    // corner world position
 };
-static_assert(sizeof(FaceFrame) == 64 && sizeof(FaceStatic) == 64, "two sectors each");
+static_assert(sizeof(FaceFrame) == 96 && sizeof(FaceStatic) == 64, "whole 32-byte sectors");
 constexpr uint32_t kZ24 = 0xFFFFFFu;
+// Face flags, bit t for triangle t where shifted by it.
+constexpr uint32_t kFaceDrawn = 1u;      // << t: triangle drawn
+constexpr uint32_t kFaceBoundary = 4u;   // a face of one cell
+constexpr uint32_t kFaceSwapped = 8u;    // << t: vertices 1 and 2 swapped to wind it to positive area
+constexpr uint32_t kFaceOut = 32u;       // << t: wholly outside the sphere lens
 
-// Device scalars of a frame (FrameBufs::scal): 0-2 pixel scan (fragments,
-// longest list, lists above the warp sort), 3-4 resolve queue cursors (long,
-// out of order), 5 device error bits (kept across frames), 6 tiles above
-// their chosen capacity, 8-10 tile scan (bin entries, ...), 11-13 capacity
-// scan (regions' total, ...), 14 records taken from the pool, 16-18 count
-// pass statistics (fragments, longest list, lists above the warp sort).
+// Device scalars of a frame (FrameBufs::scal): 0-2 count pass (fragments,
+// longest list, lists longer than kLongList), 3 cursor of the
+// drawing pass's queue, 5 device error bits (kept across frames), 6 tiles
+// above their chosen capacity, 8-10 tile scan (bin entries, ...), 11-13
+// capacity scan (regions' total, ...), 14 records taken from the pool, 15 tiles
+// counted. The count pass's statistics follow them: kStatCopies copies of
+// (fragments, longest list, long lists, unused), one per tile % kStatCopies
+// (tiles adding into one address would queue on it), summed by its last block.
 constexpr int kScal = 24;
-// Copies of the count pass's frame statistics (fragments, longest list, long
-// lists, unused), one per tile % kStatCopies, summed on the host: tiles
-// adding into one address would queue on it.
 constexpr int kStatCopies = 32;
+constexpr int kScalAll = kScal + 4 * kStatCopies;
 __host__ __device__ inline uint32_t face_edge_flags(const uint4& z) { return z.x >> 24; }
+__host__ __device__ inline uint32_t face_flags(const uint4& z) { return z.y >> 24; }
 __host__ __device__ inline uint32_t face_tris(const uint4& z) { return (z.y >> 24) & 3u; }
-__host__ __device__ inline uint32_t face_boundary(const uint4& z) { return (z.y >> 26) & 1u; }
 constexpr uint32_t kNoDepth = 0xFFFFFFFFu;   // no boundary fragment at a pixel
 
 // Resident mesh (device pointers), see hexfc_upload_mesh.
@@ -97,7 +109,11 @@ struct DevMesh {
     int4* fverts = nullptr;        // [F] canonical corners
     int4* fedges = nullptr;        // [F] unique edge id of local edge k = (c_k, c_k+1)
     uint8_t* fbound = nullptr;     // [F] 1: a boundary face (one cell)
-    FaceStatic* fstat = nullptr;   // [F] static face records
+    // [F] static face records. A frame keeps the records it was drawn with (its
+    // lists are rebuilt from them on request), so an importance update writes
+    // records that no frame keeps: at most one set per context and one more.
+    std::shared_ptr<FaceStatic> fstat;
+    std::vector<std::shared_ptr<FaceStatic>> fstat_sets;   // all sets, fstat among them
 };
 
 // Tile-capacity network (4 -> 64 -> 64 -> 1): FP32 master weights, the FP16
@@ -130,7 +146,7 @@ struct FrameBufs {
     int64_t v_cap = 0;
     // faces
     FaceFrame* fframe = nullptr;    // [F] per-frame face records
-    uint32_t* tzsum = nullptr;      // [2F] per triangle (2 face + tri): sum of its window depths
+    uint32_t* tzsum = nullptr;      // [2F] per triangle (2 face + tri): its depths (pack_depths)
     int64_t f_cap = 0;
     // tiles
     uint32_t* tile_cnt = nullptr;   // [T+1]
@@ -149,27 +165,22 @@ struct FrameBufs {
     bool scal_fresh = false;        // scal just allocated (undefined contents)
     int64_t bin_cap = 0;
     uint32_t* masks = nullptr;      // per chunk of a tile list: 256 per-pixel coverage masks
-    uint64_t* seg = nullptr;        // per chunk and warp group of 32 pixels: the first fragment of its records
-    int64_t seg_cap = 0;
+    uint32_t* zsuf = nullptr;       // per chunk: a lower bound of the depths of its tile's triangles from it on
+    int64_t zsuf_cap = 0;
     int64_t mask_cap = 0;
     // pixels (tile-major)
     uint32_t* cnt = nullptr;        // [P]
-    uint64_t* off = nullptr;        // [P]
     int64_t p_cap = 0;
     uint64_t* part = nullptr;       // scan partials
     uint32_t* part_max = nullptr;
     int64_t part_cap = 0;
-    uint32_t* long_q = nullptr;     // queue of pixels with long lists
-    uint32_t* fix_q = nullptr;      // queue of pixels whose list arrived out of order
     uint32_t* zsil = nullptr;       // [P] depth of the nearest boundary fragment (silhouettes), kNoDepth if none
-    // fragments
-    uint64_t* key = nullptr;
-    float4* rgba = nullptr;
+    uint32_t* redo = nullptr;       // [P] queue of the pixels that met their fragments out of order
+    // fragments: the drawing pass stores none; what a frame's lists would take (24 bytes a fragment) is
+    // accounted against the memory budget and the chosen capacities
     int64_t frag_cap = 0;
-    // small device scalars: [0] total fragments, [1] max list, [2] long lists, [3] long queue cursor,
-    // [4] out-of-order queue cursor, [5] error bits (kept across frames), [8..10] tile scan totals
-    uint64_t* scal = nullptr;       // kScal device scalars (slots: see kScal)
-    uint64_t* cstat = nullptr;      // [4 * kStatCopies] count pass statistics (predicted frames)
+    bool frag_sized = false;
+    uint64_t* scal = nullptr;       // kScalAll device scalars (slots: see kScal)
     uint64_t* h_scal = nullptr;     // pinned mirror
 };
 
@@ -192,54 +203,37 @@ struct CountItem {
     uint32_t* cnt;
     uint32_t* masks;
     uint32_t* tile_frag;
-    int tiles_x, W, H;
+    unsigned long long* scal;
+    int tiles_x, W, H, n_tiles;
 };
 struct CountBatch {
     CountItem it[kBatchLaunchMax];
     uint32_t tile_begin[kBatchLaunchMax + 1];
     int n;
 };
-struct FillItem {
+// What the drawing pass needs of a frame.
+struct DrawItem {
     const uint64_t* tile_off;
     const uint32_t* bins;
     const uint32_t* masks;
+    const uint32_t* zsuf;
     const FaceFrame* fframe;
     const FaceStatic* fstat;
     const uint32_t* order;
-    const uint64_t* off;
     const uint32_t* cnt;
-    uint64_t* key;
-    float4* rgba;
-    uint64_t* seg;
-    unsigned long long* err;
     uint32_t* zsil;   // nullptr: no silhouettes
-    ShadeParams sp;
-    int tiles_x, W, H;
-};
-struct FillBatch {
-    FillItem it[kBatchLaunchMax];
-    uint32_t tile_begin[kBatchLaunchMax + 1];
-    int n;
-};
-struct CompositeItem {
-    const uint32_t* cnt;
-    const uint64_t* seg;
-    const uint64_t* tile_off;
-    const uint32_t* masks;
-    const uint64_t* key;
-    const float4* rgba;
     float4* out;
-    uint32_t* long_q;
-    unsigned long long* long_cursor;
-    uint32_t* fix_q;
-    unsigned long long* fix_cursor;
-    uint64_t frag_cap;
-    float bg[3];
+    uint32_t* redo;   // queue of the pixels that met their fragments out of order
+    unsigned long long* redo_cursor;
+    const unsigned long long* scal;
+    unsigned long long* err;
+    uint64_t limit;   // most fragments the frame may have (memory budget)
+    ShadeParams sp;
     OutWin win;
     int tiles_x, W, H;
 };
-struct CompositeBatch {
-    CompositeItem it[kBatchLaunchMax];
+struct DrawBatch {
+    DrawItem it[kBatchLaunchMax];
     uint32_t tile_begin[kBatchLaunchMax + 1];
     int n;
 };
@@ -254,7 +248,7 @@ __device__ __forceinline__ int batch_item(const uint32_t* begin, int n, uint32_t
     }
     return lo;
 }
-static_assert(sizeof(FillBatch) < 30000 && sizeof(CompositeBatch) < 30000 && sizeof(CountBatch) < 30000,
+static_assert(sizeof(DrawBatch) < 30000 && sizeof(CountBatch) < 30000,
               "a batch's parameters fit a kernel's parameter space");
 
 // ---- launches (each returns cudaGetLastError()) -----------------------------------------
@@ -264,30 +258,30 @@ cudaError_t launch_cell_quality(const DevMesh& m, int metric, float* out, cudaSt
 cudaError_t launch_importance(const DevMesh& m, bool positions, cudaStream_t s);
 
 cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, cudaStream_t s);
-cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, int lod, float delta,
-                              FrameBufs& fb, int tiles_x, int tiles_y, cudaStream_t s);
+cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const ShadeParams& sp, FrameBufs& fb,
+                              int tiles_x, int tiles_y, cudaStream_t s);
 cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, int reverse,
                             cudaStream_t s);
 // Kernel attributes (dynamic shared memory limits), once per device context.
 cudaError_t prepare_raster_kernels();
-cudaError_t prepare_fill_kernels();
-cudaError_t prepare_composite_kernels();
+cudaError_t prepare_draw_kernels();
 
-cudaError_t launch_bin_sort(const DevMesh& m, FrameBufs& fb, int tiles_x, int tiles_y, int buckets,
+cudaError_t launch_bin_sort(const DevMesh& m, FrameBufs& fb, int tiles_x, int tiles_y, int64_t n_bins, int buckets,
                             cudaStream_t s);
 cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s);
-cudaError_t launch_count(const DevMesh& m, FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, bool stats,
-                         cudaStream_t s);
-// The count, fill and main resolve pass of several frames, each one launch.
+CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H);
+cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, cudaStream_t s);
+// The count and the drawing pass of several frames, each one launch.
 cudaError_t launch_count_batch(const CountBatch& b, cudaStream_t s);
-cudaError_t launch_fill_batch(const FillBatch& b, bool sil, cudaStream_t s);
-cudaError_t launch_composite_batch(const CompositeBatch& b, int window, cudaStream_t s);
-// The second passes of one frame's resolve (out-of-order and long lists).
-cudaError_t launch_composite_tail(FrameBufs& fb, const ShadeParams& sp, int tiles_x, float* out, uint32_t n_long,
-                                  OutWin win, cudaStream_t s);
+cudaError_t launch_draw_batch(const DrawBatch& b, bool sil, int window, cudaStream_t s);
+// The drawing pass of a frame, and its second pass (pixels out of order).
+cudaError_t launch_draw(const DrawItem& a, int64_t n_tiles, int window, cudaStream_t s);
+cudaError_t launch_draw_tail(const DrawItem& a, cudaStream_t s);
 // Tile capacities from the previous frame's exact counts, or `uniform` (> 0) per tile.
 cudaError_t launch_capacity_from_previous(FrameBufs& fb, int64_t n_tiles, float margin, uint32_t pad,
                                           uint32_t uniform, cudaStream_t s);
+// The frame's exact tile counts against the chosen capacities.
+cudaError_t launch_capacity_check(FrameBufs& fb, int64_t n_tiles, cudaStream_t s);
 cudaError_t launch_cap_features(FrameBufs& fb, int64_t n_tiles, int tiles_x, float lens_x, float lens_y,
                                 float inv_diag, float motion, cudaStream_t s);
 cudaError_t launch_cap_forward(const CapNet& net, FrameBufs& fb, int64_t n_tiles, float margin, uint32_t pad,
@@ -295,19 +289,14 @@ cudaError_t launch_cap_forward(const CapNet& net, FrameBufs& fb, int64_t n_tiles
 cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, cudaStream_t s);
 cudaError_t launch_cap_adam(CapNet& net, float lr, cudaStream_t s);
 cudaError_t launch_cap_to_half(CapNet& net, cudaStream_t s);
-// sil: record each pixel's nearest boundary-fragment depth into fb.zsil.
-cudaError_t launch_fill(const DevMesh& m, FrameBufs& fb, const ShadeParams& sp, int tiles_x, int tiles_y, int W,
-                        int H, bool regions, bool sil, cudaStream_t s);
-cudaError_t launch_composite(FrameBufs& fb, const ShadeParams& sp, int tiles_x, int tiles_y, int W, int H,
-                             float* out, uint32_t n_long, int window, OutWin win, cudaStream_t s);
 // White silhouettes over the output (Section "Blending Focus and Context"):
-// from the boundary surface's depths fb.zsil of the drawn rectangle, which sits
+// from the boundary surface's depths zsil of the drawn rectangle, which sits
 // at (fx0, fy0) of a frame_w x frame_h frame.
-cudaError_t launch_silhouette(FrameBufs& fb, int tiles_x, int fx0, int fy0, int frame_w, int frame_h, float alpha,
-                              float threshold, float* out, OutWin win, cudaStream_t s);
-cudaError_t launch_debug_gather(FrameBufs& fb, const int32_t* d_px, const int32_t* d_py, int64_t n,
-                                const uint64_t* d_dst_off, int tiles_x, int W, int H,
-                                uint64_t* d_keys, float4* d_rgba, uint32_t* d_counts,
+cudaError_t launch_silhouette(const uint32_t* zsil, int tiles_x, int fx0, int fy0, int frame_w, int frame_h,
+                              float alpha, float threshold, float* out, OutWin win, cudaStream_t s);
+// The sorted lists of n pixels of a frame drawn as `a` (or their lengths, if d_counts).
+cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const int32_t* d_py, int64_t n,
+                                const uint64_t* d_dst_off, uint64_t* d_keys, float4* d_rgba, uint32_t* d_counts,
                                 cudaStream_t s);
 
 // scans

@@ -200,7 +200,50 @@ __global__ void k_cap_to_half(const float* __restrict__ w, __half* __restrict__ 
     if (p < kCapParams) w16[p] = __float2half_rn(w[p]);
 }
 
+// Capacities from the previous frame's exact tile counts: prev * (1 + margin)
+// + pad; or, given a uniform count (> 0), that count for every tile instead.
+__global__ void k_capacity_from_previous(const uint32_t* __restrict__ prev, int64_t n_tiles, float margin,
+                                         uint32_t pad, uint32_t uniform, uint32_t* __restrict__ cap)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n_tiles) return;
+    const float c = uniform ? (float)uniform : (float)prev[t];
+    cap[t] = (uint32_t)fminf(c * (1.f + margin) + (float)pad, 4.0e9f);
+}
+
+// The exact tile counts against the chosen capacities: a tile's lists go to its
+// region [cap_off[t], cap_off[t+1]), or to the pool after all regions (scal[14]
+// records taken, scal[6] tiles) if they do not fit; a frame whose pool runs out
+// is not drawn (error bit kErrPool) but drawn again without capacities.
+constexpr unsigned long long kErrPool = 16ull;
+__global__ void k_capacity_check(const uint32_t* __restrict__ tile_frag, const uint64_t* __restrict__ cap_off,
+                                 int64_t n_tiles, uint64_t frag_cap, unsigned long long* __restrict__ scal)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n_tiles) return;
+    const uint64_t total = tile_frag[t], region = cap_off[t];
+    if (region + total <= cap_off[t + 1] && region + total <= frag_cap) return;
+    const uint64_t p = atomicAdd(&scal[14], (unsigned long long)total);
+    atomicAdd(&scal[6], 1ull);
+    if (cap_off[n_tiles] + p + total > frag_cap) atomicOr(&scal[5], kErrPool);
+}
+
 }  // namespace
+
+cudaError_t launch_capacity_from_previous(FrameBufs& fb, int64_t n_tiles, float margin, uint32_t pad, uint32_t uniform,
+                                          cudaStream_t s)
+{
+    k_capacity_from_previous<<<grid_for(n_tiles, 256), 256, 0, s>>>(fb.tile_frag, n_tiles, margin, pad, uniform,
+                                                                     fb.tile_cap);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_capacity_check(FrameBufs& fb, int64_t n_tiles, cudaStream_t s)
+{
+    k_capacity_check<<<grid_for(n_tiles, 256), 256, 0, s>>>(fb.tile_frag, fb.cap_off, n_tiles, (uint64_t)fb.frag_cap,
+                                                            reinterpret_cast<unsigned long long*>(fb.scal));
+    return cudaGetLastError();
+}
 
 cudaError_t launch_cap_features(FrameBufs& fb, int64_t n_tiles, int tiles_x, float lens_x, float lens_y,
                                 float inv_diag, float motion, cudaStream_t s)

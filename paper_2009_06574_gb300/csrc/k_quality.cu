@@ -161,7 +161,7 @@ cudaError_t launch_importance(const DevMesh& m, bool positions, cudaStream_t s)
                                                                    m.n_cells, m.vkey, m.ekey);
     k_key_to_float<<<grid_for(nk, 256), 256, 0, s>>>(m.vkey, m.vimp, m.n_verts, m.ekey, m.eattr, m.n_edges);
     k_face_static<<<grid_for(m.n_faces, 256), 256, 0, s>>>(m.fverts, m.vimp, m.verts, m.n_faces, positions,
-                                                           m.fstat);
+                                                           m.fstat.get());
     return cudaGetLastError();
 }
 

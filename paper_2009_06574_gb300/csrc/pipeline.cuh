@@ -1,12 +1,11 @@
-// Shared-memory barriers and asynchronous copies (inline PTX, sm_90+) used by
-// the producer/consumer pipelines of this library. Every wait is bounded.
+// Shared-memory barriers (inline PTX, sm_90+) of the drawing pass. Every wait is
+// bounded.
 #pragma once
 #include <stdint.h>
 
 namespace hexfc {
 
-constexpr uint32_t kWaitPolls = 1u << 26;          // bounded mbarrier polls
-constexpr long long kWaitCycles = 1ll << 30;       // and about half a second of SM clock
+constexpr long long kWaitCycles = 1ll << 30;       // about half a second of SM clock
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -23,40 +22,16 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_addr(bar)) : "memory");
 }
-// Waits for the phase with parity `parity` to complete; false if the bound ran out.
-__device__ __forceinline__ bool mbar_try(unsigned a, unsigned parity)
+// Whether the phase with parity `parity` has completed (does not wait).
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, unsigned parity)
 {
     unsigned done;
     asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
-        : "r"(a), "r"(parity)
+        : "r"(smem_addr(bar)), "r"(parity)
         : "memory");
     return done != 0;
 }
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity)
-{
-    const unsigned a = smem_addr(bar);
-    if (mbar_try(a, parity)) return true;
-    const long long t0 = clock64();
-    for (uint32_t it = 0; it < kWaitPolls && clock64() - t0 < kWaitCycles; ++it) {
-        unsigned done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-// Per-thread asynchronous copy global -> shared (16 bytes, 16-byte aligned).
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 }  // namespace hexfc

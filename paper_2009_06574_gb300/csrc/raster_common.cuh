@@ -38,8 +38,8 @@ struct TriGeom {
     bool valid;
 };
 
-__device__ __forceinline__ void tri_setup(const int32_t FX[4], const int32_t FY[4], int tri, int W, int H,
-                                          TriGeom& t)
+// Vertices, winding and area of the triangle (the rest of t is left alone).
+__device__ __forceinline__ void tri_wind(const int32_t FX[4], const int32_t FY[4], int tri, TriGeom& t)
 {
     int i1 = tri == 0 ? 1 : 2, i2 = tri == 0 ? 2 : 3;
     t.vi[0] = 0; t.vi[1] = i1; t.vi[2] = i2;
@@ -56,6 +56,12 @@ __device__ __forceinline__ void tri_setup(const int32_t FX[4], const int32_t FY[
         a = -a;
     }
     t.area = a;
+}
+
+__device__ __forceinline__ void tri_setup(const int32_t FX[4], const int32_t FY[4], int tri, int W, int H,
+                                          TriGeom& t)
+{
+    tri_wind(FX, FY, tri, t);
     int32_t xmin = min(t.X[0], min(t.X[1], t.X[2])), xmax = max(t.X[0], max(t.X[1], t.X[2]));
     int32_t ymin = min(t.Y[0], min(t.Y[1], t.Y[2])), ymax = max(t.Y[0], max(t.Y[1], t.Y[2]));
     // pixel p has its centre at 256 p + 128
@@ -68,7 +74,7 @@ __device__ __forceinline__ void tri_setup(const int32_t FX[4], const int32_t FY[
     bx1 = min(bx1, (int64_t)W - 1);
     by1 = min(by1, (int64_t)H - 1);
     t.bx0 = (int32_t)bx0; t.by0 = (int32_t)by0; t.bx1 = (int32_t)bx1; t.by1 = (int32_t)by1;
-    t.valid = (a != 0) && bx0 <= bx1 && by0 <= by1;
+    t.valid = (t.area != 0) && bx0 <= bx1 && by0 <= by1;
 }
 
 // Exact floor(n / a) for a > 0 and |n / a| < 2^25, with |n| < 2^63:
@@ -102,11 +108,11 @@ __device__ __forceinline__ float i64_to_f32(int64_t v)
     return v < 0 ? -m : m;
 }
 
-// Per-sample depth: z0 + floor((l1 (z1 - z0) + l2 (z2 - z0)) / area), exact.
-__device__ __forceinline__ uint32_t sample_depth(uint32_t z0, uint32_t z1, uint32_t z2, int64_t l1, int64_t l2,
+// Per-sample depth: z0 + floor((l1 d1 + l2 d2) / area), exact, with d1, d2 the
+// depths of vertices 1, 2 less vertex 0's.
+__device__ __forceinline__ uint32_t sample_depth(uint32_t z0, int64_t d1, int64_t d2, int64_t l1, int64_t l2,
                                                  int64_t area, bool& bad)
 {
-    int64_t d1 = (int64_t)z1 - (int64_t)z0, d2 = (int64_t)z2 - (int64_t)z0;
     int64_t q;
     if (area < (1ll << 38)) {
         // |l| <= area < 2^38 and |d| < 2^24: the numerator fits in int64
@@ -131,12 +137,11 @@ __device__ __forceinline__ uint32_t sample_depth(uint32_t z0, uint32_t z1, uint3
 // deltas dz1, dz2 (same result). With lam within 5 ulp and 0 <= lam <= 1,
 // |d| < 2^24, the float estimate is within 8 of the quotient; the integer
 // remainder then corrects it.
-__device__ __forceinline__ uint32_t sample_depth_lam(uint32_t z0, uint32_t z1, uint32_t z2, int64_t l1, int64_t l2,
+__device__ __forceinline__ uint32_t sample_depth_lam(uint32_t z0, int32_t d1, int32_t d2, int64_t l1, int64_t l2,
                                                      int64_t area, float lam1, float lam2, float dz1, float dz2,
                                                      bool& bad)
 {
-    if (area >= (1ll << 38)) return sample_depth(z0, z1, z2, l1, l2, area, bad);
-    const int32_t d1 = (int32_t)(z1 - z0), d2 = (int32_t)(z2 - z0);
+    if (area >= (1ll << 38)) return sample_depth(z0, d1, d2, l1, l2, area, bad);
     int64_t q = __float2int_rd(fmaf(lam1, dz1, lam2 * dz2));
     // |l| <= area < 2^38 and |d| < 2^24: the numerator fits in int64
     int64_t r = l1 * d1 + l2 * d2 - q * area;
@@ -146,25 +151,6 @@ __device__ __forceinline__ uint32_t sample_depth_lam(uint32_t z0, uint32_t z1, u
     for (int it = 0; it < 16 && r >= area; ++it) { ++q; r -= area; }
     if (r < 0 || r >= area) bad = true;
     return (uint32_t)((int64_t)z0 + q);
-}
-
-// sample_depth_lam for a triangle with area < 2^26 (16.8 units squared: below
-// 512 square pixels), in 32-bit arithmetic: its weights satisfy 0 <= l <=
-// area < 2^26, the float estimate is within 8 of the quotient, so the exact
-// remainder l1 d1 + l2 d2 - q area lies within (-9, 9) areas, below 2^30 in
-// magnitude, and its value modulo 2^32 read as a signed integer is exact.
-__device__ __forceinline__ uint32_t sample_depth_small(uint32_t z0, uint32_t z1, uint32_t z2, uint32_t l1,
-                                                       uint32_t l2, uint32_t area, float lam1, float lam2, float dz1,
-                                                       float dz2, bool& bad)
-{
-    int32_t q = __float2int_rd(fmaf(lam1, dz1, lam2 * dz2));
-    int32_t r = (int32_t)(l1 * (z1 - z0) + l2 * (z2 - z0) - (uint32_t)q * area);
-#pragma unroll 1
-    for (int it = 0; it < 16 && r < 0; ++it) { --q; r += (int32_t)area; }
-#pragma unroll 1
-    for (int it = 0; it < 16 && r >= (int32_t)area; ++it) { ++q; r -= (int32_t)area; }
-    if (r < 0 || r >= (int32_t)area) bad = true;
-    return z0 + (uint32_t)q;
 }
 
 }  // namespace hexfc

@@ -1,8 +1,6 @@
-// Per-tile rasterisation shared by the count and fill passes: exact
-// coverage data of a chunk of triangles, and the producer/consumer ring of
-// the fill pipeline.
+// Per-tile rasterisation of the count pass: exact coverage data of a chunk of
+// triangles.
 #pragma once
-#include "pipeline.cuh"
 #include "raster_common.cuh"
 
 namespace hexfc {
@@ -49,32 +47,6 @@ __device__ __forceinline__ void stage_cov(int4 a, int4 b, uint32_t f2t, int W, i
     c.box[j] = (x0 - px0) | ((y0 - py0) << 8) | ((x1 - x0 + 1) << 16) | ((y1 - y0 + 1) << 24);
 }
 
-// ------------------------------------------------------------------ tile passes
-//
-// k_fill runs one block per tile as a pipeline: a producer warp stages each
-// chunk of 32 triangles of the tile's (depth-ordered) list into a ring of
-// kRing slots in shared memory, while the eight consumer warps shade the
-// covered samples of earlier chunks. Slots are handed over with mbarriers
-// (full: the 32 producer lanes arrive; empty: lane 0 of each consumer warp
-// arrives once no sample in its warp's queue refers to the slot), so the
-// producer runs up to kRing chunks ahead. Every wait is bounded; a wait that runs out sets an error bit
-// and ends the kernel's loops.
-
-constexpr int kRing = 6;
-constexpr int kConsumerWarps = kTilePix / 32;
-constexpr int kPipeThreads = kTilePix + 32;
-constexpr unsigned long long kErrWait = 4ull;
-
-__device__ __forceinline__ void pipe_init(uint64_t* full, uint64_t* empty)
-{
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kRing; ++s) {
-            mbar_init(&full[s], 32);
-            mbar_init(&empty[s], kConsumerWarps);   // lane 0 of each consumer warp
-        }
-        mbar_init_fence();
-    }
-    __syncthreads();
-}
+constexpr int kConsumerWarps = kTilePix / 32;   // warps of the count pass
 
 }  // namespace hexfc
