@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "hexfc.h"
+#include "vertex_stage.h"
 
 namespace hexfc {
 
@@ -22,14 +23,6 @@ constexpr int kLongList = 256;             // lists longer than this are counted
 constexpr uint64_t kPadKey = ~0ull;
 constexpr int kChunk = 32;                // triangles per raster chunk (one coverage bit each)
 constexpr uint32_t kPadBin = 0xFFFFFFFFu; // empty slot: tile lists are padded to whole chunks
-
-// Camera constants of the vertex stage (double, evaluated without FMA).
-struct CamParams {
-    double eye[3], R[3], U[3], F[3];
-    double focal, scale, cx, cy, znear, zfar, zf_over;
-    int ortho, W, H;   // W, H: size of the drawn rectangle (the frame's unless a sub-rectangle is drawn)
-    int ox, oy;   // drawn rectangle's offset in the frame (pixels): window positions are shifted by it
-};
 
 // Focus+context constants of the fragment stage (float).
 struct ShadeParams {

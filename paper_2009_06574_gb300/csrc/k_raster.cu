@@ -27,40 +27,19 @@ inline unsigned grid_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b);
 
 // ------------------------------------------------------------------ vertex stage
 
-__global__ void k_vertex_setup(const float* __restrict__ verts, int64_t n, CamParams cam,
-                               int4* __restrict__ vproj, float* __restrict__ ved)
+// Thread per vertex: window position on 1/256 pixel, 24-bit depth, eye depth.
+__global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ verts, int64_t n,
+                                                      const __grid_constant__ CamParams cam,
+                                                      const __grid_constant__ CamPairs pairs,
+                                                      int4* __restrict__ vproj, float* __restrict__ ved)
 {
-    int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n) return;
-    double dx = __dsub_rn((double)verts[3 * v], cam.eye[0]);
-    double dy = __dsub_rn((double)verts[3 * v + 1], cam.eye[1]);
-    double dz = __dsub_rn((double)verts[3 * v + 2], cam.eye[2]);
-    double ex = __dadd_rn(__dadd_rn(__dmul_rn(dx, cam.R[0]), __dmul_rn(dy, cam.R[1])), __dmul_rn(dz, cam.R[2]));
-    double ey = __dadd_rn(__dadd_rn(__dmul_rn(dx, cam.U[0]), __dmul_rn(dy, cam.U[1])), __dmul_rn(dz, cam.U[2]));
-    double ed = __dadd_rn(__dadd_rn(__dmul_rn(dx, cam.F[0]), __dmul_rn(dy, cam.F[1])), __dmul_rn(dz, cam.F[2]));
-    double xw, yw, z;
-    if (cam.ortho) {
-        xw = __dadd_rn(cam.cx, __dmul_rn(ex, cam.scale));
-        yw = __dsub_rn(cam.cy, __dmul_rn(ey, cam.scale));
-        z = __ddiv_rn(__dsub_rn(ed, cam.znear), __dsub_rn(cam.zfar, cam.znear));
-    } else {
-        xw = __dadd_rn(cam.cx, __dmul_rn(__ddiv_rn(ex, ed), cam.focal));
-        yw = __dsub_rn(cam.cy, __dmul_rn(__ddiv_rn(ey, ed), cam.focal));
-        z = __dmul_rn(cam.zf_over, __dsub_rn(1.0, __ddiv_rn(cam.znear, ed)));
-    }
-    bool valid = (ed > cam.znear) && (ed < cam.zfar) && (fabs(xw) <= 16384.0) && (fabs(yw) <= 16384.0);
-    int4 o = make_int4(0, 0, 0, 0);
-    if (valid) {
-        z = fmin(fmax(z, 0.0), 1.0);
-        // snapped in frame coordinates, then moved by whole pixels into the drawn
-        // rectangle: coverage, depth and edge distances are those of the frame
-        o.x = (int32_t)rint(__dmul_rn(xw, 256.0)) - 256 * cam.ox;
-        o.y = (int32_t)rint(__dmul_rn(yw, 256.0)) - 256 * cam.oy;
-        o.z = (int32_t)(uint32_t)rint(__dmul_rn(z, 16777215.0));
-        o.w = 1;
-    }
-    vproj[v] = o;
-    ved[v] = (float)ed;
+    const float x = verts[3 * v], y = verts[3 * v + 1], z = verts[3 * v + 2];
+    ProjVertex o;
+    if (!pairs.usable || !vertex_pairs(x, y, z, pairs, cam, o)) vertex_double(x, y, z, cam, o);
+    vproj[v] = make_int4(o.x, o.y, o.z, o.valid);
+    ved[v] = o.depth;
 }
 
 // ------------------------------------------------------------------ face stage
@@ -606,7 +585,7 @@ cudaError_t prepare_raster_kernels()
 
 cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, cudaStream_t s)
 {
-    k_vertex_setup<<<grid_for(m.n_verts, 256), 256, 0, s>>>(m.verts, m.n_verts, cam, fb.vproj, fb.ved);
+    k_vertex_setup<<<grid_for(m.n_verts, 256), 256, 0, s>>>(m.verts, m.n_verts, cam, cam_pairs(cam), fb.vproj, fb.ved);
     return cudaGetLastError();
 }
 
