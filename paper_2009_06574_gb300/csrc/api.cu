@@ -187,8 +187,8 @@ void free_mesh(DevMesh* m)
 
 void free_frame(FrameBufs& f)
 {
-    dfree(f.vproj); dfree(f.ved); dfree(f.fframe); dfree(f.tzsum);
-    dfree(f.tile_cnt); dfree(f.tile_off); dfree(f.tile_cur); dfree(f.tile_order); dfree(f.tile_frag); dfree(f.tile_cap); dfree(f.cap_off); dfree(f.tile_zr); dfree(f.cap_x);
+    dfree(f.vproj); dfree(f.ved); dfree(f.fframe); dfree(f.tzsum); dfree(f.trange); dfree(f.slots); dfree(f.fextra); dfree(f.tile_big);
+    dfree(f.tile_cnt); dfree(f.tile_off); dfree(f.tile_cur); dfree(f.tile_order); dfree(f.tile_frag); dfree(f.tile_cap); dfree(f.cap_off); dfree(f.cap_x);
     dfree(f.bins); dfree(f.bins_tmp); dfree(f.masks); dfree(f.zsuf); dfree(f.cnt); dfree(f.zsil);
     dfree(f.part); dfree(f.part_max); dfree(f.redo); dfree(f.scal);
     if (f.h_scal) cudaFreeHost(f.h_scal);
@@ -218,6 +218,14 @@ hexfc_status own_fstat(DevMesh& m, bool* fresh)
     }
     *fresh = true;
     return HEXFC_OK;
+}
+
+void free_slots(FrameBufs& f)
+{
+    dfree(f.trange);
+    dfree(f.slots);
+    dfree(f.fextra);
+    f.slot_cap = 0;
 }
 
 DevMesh* get_mesh(hexfc_ctx* ctx, int32_t id)
@@ -388,6 +396,7 @@ struct FrameJob {
     float lens_x = 0.f, lens_y = 0.f, inv_diag = 0.f, motion = 0.f;   // capacity-network features
     bool prev_counts = false;   // fb.tile_frag holds the previous frame's counts for this tile grid
     uint64_t budget = 0;
+    bool may_drop_slots = true;   // phase 1 can be run again without the binning's places
     float* out = nullptr;
     OutWin win{};                  // output pixels of the drawn rectangle (the rest: the apron)
     float sil_alpha = 0.f, sil_threshold = 0.f;   // silhouettes (off at alpha 0)
@@ -482,14 +491,26 @@ FrameJob make_job(hexfc_ctx* ctx, FrameBufs* fb, DevMesh* m, float* out)
     return j;
 }
 
-// Capacity features of the frame (before its count overwrites the previous counts).
-hexfc_status job_features(FrameJob& j, cudaStream_t s)
+// Device memory of a context's frame buffers, with the lists of `frags`
+// fragments (24 bytes each: key and colour). The drawing pass does not store
+// the lists; they count towards the budget all the same, so that what fits a
+// budget does not depend on whether they are asked for (hexfc_debug_pixels). The
+// places of the binning and the faces' extras are not counted: a frame does
+// without them if need be.
+constexpr uint64_t kFragBytes = sizeof(uint64_t) + sizeof(float4);
+constexpr uint64_t kSlotBytes = 2 * (sizeof(uint32_t) + sizeof(uint4)) + sizeof(FaceExtra);   // a face's places, extras
+uint64_t frame_bytes(const FrameBufs& f, int64_t frags)
 {
-    FrameBufs& fb = *j.fb;
-    if (!j.prev_counts) CK(cudaMemsetAsync(fb.tile_frag, 0, sizeof(uint32_t) * (size_t)j.n_tiles, s));
-    CK(launch_cap_features(fb, j.n_tiles, j.tiles_x, j.lens_x, j.lens_y, j.inv_diag, j.motion, s));
-    j.launches += 1;
-    return HEXFC_OK;
+    uint64_t b = 0;
+    b += (uint64_t)f.v_cap * (sizeof(int4) + sizeof(float));
+    b += (uint64_t)f.f_cap * (sizeof(FaceFrame) + 2 * sizeof(uint32_t));
+    b += (uint64_t)f.t_cap * (9 * sizeof(uint32_t) + sizeof(uint64_t) + sizeof(uint32_t));
+    b += (uint64_t)f.bin_cap * 2 * sizeof(uint32_t) + (uint64_t)f.mask_cap * sizeof(uint32_t) +
+         (uint64_t)f.zsuf_cap * sizeof(uint32_t);
+    b += (uint64_t)f.p_cap * (3 * sizeof(uint32_t));
+    b += (uint64_t)f.part_cap * (sizeof(uint64_t) + sizeof(uint32_t));
+    b += (uint64_t)frags * kFragBytes;
+    return b;
 }
 
 // Buffers whose size follows from the mesh and the view.
@@ -509,17 +530,18 @@ hexfc_status job_alloc(FrameJob& j)
         dfree(fb.tzsum);
         if ((st = ensure(&fb.fframe, &fb.f_cap, m->n_faces)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.tzsum, &c1, 2 * fb.f_cap)) != HEXFC_OK) return st;
+        free_slots(fb);
     }
     if (!fb.tile_cnt || fb.t_cap < j.n_tiles + 1) {
         int64_t c1 = 0, c2 = 0, c3 = 0, c4 = 0, c5 = 0, c6 = 0;
-        dfree(fb.tile_off); dfree(fb.tile_cur); dfree(fb.tile_order); dfree(fb.tile_frag); dfree(fb.tile_zr);
+        dfree(fb.tile_off); dfree(fb.tile_cur); dfree(fb.tile_order); dfree(fb.tile_frag); dfree(fb.tile_big);
         dfree(fb.cap_x);
         if ((st = ensure(&fb.tile_cnt, &fb.t_cap, j.n_tiles + 1)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.tile_off, &c1, fb.t_cap)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.tile_cur, &c2, fb.t_cap)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.tile_order, &c3, fb.t_cap)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.tile_frag, &c4, fb.t_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.tile_zr, &c5, fb.t_cap)) != HEXFC_OK) return st;
+        if ((st = ensure(&fb.tile_big, &c5, fb.t_cap)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.cap_x, &c6, 4 * fb.t_cap)) != HEXFC_OK) return st;
     }
     if (!fb.cnt || fb.p_cap < j.n_pix + 1) {
@@ -536,6 +558,19 @@ hexfc_status job_alloc(FrameJob& j)
         if ((st = ensure(&fb.part, &fb.part_cap, 2 * nparts)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.part_max, &c1, fb.part_cap)) != HEXFC_OK) return st;
     }
+    // places of the binning and the faces' extras: faster, not needed (72 bytes a
+    // face): only in what a budget leaves
+    const bool room = !j.budget || (j.may_drop_slots && fb.slots_refused != j.budget &&
+                                    frame_bytes(fb, 0) + (uint64_t)fb.f_cap * kSlotBytes <= j.budget);
+    if (fb.slots && !room) free_slots(fb);
+    if (!fb.slots && room) {
+        int64_t c1 = 0, c2 = 0, c3 = 0;
+        if (ensure(&fb.trange, &c1, 2 * fb.f_cap) == HEXFC_OK && ensure(&fb.slots, &c2, 2 * fb.f_cap) == HEXFC_OK &&
+            ensure(&fb.fextra, &c3, fb.f_cap) == HEXFC_OK)
+            fb.slot_cap = fb.f_cap;
+        else
+            free_slots(fb);
+    }
     if (!fb.scal) {
         if ((st = dalloc(&fb.scal, kScalAll)) != HEXFC_OK) return st;
         CK(cudaMallocHost((void**)&fb.h_scal, kScal * sizeof(uint64_t)));
@@ -548,33 +583,28 @@ hexfc_status job_phase1(FrameJob& j, cudaStream_t s)
 {
     FrameBufs& fb = *j.fb;
     job_mark(j, 0, s);
-    CK(cudaMemsetAsync(fb.tile_cnt, 0, sizeof(uint32_t) * (size_t)j.n_tiles, s));
-    CK(cudaMemsetAsync(fb.tile_cur, 0, sizeof(uint32_t) * (size_t)j.n_tiles, s));
     // scal[5] (device error bits) is kept across frames so that errors of the
     // last passes of a frame are reported by the next call (hexfc_render_host
-    // reads them at the end of its own frame)
+    // reads them at the end of its own frame); the vertex stage clears the rest
     if (fb.scal_fresh) {
         CK(cudaMemsetAsync(fb.scal, 0, sizeof(uint64_t) * kScalAll, s));
         fb.scal_fresh = false;
-    } else {
-        CK(cudaMemsetAsync(fb.scal, 0, sizeof(uint64_t) * 5, s));
-        CK(cudaMemsetAsync(fb.scal + 6, 0, sizeof(uint64_t) * (kScalAll - 6), s));
     }
-    CK(launch_vertex_setup(*j.m, j.cam, fb, s));
+    CK(launch_vertex_setup(*j.m, j.cam, fb, j.n_tiles, s));
     job_mark(j, 1, s);
-    CK(launch_face_setup(*j.m, j.cam, j.sp, fb, j.tiles_x, j.tiles_y, s));
+    CK(launch_face_setup(*j.m, j.cam, j.sp, fb, j.tiles_x, j.tiles_y, j.reverse, s));
     job_mark(j, 2, s);
-    CK(scan_u32_to_u64(fb.tile_cnt, fb.tile_off, j.n_tiles, fb.part, fb.part_max, fb.scal + 8, 0xFFFFFFFFu, s,
-                       (uint32_t)kChunk));
+    CK(launch_tile_scan(fb, j.n_tiles, &j.order_done, s));
     job_mark(j, 3, s);
-    j.launches = 5;
+    j.launches = j.order_done ? 3 : 5;
     CK(cudaMemcpyAsync(fb.h_scal + 8, fb.scal + 8, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    j.order_done = false;
     if (j.p1_done) {
         CK(cudaEventRecord(j.p1_done, s));
-        CK(launch_tile_order(fb, j.n_tiles, s));
-        j.order_done = true;
-        j.launches += 1;
+        if (!j.order_done) {
+            CK(launch_tile_order(fb, j.n_tiles, s));
+            j.order_done = true;
+            j.launches += 1;
+        }
     }
     return HEXFC_OK;
 }
@@ -606,21 +636,38 @@ hexfc_status job_read1(FrameJob& j)
     return HEXFC_OK;
 }
 
+// Whether the frame's buffers, now that the bins are known, exceed its budget
+// for the binning's places alone: they are given back, and phase 1 has to run
+// once more without them.
+bool drop_slots(FrameJob& j)
+{
+    FrameBufs& fb = *j.fb;
+    if (!j.budget || !fb.slots || frame_bytes(fb, 0) + (uint64_t)fb.slot_cap * kSlotBytes <= j.budget) return false;
+    free_slots(fb);
+    fb.slots_refused = j.budget;
+    return true;
+}
+
 // Phase 2 up to the count: the bins in depth order, the tile order, the capacity features.
 hexfc_status job_phase2_bins(FrameJob& j, cudaStream_t s)
 {
     FrameBufs& fb = *j.fb;
     job_mark(j, 4, s);
-    CK(cudaMemsetAsync(fb.bins, 0xFF, sizeof(uint32_t) * (size_t)j.n_bins, s));   // padding slots = kPadBin
-    CK(launch_bin_fill(*j.m, fb, j.tiles_x, j.W, j.H, j.reverse, s));
-    CK(launch_bin_sort(*j.m, fb, j.tiles_x, j.tiles_y, (int64_t)j.n_bins, j.buckets, s));
+    CK(launch_bin_fill(*j.m, fb, j.tiles_x, j.W, j.H, s));
+    CapFeatures cf{};   // (before the count overwrites the previous frame's)
+    cf.prev = j.prev_counts ? fb.tile_frag : nullptr;
+    cf.X = fb.cap_x;
+    cf.lens_x = j.lens_x;
+    cf.lens_y = j.lens_y;
+    cf.inv_diag = j.inv_diag;
+    cf.motion = j.motion;
+    cf.tiles_x = j.tiles_x;
+    CK(launch_bin_sort(fb, j.n_tiles, (int64_t)j.n_bins, j.buckets, cf, s));
     if (!j.order_done) {
         CK(launch_tile_order(fb, j.n_tiles, s));
         j.launches += 1;
     }
     j.launches += 2;
-    hexfc_status fst = job_features(j, s);
-    if (fst != HEXFC_OK) return fst;
     job_mark(j, 5, s);
     return HEXFC_OK;
 }
@@ -642,25 +689,6 @@ hexfc_status job_phase2(FrameJob& j, cudaStream_t s)
     if ((st = job_phase2_bins(j, s)) != HEXFC_OK) return st;
     CK(launch_count(*j.fb, j.tiles_x, j.tiles_y, j.W, j.H, s));
     return job_phase2_totals(j, s);
-}
-
-// Device memory of a context's frame buffers, with the lists of `frags`
-// fragments (24 bytes each: key and colour). The drawing pass does not store
-// the lists; they count towards the budget all the same, so that what fits a
-// budget does not depend on whether they are asked for (hexfc_debug_pixels).
-constexpr uint64_t kFragBytes = sizeof(uint64_t) + sizeof(float4);
-uint64_t frame_bytes(const FrameBufs& f, int64_t frags)
-{
-    uint64_t b = 0;
-    b += (uint64_t)f.v_cap * (sizeof(int4) + sizeof(float));
-    b += (uint64_t)f.f_cap * (sizeof(FaceFrame) + 2 * sizeof(uint32_t));
-    b += (uint64_t)f.t_cap * (9 * sizeof(uint32_t) + sizeof(uint64_t) + sizeof(uint32_t));
-    b += (uint64_t)f.bin_cap * 2 * sizeof(uint32_t) + (uint64_t)f.mask_cap * sizeof(uint32_t) +
-         (uint64_t)f.zsuf_cap * sizeof(uint32_t);
-    b += (uint64_t)f.p_cap * (3 * sizeof(uint32_t));
-    b += (uint64_t)f.part_cap * (sizeof(uint64_t) + sizeof(uint32_t));
-    b += (uint64_t)frags * kFragBytes;
-    return b;
 }
 
 // The most fragments the frame may have (what job_read2 refuses, the drawing
@@ -735,6 +763,7 @@ DrawItem draw_item(const FrameJob& j, uint64_t limit)
     it.zsuf = fb.zsuf;
     it.fframe = fb.fframe;
     it.fstat = j.m->fstat.get();
+    it.fextra = fb.fextra;
     it.order = fb.tile_order;
     it.cnt = fb.cnt;
     it.zsil = j.sil_alpha > 0.f ? fb.zsil : nullptr;
@@ -854,6 +883,10 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
         }
     }
     if ((st = job_read1(j)) != HEXFC_OK) return st;
+    if (drop_slots(j)) {
+        if ((st = job_phase1(j, s)) != HEXFC_OK) return st;
+        if ((st = job_wait1(ctx, j, s)) != HEXFC_OK) return st;
+    }
     if ((st = job_phase2(j, s)) != HEXFC_OK) return st;
     if (!ctx->ev_p2) CK(cudaEventCreateWithFlags(&ctx->ev_p2, cudaEventDisableTiming));
     CK(cudaEventRecord(ctx->ev_p2, s));
@@ -927,6 +960,10 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
         }
     }
     if ((st = job_read1(j)) != HEXFC_OK) return st;
+    if (drop_slots(j)) {
+        if ((st = job_phase1(j, s)) != HEXFC_OK) return st;
+        if ((st = job_wait1(ctx, j, s)) != HEXFC_OK) return st;
+    }
     // room for the regions of this frame (previous counts * margin + pad) and a
     // pool after them for the tiles above their capacity (the previous frame's
     // fragment total, now verified, scaled to this frame's pixels)
@@ -1392,6 +1429,7 @@ hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_ite
         j.buckets = ctx->depth_buckets;
         j.window = ctx->window;
         j.budget = ctx->budget;
+        j.may_drop_slots = false;
         j.out = it.out_rgba;
         j.win = OutWin{0, 0, j.W, j.H};   // whole frames
         j.sil_alpha = it.style.sil_alpha;
@@ -1572,9 +1610,12 @@ hexfc_status hexfc_capacity_train(hexfc_ctx* ctx, int32_t steps, float lr, float
 hexfc_status hexfc_frame_memory(const hexfc_ctx* ctx, uint64_t* bytes)
 {
     if (!ctx || !bytes) return HEXFC_ERR_ARG;
-    uint64_t b = frame_bytes(ctx->fb, ctx->fb.frag_cap);
+    auto held = [](const FrameBufs& f) {   // with the lists' room, or the binning's places if those are more
+        return std::max(frame_bytes(f, f.frag_cap), frame_bytes(f, 0) + (uint64_t)f.slot_cap * kSlotBytes);
+    };
+    uint64_t b = held(ctx->fb);
     b += (uint64_t)ctx->d_out_cap * sizeof(float);
-    for (const auto& bs : ctx->batch) b += frame_bytes(bs->fb, bs->fb.frag_cap);
+    for (const auto& bs : ctx->batch) b += held(bs->fb);
     *bytes = b;
     return HEXFC_OK;
 }
@@ -2034,29 +2075,25 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     fb.tile_cur = a.take<uint32_t>((size_t)n_tiles + 1);
     fb.tile_order = a.take<uint32_t>((size_t)n_tiles + 1);
     fb.tile_frag = a.take<uint32_t>((size_t)n_tiles + 1);
-    fb.tile_zr = a.take<float>((size_t)n_tiles + 1);
+    fb.tile_big = a.take<uint32_t>((size_t)n_tiles + 1);
     fb.cnt = a.take<uint32_t>((size_t)n_pix + 1);
     fb.redo = a.take<uint32_t>((size_t)n_pix + 1);
     fb.zsil = sil ? a.take<uint32_t>((size_t)n_pix) : nullptr;
     fb.part = a.take<uint64_t>(2 * (size_t)nparts);
     fb.part_max = a.take<uint32_t>(2 * (size_t)nparts);
     if (!fb.vproj || !fb.ved || !fb.fframe || !fb.tzsum || !fb.tile_cnt ||
-        !fb.tile_off || !fb.tile_cur || !fb.tile_order || !fb.tile_frag || !fb.tile_zr || !fb.cnt || !fb.redo || (sil && !fb.zsil) || !fb.part || !fb.part_max ||
+        !fb.tile_off || !fb.tile_cur || !fb.tile_order || !fb.tile_frag || !fb.tile_big || !fb.cnt || !fb.redo || (sil && !fb.zsil) || !fb.part || !fb.part_max ||
         !fb.scal)
         return HEXFC_ERR_OVERFLOW;
-    // the array keeps the previous call's contents: clear what must start at zero
-    CK(cudaMemsetAsync(fb.tile_cnt, 0, sizeof(uint32_t) * (size_t)n_tiles, s));
-    CK(cudaMemsetAsync(fb.tile_cur, 0, sizeof(uint32_t) * (size_t)n_tiles, s));
-    // all device scalars but the error word (slot 5): the fill and the composite
-    // of the previous call on this device may have set bits there after that
-    // call returned, and they are reported below, by this call (the array starts
-    // zeroed when the module is loaded)
-    CK(cudaMemsetAsync(fb.scal, 0, sizeof(uint64_t) * 5, s));
-    CK(cudaMemsetAsync(fb.scal + 6, 0, sizeof(uint64_t) * (kScalAll - 6), s));
-    CK(launch_vertex_setup(*m, ctx->cam, fb, s));
-    CK(launch_face_setup(*m, ctx->cam, make_shade(ctx), fb, tiles_x, tiles_y, s));
-    CK(scan_u32_to_u64(fb.tile_cnt, fb.tile_off, n_tiles, fb.part, fb.part_max, fb.scal + 8, 0xFFFFFFFFu, s,
-                       (uint32_t)kChunk));
+    // the array keeps the previous call's contents: the vertex stage clears what
+    // must start at zero, all device scalars but the error word (slot 5): the
+    // drawing passes of the previous call on this device may have set bits there
+    // after that call returned, and they are reported below, by this call (the
+    // array starts zeroed when the module is loaded)
+    CK(launch_vertex_setup(*m, ctx->cam, fb, n_tiles, s));
+    CK(launch_face_setup(*m, ctx->cam, make_shade(ctx), fb, tiles_x, tiles_y, ctx->reverse_bins, s));
+    bool ordered = false;
+    CK(launch_tile_scan(fb, n_tiles, &ordered, s));
     uint64_t h[16] = {};  // pageable host copy of the totals (no pinned allocation)
     CK(cudaMemcpyAsync(h + 8, fb.scal + 8, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -2073,10 +2110,9 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
         if (stats) *stats = fs;
         return HEXFC_ERR_OVERFLOW;
     }
-    CK(cudaMemsetAsync(fb.bins, 0xFF, sizeof(uint32_t) * (size_t)n_bins, s));   // padding slots = kPadBin
-    CK(launch_bin_fill(*m, fb, tiles_x, W, H, ctx->reverse_bins, s));
-    CK(launch_bin_sort(*m, fb, tiles_x, tiles_y, (int64_t)n_bins, ctx->depth_buckets, s));
-    CK(launch_tile_order(fb, n_tiles, s));
+    CK(launch_bin_fill(*m, fb, tiles_x, W, H, s));
+    CK(launch_bin_sort(fb, n_tiles, (int64_t)n_bins, ctx->depth_buckets, CapFeatures{}, s));
+    if (!ordered) CK(launch_tile_order(fb, n_tiles, s));
     CK(launch_count(fb, tiles_x, tiles_y, W, H, s));
     CK(cudaMemcpyAsync(h, fb.scal, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -2091,7 +2127,7 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     fs.fragments = total;
     fs.max_list = (uint32_t)h[1];
     fs.long_lists = n_long;
-    fs.kernel_launches = 11 + (sil ? 1u : 0u);
+    fs.kernel_launches = (ordered ? 8 : 11) + (sil ? 1u : 0u);
     if (stats) *stats = fs;
     if (fs.max_list > HEXFC_MAX_LIST) return HEXFC_ERR_OVERFLOW;
     // (the lists must fit the array too, though the drawing pass does not store them)

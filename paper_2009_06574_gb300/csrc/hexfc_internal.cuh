@@ -44,18 +44,20 @@ struct ShadeParams {
     int px_off, py_off;   // drawn rectangle's offset in the frame: pixel (x, y) is frame pixel (x + px_off, ...)
 };
 
-// A face as two records: the per-frame one, written by the face stage of every
-// frame into the rendering context's buffers (with what a triangle's shading
-// record needs that does not depend on the tile, so that it is found once per
-// face and not for every tile the face touches), and the static one (corner
-// importance and world position), owned by the mesh and rewritten only when
-// importance changes, so that contexts can render one resident mesh at the
-// same time.
-struct __align__(32) FaceFrame {
+// A face as two 64-byte records: the per-frame one (window corners, depths,
+// flags, eye depths), written by the face stage of every frame into the
+// rendering context's buffers, and the static one (corner importance and world
+// position), owned by the mesh and rewritten only when importance changes, so
+// that contexts can render one resident mesh at the same time.
+struct __align__(64) FaceFrame {
     int4 X, Y;            // corner window position, 16.8 fixed point
     uint4 Z;              // bits 0-23: corner window depth (z24). Bits 24-31 of Z.x: edge flags (bits 0-3
                           // visible in focus, 4-7 visible in context); of Z.y: face flags (kFace...)
     float4 q;             // 1 / corner eye depth (1 in an orthographic view)
+};
+// What a triangle's shading record needs besides, found once per face instead of
+// for every tile it touches where there is room for it.
+struct __align__(32) FaceExtra {
     float4 nl;            // -1 / squared length of window edge k -> k+1 (0: degenerate)
     uint4 area;           // triangle 0, 1: twice the area if below 2^26, else 0; 1 / the same (float bits)
 };
@@ -63,7 +65,7 @@ struct __align__(64) FaceStatic {
     float4 imp;           // corner importance
     float4 px, py, pz;    // corner world position
 };
-static_assert(sizeof(FaceFrame) == 96 && sizeof(FaceStatic) == 64, "whole 32-byte sectors");
+static_assert(sizeof(FaceFrame) == 64 && sizeof(FaceStatic) == 64, "two sectors each");
 constexpr uint32_t kZ24 = 0xFFFFFFu;
 // Face flags, bit t for triangle t where shifted by it.
 constexpr uint32_t kFaceDrawn = 1u;      // << t: triangle drawn
@@ -141,13 +143,20 @@ struct FrameBufs {
     FaceFrame* fframe = nullptr;    // [F] per-frame face records
     uint32_t* tzsum = nullptr;      // [2F] per triangle (2 face + tri): its depths (pack_depths)
     int64_t f_cap = 0;
+    // binning of triangles that touch at most 2x2 tiles: each pair's place in its tile's list is found
+    // with its count (nullptr: all places are found in a second pass)
+    uint32_t* trange = nullptr;     // [2F] the triangle's tiles (kRange...)
+    uint4* slots = nullptr;         // [2F] places in the lists of its 2x2 tiles
+    FaceExtra* fextra = nullptr;    // [F]
+    int64_t slot_cap = 0;           // faces of these three
+    uint64_t slots_refused = 0;     // the budget that had no room for them
     // tiles
-    uint32_t* tile_cnt = nullptr;   // [T+1]
+    uint32_t* tile_cnt = nullptr;   // [T+1] pairs whose place is known
+    uint32_t* tile_big = nullptr;   // [T+1] the others
     uint64_t* tile_off = nullptr;   // [T+1]
     uint32_t* tile_cur = nullptr;   // [T]
     uint32_t* tile_order = nullptr; // [T] tiles by decreasing chunk count
     uint32_t* tile_frag = nullptr;  // [T] exact fragments per tile (the count's or the fused pass's)
-    float* tile_zr = nullptr;       // [T] depth range of the tile's triangles (fraction of the z24 sum range)
     float* cap_x = nullptr;         // [4T] capacity-network features of the frame
     uint32_t* tile_cap = nullptr;   // [T+1] chosen fragment capacity per tile (predicted frames)
     uint64_t* cap_off = nullptr;    // [T+1] its exclusive prefix
@@ -212,6 +221,7 @@ struct DrawItem {
     const uint32_t* zsuf;
     const FaceFrame* fframe;
     const FaceStatic* fstat;
+    const FaceExtra* fextra;   // nullptr: not kept
     const uint32_t* order;
     const uint32_t* cnt;
     uint32_t* zsil;   // nullptr: no silhouettes
@@ -250,16 +260,24 @@ cudaError_t launch_cell_quality(const DevMesh& m, int metric, float* out, cudaSt
 // positions: also the corners' world positions (once, at the upload).
 cudaError_t launch_importance(const DevMesh& m, bool positions, cudaStream_t s);
 
-cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, cudaStream_t s);
+cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, int64_t n_tiles, cudaStream_t s);
 cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const ShadeParams& sp, FrameBufs& fb,
-                              int tiles_x, int tiles_y, cudaStream_t s);
-cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, int reverse,
-                            cudaStream_t s);
+                              int tiles_x, int tiles_y, int reverse, cudaStream_t s);
+// Tile offsets (whole chunks) and their total into scal[8]; true in *ordered if the tile order is done too.
+cudaError_t launch_tile_scan(FrameBufs& fb, int64_t n_tiles, bool* ordered, cudaStream_t s);
+cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, cudaStream_t s);
+// Constants of the capacity network's features (CapFeatures::X == nullptr: not wanted).
+struct CapFeatures {
+    const uint32_t* prev;   // the previous frame's tile counts, nullptr: none
+    float* X;
+    float lens_x, lens_y, inv_diag, motion;
+    int tiles_x;
+};
 // Kernel attributes (dynamic shared memory limits), once per device context.
 cudaError_t prepare_raster_kernels();
 cudaError_t prepare_draw_kernels();
 
-cudaError_t launch_bin_sort(const DevMesh& m, FrameBufs& fb, int tiles_x, int tiles_y, int64_t n_bins, int buckets,
+cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int buckets, const CapFeatures& cf,
                             cudaStream_t s);
 cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s);
 CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H);
@@ -275,8 +293,6 @@ cudaError_t launch_capacity_from_previous(FrameBufs& fb, int64_t n_tiles, float 
                                           uint32_t uniform, cudaStream_t s);
 // The frame's exact tile counts against the chosen capacities.
 cudaError_t launch_capacity_check(FrameBufs& fb, int64_t n_tiles, cudaStream_t s);
-cudaError_t launch_cap_features(FrameBufs& fb, int64_t n_tiles, int tiles_x, float lens_x, float lens_y,
-                                float inv_diag, float motion, cudaStream_t s);
 cudaError_t launch_cap_forward(const CapNet& net, FrameBufs& fb, int64_t n_tiles, float margin, uint32_t pad,
                                cudaStream_t s);
 cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, cudaStream_t s);
@@ -295,7 +311,7 @@ cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const in
 // scans
 cudaError_t scan_u32_to_u64(const uint32_t* in, uint64_t* out, int64_t n, uint64_t* part,
                             uint32_t* part_max, uint64_t* total_and_max, uint32_t long_threshold,
-                            cudaStream_t s, uint32_t round_to = 0);
+                            cudaStream_t s, uint32_t round_to = 0, const uint32_t* in2 = nullptr);
 int64_t scan_partials_needed(int64_t n);
 
 }  // namespace hexfc

@@ -4,10 +4,11 @@
 // Weights are used in FP16 (staged in shared memory), sums in FP32; training
 // keeps an FP32 master copy and Adam moments. No counterpart in the paper.
 //
-//   k_cap_features  per tile: log1p(previous frame's count) / 12, the depth
-//                   range of its triangles, the distance from the tile to the
-//                   lens on screen / screen diagonal, the camera's motion
-//                   since the previous frame
+// The features (left by the depth order of the tile lists): log1p(previous
+// frame's count) / 12, the depth range of its triangles, the distance from the
+// tile to the lens on screen / screen diagonal, the camera's motion since the
+// previous frame.
+//
 //   k_cap_forward   per tile: y and the capacity expm1(y) (1 + margin) + pad
 //   k_cap_backward  per tile: mean-squared loss on log1p(exact count); stores
 //                   the layer values and the back-propagated errors
@@ -35,21 +36,6 @@ __device__ __forceinline__ void load_weights(const __half* __restrict__ w16, flo
 {
     for (int i = threadIdx.x; i < kCapParams; i += blockDim.x) s_w[i] = __half2float(w16[i]);
     __syncthreads();
-}
-
-__global__ void k_cap_features(int64_t n_tiles, int tiles_x, const uint32_t* __restrict__ prev,
-                               const float* __restrict__ zr, float lens_x, float lens_y, float inv_diag,
-                               float motion, float* __restrict__ X)
-{
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_tiles) return;
-    const float cx = (float)((t % tiles_x) * kTileW) + 0.5f * kTileW;
-    const float cy = (float)((t / tiles_x) * kTileH) + 0.5f * kTileH;
-    const float dx = cx - lens_x, dy = cy - lens_y;
-    X[4 * t + 0] = log1pf((float)prev[t]) * (1.f / 12.f);
-    X[4 * t + 1] = zr[t];
-    X[4 * t + 2] = fminf(sqrtf(dx * dx + dy * dy) * inv_diag, 2.f);
-    X[4 * t + 3] = motion;
 }
 
 __global__ void __launch_bounds__(256) k_cap_forward(const float* __restrict__ X, int64_t n,
@@ -242,14 +228,6 @@ cudaError_t launch_capacity_check(FrameBufs& fb, int64_t n_tiles, cudaStream_t s
 {
     k_capacity_check<<<grid_for(n_tiles, 256), 256, 0, s>>>(fb.tile_frag, fb.cap_off, n_tiles, (uint64_t)fb.frag_cap,
                                                             reinterpret_cast<unsigned long long*>(fb.scal));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cap_features(FrameBufs& fb, int64_t n_tiles, int tiles_x, float lens_x, float lens_y,
-                                float inv_diag, float motion, cudaStream_t s)
-{
-    k_cap_features<<<grid_for(n_tiles, 256), 256, 0, s>>>(n_tiles, tiles_x, fb.tile_frag, fb.tile_zr, lens_x, lens_y,
-                                                          inv_diag, motion, fb.cap_x);
     return cudaGetLastError();
 }
 

@@ -235,7 +235,7 @@ __device__ __forceinline__ uint64_t fragment_key(const DrawItem& a, const PixelR
 __device__ __noinline__ float4 fragment_colour(const DrawItem& a, const PixelRef& r, uint32_t f2t, bool& bad)
 {
     ShadeRec R;
-    make_record(a.fframe[f2t >> 1], a.fstat[f2t >> 1], f2t, r.px0, r.py0, a.sp, R);
+    make_record(a.fframe[f2t >> 1], a.fstat[f2t >> 1], nullptr, f2t, r.px0, r.py0, a.sp, R);
     const Sample s = sample_of(R, R.zf, R.ha, (uint32_t)r.lx << 8, (uint32_t)r.ly << 8, true, bad);
     const int x = r.px0 + r.lx, y = r.py0 + r.ly;
     const float dist = a.sp.lens_mode == HEXFC_LENS_SCREEN ? screen_lens_dist(x, y, a.sp) : 0.f;
@@ -386,7 +386,8 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, in
         uint4* md = reinterpret_cast<uint4*>(&D.mask[((my / 4) * (kTileW / 8) + mx / 8) * 32 + (my % 4) * 8]);
         const uint4 ma = mp[0], mb = mp[1];
         if (f2t_m != kPadBin)
-            make_record(a.fframe[f2t_m >> 1], a.fstat[f2t_m >> 1], f2t_m, px0, py0, a.sp, D.sh[lane]);
+            make_record(a.fframe[f2t_m >> 1], a.fstat[f2t_m >> 1], a.fextra ? a.fextra + (f2t_m >> 1) : nullptr, f2t_m, px0,
+                        py0, a.sp, D.sh[lane]);
         md[0] = ma;
         md[1] = mb;
         mbar_arrive(&S.full[warp]);

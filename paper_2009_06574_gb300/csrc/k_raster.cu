@@ -5,9 +5,9 @@
 //   k_face_setup    per unique face: gather the 4 projected corners, edge
 //                   visibility masks of Eq. 1, triangle validity, and the
 //                   number of raster tiles each triangle's box touches.
-//   k_bin_fill      per face: append 2*face+tri to the list of every touched tile.
+//   k_tile_scan     the tiles' offsets, and the tiles by decreasing work.
+//   k_bin_fill      per triangle: into the list of every touched tile.
 //   k_bin_sort      per tile: counting sort of the tile's triangles by depth.
-//   k_tile_order    the tiles by decreasing work (for count and draw).
 //   k_count         per tile: exact coverage as per-chunk masks and per-pixel
 //                   counts.
 //
@@ -18,7 +18,10 @@
 // Section "GPU Implementation"), and the fragment shader computes focus from
 // the lens, the edge distance to the four face edges ignoring invisible ones,
 // and Eqs. 1-4 (Section "Focus+Context").
+#include <algorithm>
+
 #include "count_tiles.cuh"
+#include "shade.cuh"
 
 namespace hexfc {
 namespace {
@@ -28,12 +31,24 @@ inline unsigned grid_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b);
 // ------------------------------------------------------------------ vertex stage
 
 // Thread per vertex: window position on 1/256 pixel, 24-bit depth, eye depth.
+// It also clears the frame's counters (tile_cnt, tile_big, tile_cur, and the
+// device scalars but the error word), which every frame starts from zero.
 __global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ verts, int64_t n,
                                                       const __grid_constant__ CamParams cam,
                                                       const __grid_constant__ CamPairs pairs,
-                                                      int4* __restrict__ vproj, float* __restrict__ ved)
+                                                      int4* __restrict__ vproj, float* __restrict__ ved,
+                                                      uint32_t* __restrict__ tile_cnt,
+                                                      uint32_t* __restrict__ tile_big,
+                                                      uint32_t* __restrict__ tile_cur, int64_t n_tiles,
+                                                      uint64_t* __restrict__ scal)
 {
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (int64_t i = v; i < n_tiles; i += (int64_t)gridDim.x * blockDim.x) {
+        tile_cnt[i] = 0;
+        tile_big[i] = 0;
+        tile_cur[i] = 0;
+    }
+    if (v < kScalAll && v != 5) scal[v] = 0;
     if (v >= n) return;
     const float x = verts[3 * v], y = verts[3 * v + 1], z = verts[3 * v + 2];
     ProjVertex o;
@@ -43,20 +58,6 @@ __global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ 
 }
 
 // ------------------------------------------------------------------ face stage
-
-// atomicAdd(ctr + idx, 1) for every calling lane, one atomic per distinct idx
-// among the lanes that call together; returns the value this lane's own
-// increment would have returned (lanes of one index in lane order).
-__device__ __forceinline__ uint32_t agg_inc(uint32_t* ctr, int idx)
-{
-    const unsigned act = __activemask();
-    const unsigned peers = __match_any_sync(act, idx);
-    const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(ctr + idx, (uint32_t)__popc(peers));
-    base = __shfl_sync(peers, base, leader);
-    return base + (uint32_t)__popc(peers & ((1u << lane) - 1u));
-}
 
 __device__ __forceinline__ void tile_range(const TriGeom& t, int& tx0, int& ty0, int& tx1, int& ty1)
 {
@@ -112,56 +113,120 @@ __device__ __forceinline__ bool outside_lens(const float (&o)[3][3], const float
     return (ortho || e_lo > 0.f) && lo * inv_r >= 1.0001f + 8e-6f * far * inv_r * ratio;
 }
 
-__global__ void k_face_setup(const int4* __restrict__ fverts, const int4* __restrict__ fedges,
-                             const uint8_t* __restrict__ fbound, const FaceStatic* __restrict__ fstat,
-                             const uint8_t* __restrict__ elevel, const float* __restrict__ eattr,
-                             const int4* __restrict__ vproj, const float* __restrict__ ved, int64_t n_faces,
-                             const __grid_constant__ ShadeParams sp, int W, int H, int tiles_x,
-                             FaceFrame* __restrict__ fframe, uint32_t* __restrict__ tzsum,
-                             uint32_t* __restrict__ tile_cnt)
+// A triangle's tiles in one word: the first one's column and row, whether it
+// touches a second column and row (kRangeSmall), or that there are more than
+// 2x2 (kRangeBig: found again in the second pass).
+constexpr uint32_t kRangeSmall = 1u << 24, kRangeBig = 1u << 25;
+__device__ __forceinline__ uint32_t pack_range(int tx0, int ty0, int tx1, int ty1)
 {
-    int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= n_faces) return;
-    int4 c = fverts[f];
-    int id[4] = {c.x, c.y, c.z, c.w};
+    return (uint32_t)tx0 | ((uint32_t)ty0 << 11) | ((uint32_t)(tx1 - tx0) << 22) | ((uint32_t)(ty1 - ty0) << 23) |
+           kRangeSmall;
+}
+static_assert(16384 / 8 <= 2048, "eleven bits of tile column and row");
+
+// Each lane's place in the counters of up to four tiles (tile < 0: none): one
+// atomic per distinct tile of the warp, lanes of one tile in lane order. All
+// lanes of the warp call it. The four tiles' atomics are in flight together.
+__device__ __forceinline__ uint4 count_places(uint32_t* ctr, const int (&tile)[4])
+{
+    const int lane = threadIdx.x & 31;
+    unsigned peers[4];
+    uint32_t base[4], place[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        peers[k] = __match_any_sync(0xffffffffu, tile[k]);
+        base[k] = 0;
+        if (tile[k] >= 0 && lane == __ffs(peers[k]) - 1) base[k] = atomicAdd(ctr + tile[k], (uint32_t)__popc(peers[k]));
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        place[k] = __shfl_sync(0xffffffffu, base[k], __ffs(peers[k]) - 1) +
+                   (uint32_t)__popc(peers[k] & ((1u << lane) - 1u));
+    return make_uint4(place[0], place[1], place[2], place[3]);
+}
+
+// f(tile) for every tile of the box of each lane that has `big` set, the warp
+// on one lane's box at a time: a triangle over the whole frame is no serial loop.
+template <class F>
+__device__ __forceinline__ void for_big_tiles(bool big, int tx0, int ty0, int tx1, int ty1, int tiles_x, F&& f)
+{
+    const int lane = threadIdx.x & 31;
+    for (unsigned todo = __ballot_sync(0xffffffffu, big); todo != 0; todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        const int x0 = __shfl_sync(0xffffffffu, tx0, src), y0 = __shfl_sync(0xffffffffu, ty0, src);
+        const int w = __shfl_sync(0xffffffffu, tx1, src) - x0 + 1, h = __shfl_sync(0xffffffffu, ty1, src) - y0 + 1;
+        for (int i = lane; i < w * h; i += 32) f((y0 + i / w) * tiles_x + x0 + i % w, src);
+    }
+}
+
+// Thread per face: its record of the frame, its triangles' depths, and the
+// counts of the tiles they touch. Bound by the latency of its gathers and
+// atomics (39% of the issue slots). A triangle of at most 2x2 tiles keeps the
+// places its counts gave it, so that the binning needs no second round of
+// atomics: that pass 64 -> 36 us at 64^3 and 1920x1080, of which the scattered
+// 4-byte writes into 8160 lists remain. Triangles of more tiles are counted by
+// their whole warp (a 4^3 grid at 256x256, one block: 25 + 31 us for both passes
+// with a loop per thread, 12 + 8 us now).
+__global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fverts, const int4* __restrict__ fedges,
+                                                    const uint8_t* __restrict__ fbound,
+                                                    const FaceStatic* __restrict__ fstat,
+                                                    const uint8_t* __restrict__ elevel,
+                                                    const float* __restrict__ eattr, const int4* __restrict__ vproj,
+                                                    const float* __restrict__ ved, int64_t n_faces,
+                                                    const __grid_constant__ ShadeParams sp, int W, int H, int tiles_x,
+                                                    int reverse, FaceFrame* __restrict__ fframe,
+                                                    uint32_t* __restrict__ tzsum, uint32_t* __restrict__ trange,
+                                                    uint4* __restrict__ slots, FaceExtra* __restrict__ fextra,
+                                                    uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_big)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = i < n_faces;
+    const int64_t f = !in ? 0 : reverse ? n_faces - 1 - i : i;
+    const int4 c = fverts[f], e = fedges[f];
+    const int id[4] = {c.x, c.y, c.z, c.w}, eid[4] = {e.x, e.y, e.z, e.w};
     int32_t X[4], Y[4];
     uint32_t Z[4];
     float E[4];
     bool ok[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        int4 p = vproj[id[k]];
-        X[k] = p.x; Y[k] = p.y; Z[k] = (uint32_t)p.z & kZ24; ok[k] = p.w != 0;
+        const int4 p = vproj[id[k]];
+        X[k] = p.x; Y[k] = p.y; Z[k] = (uint32_t)p.z & kZ24; ok[k] = in && p.w != 0;
         E[k] = ved[id[k]];
     }
-    int4 e = fedges[f];
-    int eid[4] = {e.x, e.y, e.z, e.w};
     uint32_t edges = 0, flags = fbound[f] ? kFaceBoundary : 0u;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        bool vis_c = (int)elevel[eid[k]] >= sp.lod;
-        bool vis_f = vis_c || eattr[eid[k]] >= sp.delta;
+        const bool vis_c = (int)elevel[eid[k]] >= sp.lod;
+        const bool vis_f = vis_c || eattr[eid[k]] >= sp.delta;
         edges |= (vis_f ? 1u : 0u) << k;
         edges |= (vis_c ? 1u : 0u) << (4 + k);
     }
-    uint32_t area[2] = {0u, 0u};
-    float ia[2] = {0.f, 0.f};
+    uint32_t range[2] = {0u, 0u}, area[2] = {0u, 0u};
+    uint4 place[2];
 #pragma unroll
     for (int tri = 0; tri < 2; ++tri) {
-        bool vok = ok[0] && (tri == 0 ? (ok[1] && ok[2]) : (ok[2] && ok[3]));
-        if (!vok) continue;
+        const bool vok = ok[0] && ok[1 + tri] && ok[2 + tri];
         TriGeom t;
         tri_setup(X, Y, tri, W, H, t);
-        if (!t.valid) continue;
-        flags |= kFaceDrawn << tri;
-        if (t.vi[1] != 1 + tri) flags |= kFaceSwapped << tri;
-        area[tri] = t.area < (1ll << 26) ? (uint32_t)t.area : 0u;
-        ia[tri] = 1.f / u64_to_f32((uint64_t)t.area);
-        int tx0, ty0, tx1, ty1;
-        tile_range(t, tx0, ty0, tx1, ty1);
-        for (int ty = ty0; ty <= ty1; ++ty)
-            for (int tx = tx0; tx <= tx1; ++tx) agg_inc(tile_cnt, ty * tiles_x + tx);
+        const bool drawn = vok && t.valid;
+        int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
+        if (drawn) {
+            flags |= kFaceDrawn << tri;
+            if (t.vi[1] != 1 + tri) flags |= kFaceSwapped << tri;
+            area[tri] = t.area < (1ll << 26) ? (uint32_t)t.area : 0u;
+            tile_range(t, tx0, ty0, tx1, ty1);
+        }
+        const bool small = drawn && slots && tx1 - tx0 <= 1 && ty1 - ty0 <= 1;
+        if (small) range[tri] = pack_range(tx0, ty0, tx1, ty1);
+        else if (drawn) range[tri] = kRangeBig;
+        const int t0 = ty0 * tiles_x + tx0;
+        const bool c2 = small && tx1 > tx0, r2 = small && ty1 > ty0;
+        const int tile[4] = {small ? t0 : -1, c2 ? t0 + 1 : -1, r2 ? t0 + tiles_x : -1, c2 && r2 ? t0 + tiles_x + 1 : -1};
+        place[tri] = count_places(tile_cnt, tile);
+        for_big_tiles(drawn && !small, tx0, ty0, tx1, ty1, tiles_x, [&](int at, int) { atomicAdd(tile_big + at, 1u); });
     }
+    if (!in) return;
     if (sp.lens_mode == HEXFC_LENS_SPHERE && sp.bounded && (flags & (3u * kFaceDrawn))) {
         const float4 px = fstat[f].px, py = fstat[f].py, pz = fstat[f].pz;
         const float o[4][3] = {{px.x - sp.lens_c[0], py.x - sp.lens_c[1], pz.x - sp.lens_c[2]},
@@ -177,218 +242,305 @@ __global__ void k_face_setup(const int4* __restrict__ fverts, const int4* __rest
             if (outside_lens(v, d, sp.ortho != 0, sp.lens_inv_r)) flags |= kFaceOut << tri;
         }
     }
-    float nl[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int k1 = (k + 1) & 3;
-        const int32_t ex = X[k1] - X[k], ey = Y[k1] - Y[k];
-        const float l2 = u64_to_f32((uint64_t)((int64_t)ex * ex + (int64_t)ey * ey));
-        nl[k] = l2 > 0.f ? -(1.f / l2) : 0.f;
-    }
     FaceFrame& r = fframe[f];
     r.X = make_int4(X[0], X[1], X[2], X[3]);
     r.Y = make_int4(Y[0], Y[1], Y[2], Y[3]);
     r.Z = make_uint4(Z[0] | (edges << 24), Z[1] | (flags << 24), Z[2], Z[3]);
-    r.q = sp.ortho ? make_float4(1.f, 1.f, 1.f, 1.f) : make_float4(1.f / E[0], 1.f / E[1], 1.f / E[2], 1.f / E[3]);
-    r.nl = make_float4(nl[0], nl[1], nl[2], nl[3]);
-    r.area = make_uint4(area[0], area[1], __float_as_uint(ia[0]), __float_as_uint(ia[1]));
+    r.q = sp.ortho ? make_float4(1.f, 1.f, 1.f, 1.f)
+                   : make_float4(__frcp_rn(E[0]), __frcp_rn(E[1]), __frcp_rn(E[2]), __frcp_rn(E[3]));
     reinterpret_cast<uint2*>(tzsum)[f] = make_uint2(pack_depths(Z[0], Z[1], Z[2]), pack_depths(Z[0], Z[2], Z[3]));
+    if (slots) {
+        reinterpret_cast<uint2*>(trange)[f] = make_uint2(range[0], range[1]);
+        fextra[f].nl = edge_scales(r.X, r.Y);
+        fextra[f].area = make_uint4(area[0], area[1], __float_as_uint(__frcp_rn((float)area[0])),
+                                    __float_as_uint(__frcp_rn((float)area[1])));
+        if (range[0] & kRangeSmall) slots[2 * f] = place[0];
+        if (range[1] & kRangeSmall) slots[2 * f + 1] = place[1];
+    }
 }
 
-__global__ void k_bin_fill(const FaceFrame* __restrict__ fframe, int64_t n_faces, int W, int H, int tiles_x,
-                           int reverse, const uint64_t* __restrict__ tile_off, uint32_t* __restrict__ tile_cur,
-                           uint32_t* __restrict__ bins)
+// Thread per triangle (2 face + triangle): into the lists of its tiles.
+__global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ fframe,
+                                                  const uint32_t* __restrict__ trange, const uint4* __restrict__ slots,
+                                                  int64_t n_tris, int W, int H, int tiles_x,
+                                                  const uint64_t* __restrict__ tile_off,
+                                                  const uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_cur,
+                                                  uint32_t* __restrict__ bins)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_faces) return;
-    int64_t f = reverse ? (n_faces - 1 - i) : i;
-    const uint32_t tris = face_tris(fframe[f].Z);
-    if (tris == 0) return;
-    int4 a = fframe[f].X, b = fframe[f].Y;
-    int32_t X[4] = {a.x, a.y, a.z, a.w}, Y[4] = {b.x, b.y, b.z, b.w};
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t range = 0;
+    if (t < n_tris)
+        range = trange ? trange[t] : (face_tris(fframe[t >> 1].Z) >> (t & 1)) & 1u ? kRangeBig : 0u;
+    if (range & kRangeSmall) {
+        const uint4 p = slots[t];
+        const int tile = (int)((range >> 11) & 2047u) * tiles_x + (int)(range & 2047u);
+        const bool c2 = (range >> 22) & 1u, r2 = (range >> 23) & 1u;
+        bins[tile_off[tile] + p.x] = (uint32_t)t;
+        if (c2) bins[tile_off[tile + 1] + p.y] = (uint32_t)t;
+        if (r2) bins[tile_off[tile + tiles_x] + p.z] = (uint32_t)t;
+        if (c2 && r2) bins[tile_off[tile + tiles_x + 1] + p.w] = (uint32_t)t;
+    }
+    int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
+    if (range & kRangeBig) {
+        const int4 a = fframe[t >> 1].X, b = fframe[t >> 1].Y;
+        const int32_t X[4] = {a.x, a.y, a.z, a.w}, Y[4] = {b.x, b.y, b.z, b.w};
+        TriGeom g;
+        tri_setup(X, Y, (int)(t & 1), W, H, g);
+        tile_range(g, tx0, ty0, tx1, ty1);
+    }
+    const int64_t first = t - (threadIdx.x & 31);
+    for_big_tiles(range & kRangeBig, tx0, ty0, tx1, ty1, tiles_x, [&](int tile, int src) {
+        bins[tile_off[tile] + tile_cnt[tile] + atomicAdd(tile_cur + tile, 1u)] = (uint32_t)(first + src);
+    });
+}
+
+// ------------------------------------------------------------------ tile offsets and order
+
+constexpr int kScanTiles = 16384;   // most tiles of the one-block scan (16 a thread)
+
+// One block: the tiles' offsets in the bins (each list padded to whole chunks)
+// and the tiles in decreasing order of their chunks (a counting sort into 1024
+// classes; order inside a class is arbitrary, no result depends on it), so that
+// the per-tile passes start the longest tiles first and the shortest ones fill
+// the tail of the launch. One launch for what four took (64^3 at 1920x1080, 8160
+// tiles: 14 us, before 13 for the scan and 19 for the order).
+__global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__ tile_cnt,
+                                                    const uint32_t* __restrict__ tile_big, int n,
+                                                    uint64_t* __restrict__ tile_off, uint32_t* __restrict__ order,
+                                                    uint64_t* __restrict__ total)
+{
+    constexpr int kPer = kScanTiles / 1024;
+    __shared__ uint32_t s_hist[1024], s_warp[32], s_max[32], s_empty;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (n + 1023) / 1024, t0 = threadIdx.x * per;
+    uint32_t nc[kPer], sum = 0, mx = 0;
 #pragma unroll
-    for (int tri = 0; tri < 2; ++tri) {
-        if (!(tris & (1u << tri))) continue;
-        TriGeom t;
-        tri_setup(X, Y, tri, W, H, t);
-        int tx0, ty0, tx1, ty1;
-        tile_range(t, tx0, ty0, tx1, ty1);
-        for (int ty = ty0; ty <= ty1; ++ty)
-            for (int tx = tx0; tx <= tx1; ++tx) {
-                int tile = ty * tiles_x + tx;
-                const uint32_t slot = agg_inc(tile_cur, tile);
-                bins[tile_off[tile] + slot] = (uint32_t)(2 * f + tri);
+    for (int k = 0; k < kPer; ++k) {
+        const int t = t0 + k;
+        nc[k] = k < per && t < n ? (tile_cnt[t] + tile_big[t] + kChunk - 1) / kChunk : 0u;
+        sum += nc[k];
+        mx = max(mx, nc[k]);
+    }
+    s_hist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_empty = 0;
+    auto block_scan = [&](uint32_t v) -> uint32_t {   // exclusive, over the block's threads
+        uint32_t incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        __syncthreads();
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        uint32_t w = s_warp[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        const uint32_t before = __shfl_sync(0xffffffffu, w, warp - 1);
+        return incl - v + (warp > 0 ? before : 0u);
+    };
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) s_max[warp] = mx;
+    uint64_t at = block_scan(sum);   // (fewer than 2^32 chunks: its barriers publish s_max, s_hist, s_empty too)
+    mx = __reduce_max_sync(0xffffffffu, s_max[lane]);
+    int shift = 0;
+    while ((mx >> shift) >= 1024u) ++shift;
+    uint32_t rank[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int t = t0 + k;
+        const bool here = k < per && t < n;
+        if (here) tile_off[t] = at * kChunk;
+        at += nc[k];
+        // empty tiles (often most of them) are counted by the warp, the others one by one
+        rank[k] = 0;
+        if (k < per) {
+            const unsigned none = __ballot_sync(0xffffffffu, here && nc[k] == 0);
+            uint32_t base = 0;
+            if (none && lane == 0) base = atomicAdd(&s_empty, (uint32_t)__popc(none));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (here) {
+                if (nc[k] == 0) rank[k] = base + (uint32_t)__popc(none & ((1u << lane) - 1u));
+                else rank[k] = atomicAdd(&s_hist[1023u - (nc[k] >> shift)], 1u);
             }
+        }
+    }
+    if (threadIdx.x == 1023) {
+        tile_off[n] = at * kChunk;
+        *total = at * kChunk;
+    }
+    __syncthreads();
+    const uint32_t h = s_hist[threadIdx.x];
+    const uint32_t first = block_scan(h);
+    s_hist[threadIdx.x] = first;
+    __syncthreads();
+    const uint32_t filled = (uint32_t)n - s_empty;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int t = t0 + k;
+        if (k < per && t < n)
+            order[(nc[k] == 0 ? filled : s_hist[1023u - (nc[k] >> shift)]) + rank[k]] = (uint32_t)t;
     }
 }
 
 // ------------------------------------------------------------------ bin order
 
-constexpr int kBinSortMax = 4096;   // longer tile lists are sorted through global scratch
 constexpr int kDepthBucketsMax = 4096;
+__host__ __device__ constexpr size_t sort_smem(int threads, int items, int nb)
+{
+    const size_t cap = (size_t)threads * items;
+    return sizeof(uint32_t) * (cap + (size_t)(nb < threads ? threads : nb) + cap / kChunk + 64);
+}
 
 // Orders each tile's list front to back by a counting sort of the triangles
-// into nb buckets (a power of two, 256..kDepthBucketsMax) of their depth (sum of the three window depths)
-// over the tile's depth range; the padding slots stay at the end. Any order
-// gives the same image; this one makes every pixel meet its fragments sorted or
-// nearly sorted (order within a bucket is arbitrary). zsuf receives, per chunk,
-// a lower bound of the depths of the triangles from that chunk on: a pixel that
-// is opaque in front of it is finished.
-__global__ void __launch_bounds__(256) k_bin_sort(const uint64_t* __restrict__ tile_off,
-                                                  const uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ bins,
-                                                  const uint32_t* __restrict__ tzsum, int nb,
-                                                  float* __restrict__ tile_zr, uint32_t* __restrict__ tmp,
-                                                  uint32_t* __restrict__ zsuf)
+// into nb buckets (a power of two, 256..kDepthBucketsMax) of their depth (sum of
+// the three window depths) over the tile's depth range, and pads it to whole
+// chunks. Any order gives the same image; this one makes every pixel meet its
+// fragments sorted or nearly sorted (order within a bucket is arbitrary). zsuf
+// receives, per chunk, a lower bound of the depths of the triangles from that
+// chunk on: a pixel that is opaque in front of it is finished. nb 0: no order.
+//
+// A block of kT threads holds up to kT * kItems entries in registers (read
+// once); longer lists go through global scratch. The block also leaves the tile's
+// features of the capacity network (cf).
+template <int kT, int kItems>
+__global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bin_sort(const uint64_t* __restrict__ tile_off,
+                                                            const uint32_t* __restrict__ tile_cnt,
+                                                 const uint32_t* __restrict__ tile_big, uint32_t* __restrict__ bins,
+                                                 const uint32_t* __restrict__ tzsum, int nb,
+                                                 uint32_t* __restrict__ tmp, uint32_t* __restrict__ zsuf,
+                                                 const CapFeatures cf)
 {
-    constexpr int kItems = kBinSortMax / 256;   // entries per thread of a list held in registers
-    __shared__ uint32_t s_hist[kDepthBucketsMax];
-    __shared__ uint32_t s_out[kBinSortMax];
-    __shared__ uint32_t s_red[2][8];
-    __shared__ uint32_t s_low[kBinSortMax / kChunk];   // least depth of each chunk
+    constexpr uint32_t kMax = kT * kItems, kLow = kMax / kChunk;
+    extern __shared__ uint32_t sort_sm[];
+    uint32_t* s_out = sort_sm;                 // [kMax]
+    uint32_t* s_low = s_out + kMax;            // [kLow] least depth of each chunk
+    uint32_t* s_red = s_low + kLow;            // [2][32]
+    uint32_t* s_hist = s_red + 64;             // [max(nb, kT)]
     const int tile = blockIdx.x;
     const uint64_t beg = tile_off[tile];
-    const uint32_t n = tile_cnt[tile];   // real entries; the rest of the padded list is kPadBin
-    if (n < 2) {   // nothing to order; depth range 0
-        if (threadIdx.x == 0) {
-            tile_zr[tile] = 0.f;
-            if (n) zsuf[beg / kChunk] = 0u;
-        }
-        return;
-    }
+    const uint32_t n = tile_cnt[tile] + tile_big[tile];
     const uint32_t n_chunks = (n + kChunk - 1) / kChunk;
-    const bool big = n > (uint32_t)kBinSortMax;   // entries re-read, scatter through tmp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // a list of up to kBinSortMax entries is read once: entry tid + 256 k of
-    // the list and its triangle's depth sum (sum of the three window depths)
-    // stay in this thread's registers
-    uint32_t f2t[kItems], zs[kItems];
+    for (uint32_t i = n + threadIdx.x; i < n_chunks * kChunk; i += kT) bins[beg + i] = kPadBin;
     uint32_t zmin = 0xFFFFFFFFu, zmax = 0;
-    if (!big) {
+    if (n < 2 || nb == 0) {   // nothing to order
+        for (uint32_t i = threadIdx.x; i < n_chunks; i += kT) zsuf[beg / kChunk + i] = 0u;
+        zmin = 0;
+    } else {
+        const bool big = n > kMax;   // entries re-read, scatter through tmp
+        uint32_t f2t[kItems], zs[kItems];
+        if (!big) {
 #pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            const uint32_t i = threadIdx.x + 256u * k;
-            f2t[k] = i < n ? bins[beg + i] : 0u;
-        }
+            for (int k = 0; k < kItems; ++k) {
+                const uint32_t i = threadIdx.x + (uint32_t)(kT * k);
+                if (kT * k >= (int)n) break;   // (the same for the block)
+                f2t[k] = i < n ? bins[beg + i] : 0u;
+            }
 #pragma unroll
-        for (int k = 0; k < kItems; ++k) {
-            const uint32_t i = threadIdx.x + 256u * k;
-            zs[k] = i < n ? tzsum[f2t[k]] : 0u;
-            if (i < n) {
-                zmin = min(zmin, zs[k] & kZSum);
+            for (int k = 0; k < kItems; ++k) {
+                if (kT * k >= (int)n) break;
+                const bool in = threadIdx.x + (uint32_t)(kT * k) < n;
+                zs[k] = in ? tzsum[f2t[k]] : 0u;
+                zmin = min(zmin, in ? zs[k] & kZSum : 0xFFFFFFFFu);
                 zmax = max(zmax, zs[k] & kZSum);
             }
-        }
-    } else {
-        for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-            const uint32_t z = tzsum[bins[beg + i]] & kZSum;
-            zmin = min(zmin, z);
-            zmax = max(zmax, z);
-        }
-    }
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) s_hist[i] = 0;
-    if (threadIdx.x < kBinSortMax / kChunk) s_low[threadIdx.x] = 0xFFFFFFFFu;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        zmin = min(zmin, __shfl_xor_sync(0xffffffffu, zmin, o));
-        zmax = max(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
-    }
-    if (lane == 0) { s_red[0][warp] = zmin; s_red[1][warp] = zmax; }
-    __syncthreads();
-    zmin = s_red[0][0];
-    zmax = s_red[1][0];
-    for (int w = 1; w < 8; ++w) { zmin = min(zmin, s_red[0][w]); zmax = max(zmax, s_red[1][w]); }
-    const float scale = (float)nb / (float)(zmax - zmin + 1);
-    if (threadIdx.x == 0) tile_zr[tile] = (float)(zmax - zmin) * (1.f / 50331648.f);   // of 3 * 2^24
-    auto bucket = [&](uint32_t z) -> int { return min((int)((float)((z & kZSum) - zmin) * scale), nb - 1); };
-    // histogram
-    if (!big) {
-#pragma unroll
-        for (int k = 0; k < kItems; ++k)
-            if (threadIdx.x + 256u * k < n) atomicAdd(&s_hist[bucket(zs[k])], 1u);
-    } else {
-        for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&s_hist[bucket(tzsum[bins[beg + i]])], 1u);
-    }
-    __syncthreads();
-    // exclusive scan of the histogram: nb / 256 buckets per thread
-    {
-        const int per = nb / 256;
-        uint32_t v[kDepthBucketsMax / 256], sum = 0;
-#pragma unroll
-        for (int k = 0; k < kDepthBucketsMax / 256; ++k) {
-            v[k] = k < per ? s_hist[threadIdx.x * per + k] : 0u;
-            sum += v[k];
-        }
-        uint32_t incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        __syncthreads();   // everyone has read s_hist
-        if (lane == 31) s_red[0][warp] = incl;
-        __syncthreads();
-        uint32_t base = incl - sum;
-        for (int w = 0; w < warp; ++w) base += s_red[0][w];
-#pragma unroll
-        for (int k = 0; k < kDepthBucketsMax / 256; ++k) {
-            if (k < per) s_hist[threadIdx.x * per + k] = base;
-            base += v[k];
-        }
-    }
-    __syncthreads();
-    // scatter (arbitrary order inside a bucket), then write back
-    if (!big) {
-#pragma unroll
-        for (int k = 0; k < kItems; ++k)
-            if (threadIdx.x + 256u * k < n) {
-                const uint32_t at = atomicAdd(&s_hist[bucket(zs[k])], 1u);
-                s_out[at] = f2t[k];
-                atomicMin(&s_low[at / kChunk], packed_least(zs[k]));
+        } else {
+            for (uint32_t i = threadIdx.x; i < n; i += kT) {
+                const uint32_t z = tzsum[bins[beg + i]] & kZSum;
+                zmin = min(zmin, z);
+                zmax = max(zmax, z);
             }
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) bins[beg + i] = s_out[i];
-        if (warp == 0) {   // the least from each chunk on: four chunks a lane
-            constexpr int kPer = kBinSortMax / kChunk / 32;
-            uint32_t v[kPer], low = 0xFFFFFFFFu;
-#pragma unroll
-            for (int k = kPer - 1; k >= 0; --k) {
-                low = min(low, s_low[lane * kPer + k]);
-                v[k] = low;
-            }
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {   // over the higher lanes
-                const uint32_t y = __shfl_down_sync(0xffffffffu, low, o);
-                if (lane + o < 32) low = min(low, y);
-            }
-            uint32_t after = __shfl_down_sync(0xffffffffu, low, 1);
-            if (lane == 31) after = 0xFFFFFFFFu;
-#pragma unroll
-            for (int k = 0; k < kPer; ++k)
-                if ((uint32_t)(lane * kPer + k) < n_chunks) zsuf[beg / kChunk + lane * kPer + k] = min(v[k], after);
         }
-    } else {
-        for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-            const uint32_t f = bins[beg + i];
-            tmp[beg + atomicAdd(&s_hist[bucket(tzsum[f])], 1u)] = f;
+        for (int i = threadIdx.x; i < nb; i += kT) s_hist[i] = 0;
+        for (uint32_t i = threadIdx.x; i < kLow; i += kT) s_low[i] = 0xFFFFFFFFu;
+        zmin = __reduce_min_sync(0xffffffffu, zmin);
+        zmax = __reduce_max_sync(0xffffffffu, zmax);
+        if (lane == 0) {
+            s_red[warp] = zmin;
+            s_red[32 + warp] = zmax;
         }
         __syncthreads();
-        for (uint32_t i = threadIdx.x; i < n_chunks * kChunk; i += blockDim.x) {   // (a warp: one chunk)
-            uint32_t low = 0xFFFFFFFFu;
-            if (i < n) {
-                const uint32_t f = tmp[beg + i];
-                bins[beg + i] = f;
-                low = packed_least(tzsum[f]);
+        zmin = __reduce_min_sync(0xffffffffu, s_red[lane % (kT / 32)]);
+        zmax = __reduce_max_sync(0xffffffffu, s_red[32 + lane % (kT / 32)]);
+        const float scale = (float)nb / (float)(zmax - zmin + 1);
+        auto bucket = [&](uint32_t z) -> int { return min((int)((float)((z & kZSum) - zmin) * scale), nb - 1); };
+        // histogram
+        if (!big) {
+#pragma unroll
+            for (int k = 0; k < kItems; ++k) {
+                if (kT * k >= (int)n) break;
+                if (threadIdx.x + (uint32_t)(kT * k) < n) atomicAdd(&s_hist[bucket(zs[k])], 1u);
             }
-            low = __reduce_min_sync(0xffffffffu, low);
-            if (lane == 0) zsuf[(beg + i) / kChunk] = low;
+        } else {
+            for (uint32_t i = threadIdx.x; i < n; i += kT) atomicAdd(&s_hist[bucket(tzsum[bins[beg + i]])], 1u);
+        }
+        __syncthreads();
+        // exclusive scan of the histogram: nb / kT buckets a thread (at least one)
+        {
+            const int per = nb >= kT ? nb / kT : 1;
+            const bool mine = (int)threadIdx.x * per < nb;
+            uint32_t* h = s_hist + threadIdx.x * per;
+            uint32_t sum = 0;
+            for (int k = 0; k < per && mine; ++k) sum += h[k];
+            uint32_t incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            __syncthreads();   // s_red has been read
+            if (lane == 31) s_red[warp] = incl;
+            __syncthreads();
+            const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? s_red[lane] : 0u);
+            uint32_t base = before + incl - sum;
+            for (int k = 0; k < per && mine; ++k) {
+                const uint32_t v = h[k];
+                h[k] = base;
+                base += v;
+            }
+        }
+        __syncthreads();
+        // scatter (arbitrary order inside a bucket), then write back
+        if (!big) {
+#pragma unroll
+            for (int k = 0; k < kItems; ++k) {
+                if (kT * k >= (int)n) break;
+                if (threadIdx.x + (uint32_t)(kT * k) < n) {
+                    const uint32_t at = atomicAdd(&s_hist[bucket(zs[k])], 1u);
+                    s_out[at] = f2t[k];
+                    atomicMin(&s_low[at / kChunk], packed_least(zs[k]));
+                }
+            }
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < n; i += kT) bins[beg + i] = s_out[i];
+        } else {
+            for (uint32_t i = threadIdx.x; i < n; i += kT) {
+                const uint32_t f = bins[beg + i];
+                tmp[beg + atomicAdd(&s_hist[bucket(tzsum[f])], 1u)] = f;
+            }
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < n_chunks * kChunk; i += kT) {   // (a warp: one chunk)
+                uint32_t low = 0xFFFFFFFFu;
+                if (i < n) {
+                    const uint32_t f = tmp[beg + i];
+                    bins[beg + i] = f;
+                    low = packed_least(tzsum[f]);
+                }
+                low = __reduce_min_sync(0xffffffffu, low);
+                if (lane == 0) zsuf[(beg + i) / kChunk] = low;
+            }
         }
         __syncthreads();
         if (warp == 0) {   // the least from each chunk on, 32 chunks at a time from the end
             uint32_t after = 0xFFFFFFFFu;
             for (int c0 = (int)((n_chunks - 1) & ~31u); c0 >= 0; c0 -= 32) {
-                uint32_t* z = zsuf + beg / kChunk + c0 + lane;
                 const bool in = (uint32_t)(c0 + lane) < n_chunks;
-                uint32_t low = in ? *z : 0xFFFFFFFFu;
+                uint32_t* z = zsuf + beg / kChunk + c0 + lane;
+                uint32_t low = !in ? 0xFFFFFFFFu : big ? *z : s_low[c0 + lane];
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const uint32_t y = __shfl_down_sync(0xffffffffu, low, o);
@@ -399,6 +551,19 @@ __global__ void __launch_bounds__(256) k_bin_sort(const uint64_t* __restrict__ t
                 after = __shfl_sync(0xffffffffu, low, 0);
             }
         }
+    }
+    if (cf.X && threadIdx.x == 0) {
+        // log of the previous frame's count, the tile's depth range (of 3 * 2^24), its
+        // distance to the lens on screen, the camera's motion
+        const float cx = (float)((tile % cf.tiles_x) * kTileW) + 0.5f * kTileW;
+        const float cy = (float)((tile / cf.tiles_x) * kTileH) + 0.5f * kTileH;
+        const float dx = cx - cf.lens_x, dy = cy - cf.lens_y;
+        float4 x;
+        x.x = log1pf(cf.prev ? (float)cf.prev[tile] : 0.f) * (1.f / 12.f);
+        x.y = (float)(zmax - zmin) * (1.f / 50331648.f);
+        x.z = fminf(sqrtf(dx * dx + dy * dy) * cf.inv_diag, 2.f);
+        x.w = cf.motion;
+        reinterpret_cast<float4*>(cf.X)[tile] = x;
     }
 }
 
@@ -421,10 +586,8 @@ __device__ __forceinline__ uint32_t warp_add_same(uint32_t* s, uint32_t b, bool 
     return base + (uint32_t)__popc(peers & ((1u << lane) - 1u));
 }
 
-// The tiles in decreasing order of their number of chunks (a counting sort),
-// so that the per-tile passes start the longest tiles first and the shortest
-// ones fill the tail of the launch. Order inside a class is arbitrary; no
-// result depends on it. One block.
+// The tiles in decreasing order of their number of chunks, as k_tile_scan
+// leaves them, for frames of more tiles than that takes. One block.
 __global__ void __launch_bounds__(1024) k_tile_order(const uint64_t* __restrict__ tile_off, int n_tiles,
                                                      uint32_t* __restrict__ order)
 {
@@ -578,46 +741,67 @@ cudaError_t prepare_raster_kernels()
     cudaError_t e = cudaFuncSetAttribute(k_count, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(kConsumerWarps * sizeof(CountWarp)));
     if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_bin_sort<1024, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sort_smem(1024, 16, kDepthBucketsMax));
+    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_count_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(kConsumerWarps * sizeof(CountWarp)));
     return e;
 }
 
-cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, cudaStream_t s)
+cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, int64_t n_tiles, cudaStream_t s)
 {
-    k_vertex_setup<<<grid_for(m.n_verts, 256), 256, 0, s>>>(m.verts, m.n_verts, cam, cam_pairs(cam), fb.vproj, fb.ved);
+    const unsigned tiles = std::min(grid_for(n_tiles, 256), 1216u);   // (two blocks' worth of clears an SM at most)
+    k_vertex_setup<<<std::max(grid_for(m.n_verts, 256), tiles), 256, 0, s>>>(m.verts, m.n_verts, cam, cam_pairs(cam),
+                                                                             fb.vproj, fb.ved, fb.tile_cnt, fb.tile_big,
+                                                                             fb.tile_cur, n_tiles, fb.scal);
     return cudaGetLastError();
 }
 
 cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const ShadeParams& sp, FrameBufs& fb,
-                              int tiles_x, int tiles_y, cudaStream_t s)
+                              int tiles_x, int tiles_y, int reverse, cudaStream_t s)
 {
     (void)tiles_y;
     k_face_setup<<<grid_for(m.n_faces, 256), 256, 0, s>>>(m.fverts, m.fedges, m.fbound, m.fstat.get(), m.elevel,
                                                            m.eattr, fb.vproj, fb.ved, m.n_faces, sp, cam.W, cam.H,
-                                                           tiles_x, fb.fframe, fb.tzsum, fb.tile_cnt);
+                                                           tiles_x, reverse, fb.fframe, fb.tzsum, fb.trange, fb.slots, fb.fextra,
+                                                           fb.tile_cnt, fb.tile_big);
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, int reverse,
-                            cudaStream_t s)
+cudaError_t launch_tile_scan(FrameBufs& fb, int64_t n_tiles, bool* ordered, cudaStream_t s)
 {
-    k_bin_fill<<<grid_for(m.n_faces, 256), 256, 0, s>>>(fb.fframe, m.n_faces, W, H, tiles_x, reverse,
-                                                         fb.tile_off, fb.tile_cur, fb.bins);
+    *ordered = n_tiles <= kScanTiles;
+    if (!*ordered)
+        return scan_u32_to_u64(fb.tile_cnt, fb.tile_off, n_tiles, fb.part, fb.part_max, fb.scal + 8, 0xFFFFFFFFu, s,
+                               (uint32_t)kChunk, fb.tile_big);
+    k_tile_scan<<<1, 1024, 0, s>>>(fb.tile_cnt, fb.tile_big, (int)n_tiles, fb.tile_off, fb.tile_order, fb.scal + 8);
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin_sort(const DevMesh& m, FrameBufs& fb, int tiles_x, int tiles_y, int64_t n_bins, int buckets,
+cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, cudaStream_t s)
+{
+    k_bin_fill<<<grid_for(2 * m.n_faces, 256), 256, 0, s>>>(fb.fframe, fb.trange, fb.slots, 2 * m.n_faces, W, H,
+                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int buckets, const CapFeatures& cf,
                             cudaStream_t s)
 {
-    (void)m;
-    if (buckets == 0) {   // no depth order (lists keep the faces' arrival order); depth ranges unknown
-        const cudaError_t e = cudaMemsetAsync(fb.tile_zr, 0, sizeof(float) * (size_t)tiles_x * tiles_y, s);
-        if (e != cudaSuccess) return e;
-        return cudaMemsetAsync(fb.zsuf, 0, sizeof(uint32_t) * (size_t)(n_bins / kChunk), s);
-    }
-    k_bin_sort<<<(unsigned)(tiles_x * tiles_y), 256, 0, s>>>(fb.tile_off, fb.tile_cnt, fb.bins, fb.tzsum, buckets,
-                                                              fb.tile_zr, fb.bins_tmp, fb.zsuf);
+    auto go = [&](auto kernel, int threads, int items) {
+        kernel<<<(unsigned)n_tiles, threads, sort_smem(threads, items, buckets), s>>>(
+            fb.tile_off, fb.tile_cnt, fb.tile_big, fb.bins, fb.tzsum, buckets, fb.bins_tmp, fb.zsuf, cf);
+    };
+    // Many tiles: several blocks an SM, to go on with others while one waits at its
+    // barriers; 16 entries a thread where lists of more than 8 x 256 are common
+    // (128^3 at 3840x2160, 1050 a tile: 0.45 ms, with 8 entries 0.85; 64^3 at
+    // 1920x1080, 500 a tile: 8 entries 0.061 ms, 16 entries 0.076). Few tiles with
+    // long lists (a large mesh drawn small): most of an SM for each (96^3 at
+    // 320x180: 0.51 ms with 256 threads, 0.07 with 1024).
+    if (n_bins <= 768 * n_tiles) go(k_bin_sort<256, 8>, 256, 8);
+    else if (n_tiles > 1024) go(k_bin_sort<256, 16>, 256, 16);
+    else go(k_bin_sort<1024, 16>, 1024, 16);
     return cudaGetLastError();
 }
 

@@ -38,21 +38,35 @@ constexpr uint32_t kRecEdge = 1u << 30;    // an edge of the face is visible in 
 constexpr uint32_t kRecBound = 1u << 29;   // a boundary face
 constexpr uint32_t kRecArea = (1u << 26) - 1u;
 
-// The record of triangle f2t (from the records F, S of its face) for the tile
-// whose first pixel is (px0, py0). The positions are read only where the
-// sphere lens may reach.
-__device__ __forceinline__ void make_record(const FaceFrame& F, const FaceStatic& S, uint32_t f2t, int px0, int py0,
-                                            const ShadeParams& sp, ShadeRec& R)
+// -1 / the squared lengths of a face's window edges, k -> k + 1.
+__device__ __forceinline__ float4 edge_scales(const int4& X, const int4& Y)
+{
+    const int32_t FX[4] = {X.x, X.y, X.z, X.w}, FY[4] = {Y.x, Y.y, Y.z, Y.w};
+    float nl[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int32_t ex = FX[(k + 1) & 3] - FX[k], ey = FY[(k + 1) & 3] - FY[k];
+        const float l2 = u64_to_f32((uint64_t)((int64_t)ex * ex + (int64_t)ey * ey));
+        nl[k] = l2 > 0.f ? -__frcp_rn(l2) : 0.f;
+    }
+    return make_float4(nl[0], nl[1], nl[2], nl[3]);
+}
+
+// The record of triangle f2t (from the records F, S of its face, E if kept) for
+// the tile whose first pixel is (px0, py0). The positions are read only where
+// the sphere lens may reach.
+__device__ __forceinline__ void make_record(const FaceFrame& F, const FaceStatic& S, const FaceExtra* E, uint32_t f2t,
+                                            int px0, int py0, const ShadeParams& sp, ShadeRec& R)
 {
     const int4 X = F.X, Y = F.Y;
-    const uint4 Z = F.Z, A = F.area;
+    const uint4 Z = F.Z;
     const float4 fq = F.q, imp = S.imp;
     const bool second = f2t & 1u;
     const uint32_t flags = face_flags(Z) >> (f2t & 1u);   // this triangle's bits in triangle 0's places
     // |coordinate| <= 2^22: exact in float
     R.nx = make_float4(-(float)X.x, -(float)X.y, -(float)X.z, -(float)X.w);
     R.ny = make_float4(-(float)Y.x, -(float)Y.y, -(float)Y.z, -(float)Y.w);
-    R.nl = F.nl;
+    R.nl = E ? E->nl : edge_scales(X, Y);
     // vertices 1 and 2: corners (1, 2) or (2, 3), swapped if the triangle winds the other way
     const bool sw = flags & kFaceSwapped;
     auto pick = [&](auto b, auto c, auto d, auto& v1, auto& v2) {
@@ -82,11 +96,19 @@ __device__ __forceinline__ void make_record(const FaceFrame& F, const FaceStatic
     R.ev = make_int4(dx1, dy1, dx2, dy2);
     const int32_t d1 = (int32_t)(z1 - z0), d2 = (int32_t)(z2 - z0);
     R.zf = make_uint4(z0 | (face_edge_flags(Z) << 24), (uint32_t)d1, (uint32_t)d2, f2t);
-    const uint32_t area = second ? A.y : A.x;
     const bool lens = !(flags & kFaceOut) && sp.lens_mode == HEXFC_LENS_SPHERE;
-    uint32_t iw = second ? A.w : A.z;
+    uint32_t area, iw;
+    if (E) {
+        const uint4 A = E->area;
+        area = second ? A.y : A.x;
+        iw = second ? A.w : A.z;
+    } else {
+        const uint64_t twice = (uint64_t)edge_fn(X.x, Y.x, x1, y1, x2, y2);
+        area = twice < (1ull << 26) ? (uint32_t)twice : 0u;
+        iw = __float_as_uint(__frcp_rn((float)area));
+    }
     uint4 p2 = make_uint4(0u, 0u, 0u, 0u);
-    if (area == 0) {   // a large triangle: 64-bit edge functions and area
+    if (area == 0) {   // a large triangle: 64-bit edge functions and area (wound: positive)
         const int64_t f1 = edge_fn(x2, y2, X.x, Y.x, sx, sy), f2 = edge_fn(X.x, Y.x, x1, y1, sx, sy);
         const uint64_t big = (uint64_t)edge_fn(X.x, Y.x, x1, y1, x2, y2);
         p2 = make_uint4(0u, (uint32_t)((uint64_t)f1 >> 32), (uint32_t)((uint64_t)f2 >> 32), (uint32_t)(big >> 32));
@@ -121,7 +143,7 @@ struct Sample {
 };
 // The parts of sample_of that few samples need: a large triangle (64-bit
 // weights), or a depth whose float estimate q was off (remainder r).
-__device__ __noinline__ Sample sample_rare(const ShadeRec& R, Sample s, int32_t r, uint32_t sx8, uint32_t sy8, bool& bad)
+static __device__ __noinline__ Sample sample_rare(const ShadeRec& R, Sample s, int32_t r, uint32_t sx8, uint32_t sy8, bool& bad)
 {
     const uint4 zf = R.zf, ha = R.ha, aw = R.aw, hw = R.p2;
     const int32_t area = (int32_t)(ha.z & kRecArea);
