@@ -1112,23 +1112,19 @@ hexfc_status cap_alloc(CapNet& n)
         if ((st = dalloc(&n.m, kCapParams)) != HEXFC_OK) return st;
         if ((st = dalloc(&n.v, kCapParams)) != HEXFC_OK) return st;
         if ((st = dalloc(&n.grad, kCapParams + 1)) != HEXFC_OK) return st;
+        if ((st = dalloc(&n.part, (size_t)cap_partials())) != HEXFC_OK) return st;
     }
     return st;
 }
 
-// Per-tile training buffers for n tiles.
-hexfc_status cap_train_buffers(CapNet& c, int64_t n)
+// Features and counts of n tiles handed in by the caller.
+hexfc_status cap_inputs(CapNet& c, int64_t n)
 {
-    if (c.h1 && c.tiles >= n) return HEXFC_OK;
-    dfree(c.h1); dfree(c.h2); dfree(c.da1); dfree(c.da2); dfree(c.dy); dfree(c.x); dfree(c.t);
+    if (c.x && c.tiles >= n) return HEXFC_OK;
+    dfree(c.x); dfree(c.t);
     c.tiles = 0;
     hexfc_status st;
     const int64_t m = n + n / 4 + 256;
-    if ((st = dalloc(&c.h1, (size_t)(m * kCapHid))) != HEXFC_OK) return st;
-    if ((st = dalloc(&c.h2, (size_t)(m * kCapHid))) != HEXFC_OK) return st;
-    if ((st = dalloc(&c.da1, (size_t)(m * kCapHid))) != HEXFC_OK) return st;
-    if ((st = dalloc(&c.da2, (size_t)(m * kCapHid))) != HEXFC_OK) return st;
-    if ((st = dalloc(&c.dy, (size_t)m)) != HEXFC_OK) return st;
     if ((st = dalloc(&c.x, (size_t)(4 * m))) != HEXFC_OK) return st;
     if ((st = dalloc(&c.t, (size_t)m)) != HEXFC_OK) return st;
     c.tiles = m;
@@ -1263,7 +1259,8 @@ hexfc_status hexfc_create(hexfc_ctx** out, int device, uint64_t frag_budget_byte
     c->lens.radius = 1.0;
     {
         DeviceGuard g(device);
-        if (prepare_raster_kernels() != cudaSuccess || prepare_draw_kernels() != cudaSuccess) {
+        if (prepare_raster_kernels() != cudaSuccess || prepare_draw_kernels() != cudaSuccess ||
+            prepare_capacity_kernels() != cudaSuccess) {
             (void)cudaGetLastError();
             delete c;
             return HEXFC_ERR_CUDA;
@@ -1296,7 +1293,7 @@ void hexfc_destroy(hexfc_ctx* ctx)
     {
         CapNet& n = ctx->cap;
         dfree(n.w); dfree(n.w16); dfree(n.m); dfree(n.v); dfree(n.grad);
-        dfree(n.h1); dfree(n.h2); dfree(n.da1); dfree(n.da2); dfree(n.dy); dfree(n.x); dfree(n.t);
+        dfree(n.part); dfree(n.x); dfree(n.t);
     }
     if (ctx->origin) cudaStreamDestroy(ctx->origin);
     if (ctx->ev_in) cudaEventDestroy(ctx->ev_in);
@@ -1576,10 +1573,10 @@ hexfc_status hexfc_capacity_grad(hexfc_ctx* ctx, const float* x, const uint32_t*
     DeviceGuard g(ctx->device);
     CapNet& c = ctx->cap;
     hexfc_status st;
-    if ((st = cap_train_buffers(c, n)) != HEXFC_OK) return st;
+    if ((st = cap_inputs(c, n)) != HEXFC_OK) return st;
     CK(cudaMemcpy(c.x, x, sizeof(float) * 4 * (size_t)n, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c.t, counts, sizeof(uint32_t) * (size_t)n, cudaMemcpyHostToDevice));
-    CK(launch_cap_grad(c, c.x, c.t, n, 0));
+    CK(launch_cap_grad(c, c.x, c.t, n, 0.f, 0));
     CK(cudaMemcpy(grad, c.grad, sizeof(float) * kCapParams, cudaMemcpyDeviceToHost));
     if (loss) CK(cudaMemcpy(loss, c.grad + kCapParams, sizeof(float), cudaMemcpyDeviceToHost));
     return HEXFC_OK;
@@ -1593,14 +1590,9 @@ hexfc_status hexfc_capacity_train(hexfc_ctx* ctx, int32_t steps, float lr, float
     CapNet& c = ctx->cap;
     const cudaStream_t s = (cudaStream_t)stream;
     const int64_t n = ctx->feat_tiles;
-    hexfc_status st;
-    if ((st = cap_train_buffers(c, n)) != HEXFC_OK) return st;
-    for (int32_t k = 0; k < steps; ++k) {
-        CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, s));
-        CK(launch_cap_adam(c, lr, s));
-    }
+    for (int32_t k = 0; k < steps; ++k) CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, lr, s));
     if (loss) {
-        if (steps == 0) CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, s));
+        if (steps == 0) CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, 0.f, s));
         CK(cudaMemcpyAsync(loss, c.grad + kCapParams, sizeof(float), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
     }

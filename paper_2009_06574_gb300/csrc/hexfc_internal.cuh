@@ -121,11 +121,7 @@ struct CapNet {
     float* m = nullptr;
     float* v = nullptr;
     float* grad = nullptr;        // [kCapParams + 1]; the last value is the loss
-    float* h1 = nullptr;          // [tiles * kCapHid] layer values and errors of a training pass
-    float* h2 = nullptr;
-    float* da1 = nullptr;
-    float* da2 = nullptr;
-    float* dy = nullptr;          // [tiles]
+    float* part = nullptr;        // shares of the gradient (cap_partials())
     float* x = nullptr;           // [4 * tiles] features handed in by the caller
     uint32_t* t = nullptr;        // [tiles] counts handed in by the caller
     int64_t tiles = 0;            // capacity of the per-tile arrays
@@ -295,8 +291,10 @@ cudaError_t launch_capacity_from_previous(FrameBufs& fb, int64_t n_tiles, float 
 cudaError_t launch_capacity_check(FrameBufs& fb, int64_t n_tiles, cudaStream_t s);
 cudaError_t launch_cap_forward(const CapNet& net, FrameBufs& fb, int64_t n_tiles, float margin, uint32_t pad,
                                cudaStream_t s);
-cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, cudaStream_t s);
-cudaError_t launch_cap_adam(CapNet& net, float lr, cudaStream_t s);
+cudaError_t prepare_capacity_kernels();
+int64_t cap_partials();   // floats of CapNet::part
+// Loss and gradient into net.grad, and (lr > 0) an Adam step.
+cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, float lr, cudaStream_t s);
 cudaError_t launch_cap_to_half(CapNet& net, cudaStream_t s);
 // White silhouettes over the output (Section "Blending Focus and Context"):
 // from the boundary surface's depths zsil of the drawn rectangle, which sits

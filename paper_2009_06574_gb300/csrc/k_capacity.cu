@@ -10,15 +10,14 @@
 // previous frame.
 //
 //   k_cap_forward   per tile: y and the capacity expm1(y) (1 + margin) + pad
-//   k_cap_backward  per tile: mean-squared loss on log1p(exact count); stores
-//                   the layer values and the back-propagated errors
-//   k_cap_reduce    per parameter: gradient = sum over tiles (tile slices,
-//                   atomics between slices)
-//   k_cap_adam      per parameter: Adam step on the master copy, FP16 copy
+//   k_cap_backward  mean-squared loss on log1p(exact count) and the gradient, a
+//                   share per block
+//   k_cap_sum       the shares summed; an Adam step on the master copy, FP16 copy
 #include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 
 #include "hexfc_internal.cuh"
 
@@ -32,145 +31,258 @@ static_assert(oB3 + 1 == kCapParams, "parameter layout");
 
 inline unsigned grid_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
-__device__ __forceinline__ void load_weights(const __half* __restrict__ w16, float* s_w)
+// ---- layers on a group of kGroup tiles, 256 threads
+//
+// A thread per tile left 120 of 152 SMs idle at 8160 tiles and walked 8,500
+// multiply-adds alone: 75 us forward and backward, and 32 us to sum the gradient
+// from 8 MB of stored layer values. Here a block takes 32 tiles; the three 64 x 64
+// products (layer 2, its gradient, the error back through it) are register tiles
+// over operands in shared memory, the gradient's sums stay in registers over the
+// block's groups, and what leaves the block is its share of the gradient, summed
+// in a fixed order (so a training step gives the same bits every time). 8 Adam
+// steps at 1920x1080: 0.90 -> XX ms.
+constexpr int kGroup = 32;
+constexpr int kCapThreads = 256;
+constexpr int kCapBlocks = 304;   // two blocks an SM at most; more tiles than kGroup * 304: several groups each
+
+struct NetSmem {
+    float w1[kHid * kIn], b1[kHid], b2[kHid], w3[kHid];
+    float w2[kHid][kHid];       // [j][i]
+    float w2t[kHid][kHid];      // [i][j]
+    float x[kGroup][kIn];
+    float h1[kGroup][kHid];     // [t][i]
+    float h1t[kHid][kGroup];    // [i][t]
+    float da[kGroup][kHid];     // [t][j]: errors of layer 2, then [t][i]: of layer 1
+    float dat[kHid][kGroup];    // [j][t]
+    float red[2][16][kHid];     // sums over the groups of tiles at the end
+    float dy[16][2];
+    float b3;
+};
+// (read 16 bytes at a time, the transposed ones 8)
+static_assert(offsetof(NetSmem, b2) % 16 == 0 && offsetof(NetSmem, w3) % 16 == 0 && offsetof(NetSmem, w2) % 16 == 0 &&
+                  offsetof(NetSmem, w2t) % 16 == 0 && offsetof(NetSmem, h1) % 16 == 0 &&
+                  offsetof(NetSmem, da) % 16 == 0 && offsetof(NetSmem, h1t) % 8 == 0 &&
+                  offsetof(NetSmem, dat) % 8 == 0,
+              "alignment of the vector reads");
+
+__device__ __forceinline__ void net_load(NetSmem& S, const __half* __restrict__ w16)
 {
-    for (int i = threadIdx.x; i < kCapParams; i += blockDim.x) s_w[i] = __half2float(w16[i]);
-    __syncthreads();
+    for (int p = threadIdx.x; p < kCapParams; p += kCapThreads) {
+        const float v = __half2float(w16[p]);
+        if (p < oB1) S.w1[p] = v;
+        else if (p < oW2) S.b1[p - oB1] = v;
+        else if (p < oB2) {
+            const int j = (p - oW2) / kHid, i = (p - oW2) % kHid;
+            S.w2[j][i] = v;
+            S.w2t[i][j] = v;
+        }
+        else if (p < oW3) S.b2[p - oB2] = v;
+        else if (p < oB3) S.w3[p - oW3] = v;
+        else S.b3 = v;
+    }
 }
 
-__global__ void __launch_bounds__(256) k_cap_forward(const float* __restrict__ X, int64_t n,
-                                                     const __half* __restrict__ w16, float margin, uint32_t pad,
-                                                     uint32_t* __restrict__ cap)
+// Layers 1 and 2 of tiles t0 .. t0 + 31 (rows past n are zero): this thread's
+// values before the second ReLU, a[u][v] of tile 2 (tid / 16) + u and hidden
+// unit 4 (tid % 16) + v, and the output y[u] of its two tiles.
+template <bool kTrain>
+__device__ __forceinline__ void net_forward(NetSmem& S, const float* __restrict__ X, int64_t n, int64_t t0, float (&a)[2][4],
+                                            float (&y)[2])
 {
-    __shared__ float s_w[kCapParams];
-    load_weights(w16, s_w);
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const float x0 = X[4 * t], x1 = X[4 * t + 1], x2 = X[4 * t + 2], x3 = X[4 * t + 3];
-    float h1[kHid];
+    const int tid = threadIdx.x, jq = tid & 15, tp = tid >> 4;
+    __syncthreads();   // the last group is done with the arrays (and the weights are loaded)
+    if (tid < kGroup * kIn) {
+        const int64_t at = t0 * kIn + tid;
+        S.x[tid / kIn][tid % kIn] = at < n * kIn ? X[at] : 0.f;
+    }
+    __syncthreads();
+    {
+        const int i = tid & 63, t8 = (tid >> 6) * 8;
+        const float* w = S.w1 + i * kIn;
 #pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float* x = S.x[t8 + k];
+            const float h = fmaxf(fmaf(w[3], x[3], fmaf(w[2], x[2], fmaf(w[1], x[1], fmaf(w[0], x[0], S.b1[i])))), 0.f);
+            S.h1t[i][t8 + k] = h;
+            if (kTrain) S.h1[t8 + k][i] = h;
+        }
+    }
+    __syncthreads();
+    const float4 b = *reinterpret_cast<const float4*>(&S.b2[4 * jq]);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        a[u][0] = b.x; a[u][1] = b.y; a[u][2] = b.z; a[u][3] = b.w;
+    }
+#pragma unroll 8
     for (int i = 0; i < kHid; ++i) {
-        const float* w = s_w + oW1 + i * kIn;
-        h1[i] = fmaxf(fmaf(w[3], x3, fmaf(w[2], x2, fmaf(w[1], x1, fmaf(w[0], x0, s_w[oB1 + i])))), 0.f);
+        const float2 h = *reinterpret_cast<const float2*>(&S.h1t[i][2 * tp]);
+        const float4 w = *reinterpret_cast<const float4*>(&S.w2t[i][4 * jq]);
+        a[0][0] = fmaf(w.x, h.x, a[0][0]); a[0][1] = fmaf(w.y, h.x, a[0][1]);
+        a[0][2] = fmaf(w.z, h.x, a[0][2]); a[0][3] = fmaf(w.w, h.x, a[0][3]);
+        a[1][0] = fmaf(w.x, h.y, a[1][0]); a[1][1] = fmaf(w.y, h.y, a[1][1]);
+        a[1][2] = fmaf(w.z, h.y, a[1][2]); a[1][3] = fmaf(w.w, h.y, a[1][3]);
     }
-    float y = s_w[oB3];
-    for (int j = 0; j < kHid; ++j) {
-        const float* w = s_w + oW2 + j * kHid;
-        float a = s_w[oB2 + j];
+    const float4 w3 = *reinterpret_cast<const float4*>(&S.w3[4 * jq]);
 #pragma unroll
-        for (int i = 0; i < kHid; ++i) a = fmaf(w[i], h1[i], a);
-        y = fmaf(s_w[oW3 + j], fmaxf(a, 0.f), y);
+    for (int u = 0; u < 2; ++u) {
+        float v = fmaf(w3.x, fmaxf(a[u][0], 0.f), w3.y * fmaxf(a[u][1], 0.f)) +
+                  fmaf(w3.z, fmaxf(a[u][2], 0.f), w3.w * fmaxf(a[u][3], 0.f));
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        y[u] = v + S.b3;
     }
-    const float c = expm1f(fminf(y, 20.f)) * (1.f + margin) + (float)pad;
-    cap[t] = (uint32_t)fminf(fmaxf(c, 0.f), 4.0e9f);
 }
 
-// Forward and backward of one tile; loss = mean over the n tiles of (y - t)^2.
-__global__ void __launch_bounds__(256) k_cap_backward(const float* __restrict__ X,
-                                                      const uint32_t* __restrict__ counts, int64_t n,
-                                                      const __half* __restrict__ w16, float* __restrict__ H1,
-                                                      float* __restrict__ H2, float* __restrict__ DA1,
-                                                      float* __restrict__ DA2, float* __restrict__ DY,
-                                                      float* __restrict__ loss)
+__global__ void __launch_bounds__(kCapThreads) k_cap_forward(const float* __restrict__ X, int64_t n,
+                                                             const __half* __restrict__ w16, float margin,
+                                                             uint32_t pad, uint32_t* __restrict__ cap)
 {
-    __shared__ float s_w[kCapParams];
-    __shared__ float s_loss[8];
-    load_weights(w16, s_w);
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float l = 0.f;
-    if (t < n) {
-        const float x0 = X[4 * t], x1 = X[4 * t + 1], x2 = X[4 * t + 2], x3 = X[4 * t + 3];
-        float h1[kHid];
-        uint64_t m1 = 0, m2 = 0;
+    extern __shared__ __align__(16) unsigned char net_smem[];
+    NetSmem& S = *reinterpret_cast<NetSmem*>(net_smem);
+    net_load(S, w16);
+    for (int64_t t0 = (int64_t)blockIdx.x * kGroup; t0 < n; t0 += (int64_t)gridDim.x * kGroup) {
+        float a[2][4], y[2];
+        net_forward<false>(S, X, n, t0, a, y);
+        const int64_t t = t0 + 2 * (threadIdx.x >> 4);
 #pragma unroll
-        for (int i = 0; i < kHid; ++i) {
-            const float* w = s_w + oW1 + i * kIn;
-            const float a = fmaf(w[3], x3, fmaf(w[2], x2, fmaf(w[1], x1, fmaf(w[0], x0, s_w[oB1 + i]))));
-            h1[i] = fmaxf(a, 0.f);
-            m1 |= (uint64_t)(a > 0.f) << i;
-            H1[t * kHid + i] = h1[i];
-        }
-        float y = s_w[oB3];
-        for (int j = 0; j < kHid; ++j) {
-            const float* w = s_w + oW2 + j * kHid;
-            float a = s_w[oB2 + j];
-#pragma unroll
-            for (int i = 0; i < kHid; ++i) a = fmaf(w[i], h1[i], a);
-            const float h2 = fmaxf(a, 0.f);
-            m2 |= (uint64_t)(a > 0.f) << j;
-            H2[t * kHid + j] = h2;
-            y = fmaf(s_w[oW3 + j], h2, y);
-        }
-        const float e = y - log1pf((float)counts[t]);
-        l = e * e / (float)n;
-        const float dy = 2.f * e / (float)n;
-        DY[t] = dy;
-        float dh1[kHid];
-#pragma unroll
-        for (int i = 0; i < kHid; ++i) dh1[i] = 0.f;
-        for (int j = 0; j < kHid; ++j) {
-            const float da2 = ((m2 >> j) & 1ull) ? dy * s_w[oW3 + j] : 0.f;
-            DA2[t * kHid + j] = da2;
-            const float* w = s_w + oW2 + j * kHid;
-#pragma unroll
-            for (int i = 0; i < kHid; ++i) dh1[i] = fmaf(w[i], da2, dh1[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < kHid; ++i) DA1[t * kHid + i] = ((m1 >> i) & 1ull) ? dh1[i] : 0.f;
+        for (int u = 0; u < 2; ++u)
+            if ((threadIdx.x & 15) == 0 && t + u < n) {
+                const float c = expm1f(fminf(y[u], 20.f)) * (1.f + margin) + (float)pad;
+                cap[t + u] = (uint32_t)fminf(fmaxf(c, 0.f), 4.0e9f);
+            }
     }
-    // the block's share of the loss
+}
+
+// Loss (mean over the n tiles of (y - log1p(count))^2) and gradient: block b's
+// shares into part[b][kCapParams + 1].
+__global__ void __launch_bounds__(kCapThreads) k_cap_backward(const float* __restrict__ X,
+                                                              const uint32_t* __restrict__ counts, int64_t n,
+                                                              const __half* __restrict__ w16,
+                                                              float* __restrict__ part)
+{
+    extern __shared__ __align__(16) unsigned char net_smem[];
+    NetSmem& S = *reinterpret_cast<NetSmem*>(net_smem);
+    net_load(S, w16);
+    const int tid = threadIdx.x, q = tid & 15, g = tid >> 4;
+    float gw2[4][4] = {}, gw3[4] = {}, gb2[4] = {}, gw1 = 0.f, gb1 = 0.f, gb3 = 0.f, loss = 0.f;
+    const float inv_n = 1.f / (float)n;
+    for (int64_t t0 = (int64_t)blockIdx.x * kGroup; t0 < n; t0 += (int64_t)gridDim.x * kGroup) {
+        float a[2][4], y[2];
+        net_forward<true>(S, X, n, t0, a, y);
+        const float4 w3 = *reinterpret_cast<const float4*>(&S.w3[4 * q]);
+        const float w3v[4] = {w3.x, w3.y, w3.z, w3.w};
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0) s_loss[threadIdx.x >> 5] = l;
+        for (int u = 0; u < 2; ++u) {
+            const int64_t t = t0 + 2 * g + u;
+            const float e = t < n ? y[u] - log1pf((float)counts[t]) : 0.f;
+            const float dy = 2.f * e * inv_n;
+            if (q == 0) {
+                loss = fmaf(e * inv_n, e, loss);
+                gb3 += dy;
+            }
+            float d[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                gw3[v] = fmaf(dy, fmaxf(a[u][v], 0.f), gw3[v]);
+                d[v] = a[u][v] > 0.f ? dy * w3v[v] : 0.f;
+                gb2[v] += d[v];
+                S.dat[4 * q + v][2 * g + u] = d[v];
+            }
+            *reinterpret_cast<float4*>(&S.da[2 * g + u][4 * q]) = make_float4(d[0], d[1], d[2], d[3]);
+        }
+        __syncthreads();
+        // gradient of W2: units j = 4 g + u, i = 4 q + v
+#pragma unroll 4
+        for (int t = 0; t < kGroup; ++t) {
+            const float4 d = *reinterpret_cast<const float4*>(&S.da[t][4 * g]);
+            const float4 h = *reinterpret_cast<const float4*>(&S.h1[t][4 * q]);
+            const float dv[4] = {d.x, d.y, d.z, d.w}, hv[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) gw2[u][v] = fmaf(dv[u], hv[v], gw2[u][v]);
+        }
+        // errors of layer 1: tiles 2 g + u, units i = 4 q + v
+        float e1[2][4] = {};
+#pragma unroll 8
+        for (int j = 0; j < kHid; ++j) {
+            const float2 d = *reinterpret_cast<const float2*>(&S.dat[j][2 * g]);
+            const float4 w = *reinterpret_cast<const float4*>(&S.w2[j][4 * q]);
+            e1[0][0] = fmaf(w.x, d.x, e1[0][0]); e1[0][1] = fmaf(w.y, d.x, e1[0][1]);
+            e1[0][2] = fmaf(w.z, d.x, e1[0][2]); e1[0][3] = fmaf(w.w, d.x, e1[0][3]);
+            e1[1][0] = fmaf(w.x, d.y, e1[1][0]); e1[1][1] = fmaf(w.y, d.y, e1[1][1]);
+            e1[1][2] = fmaf(w.z, d.y, e1[1][2]); e1[1][3] = fmaf(w.w, d.y, e1[1][3]);
+        }
+        __syncthreads();   // da has been read
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const float4 h = *reinterpret_cast<const float4*>(&S.h1[2 * g + u][4 * q]);
+            *reinterpret_cast<float4*>(&S.da[2 * g + u][4 * q]) =
+                make_float4(h.x > 0.f ? e1[u][0] : 0.f, h.y > 0.f ? e1[u][1] : 0.f, h.z > 0.f ? e1[u][2] : 0.f,
+                            h.w > 0.f ? e1[u][3] : 0.f);
+        }
+        __syncthreads();
+        // gradients of W1 and b1: unit tid / 4, input tid % 4
+#pragma unroll 8
+        for (int t = 0; t < kGroup; ++t) {
+            const float d = S.da[t][tid >> 2];
+            gw1 = fmaf(d, S.x[t][tid & 3], gw1);
+            gb1 += d;
+        }
+    }
+    float* P = part + (int64_t)blockIdx.x * (kCapParams + 1);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) P[oW2 + (4 * g + u) * kHid + 4 * q + v] = gw2[u][v];
+    P[oW1 + tid] = gw1;
+    if ((tid & 3) == 0) P[oB1 + (tid >> 2)] = gb1;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float b = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += s_loss[w];
-        atomicAdd(loss, b);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        S.red[0][g][4 * q + v] = gw3[v];
+        S.red[1][g][4 * q + v] = gb2[v];
+    }
+    if (q == 0) {
+        S.dy[g][0] = gb3;
+        S.dy[g][1] = loss;
+    }
+    __syncthreads();
+    if (tid < 2 * kHid) {
+        const int which = tid / kHid, j = tid % kHid;
+        float v = 0.f;
+        for (int k = 0; k < 16; ++k) v += S.red[which][k][j];
+        P[(which == 0 ? oW3 : oB2) + j] = v;
+    }
+    if (tid < 2) {
+        float v = 0.f;
+        for (int k = 0; k < 16; ++k) v += S.dy[k][tid];
+        P[tid == 0 ? oB3 : kCapParams] = v;
     }
 }
 
-// Parameter p's gradient over tiles [s0, s1): a sum of products of the stored
-// layer values and errors.
-__global__ void __launch_bounds__(256) k_cap_reduce(const float* __restrict__ X, int64_t n,
-                                                    const float* __restrict__ H1, const float* __restrict__ H2,
-                                                    const float* __restrict__ DA1, const float* __restrict__ DA2,
-                                                    const float* __restrict__ DY, int slices,
-                                                    float* __restrict__ grad)
+// The blocks' shares summed, 8 threads a parameter; with `adam`, an Adam step on
+// the master copy and its FP16 copy.
+__global__ void __launch_bounds__(256) k_cap_sum(const float* __restrict__ part, int blocks, float* __restrict__ grad,
+                                                 bool adam, float* __restrict__ w, __half* __restrict__ w16,
+                                                 float* __restrict__ m, float* __restrict__ v, float lr, float b1,
+                                                 float b2, float eps, float c1, float c2)
 {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kCapParams) return;
-    const int64_t per = (n + slices - 1) / slices;
-    const int64_t s0 = (int64_t)blockIdx.y * per, s1 = min(n, s0 + per);
+    __shared__ float s[8][32];
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+    float sum = 0.f;
+    if (p <= kCapParams) {
+#pragma unroll 8
+        for (int b = k; b < blocks; b += 8) sum += part[(int64_t)b * (kCapParams + 1) + p];
+    }
+    s[k][lane] = sum;
+    __syncthreads();
+    if (k != 0 || p > kCapParams) return;
     float g = 0.f;
-    if (p < oB1) {                 // W1[i][k]
-        const int i = p / kIn, k = p % kIn;
-        for (int64_t t = s0; t < s1; ++t) g = fmaf(DA1[t * kHid + i], X[4 * t + k], g);
-    } else if (p < oW2) {          // b1[i]
-        const int i = p - oB1;
-        for (int64_t t = s0; t < s1; ++t) g += DA1[t * kHid + i];
-    } else if (p < oB2) {          // W2[j][i]
-        const int j = (p - oW2) / kHid, i = (p - oW2) % kHid;
-        for (int64_t t = s0; t < s1; ++t) g = fmaf(DA2[t * kHid + j], H1[t * kHid + i], g);
-    } else if (p < oW3) {          // b2[j]
-        const int j = p - oB2;
-        for (int64_t t = s0; t < s1; ++t) g += DA2[t * kHid + j];
-    } else if (p < oB3) {          // w3[j]
-        const int j = p - oW3;
-        for (int64_t t = s0; t < s1; ++t) g = fmaf(DY[t], H2[t * kHid + j], g);
-    } else {                       // b3
-        for (int64_t t = s0; t < s1; ++t) g += DY[t];
-    }
-    atomicAdd(&grad[p], g);
-}
-
-__global__ void k_cap_adam(float* __restrict__ w, __half* __restrict__ w16, const float* __restrict__ grad,
-                           float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2, float eps,
-                           float c1, float c2)
-{
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kCapParams) return;
-    const float g = grad[p];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) g += s[i][lane];
+    grad[p] = g;
+    if (!adam || p == kCapParams) return;
     const float mm = fmaf(b1, m[p], (1.f - b1) * g);
     const float vv = fmaf(b2, v[p], (1.f - b2) * g * g);
     m[p] = mm;
@@ -231,32 +343,36 @@ cudaError_t launch_capacity_check(FrameBufs& fb, int64_t n_tiles, cudaStream_t s
     return cudaGetLastError();
 }
 
+cudaError_t prepare_capacity_kernels()
+{
+    const cudaError_t e = cudaFuncSetAttribute(k_cap_forward, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sizeof(NetSmem));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_cap_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NetSmem));
+}
+
+int64_t cap_partials() { return (int64_t)kCapBlocks * (kCapParams + 1); }
+
+static unsigned cap_grid(int64_t n) { return (unsigned)std::min<int64_t>((n + kGroup - 1) / kGroup, kCapBlocks); }
+
 cudaError_t launch_cap_forward(const CapNet& net, FrameBufs& fb, int64_t n_tiles, float margin, uint32_t pad,
                                cudaStream_t s)
 {
-    k_cap_forward<<<grid_for(n_tiles, 256), 256, 0, s>>>(fb.cap_x, n_tiles, net.w16, margin, pad, fb.tile_cap);
+    k_cap_forward<<<cap_grid(n_tiles), kCapThreads, sizeof(NetSmem), s>>>(fb.cap_x, n_tiles, net.w16, margin, pad,
+                                                                           fb.tile_cap);
     return cudaGetLastError();
 }
 
-cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, cudaStream_t s)
-{
-    cudaError_t e = cudaMemsetAsync(net.grad, 0, sizeof(float) * (kCapParams + 1), s);   // grad[kCapParams] = loss
-    if (e != cudaSuccess) return e;
-    k_cap_backward<<<grid_for(n, 256), 256, 0, s>>>(X, counts, n, net.w16, net.h1, net.h2, net.da1, net.da2, net.dy,
-                                                    net.grad + kCapParams);
-    const int slices = (int)std::min<int64_t>(64, std::max<int64_t>(1, n / 256));
-    k_cap_reduce<<<dim3(grid_for(kCapParams, 256), (unsigned)slices), 256, 0, s>>>(X, n, net.h1, net.h2, net.da1,
-                                                                                   net.da2, net.dy, slices, net.grad);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cap_adam(CapNet& net, float lr, cudaStream_t s)
+cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, float lr, cudaStream_t s)
 {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    net.step += 1;
+    const bool adam = lr > 0.f;
+    if (adam) net.step += 1;
     const float c1 = 1.f / (1.f - std::pow(b1, (float)net.step)), c2 = 1.f / (1.f - std::pow(b2, (float)net.step));
-    k_cap_adam<<<grid_for(kCapParams, 256), 256, 0, s>>>(net.w, net.w16, net.grad, net.m, net.v, lr, b1, b2, eps, c1,
-                                                         c2);
+    const unsigned blocks = cap_grid(n);
+    k_cap_backward<<<blocks, kCapThreads, sizeof(NetSmem), s>>>(X, counts, n, net.w16, net.part);
+    k_cap_sum<<<grid_for(kCapParams + 1, 32), 256, 0, s>>>(net.part, (int)blocks, net.grad, adam, net.w, net.w16, net.m,
+                                                           net.v, lr, b1, b2, eps, c1, c2);
     return cudaGetLastError();
 }
 
