@@ -687,7 +687,7 @@ hexfc_status job_phase2(FrameJob& j, cudaStream_t s)
 {
     hexfc_status st;
     if ((st = job_phase2_bins(j, s)) != HEXFC_OK) return st;
-    CK(launch_count(*j.fb, j.tiles_x, j.tiles_y, j.W, j.H, s));
+    CK(launch_count(*j.fb, j.tiles_x, j.tiles_y, j.W, j.H, (int64_t)j.n_bins, s));
     return job_phase2_totals(j, s);
 }
 
@@ -985,7 +985,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     }
     CK(scan_u32_to_u64(fb.tile_cap, fb.cap_off, j.n_tiles, fb.part, fb.part_max, fb.scal + 11, 0xFFFFFFFFu, s));
     job_mark(j, 5, s);
-    CK(launch_count(fb, j.tiles_x, j.tiles_y, j.W, j.H, s));
+    CK(launch_count(fb, j.tiles_x, j.tiles_y, j.W, j.H, (int64_t)j.n_bins, s));
     job_mark(j, 6, s);
     CK(launch_capacity_check(fb, j.n_tiles, s));
     job_mark(j, 7, s);
@@ -2105,7 +2105,7 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     CK(launch_bin_fill(*m, fb, tiles_x, W, H, s));
     CK(launch_bin_sort(fb, n_tiles, (int64_t)n_bins, ctx->depth_buckets, CapFeatures{}, s));
     if (!ordered) CK(launch_tile_order(fb, n_tiles, s));
-    CK(launch_count(fb, tiles_x, tiles_y, W, H, s));
+    CK(launch_count(fb, tiles_x, tiles_y, W, H, (int64_t)n_bins, s));
     CK(cudaMemcpyAsync(h, fb.scal, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (h[5] != 0) {   // this call's count pass, or the previous call's fill or composite

@@ -1,150 +1,95 @@
 // The coverage count of one tile (warp-level).
 #pragma once
-#include "raster_tiles.cuh"
+#include "raster_common.cuh"
+#include "row_span.h"
 
 namespace hexfc {
 
+constexpr int kConsumerWarps = kTilePix / 32;   // warps of the count pass
+constexpr int kCountBlocks = 4;                 // its blocks an SM (64 registers a thread; 5: 2-6% slower)
+constexpr int kCountSlices = 8;                 // blocks a tile at most
+
 // Per tile: coverage of every chunk of 32 triangles as per-pixel bit masks;
 // the masks are kept for the drawing pass and their bit counts are the
-// per-pixel list lengths. Warp w takes chunks w, w + 8, ... of the tile's list
+// per-pixel list lengths. A warp takes every so-many-th chunk of the tile's list
 // on its own: its 32 lanes stage the chunk's triangles, then take the
-// triangles' box rows (clipped to the tile) one per lane: a triangle covers
-// one run of samples in a row, found from its three edges' crossings of the
-// row, and the lane sets bit j of those pixels in the warp's private masks.
-// No block barrier until the per-pixel totals are summed at the end.
+// triangles' row pairs (clipped to the tile) one per lane: a triangle covers
+// one run of samples in a row, found from where its three edges cross the row,
+// and the lane writes the runs as bits of the triangle's tile bitmap (256 bits,
+// pixel ly * kTileW + lx). Eight 32 x 32 bit transposes turn the 32 bitmaps into
+// the 256 pixels' masks. No block barrier until the per-pixel totals are summed.
+//
+// Bound by instruction issue. What it spends a row on was cut: values that fit 32
+// bits (all but triangles that reach 64 pixels beyond the tile's corner), one
+// estimate and one exact remainder an edge instead of an error bound and its
+// slow path, two rows a lane's turn, a store a row pair instead of an atomic per
+// covered sample. 64^3 at 1920x1080 (127,000 chunks): 0.248 -> 0.156 ms; 128^3 at
+// 3840x2160: 1.80 -> 1.07 ms.
 struct CountWarp {
-    CovSoA c;
-    // per edge, float data of its crossing with a sample row: (e0f, fb, rfa,
-    // eps). The edge value at box column rx of row ry is E = e0f + fb*ry +
-    // fa*rx (fa = -256 dy, fb = 256 dx, e0f ~ e0), so it crosses 0 at column
-    // t = -(e0f + fb*ry) * rfa, rfa = 1 / fa; eps bounds |t - t_exact|. An
-    // edge parallel to the rows (dy = 0) has rfa = 0 and eps = the bound on
-    // the float error of its (constant) value.
-    float4 ef[3][kChunk];
-    // the chunk's rows as one sequence: triangle j's rows start at seq[j].x
-    // (seq[j] = start, -, box, -); r2j maps the rank of a non-empty triangle
-    // to its index
-    uint4 seq[kChunk];
+    int4 edge[3][kChunk];   // stage_edges
+    // the chunk's row pairs as one sequence: triangle j's start at seq[j].x; its box seq[j].y. r2j maps
+    // the rank of a non-empty triangle to its index.
+    uint2 seq[kChunk];
     uint8_t r2j[kChunk];
-    uint32_t mask[kTilePix];   // coverage bits of the chunk; after the last chunk, the warp's per-pixel counts
+    uint32_t rows[kTilePix / 32][kChunk];   // [w][j]: pixels 32 w .. of triangle j's bitmap; at the end the
+                                            // warp's counts of the 256 pixels
 };
 
-// Float crossing data of triangle j's edges in the warp's staging slot. e0f
-// is within 0.75 ulp of e0 and fmaf(fb, ry, e0f) adds one rounding, all of
-// magnitudes at most M = |e0| + TW |fa| + TH |fb| (tile TW x TH): within
-// tol = 8 units of 2^-24 M of the exact value. Dividing by fa (rfa within 0.5
-// ulp, one more rounding of t) moves t by at most tol |rfa| + 2^-22 |t|, and
-// |t| <= TW + 1 wherever it matters (columns 0..TW-1): eps = tol |rfa|
-// (1 + 2^-10) + 2^-17 for TW <= 16 (17 * 2^-22 < 2^-17), + 2^-16 for TW = 32.
-__device__ __forceinline__ void stage_rows(const CovSoA& c, float4 (*ef)[kChunk], int j)
+// 32 x 32 bit transpose over a warp: bit i of lane l becomes bit l of lane i
+// (Warren, Hacker's Delight, section 7-3, with a lane per row).
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t v, int lane)
 {
+    uint32_t o = __shfl_xor_sync(0xffffffffu, v, 16);
+    v = __byte_perm(v, o, (lane & 16) ? 0x3276 : 0x5410);
+    o = __shfl_xor_sync(0xffffffffu, v, 8);
+    v = __byte_perm(v, o, (lane & 8) ? 0x3715 : 0x6240);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float e0 = i64_to_f32(c.e0[k][j]);
-        const float fa = -256.f * (float)c.dy[k][j];   // exact: |dy| < 2^24
-        const float fb = 256.f * (float)c.dx[k][j];
-        const float tol = ldexpf(fabsf(e0) + (float)kTileW * fabsf(fa) + (float)kTileH * fabsf(fb), -21);
-        const float rfa = fa != 0.f ? __frcp_rn(fa) : 0.f;
-        constexpr float kTabs = kTileW <= 16 ? 0x1p-17f : 0x1p-16f;
-        const float eps = fa != 0.f ? fmaf(tol * fabsf(rfa), 1.f + 0x1p-10f, kTabs) : tol;
-        ef[k][j] = make_float4(e0, fb, rfa, eps);
+    for (int s = 4; s > 0; s >>= 1) {
+        const uint32_t m = s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
+        o = __shfl_xor_sync(0xffffffffu, v, s);
+        v = (lane & s) ? (v & ~m) | ((o >> s) & m) : (v & m) | ((o << s) & ~m);
     }
+    return v;
 }
 
-// Exact: does edge k of triangle j own box column rx of the row whose edge
-// value at column 0 is A (edge function > 0, or 0 on an edge the top-left rule
-// gives to the triangle)?
-__device__ __forceinline__ bool edge_in(const CovSoA& c, int k, int j, int64_t A, int rx)
-{
-    const int64_t e = A - (int64_t)c.dy[k][j] * (int64_t)(rx << 8);
-    return e > 0 || (e == 0 && ((c.meta[j] >> k) & 1u));
-}
-
-// The covered box columns [lo, hi] of box row ry of triangle j (empty if lo >
-// hi): the intersection of its three edges' half-rows. Each edge's crossing
-// is taken from the float data where it is more than eps from an integer
-// column; near one (or if eps is not small), the column is decided by exact
-// integer tests (a binary search on the monotone edge test).
-__device__ __forceinline__ void row_span(const CovSoA& c, const float4 (*ef)[kChunk], int j, int ry, int bw, int& lo,
-                                         int& hi)
-{
-    lo = 0;
-    hi = bw - 1;
-    const float fry = (float)ry;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float4 f = ef[k][j];
-        const float af = fmaf(f.y, fry, f.x);   // edge value at column 0
-        if (f.z == 0.f) {   // parallel to the rows: the whole row or nothing
-            bool in = af > f.w;
-            if (!in && af >= -f.w)
-                in = edge_in(c, k, j, c.e0[k][j] + (int64_t)c.dx[k][j] * (int64_t)(ry << 8), 0);
-            if (!in) hi = -1;
-            continue;
-        }
-        const float t = -af * f.z;
-        const float rt = rintf(t);
-        const bool exact = f.w > 0.25f || (fabsf(t - rt) <= f.w && rt >= 0.f && rt <= (float)(bw - 1));
-        int b;
-        if (!exact) {
-            const float ft = floorf(t);
-            b = f.z > 0.f ? (int)fminf(fmaxf(ft + 1.f, 0.f), (float)bw)     // first column inside
-                          : (int)fminf(fmaxf(ft, -1.f), (float)(bw - 1));   // last column inside
-        } else {
-            const int64_t A = c.e0[k][j] + (int64_t)c.dx[k][j] * (int64_t)(ry << 8);
-            if (f.z > 0.f) {   // inside from the first column that passes: search [0, bw]
-                int a = 0, z = bw;
-                while (a < z) {
-                    const int m = (a + z) >> 1;
-                    if (edge_in(c, k, j, A, m)) z = m;
-                    else a = m + 1;
-                }
-                b = a;
-            } else {           // inside up to the last column that passes: search [-1, bw - 1]
-                int a = -1, z = bw - 1;
-                while (a < z) {
-                    const int m = (a + z + 1) >> 1;
-                    if (edge_in(c, k, j, A, m)) a = m;
-                    else z = m - 1;
-                }
-                b = a;
-            }
-        }
-        if (f.z > 0.f) lo = max(lo, b);
-        else hi = min(hi, b);
-    }
-}
-
-__device__ __forceinline__ void count_chunks(CountWarp* s_w, int warp, int lane, const uint32_t* __restrict__ bins,
+__device__ __forceinline__ void count_chunks(CountWarp& me, int lane, const uint32_t* __restrict__ bins,
                                              const FaceFrame* __restrict__ fframe, uint64_t beg, uint32_t n_chunks,
-                                             int px0, int py0, int W, int H, uint32_t* __restrict__ masks)
+                                             uint32_t first, uint32_t step, int px0, int py0, int W, int H,
+                                             uint32_t* __restrict__ masks)
 {
-    CountWarp& me = s_w[warp];
-    uint32_t count[kTilePix / 32];   // pixels lane + 32 k
+    constexpr int kWords = kTilePix / 32;
+    using Row = typename std::conditional<kTileW == 8, uint8_t,
+                                          typename std::conditional<kTileW == 16, uint16_t, uint32_t>::type>::type;
+    constexpr int kRowsPerWord = 32 / kTileW;
+    static_assert(kTileW <= 32 && kTileH <= 32, "stage_edges, row_span");
+    const int rows = H - py0;   // rows of the image from the tile's first
+    uint32_t count[kWords];   // pixels lane + 32 k
 #pragma unroll
-    for (int k = 0; k < kTilePix / 32; ++k) {
-        me.mask[lane + 32 * k] = 0;
-        count[k] = 0;
-    }
-    __syncwarp();
-    uint32_t f2t = warp < (int)n_chunks ? bins[beg + (uint64_t)warp * kChunk + lane] : kPadBin;
-    for (uint32_t c = warp; c < n_chunks; c += kConsumerWarps) {
+    for (int k = 0; k < kWords; ++k) count[k] = 0;
+    uint32_t f2t = first < n_chunks ? bins[beg + (uint64_t)first * kChunk + lane] : kPadBin;
+    for (uint32_t c = first; c < n_chunks; c += step) {
         int4 a = make_int4(0, 0, 0, 0), b = a;
         if (f2t != kPadBin) { a = fframe[f2t >> 1].X; b = fframe[f2t >> 1].Y; }
         const uint32_t f2t_next =
-            c + kConsumerWarps < n_chunks ? bins[beg + (uint64_t)(c + kConsumerWarps) * kChunk + lane] : kPadBin;
+            c + step < n_chunks ? bins[beg + (uint64_t)(c + step) * kChunk + lane] : kPadBin;
+#pragma unroll
+        for (int k = 0; k < kWords; ++k) me.rows[k][lane] = 0u;
+        uint32_t box = 0u;
         if (f2t != kPadBin) {
-            TriGeom t;
-            stage_cov(a, b, f2t, W, H, px0, py0, me.c, lane, t);
-            if (me.c.box[lane] != 0) stage_rows(me.c, me.ef, lane);
-        } else {
-            me.c.box[lane] = 0;
+            const bool second = f2t & 1u;
+            const int ox = 256 * px0, oy = 256 * py0;
+            const int32_t x[3] = {a.x - ox, (second ? a.z : a.y) - ox, (second ? a.w : a.z) - ox};
+            const int32_t y[3] = {b.x - oy, (second ? b.z : b.y) - oy, (second ? b.w : b.z) - oy};
+            int4 e[3];
+            box = stage_edges(x, y, min(kTileW, W - px0), min(kTileH, rows), e);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (box) me.edge[k][lane] = e[k];
         }
         f2t = f2t_next;
-        // the box rows of the chunk's 32 triangles as one sequence, so that
-        // every round gives each lane a row whatever the boxes' sizes
-        const int bx_l = me.c.box[lane];
-        const uint32_t rows_l = (uint32_t)box_bh(bx_l);
+        // the row pairs of the chunk's 32 triangles as one sequence, so that
+        // every round gives each lane a pair whatever the boxes' sizes
+        const uint32_t rows_l = (uint32_t)box_pairs(box);
         uint32_t incl = rows_l;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -153,7 +98,7 @@ __device__ __forceinline__ void count_chunks(CountWarp* s_w, int warp, int lane,
         }
         const uint32_t start_l = incl - rows_l, total = __shfl_sync(0xffffffffu, incl, 31);
         const unsigned nonempty = __ballot_sync(0xffffffffu, rows_l != 0);
-        me.seq[lane] = make_uint4(start_l, 0u, (uint32_t)bx_l, 0u);
+        me.seq[lane] = make_uint2(start_l, box);
         if (rows_l) me.r2j[__popc(nonempty & ((1u << lane) - 1u))] = (uint8_t)lane;
         __syncwarp();
         for (uint32_t g = 0; g < total; g += 32) {
@@ -163,30 +108,42 @@ __device__ __forceinline__ void count_chunks(CountWarp* s_w, int warp, int lane,
             const int before = __popc(__ballot_sync(0xffffffffu, rows_l != 0 && start_l < g));
             const uint32_t idx = g + (uint32_t)lane;
             if (idx < total) {
-                const int c = __popc(smask & (0xffffffffu >> (31 - lane)));   // starts in [g, idx]
-                const int j = me.r2j[c > 0 ? before + c - 1 : before - 1];
-                const uint4 sq = me.seq[j];
-                const int bx = (int)sq.z;
-                const int ry = (int)(idx - sq.x);
-                int lo, hi;
-                row_span(me.c, me.ef, j, ry, box_bw(bx), lo, hi);
-                uint32_t* mrow = &me.mask[(box_ly0(bx) + ry) * kTileW + box_lx0(bx)];
-                for (int rx = lo; rx <= hi; ++rx) atomicOr(mrow + rx, 1u << j);
+                const int n = before + __popc(smask & (0xffffffffu >> (31 - lane)));   // starts in [0, idx]
+                const int j = me.r2j[n - 1];
+                const uint2 sq = me.seq[j];
+                const int ry = 2 * (int)(idx - sq.x), ly = box_ly0(sq.y) + ry;
+                int lo0 = box_lx0(sq.y), hi0 = box_lx1(sq.y), lo1 = lo0, hi1 = hi0;
+                if (sq.y & kBoxBig) {
+                    const int2 s0 = row_span_big(&me.edge[0][j], kChunk, kTileW, ry, lo0, hi0);
+                    const int2 s1 = row_span_big(&me.edge[0][j], kChunk, kTileW, ry + 1, lo1, hi1);
+                    lo0 = s0.x; hi0 = s0.y;
+                    lo1 = s1.x; hi1 = s1.y;
+                } else {
+                    const int4 e[3] = {me.edge[0][j], me.edge[1][j], me.edge[2][j]};
+                    row_span(e, ry, lo0, hi0);
+                    row_span(e, ry + 1, lo1, hi1);
+                }
+                const uint32_t r0 = lo0 <= hi0 ? ((2u << (hi0 - lo0)) - 1u) << lo0 : 0u;
+                const uint32_t r1 = lo1 <= hi1 && ly + 1 < rows ? ((2u << (hi1 - lo1)) - 1u) << lo1 : 0u;
+                if constexpr (kTileW == 16) {
+                    me.rows[ly / 2][j] = r0 | (r1 << 16);
+                } else {
+                    reinterpret_cast<Row*>(&me.rows[ly / kRowsPerWord][j])[ly % kRowsPerWord] = (Row)r0;
+                    reinterpret_cast<Row*>(&me.rows[(ly + 1) / kRowsPerWord][j])[(ly + 1) % kRowsPerWord] = (Row)r1;
+                }
             }
         }
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < kTilePix / 32; ++k) {
-            const int i = lane + 32 * k;
-            const uint32_t m = me.mask[i];
-            me.mask[i] = 0;
-            masks[(beg / kChunk + c) * kTilePix + i] = m;
+        for (int k = 0; k < kWords; ++k) {
+            const uint32_t m = warp_transpose(me.rows[k][lane], lane);
+            masks[(beg / kChunk + c) * kTilePix + 32 * k + lane] = m;
             count[k] += __popc(m);
         }
         __syncwarp();
     }
 #pragma unroll
-    for (int k = 0; k < kTilePix / 32; ++k) me.mask[lane + 32 * k] = count[k];
+    for (int k = 0; k < kWords; ++k) me.rows[k][lane] = count[k];
 }
 
 }  // namespace hexfc

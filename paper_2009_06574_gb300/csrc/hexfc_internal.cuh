@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <memory>
+#include <type_traits>
 #include <vector>
 
 #include "hexfc.h"
@@ -277,7 +278,7 @@ cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int 
                             cudaStream_t s);
 cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s);
 CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H);
-cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, cudaStream_t s);
+cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s);
 // The count and the drawing pass of several frames, each one launch.
 cudaError_t launch_count_batch(const CountBatch& b, cudaStream_t s);
 cudaError_t launch_draw_batch(const DrawBatch& b, bool sil, int window, cudaStream_t s);

@@ -20,6 +20,8 @@
 // and Eqs. 1-4 (Section "Focus+Context").
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "count_tiles.cuh"
 #include "shade.cuh"
 
@@ -662,8 +664,10 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint64_t* __restrict_
 // the device scalars scal): [0] += fragments, [1] = longest list, [2] += lists
 // longer than kLongList. The last of the frame's tiles sums the copies into
 // scal[0..2].
-// The count of one tile (the body of k_count and k_count_batch).
-__device__ __forceinline__ void count_tile(int tile, const CountItem& a)
+// The count of one tile (the body of k_count and k_count_batch), by the blocks
+// of a cluster: block `slice` of `slices` takes every slices-th run of
+// kConsumerWarps chunks, the first sums the pixels' counts.
+__device__ __forceinline__ void count_tile(int tile, const CountItem& a, uint32_t slice, uint32_t slices)
 {
     extern __shared__ __align__(16) unsigned char count_smem[];
     CountWarp* s_w = reinterpret_cast<CountWarp*>(count_smem);   // [kConsumerWarps]
@@ -671,11 +675,22 @@ __device__ __forceinline__ void count_tile(int tile, const CountItem& a)
     const uint64_t beg = a.tile_off[tile], end = a.tile_off[tile + 1];  // multiples of kChunk
     const uint32_t n_chunks = (uint32_t)((end - beg) / kChunk);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    count_chunks(s_w, warp, lane, a.bins, a.fframe, beg, n_chunks, px0, py0, a.W, a.H, a.masks);
+    count_chunks(s_w[warp], lane, a.bins, a.fframe, beg, n_chunks, slice * kConsumerWarps + warp,
+                 slices * kConsumerWarps, px0, py0, a.W, a.H, a.masks);
     __syncthreads();
     uint32_t n = 0;
 #pragma unroll
-    for (int w = 0; w < kConsumerWarps; ++w) n += s_w[w].mask[threadIdx.x];
+    for (int w = 0; w < kConsumerWarps; ++w) n += (&s_w[w].rows[0][0])[threadIdx.x];
+    if (slices > 1) {
+        const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+        __shared__ uint32_t s_cnt[kTilePix];
+        s_cnt[threadIdx.x] = n;
+        cluster.sync();
+        if (slice == 0)
+            for (uint32_t k = 1; k < slices; ++k) n += cluster.map_shared_rank(s_cnt, k)[threadIdx.x];
+        cluster.sync();   // (a block's shared memory lives until it was read)
+        if (slice != 0) return;
+    }
     a.cnt[(int64_t)tile * kTilePix + threadIdx.x] = n;
     __shared__ uint32_t s_red[3][kConsumerWarps];
     const uint32_t sum = __reduce_add_sync(0xffffffffu, n), mx = __reduce_max_sync(0xffffffffu, n);
@@ -722,16 +737,17 @@ __device__ __forceinline__ void count_tile(int tile, const CountItem& a)
     }
 }
 
-__global__ void __launch_bounds__(kTilePix, 5) k_count(const __grid_constant__ CountItem a)
+__global__ void __launch_bounds__(kTilePix, kCountBlocks) k_count(const __grid_constant__ CountItem a)
 {
-    count_tile((int)a.order[blockIdx.x], a);
+    const uint32_t slices = cooperative_groups::this_cluster().num_blocks();
+    count_tile((int)a.order[blockIdx.x / slices], a, blockIdx.x % slices, slices);
 }
 
 // The count of several frames in one grid (a batch).
-__global__ void __launch_bounds__(kTilePix, 5) k_count_batch(const __grid_constant__ CountBatch b)
+__global__ void __launch_bounds__(kTilePix, kCountBlocks) k_count_batch(const __grid_constant__ CountBatch b)
 {
     const int i = batch_item(b.tile_begin, b.n, blockIdx.x);
-    count_tile((int)b.it[i].order[blockIdx.x - b.tile_begin[i]], b.it[i]);
+    count_tile((int)b.it[i].order[blockIdx.x - b.tile_begin[i]], b.it[i], 0, 1);
 }
 
 }  // namespace
@@ -817,11 +833,30 @@ CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H
                      reinterpret_cast<unsigned long long*>(fb.scal), tiles_x, W, H, tiles_x * tiles_y};
 }
 
-cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, cudaStream_t s)
+cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s)
 {
-    k_count<<<(unsigned)(tiles_x * tiles_y), kTilePix, kConsumerWarps * sizeof(CountWarp), s>>>(
-        count_item(fb, tiles_x, tiles_y, W, H));
-    return cudaGetLastError();
+    // Few tiles with long lists: several blocks a tile, up to four times what the
+    // chip holds at once, so that the longest list does not decide alone, and a
+    // run of chunks for every warp (96^3 at 320x180, 240 tiles of up to 1500
+    // chunks: one block 0.48 ms, as many as fit at once 0.26, twice 0.15, four
+    // times 0.11). The blocks of a tile are a cluster.
+    const int64_t n_tiles = (int64_t)tiles_x * tiles_y;
+    unsigned slices = 1;
+    while (slices < kCountSlices && 2 * slices * n_tiles <= 4 * 152 * kCountBlocks &&
+           slices * n_tiles * 2 * kConsumerWarps * kChunk < n_bins)
+        slices *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)n_tiles * slices);
+    cfg.blockDim = dim3(kTilePix);
+    cfg.dynamicSmemBytes = kConsumerWarps * sizeof(CountWarp);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = slices;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_count, count_item(fb, tiles_x, tiles_y, W, H));
 }
 
 cudaError_t launch_count_batch(const CountBatch& b, cudaStream_t s)

@@ -103,3 +103,21 @@ def test_lists_survive_an_importance_update(hx):
     assert not torch.equal(again, out)
     assert not np.array_equal(r.debug_pixels(px, py)["rgba"], a["rgba"])
     r.close()
+
+
+# one block a tile's count, and clusters of 2 to 8 of them; lists that end inside a chunk, a run of chunks, a tile
+@pytest.mark.parametrize("n,w,h", [(2, 32, 32), (14, 16, 16), (26, 47, 35), (40, 320, 180), (30, 640, 250)])
+def test_counts_with_and_without_clusters(hx, n, w, h):
+    mesh = synth.hex_grid(n, jitter=0.1, warp_amp=0.2, seed=11)
+    view, lens, style = synth.orbit_view(9, 120, w, h), synth.lissajous_lens(9, 120), synth.Style(w_base=1.0)
+    r, mid = _renderer(hx, mesh, view, lens, style)
+    one = torch.full((h, w, 4), -1.0, device="cuda")
+    r.render(mid, one)
+    outs = [torch.full((h, w, 4), -1.0, device="cuda") for _ in range(2)]
+    st, per, stats = r.render_batch([(mid, view, lens, style, o) for o in outs])   # one block a tile
+    assert st == 0 and all(p == 0 for p in per)
+    for o, s in zip(outs, stats):
+        assert torch.equal(o, one)
+        for k in ("fragments", "bin_entries", "max_list", "long_lists", "covered_pixels"):
+            assert s[k] == r.last_stats[k], k
+    r.close()
