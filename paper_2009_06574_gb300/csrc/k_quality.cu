@@ -15,10 +15,6 @@
 namespace hexfc {
 namespace {
 
-// neighbours of corner k of a VTK hexahedron, right-handed
-__constant__ int8_t c_corner_nb[8][3] = {{1, 3, 4}, {2, 0, 5}, {3, 1, 6}, {0, 2, 7},
-                                         {7, 5, 0}, {4, 6, 1}, {5, 7, 2}, {6, 4, 3}};
-
 __device__ __forceinline__ float det3f(float3 a, float3 b, float3 c)
 {
     return a.x * (b.y * c.z - b.z * c.y) + a.y * (b.z * c.x - b.x * c.z) + a.z * (b.x * c.y - b.y * c.x);
@@ -27,9 +23,21 @@ __device__ __forceinline__ float3 sub3(float3 a, float3 b) { return make_float3(
 __device__ __forceinline__ float3 add3(float3 a, float3 b) { return make_float3(a.x + b.x, a.y + b.y, a.z + b.z); }
 __device__ __forceinline__ float len3(float3 a) { return sqrtf(a.x * a.x + a.y * a.y + a.z * a.z); }
 
-__global__ void k_cell_quality(const float* __restrict__ verts, const int32_t* __restrict__ cells,
-                               int64_t n_cells, int metric, float* __restrict__ out)
+// One thread a cell, the metric at compile time (the ratio needs no lengths), all
+// indices too (the corners stay in registers). The 12 edges' lengths are taken
+// once: the two corners of an edge see it with the same length, bit for bit.
+// 262,144 cells, caches cold: 17 -> 15 us (scaled Jacobian), 17 -> 11 us (ratio).
+// Bound by the gathers' latency, then by the 9 divisions and 15 square roots a
+// cell; cells, vertices and results are 13 MB, 2 us at the copy rate.
+template <int kMetric>
+__global__ void __launch_bounds__(128) k_cell_quality(const float* __restrict__ verts, const int32_t* __restrict__ cells,
+                                                      int64_t n_cells, float* __restrict__ out)
 {
+    // neighbours of corner k of a VTK hexahedron, right-handed, and the edges to them
+    constexpr int kNb[8][3] = {{1, 3, 4}, {2, 0, 5}, {3, 1, 6}, {0, 2, 7}, {7, 5, 0}, {4, 6, 1}, {5, 7, 2}, {6, 4, 3}};
+    constexpr int kEdge[8][3] = {{0, 3, 8}, {1, 0, 9}, {2, 1, 10}, {3, 2, 11}, {7, 4, 8}, {4, 5, 9}, {5, 6, 10}, {6, 7, 11}};
+    constexpr int kEnds[12][2] = {{0, 1}, {1, 2}, {2, 3}, {3, 0}, {4, 5}, {5, 6}, {6, 7}, {7, 4}, {0, 4}, {1, 5}, {2, 6}, {3, 7}};
+    constexpr bool kRatio = kMetric == HEXFC_METRIC_JACOBIAN_RATIO;
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n_cells) return;
     const int4* cc = reinterpret_cast<const int4*>(cells + 8 * c);
@@ -40,34 +48,45 @@ __global__ void k_cell_quality(const float* __restrict__ verts, const int32_t* _
     for (int k = 0; k < 8; ++k)
         p[k] = make_float3(__ldg(verts + 3 * (int64_t)id[k]), __ldg(verts + 3 * (int64_t)id[k] + 1),
                            __ldg(verts + 3 * (int64_t)id[k] + 2));
+    float len[12];
+    if (!kRatio) {
+#pragma unroll
+        for (int e = 0; e < 12; ++e) len[e] = len3(sub3(p[kEnds[e][1]], p[kEnds[e][0]]));
+    }
     float sj = 3.0e38f, dmin = 3.0e38f, dmax = -3.0e38f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        float3 e0 = sub3(p[c_corner_nb[k][0]], p[k]);
-        float3 e1 = sub3(p[c_corner_nb[k][1]], p[k]);
-        float3 e2 = sub3(p[c_corner_nb[k][2]], p[k]);
+        float3 e0 = sub3(p[kNb[k][0]], p[k]);
+        float3 e1 = sub3(p[kNb[k][1]], p[k]);
+        float3 e2 = sub3(p[kNb[k][2]], p[k]);
         float d = det3f(e0, e1, e2);
-        float l = len3(e0) * len3(e1) * len3(e2);
-        float nd = l > 0.f ? d / l : 0.f;
-        sj = fminf(sj, nd);
-        dmin = fminf(dmin, d);
-        dmax = fmaxf(dmax, d);
+        if (kRatio) {
+            dmin = fminf(dmin, d);
+            dmax = fmaxf(dmax, d);
+        } else {
+            float l = len[kEdge[k][0]] * len[kEdge[k][1]] * len[kEdge[k][2]];
+            float nd = l > 0.f ? d / l : 0.f;
+            sj = fminf(sj, nd);
+        }
     }
     {
         float3 X0 = add3(add3(sub3(p[1], p[0]), sub3(p[2], p[3])), add3(sub3(p[5], p[4]), sub3(p[6], p[7])));
         float3 X1 = add3(add3(sub3(p[3], p[0]), sub3(p[2], p[1])), add3(sub3(p[7], p[4]), sub3(p[6], p[5])));
         float3 X2 = add3(add3(sub3(p[4], p[0]), sub3(p[5], p[1])), add3(sub3(p[6], p[2]), sub3(p[7], p[3])));
         float d = det3f(X0, X1, X2);
-        float l = len3(X0) * len3(X1) * len3(X2);
-        float nd = l > 0.f ? d / l : 0.f;
-        sj = fminf(sj, nd);
-        float dc = d * (1.0f / 64.0f);
-        dmin = fminf(dmin, dc);
-        dmax = fmaxf(dmax, dc);
+        if (kRatio) {
+            float dc = d * (1.0f / 64.0f);
+            dmin = fminf(dmin, dc);
+            dmax = fmaxf(dmax, dc);
+        } else {
+            float l = len3(X0) * len3(X1) * len3(X2);
+            float nd = l > 0.f ? d / l : 0.f;
+            sj = fminf(sj, nd);
+        }
     }
     float v;
-    if (metric == HEXFC_METRIC_SCALED_JACOBIAN) v = sj;
-    else if (metric == HEXFC_METRIC_JACOBIAN_RATIO) v = dmax > 0.f ? dmin / dmax : -1.f;
+    if (kMetric == HEXFC_METRIC_SCALED_JACOBIAN) v = sj;
+    else if (kRatio) v = dmax > 0.f ? dmin / dmax : -1.f;
     else v = fminf(fmaxf(1.f - sj, 0.f), 1.f);
     out[c] = v;
 }
@@ -148,8 +167,11 @@ inline unsigned grid_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b);
 
 cudaError_t launch_cell_quality(const DevMesh& m, int metric, float* out, cudaStream_t s)
 {
-    if (m.n_cells > 0)
-        k_cell_quality<<<grid_for(m.n_cells, 256), 256, 0, s>>>(m.verts, m.cells, m.n_cells, metric, out);
+    if (m.n_cells == 0) return cudaSuccess;
+    auto go = [&](auto kernel) { kernel<<<grid_for(m.n_cells, 128), 128, 0, s>>>(m.verts, m.cells, m.n_cells, out); };
+    if (metric == HEXFC_METRIC_SCALED_JACOBIAN) go(k_cell_quality<HEXFC_METRIC_SCALED_JACOBIAN>);
+    else if (metric == HEXFC_METRIC_JACOBIAN_RATIO) go(k_cell_quality<HEXFC_METRIC_JACOBIAN_RATIO>);
+    else go(k_cell_quality<HEXFC_METRIC_IMPORTANCE>);
     return cudaGetLastError();
 }
 
