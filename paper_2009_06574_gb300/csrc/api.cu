@@ -187,7 +187,7 @@ void free_mesh(DevMesh* m)
 
 void free_frame(FrameBufs& f)
 {
-    dfree(f.vproj); dfree(f.ved); dfree(f.fframe); dfree(f.tzsum); dfree(f.trange); dfree(f.slots); dfree(f.fextra); dfree(f.tile_big);
+    dfree(f.vproj); dfree(f.ved); dfree(f.fframe); dfree(f.tzsum); dfree(f.trange); dfree(f.slots); dfree(f.fextra); dfree(f.tile_big); dfree(f.tile_skip);
     dfree(f.tile_cnt); dfree(f.tile_off); dfree(f.tile_cur); dfree(f.tile_order); dfree(f.tile_frag); dfree(f.tile_cap); dfree(f.cap_off); dfree(f.cap_x);
     dfree(f.bins); dfree(f.bins_tmp); dfree(f.masks); dfree(f.zsuf); dfree(f.cnt); dfree(f.zsil);
     dfree(f.part); dfree(f.part_max); dfree(f.redo); dfree(f.scal);
@@ -504,7 +504,7 @@ uint64_t frame_bytes(const FrameBufs& f, int64_t frags)
     uint64_t b = 0;
     b += (uint64_t)f.v_cap * (sizeof(int4) + sizeof(float));
     b += (uint64_t)f.f_cap * (sizeof(FaceFrame) + 2 * sizeof(uint32_t));
-    b += (uint64_t)f.t_cap * (9 * sizeof(uint32_t) + sizeof(uint64_t) + sizeof(uint32_t));
+    b += (uint64_t)f.t_cap * (10 * sizeof(uint32_t) + sizeof(uint64_t) + sizeof(uint32_t));
     b += (uint64_t)f.bin_cap * 2 * sizeof(uint32_t) + (uint64_t)f.mask_cap * sizeof(uint32_t) +
          (uint64_t)f.zsuf_cap * sizeof(uint32_t);
     b += (uint64_t)f.p_cap * (3 * sizeof(uint32_t));
@@ -533,8 +533,9 @@ hexfc_status job_alloc(FrameJob& j)
         free_slots(fb);
     }
     if (!fb.tile_cnt || fb.t_cap < j.n_tiles + 1) {
-        int64_t c1 = 0, c2 = 0, c3 = 0, c4 = 0, c5 = 0, c6 = 0;
+        int64_t c1 = 0, c2 = 0, c3 = 0, c4 = 0, c5 = 0, c6 = 0, c7 = 0;
         dfree(fb.tile_off); dfree(fb.tile_cur); dfree(fb.tile_order); dfree(fb.tile_frag); dfree(fb.tile_big);
+        dfree(fb.tile_skip);
         dfree(fb.cap_x);
         if ((st = ensure(&fb.tile_cnt, &fb.t_cap, j.n_tiles + 1)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.tile_off, &c1, fb.t_cap)) != HEXFC_OK) return st;
@@ -543,6 +544,7 @@ hexfc_status job_alloc(FrameJob& j)
         if ((st = ensure(&fb.tile_frag, &c4, fb.t_cap)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.tile_big, &c5, fb.t_cap)) != HEXFC_OK) return st;
         if ((st = ensure(&fb.cap_x, &c6, 4 * fb.t_cap)) != HEXFC_OK) return st;
+        if ((st = ensure(&fb.tile_skip, &c7, fb.t_cap)) != HEXFC_OK) return st;
     }
     if (!fb.cnt || fb.p_cap < j.n_pix + 1) {
         int64_t c1 = 0, c2 = 0;
@@ -758,6 +760,7 @@ DrawItem draw_item(const FrameJob& j, uint64_t limit)
     const FrameBufs& fb = *j.fb;
     DrawItem it{};
     it.tile_off = fb.tile_off;
+    it.tile_chunks = fb.tile_cur;
     it.bins = fb.bins;
     it.masks = fb.masks;
     it.zsuf = fb.zsuf;

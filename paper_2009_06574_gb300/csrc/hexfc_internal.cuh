@@ -150,8 +150,9 @@ struct FrameBufs {
     // tiles
     uint32_t* tile_cnt = nullptr;   // [T+1] pairs whose place is known
     uint32_t* tile_big = nullptr;   // [T+1] the others
+    uint32_t* tile_skip = nullptr;  // [T+1] pairs of triangles that cover no sample (with places only)
     uint64_t* tile_off = nullptr;   // [T+1]
-    uint32_t* tile_cur = nullptr;   // [T]
+    uint32_t* tile_cur = nullptr;   // [T] the binning's places without counts, then the tiles' chunks
     uint32_t* tile_order = nullptr; // [T] tiles by decreasing chunk count
     uint32_t* tile_frag = nullptr;  // [T] exact fragments per tile (the count's or the fused pass's)
     float* cap_x = nullptr;         // [4T] capacity-network features of the frame
@@ -196,6 +197,7 @@ struct OutWin {
 constexpr int kBatchLaunchMax = 64;
 struct CountItem {
     const uint64_t* tile_off;
+    const uint32_t* tile_chunks;
     const uint32_t* bins;
     const FaceFrame* fframe;
     const uint32_t* order;
@@ -213,6 +215,7 @@ struct CountBatch {
 // What the drawing pass needs of a frame.
 struct DrawItem {
     const uint64_t* tile_off;
+    const uint32_t* tile_chunks;   // chunks of the tile's list that are drawn
     const uint32_t* bins;
     const uint32_t* masks;
     const uint32_t* zsuf;
@@ -310,7 +313,7 @@ cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const in
 // scans
 cudaError_t scan_u32_to_u64(const uint32_t* in, uint64_t* out, int64_t n, uint64_t* part,
                             uint32_t* part_max, uint64_t* total_and_max, uint32_t long_threshold,
-                            cudaStream_t s, uint32_t round_to = 0, const uint32_t* in2 = nullptr);
+                            cudaStream_t s, uint32_t round_to = 0, const uint32_t* in2 = nullptr, const uint32_t* in3 = nullptr);
 int64_t scan_partials_needed(int64_t n);
 
 }  // namespace hexfc

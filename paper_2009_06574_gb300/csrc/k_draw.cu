@@ -186,7 +186,7 @@ __device__ __forceinline__ PixelRef pixel_ref(int64_t q, int tiles_x)
 template <class F>
 __device__ __forceinline__ void list_walk(const DrawItem& a, const PixelRef& r, int lane, uint32_t limit, F&& f)
 {
-    const uint64_t cb = a.tile_off[r.tile] / kChunk, ce = a.tile_off[r.tile + 1] / kChunk;
+    const uint64_t cb = a.tile_off[r.tile] / kChunk, ce = cb + a.tile_chunks[r.tile];
     uint32_t k = 0;
     for (uint64_t c0 = cb; c0 < ce; c0 += 32) {
         const uint64_t c = c0 + lane;
@@ -367,8 +367,8 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, in
 {
     const bool allowed = frame_allowed(a.scal, a.limit);
     const int px0 = (tile % a.tiles_x) * kTileW, py0 = (tile / a.tiles_x) * kTileH;
-    const uint64_t beg = a.tile_off[tile], end = a.tile_off[tile + 1];  // multiples of kChunk
-    const uint32_t n_chunks = (uint32_t)((end - beg) / kChunk);
+    const uint64_t beg = a.tile_off[tile];   // a multiple of kChunk
+    const uint32_t n_chunks = a.tile_chunks[tile];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < kRing) mbar_init(&S.full[threadIdx.x], 32);
     if (threadIdx.x < kWarps) S.rel[threadIdx.x] = 0;

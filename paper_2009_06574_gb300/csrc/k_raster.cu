@@ -33,7 +33,7 @@ inline unsigned grid_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b);
 // ------------------------------------------------------------------ vertex stage
 
 // Thread per vertex: window position on 1/256 pixel, 24-bit depth, eye depth.
-// It also clears the frame's counters (tile_cnt, tile_big, tile_cur, and the
+// It also clears the frame's counters (tile_cnt, tile_big, tile_skip, tile_cur, and the
 // device scalars but the error word), which every frame starts from zero.
 __global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ verts, int64_t n,
                                                       const __grid_constant__ CamParams cam,
@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ 
                                                       int4* __restrict__ vproj, float* __restrict__ ved,
                                                       uint32_t* __restrict__ tile_cnt,
                                                       uint32_t* __restrict__ tile_big,
+                                                      uint32_t* __restrict__ tile_skip,
                                                       uint32_t* __restrict__ tile_cur, int64_t n_tiles,
                                                       uint64_t* __restrict__ scal)
 {
@@ -48,6 +49,7 @@ __global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ 
     for (int64_t i = v; i < n_tiles; i += (int64_t)gridDim.x * blockDim.x) {
         tile_cnt[i] = 0;
         tile_big[i] = 0;
+        if (tile_skip) tile_skip[i] = 0;
         tile_cur[i] = 0;
     }
     if (v < kScalAll && v != 5) scal[v] = 0;
@@ -116,9 +118,10 @@ __device__ __forceinline__ bool outside_lens(const float (&o)[3][3], const float
 }
 
 // A triangle's tiles in one word: the first one's column and row, whether it
-// touches a second column and row (kRangeSmall), or that there are more than
-// 2x2 (kRangeBig: found again in the second pass).
-constexpr uint32_t kRangeSmall = 1u << 24, kRangeBig = 1u << 25;
+// touches a second column and row (kRangeSmall) and that it covers no sample
+// (kRangeSkip), or that there are more than 2x2 (kRangeBig: found again in the
+// second pass).
+constexpr uint32_t kRangeSmall = 1u << 24, kRangeBig = 1u << 25, kRangeSkip = 1u << 26;
 __device__ __forceinline__ uint32_t pack_range(int tx0, int ty0, int tx1, int ty1)
 {
     return (uint32_t)tx0 | ((uint32_t)ty0 << 11) | ((uint32_t)(tx1 - tx0) << 22) | ((uint32_t)(ty1 - ty0) << 23) |
@@ -128,17 +131,18 @@ static_assert(16384 / 8 <= 2048, "eleven bits of tile column and row");
 
 // Each lane's place in the counters of up to four tiles (tile < 0: none): one
 // atomic per distinct tile of the warp, lanes of one tile in lane order. All
-// lanes of the warp call it. The four tiles' atomics are in flight together.
-__device__ __forceinline__ uint4 count_places(uint32_t* ctr, const int (&tile)[4])
+// lanes of the warp call it. The four tiles' atomics are in flight together. With
+// `skip` set the lane's tiles are counted apart, in ctr_skip.
+__device__ __forceinline__ uint4 count_places(uint32_t* ctr, uint32_t* ctr_skip, bool skip, const int (&tile)[4])
 {
     const int lane = threadIdx.x & 31;
     unsigned peers[4];
     uint32_t base[4], place[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        peers[k] = __match_any_sync(0xffffffffu, tile[k]);
+        peers[k] = __match_any_sync(0xffffffffu, tile[k] >= 0 && skip ? tile[k] | (1 << 30) : tile[k]);
         base[k] = 0;
-        if (tile[k] >= 0 && lane == __ffs(peers[k]) - 1) base[k] = atomicAdd(ctr + tile[k], (uint32_t)__popc(peers[k]));
+        if (tile[k] >= 0 && lane == __ffs(peers[k]) - 1) base[k] = atomicAdd((skip ? ctr_skip : ctr) + tile[k], (uint32_t)__popc(peers[k]));
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k)
@@ -161,6 +165,19 @@ __device__ __forceinline__ void for_big_tiles(bool big, int tx0, int ty0, int tx
     }
 }
 
+// Is the triangle's sample at pixel (px, py) covered (top-left rule)?
+__device__ __forceinline__ bool covers(const TriGeom& t, int px, int py)
+{
+    bool in = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int a = (k + 1) % 3, b = (k + 2) % 3;
+        const int64_t e = edge_fn(t.X[a], t.Y[a], t.X[b], t.Y[b], 256 * px + 128, 256 * py + 128);
+        in = in && (e > 0 || (e == 0 && top_left(t.X[a], t.Y[a], t.X[b], t.Y[b])));
+    }
+    return in;
+}
+
 // Thread per face: its record of the frame, its triangles' depths, and the
 // counts of the tiles they touch. Bound by the latency of its gathers and
 // atomics (39% of the issue slots). A triangle of at most 2x2 tiles keeps the
@@ -179,7 +196,8 @@ __global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fve
                                                     int reverse, FaceFrame* __restrict__ fframe,
                                                     uint32_t* __restrict__ tzsum, uint32_t* __restrict__ trange,
                                                     uint4* __restrict__ slots, FaceExtra* __restrict__ fextra,
-                                                    uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_big)
+                                                    uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_big,
+                                                    uint32_t* __restrict__ tile_skip)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = i < n_faces;
@@ -220,12 +238,18 @@ __global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fve
             tile_range(t, tx0, ty0, tx1, ty1);
         }
         const bool small = drawn && slots && tx1 - tx0 <= 1 && ty1 - ty0 <= 1;
-        if (small) range[tri] = pack_range(tx0, ty0, tx1, ty1);
+        // A box of one or two samples, none of them covered: set aside, neither
+        // ordered nor drawn (it still counts for the tile's depth range and the
+        // frame's pairs). A third of the pairs where triangles are about a pixel
+        // (96^3 at 320x180: 4.2 -> 2.8 million, 2.01 -> 1.35 ms a frame), none at
+        // 64^3 and 1920x1080; boxes of up to four samples would be 1% more.
+        const bool skip = small && t.bx1 - t.bx0 + t.by1 - t.by0 <= 1 && !covers(t, t.bx0, t.by0) && !covers(t, t.bx1, t.by1);
+        if (small) range[tri] = pack_range(tx0, ty0, tx1, ty1) | (skip ? kRangeSkip : 0u);
         else if (drawn) range[tri] = kRangeBig;
         const int t0 = ty0 * tiles_x + tx0;
         const bool c2 = small && tx1 > tx0, r2 = small && ty1 > ty0;
         const int tile[4] = {small ? t0 : -1, c2 ? t0 + 1 : -1, r2 ? t0 + tiles_x : -1, c2 && r2 ? t0 + tiles_x + 1 : -1};
-        place[tri] = count_places(tile_cnt, tile);
+        place[tri] = count_places(tile_cnt, tile_skip, skip, tile);
         for_big_tiles(drawn && !small, tx0, ty0, tx1, ty1, tiles_x, [&](int at, int) { atomicAdd(tile_big + at, 1u); });
     }
     if (!in) return;
@@ -266,8 +290,9 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
                                                   const uint32_t* __restrict__ trange, const uint4* __restrict__ slots,
                                                   int64_t n_tris, int W, int H, int tiles_x,
                                                   const uint64_t* __restrict__ tile_off,
-                                                  const uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_cur,
-                                                  uint32_t* __restrict__ bins)
+                                                  const uint32_t* __restrict__ tile_cnt,
+                                                  const uint32_t* __restrict__ tile_big,
+                                                  uint32_t* __restrict__ tile_cur, uint32_t* __restrict__ bins)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t range = 0;
@@ -277,10 +302,14 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
         const uint4 p = slots[t];
         const int tile = (int)((range >> 11) & 2047u) * tiles_x + (int)(range & 2047u);
         const bool c2 = (range >> 22) & 1u, r2 = (range >> 23) & 1u;
-        bins[tile_off[tile] + p.x] = (uint32_t)t;
-        if (c2) bins[tile_off[tile + 1] + p.y] = (uint32_t)t;
-        if (r2) bins[tile_off[tile + tiles_x] + p.z] = (uint32_t)t;
-        if (c2 && r2) bins[tile_off[tile + tiles_x + 1] + p.w] = (uint32_t)t;
+        const bool skip = range & kRangeSkip;   // after the tile's others
+        auto put = [&](int at, uint32_t place) {
+            bins[tile_off[at] + (skip ? tile_cnt[at] + tile_big[at] : 0u) + place] = (uint32_t)t;
+        };
+        put(tile, p.x);
+        if (c2) put(tile + 1, p.y);
+        if (r2) put(tile + tiles_x, p.z);
+        if (c2 && r2) put(tile + tiles_x + 1, p.w);
     }
     int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
     if (range & kRangeBig) {
@@ -307,7 +336,8 @@ constexpr int kScanTiles = 16384;   // most tiles of the one-block scan (16 a th
 // the tail of the launch. One launch for what four took (64^3 at 1920x1080, 8160
 // tiles: 14 us, before 13 for the scan and 19 for the order).
 __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__ tile_cnt,
-                                                    const uint32_t* __restrict__ tile_big, int n,
+                                                    const uint32_t* __restrict__ tile_big,
+                                                    const uint32_t* __restrict__ tile_skip, int n,
                                                     uint64_t* __restrict__ tile_off, uint32_t* __restrict__ order,
                                                     uint64_t* __restrict__ total)
 {
@@ -319,7 +349,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
         const int t = t0 + k;
-        nc[k] = k < per && t < n ? (tile_cnt[t] + tile_big[t] + kChunk - 1) / kChunk : 0u;
+        nc[k] = k < per && t < n ? (tile_cnt[t] + tile_big[t] + (tile_skip ? tile_skip[t] : 0u) + kChunk - 1) / kChunk : 0u;
         sum += nc[k];
         mx = max(mx, nc[k]);
     }
@@ -411,7 +441,9 @@ __host__ __device__ constexpr size_t sort_smem(int threads, int items, int nb)
 template <int kT, int kItems>
 __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bin_sort(const uint64_t* __restrict__ tile_off,
                                                             const uint32_t* __restrict__ tile_cnt,
-                                                 const uint32_t* __restrict__ tile_big, uint32_t* __restrict__ bins,
+                                                 const uint32_t* __restrict__ tile_big,
+                                                 const uint32_t* __restrict__ tile_skip,
+                                                 uint32_t* __restrict__ tile_chunks, uint32_t* __restrict__ bins,
                                                  const uint32_t* __restrict__ tzsum, int nb,
                                                  uint32_t* __restrict__ tmp, uint32_t* __restrict__ zsuf,
                                                  const CapFeatures cf)
@@ -424,12 +456,16 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
     uint32_t* s_hist = s_red + 64;             // [max(nb, kT)]
     const int tile = blockIdx.x;
     const uint64_t beg = tile_off[tile];
-    const uint32_t n = tile_cnt[tile] + tile_big[tile];
+    const uint32_t n = tile_cnt[tile] + tile_big[tile], all = n + (tile_skip ? tile_skip[tile] : 0u);
     const uint32_t n_chunks = (n + kChunk - 1) / kChunk;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint32_t i = n + threadIdx.x; i < n_chunks * kChunk; i += kT) bins[beg + i] = kPadBin;
+    auto pad = [&]() {   // the last chunk, over what was read of the rest
+        for (uint32_t i = n + threadIdx.x; i < n_chunks * kChunk; i += kT) bins[beg + i] = kPadBin;
+    };
+    if (threadIdx.x == 0) tile_chunks[tile] = n_chunks;
     uint32_t zmin = 0xFFFFFFFFu, zmax = 0;
-    if (n < 2 || nb == 0) {   // nothing to order
+    if (all < 2 || nb == 0) {   // nothing to order
+        pad();
         for (uint32_t i = threadIdx.x; i < n_chunks; i += kT) zsuf[beg / kChunk + i] = 0u;
         zmin = 0;
     } else {
@@ -457,6 +493,12 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
                 zmax = max(zmax, z);
             }
         }
+        // triangles that cover no sample count for the tile's depth range only
+        for (uint32_t i = n + threadIdx.x; i < all; i += kT) {
+            const uint32_t z = tzsum[bins[beg + i]] & kZSum;
+            zmin = min(zmin, z);
+            zmax = max(zmax, z);
+        }
         for (int i = threadIdx.x; i < nb; i += kT) s_hist[i] = 0;
         for (uint32_t i = threadIdx.x; i < kLow; i += kT) s_low[i] = 0xFFFFFFFFu;
         zmin = __reduce_min_sync(0xffffffffu, zmin);
@@ -466,6 +508,7 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
             s_red[32 + warp] = zmax;
         }
         __syncthreads();
+        pad();
         zmin = __reduce_min_sync(0xffffffffu, s_red[lane % (kT / 32)]);
         zmax = __reduce_max_sync(0xffffffffu, s_red[32 + lane % (kT / 32)]);
         const float scale = (float)nb / (float)(zmax - zmin + 1);
@@ -672,8 +715,8 @@ __device__ __forceinline__ void count_tile(int tile, const CountItem& a, uint32_
     extern __shared__ __align__(16) unsigned char count_smem[];
     CountWarp* s_w = reinterpret_cast<CountWarp*>(count_smem);   // [kConsumerWarps]
     const int px0 = (tile % a.tiles_x) * kTileW, py0 = (tile / a.tiles_x) * kTileH;
-    const uint64_t beg = a.tile_off[tile], end = a.tile_off[tile + 1];  // multiples of kChunk
-    const uint32_t n_chunks = (uint32_t)((end - beg) / kChunk);
+    const uint64_t beg = a.tile_off[tile];   // a multiple of kChunk
+    const uint32_t n_chunks = a.tile_chunks[tile];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     count_chunks(s_w[warp], lane, a.bins, a.fframe, beg, n_chunks, slice * kConsumerWarps + warp,
                  slices * kConsumerWarps, px0, py0, a.W, a.H, a.masks);
@@ -770,7 +813,7 @@ cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBuf
     const unsigned tiles = std::min(grid_for(n_tiles, 256), 1216u);   // (two blocks' worth of clears an SM at most)
     k_vertex_setup<<<std::max(grid_for(m.n_verts, 256), tiles), 256, 0, s>>>(m.verts, m.n_verts, cam, cam_pairs(cam),
                                                                              fb.vproj, fb.ved, fb.tile_cnt, fb.tile_big,
-                                                                             fb.tile_cur, n_tiles, fb.scal);
+                                                                             fb.tile_skip, fb.tile_cur, n_tiles, fb.scal);
     return cudaGetLastError();
 }
 
@@ -781,7 +824,7 @@ cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const Shad
     k_face_setup<<<grid_for(m.n_faces, 256), 256, 0, s>>>(m.fverts, m.fedges, m.fbound, m.fstat.get(), m.elevel,
                                                            m.eattr, fb.vproj, fb.ved, m.n_faces, sp, cam.W, cam.H,
                                                            tiles_x, reverse, fb.fframe, fb.tzsum, fb.trange, fb.slots, fb.fextra,
-                                                           fb.tile_cnt, fb.tile_big);
+                                                           fb.tile_cnt, fb.tile_big, fb.tile_skip);
     return cudaGetLastError();
 }
 
@@ -790,15 +833,16 @@ cudaError_t launch_tile_scan(FrameBufs& fb, int64_t n_tiles, bool* ordered, cuda
     *ordered = n_tiles <= kScanTiles;
     if (!*ordered)
         return scan_u32_to_u64(fb.tile_cnt, fb.tile_off, n_tiles, fb.part, fb.part_max, fb.scal + 8, 0xFFFFFFFFu, s,
-                               (uint32_t)kChunk, fb.tile_big);
-    k_tile_scan<<<1, 1024, 0, s>>>(fb.tile_cnt, fb.tile_big, (int)n_tiles, fb.tile_off, fb.tile_order, fb.scal + 8);
+                               (uint32_t)kChunk, fb.tile_big, fb.slots ? fb.tile_skip : nullptr);
+    k_tile_scan<<<1, 1024, 0, s>>>(fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, (int)n_tiles, fb.tile_off, fb.tile_order, fb.scal + 8);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, cudaStream_t s)
 {
     k_bin_fill<<<grid_for(2 * m.n_faces, 256), 256, 0, s>>>(fb.fframe, fb.trange, fb.slots, 2 * m.n_faces, W, H,
-                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins);
+                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_big, fb.tile_cur,
+                                                             fb.bins);
     return cudaGetLastError();
 }
 
@@ -807,7 +851,7 @@ cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int 
 {
     auto go = [&](auto kernel, int threads, int items) {
         kernel<<<(unsigned)n_tiles, threads, sort_smem(threads, items, buckets), s>>>(
-            fb.tile_off, fb.tile_cnt, fb.tile_big, fb.bins, fb.tzsum, buckets, fb.bins_tmp, fb.zsuf, cf);
+            fb.tile_off, fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, fb.tile_cur, fb.bins, fb.tzsum, buckets, fb.bins_tmp, fb.zsuf, cf);
     };
     // Many tiles: several blocks an SM, to go on with others while one waits at its
     // barriers; 16 entries a thread where lists of more than 8 x 256 are common
@@ -829,7 +873,7 @@ cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s)
 
 CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H)
 {
-    return CountItem{fb.tile_off, fb.bins, fb.fframe, fb.tile_order, fb.cnt, fb.masks, fb.tile_frag,
+    return CountItem{fb.tile_off, fb.tile_cur, fb.bins, fb.fframe, fb.tile_order, fb.cnt, fb.masks, fb.tile_frag,
                      reinterpret_cast<unsigned long long*>(fb.scal), tiles_x, W, H, tiles_x * tiles_y};
 }
 

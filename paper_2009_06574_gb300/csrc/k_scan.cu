@@ -1,4 +1,4 @@
-// Exclusive prefix scan of uint32 counts (or of the sums of two) into uint64
+// Exclusive prefix scan of uint32 counts (or of the sums of up to three) into uint64
 // offsets, with the total, the maximum and the number of entries above a
 // threshold (each count can be rounded up to a power of two first). Three
 // phases: per-block reduce, scan of the block partials in one block, per-block
@@ -59,7 +59,8 @@ __device__ __forceinline__ uint64_t warp_sum(uint64_t v)
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t* __restrict__ in,
-                                                              const uint32_t* __restrict__ in2, int64_t n,
+                                                              const uint32_t* __restrict__ in2, const uint32_t* __restrict__ in3,
+                                                              int64_t n,
                                                               uint64_t* __restrict__ part,
                                                               uint32_t* __restrict__ part_max,
                                                               uint32_t long_thr, uint32_t round_mask)
@@ -72,7 +73,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t* __
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
         int64_t i = base + k;
-        uint32_t v = i < n ? ((in[i] + (in2 ? in2[i] : 0u) + round_mask) & ~round_mask) : 0u;
+        uint32_t v = i < n ? ((in[i] + (in2 ? in2[i] : 0u) + (in3 ? in3[i] : 0u) + round_mask) & ~round_mask) : 0u;
         sum += v;
         mx = max(mx, v);
         nlong += v > long_thr ? 1u : 0u;
@@ -137,7 +138,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_partials(uint64_t* __rest
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(const uint32_t* __restrict__ in,
-                                                            const uint32_t* __restrict__ in2, int64_t n,
+                                                            const uint32_t* __restrict__ in2, const uint32_t* __restrict__ in3,
+                                                              int64_t n,
                                                             const uint64_t* __restrict__ part,
                                                             uint64_t* __restrict__ out,
                                                             const uint64_t* __restrict__ scal, uint32_t round_mask)
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const uint32_t* __re
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
         int64_t i = base + k;
-        v[k] = i < n ? ((in[i] + (in2 ? in2[i] : 0u) + round_mask) & ~round_mask) : 0u;
+        v[k] = i < n ? ((in[i] + (in2 ? in2[i] : 0u) + (in3 ? in3[i] : 0u) + round_mask) & ~round_mask) : 0u;
         local += v[k];
     }
     uint64_t tot;
@@ -168,14 +170,14 @@ int64_t scan_partials_needed(int64_t n) { return (n + kScanChunk - 1) / kScanChu
 
 cudaError_t scan_u32_to_u64(const uint32_t* in, uint64_t* out, int64_t n, uint64_t* part,
                             uint32_t* part_max, uint64_t* scal, uint32_t long_thr, cudaStream_t s,
-                            uint32_t round_to, const uint32_t* in2)
+                            uint32_t round_to, const uint32_t* in2, const uint32_t* in3)
 {
     int64_t nb = scan_partials_needed(n);
     if (nb < 1) nb = 1;
     const uint32_t rm = round_to > 1 ? round_to - 1 : 0u;   // round_to: 0/1 or a power of two
-    k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, in2, n, part, part_max, long_thr, rm);
+    k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(in, in2, in3, n, part, part_max, long_thr, rm);
     k_scan_partials<<<1, kScanThreads, 0, s>>>(part, part_max, nb, scal);
-    k_scan_down<<<(unsigned)nb, kScanThreads, 0, s>>>(in, in2, n, part, out, scal, rm);
+    k_scan_down<<<(unsigned)nb, kScanThreads, 0, s>>>(in, in2, in3, n, part, out, scal, rm);
     return cudaGetLastError();
 }
 

@@ -121,3 +121,32 @@ def test_counts_with_and_without_clusters(hx, n, w, h):
         for k in ("fragments", "bin_entries", "max_list", "long_lists", "covered_pixels"):
             assert s[k] == r.last_stats[k], k
     r.close()
+
+
+# meshes drawn so small that triangles lie between samples: set aside when binned, where places are kept
+@pytest.mark.parametrize("n,w,h,radius", [(24, 33, 21, 2.0), (40, 64, 48, 2.6), (40, 16, 16, 8.0), (12, 1, 1, 2.0)])
+def test_triangles_between_samples(hx, n, w, h, radius):
+    mesh = synth.hex_grid(n, jitter=0.1, warp_amp=0.2, seed=13)
+    view, lens, style = synth.orbit_view(17, 120, w, h, radius=radius), synth.lissajous_lens(17, 120), synth.Style()
+    imgs, stats, weights = [], [], []
+    budget = 0
+    for kind in ("places", "budget", "noalloc"):
+        r = hx.Renderer(0, frag_budget_bytes=budget if kind == "budget" else 0)
+        mid = r.upload_mesh(mesh.verts, mesh.cells, mesh.cell_scalar, mesh.edge_level)
+        r.set_view(view)
+        r.set_lens(lens)
+        r.set_style(style)
+        out = torch.full((h, w, 4), -1.0, device="cuda")
+        (r.render_noalloc if kind == "noalloc" else r.render)(mid, out)
+        imgs.append(out)
+        stats.append({k: r.last_stats[k] for k in ("fragments", "bin_entries", "max_list", "covered_pixels")})
+        if kind != "noalloc":   # the network's features of the frame
+            r.capacity_reset(5)
+            r.capacity_train(4, lr=1e-2)
+            weights.append(r.capacity_get_weights())
+            budget = r.frame_memory() - 3 * n ** 3 * 16   # too little for the places (72 bytes a face)
+        r.close()
+    for img, st in zip(imgs[1:], stats[1:]):
+        assert torch.equal(img, imgs[0])
+        assert st == stats[0]
+    np.testing.assert_allclose(weights[1], weights[0], rtol=1e-5, atol=1e-7)
