@@ -80,11 +80,7 @@ __device__ __forceinline__ void count_chunks(CountWarp& me, int lane, const uint
             const int ox = 256 * px0, oy = 256 * py0;
             const int32_t x[3] = {a.x - ox, (second ? a.z : a.y) - ox, (second ? a.w : a.z) - ox};
             const int32_t y[3] = {b.x - oy, (second ? b.z : b.y) - oy, (second ? b.w : b.z) - oy};
-            int4 e[3];
-            box = stage_edges(x, y, min(kTileW, W - px0), min(kTileH, rows), e);
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-                if (box) me.edge[k][lane] = e[k];
+            box = stage_edges(x, y, min(kTileW, W - px0), min(kTileH, rows), &me.edge[0][lane], kChunk);
         }
         f2t = f2t_next;
         // the row pairs of the chunk's 32 triangles as one sequence, so that

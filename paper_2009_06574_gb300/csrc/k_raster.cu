@@ -136,13 +136,15 @@ static_assert(16384 / 8 <= 2048, "eleven bits of tile column and row");
 __device__ __forceinline__ uint4 count_places(uint32_t* ctr, uint32_t* ctr_skip, bool skip, const int (&tile)[4])
 {
     const int lane = threadIdx.x & 31;
+    const int apart = skip ? 1 << 30 : 0;   // (no tile, -1, stays -1)
+    uint32_t* const c = skip ? ctr_skip : ctr;
     unsigned peers[4];
     uint32_t base[4], place[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        peers[k] = __match_any_sync(0xffffffffu, tile[k] >= 0 && skip ? tile[k] | (1 << 30) : tile[k]);
+        peers[k] = __match_any_sync(0xffffffffu, tile[k] | apart);
         base[k] = 0;
-        if (tile[k] >= 0 && lane == __ffs(peers[k]) - 1) base[k] = atomicAdd((skip ? ctr_skip : ctr) + tile[k], (uint32_t)__popc(peers[k]));
+        if (tile[k] >= 0 && lane == __ffs(peers[k]) - 1) base[k] = atomicAdd(c + tile[k], (uint32_t)__popc(peers[k]));
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k)
@@ -290,9 +292,8 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
                                                   const uint32_t* __restrict__ trange, const uint4* __restrict__ slots,
                                                   int64_t n_tris, int W, int H, int tiles_x,
                                                   const uint64_t* __restrict__ tile_off,
-                                                  const uint32_t* __restrict__ tile_cnt,
-                                                  const uint32_t* __restrict__ tile_big,
-                                                  uint32_t* __restrict__ tile_cur, uint32_t* __restrict__ bins)
+                                                  const uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_cur,
+                                                  uint32_t* __restrict__ bins)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t range = 0;
@@ -302,10 +303,10 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
         const uint4 p = slots[t];
         const int tile = (int)((range >> 11) & 2047u) * tiles_x + (int)(range & 2047u);
         const bool c2 = (range >> 22) & 1u, r2 = (range >> 23) & 1u;
-        const bool skip = range & kRangeSkip;   // after the tile's others
-        auto put = [&](int at, uint32_t place) {
-            bins[tile_off[at] + (skip ? tile_cnt[at] + tile_big[at] : 0u) + place] = (uint32_t)t;
-        };
+        // set aside: from the end of the tile's list down
+        const uint64_t* off = range & kRangeSkip ? tile_off + 1 : tile_off;
+        const uint32_t down = range & kRangeSkip ? ~0u : 0u;   // (~place is -1 - place)
+        auto put = [&](int at, uint32_t place) { bins[(int64_t)off[at] + (int32_t)(place ^ down)] = (uint32_t)t; };
         put(tile, p.x);
         if (c2) put(tile + 1, p.y);
         if (r2) put(tile + tiles_x, p.z);
@@ -456,7 +457,7 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
     uint32_t* s_hist = s_red + 64;             // [max(nb, kT)]
     const int tile = blockIdx.x;
     const uint64_t beg = tile_off[tile];
-    const uint32_t n = tile_cnt[tile] + tile_big[tile], all = n + (tile_skip ? tile_skip[tile] : 0u);
+    const uint32_t n = tile_cnt[tile] + tile_big[tile], n_skip = tile_skip ? tile_skip[tile] : 0u;
     const uint32_t n_chunks = (n + kChunk - 1) / kChunk;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto pad = [&]() {   // the last chunk, over what was read of the rest
@@ -464,11 +465,21 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
     };
     if (threadIdx.x == 0) tile_chunks[tile] = n_chunks;
     uint32_t zmin = 0xFFFFFFFFu, zmax = 0;
-    if (all < 2 || nb == 0) {   // nothing to order
+    if (n + n_skip < 2 || nb == 0) {   // nothing to order
         pad();
         for (uint32_t i = threadIdx.x; i < n_chunks; i += kT) zsuf[beg / kChunk + i] = 0u;
         zmin = 0;
     } else {
+        // triangles that cover no sample count for the tile's depth range only
+        if (n_skip) {
+            const uint32_t* aside = bins + tile_off[tile + 1] - n_skip;
+#pragma unroll 1
+            for (uint32_t i = threadIdx.x; i < n_skip; i += kT) {
+                const uint32_t z = tzsum[aside[i]] & kZSum;
+                zmin = min(zmin, z);
+                zmax = max(zmax, z);
+            }
+        }
         const bool big = n > kMax;   // entries re-read, scatter through tmp
         uint32_t f2t[kItems], zs[kItems];
         if (!big) {
@@ -492,12 +503,6 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
                 zmin = min(zmin, z);
                 zmax = max(zmax, z);
             }
-        }
-        // triangles that cover no sample count for the tile's depth range only
-        for (uint32_t i = n + threadIdx.x; i < all; i += kT) {
-            const uint32_t z = tzsum[bins[beg + i]] & kZSum;
-            zmin = min(zmin, z);
-            zmax = max(zmax, z);
         }
         for (int i = threadIdx.x; i < nb; i += kT) s_hist[i] = 0;
         for (uint32_t i = threadIdx.x; i < kLow; i += kT) s_low[i] = 0xFFFFFFFFu;
@@ -841,8 +846,7 @@ cudaError_t launch_tile_scan(FrameBufs& fb, int64_t n_tiles, bool* ordered, cuda
 cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, cudaStream_t s)
 {
     k_bin_fill<<<grid_for(2 * m.n_faces, 256), 256, 0, s>>>(fb.fframe, fb.trange, fb.slots, 2 * m.n_faces, W, H,
-                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_big, fb.tile_cur,
-                                                             fb.bins);
+                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins);
     return cudaGetLastError();
 }
 

@@ -48,8 +48,9 @@ constexpr int32_t kSmallTri = 16384;
 // (edge vector), 1 / (64 * 256 dy) as float bits; for a large triangle low word, dx,
 // dy, high word. The value is exact, and less by one where the top-left rule does
 // not give the edge's own samples to the triangle, so that a sample is inside iff
-// no value is negative.
-HEXFC_ROW uint32_t stage_edges(const int32_t xin[3], const int32_t yin[3], int cols, int rows, int4 edge[3])
+// no value is negative. Edge k goes to edge[k * stride].
+HEXFC_ROW uint32_t stage_edges(const int32_t xin[3], const int32_t yin[3], int cols, int rows, int4* edge,
+                               int stride)
 {
     int32_t x[3] = {xin[0], xin[1], xin[2]}, y[3] = {yin[0], yin[1], yin[2]};
     const int64_t area = (int64_t)(x[1] - x[0]) * (y[2] - y[0]) - (int64_t)(y[1] - y[0]) * (x[2] - x[0]);
@@ -90,7 +91,7 @@ HEXFC_ROW uint32_t stage_edges(const int32_t xin[3], const int32_t yin[3], int c
             e.z = dy;
             e.w = (int32_t)(v >> 32);
         }
-        edge[k] = e;
+        edge[k * stride] = e;
     }
     return (uint32_t)x0 | ((uint32_t)yf << 8) | ((uint32_t)x1 << 16) | ((uint32_t)((y1 - yf) / 2 + 1) << 24) |
            (big ? kBoxBig : 0u);

@@ -22,7 +22,7 @@ extern "C" long check(const int32_t* tris, long n, int cols, int rows, int tw, l
     for (long i = 0; i < n; ++i) {
         const int32_t *x = tris + 6 * i, *y = x + 3;
         int4 e[3];
-        const uint32_t box = stage_edges(x, y, cols, rows, e);
+        const uint32_t box = stage_edges(x, y, cols, rows, e, 1);
         uint32_t got[33] = {0};
         for (int r = 0; r < 2 * box_pairs(box); ++r) {
             int lo = box_lx0(box), hi = box_lx1(box);
