@@ -30,6 +30,18 @@ namespace {
 
 inline unsigned grid_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
+// Small meshes: log2 of the threads a face or triangle gets, as many as one block
+// an SM has room for. A warp goes through the tiles of its large triangles one
+// triangle at a time, so with fewer of them a warp is done sooner, on SMs that
+// have nothing else to do (a 4^3 grid at 256x256: face setup 19 -> 5 us, binning
+// 19 -> 3.5 us).
+inline int spread_for(int64_t n)
+{
+    int spread = 0;
+    while (spread < 5 && n << (spread + 1) <= 152 * 256) ++spread;
+    return spread;
+}
+
 // ------------------------------------------------------------------ vertex stage
 
 // Thread per vertex: window position on 1/256 pixel, 24-bit depth, eye depth.
@@ -199,10 +211,10 @@ __global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fve
                                                     uint32_t* __restrict__ tzsum, uint32_t* __restrict__ trange,
                                                     uint4* __restrict__ slots, FaceExtra* __restrict__ fextra,
                                                     uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_big,
-                                                    uint32_t* __restrict__ tile_skip)
+                                                    uint32_t* __restrict__ tile_skip, int spread)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool in = i < n_faces;
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = g >> spread;
+    const bool in = i < n_faces && i << spread == g;
     const int64_t f = !in ? 0 : reverse ? n_faces - 1 - i : i;
     const int4 c = fverts[f], e = fedges[f];
     const int id[4] = {c.x, c.y, c.z, c.w}, eid[4] = {e.x, e.y, e.z, e.w};
@@ -293,11 +305,11 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
                                                   int64_t n_tris, int W, int H, int tiles_x,
                                                   const uint64_t* __restrict__ tile_off,
                                                   const uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_cur,
-                                                  uint32_t* __restrict__ bins)
+                                                  uint32_t* __restrict__ bins, int spread)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, t = g >> spread;
     uint32_t range = 0;
-    if (t < n_tris)
+    if (t < n_tris && t << spread == g)
         range = trange ? trange[t] : (face_tris(fframe[t >> 1].Z) >> (t & 1)) & 1u ? kRangeBig : 0u;
     if (range & kRangeSmall) {
         const uint4 p = slots[t];
@@ -320,9 +332,9 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
         tri_setup(X, Y, (int)(t & 1), W, H, g);
         tile_range(g, tx0, ty0, tx1, ty1);
     }
-    const int64_t first = t - (threadIdx.x & 31);
+    const int64_t first = g - (threadIdx.x & 31);
     for_big_tiles(range & kRangeBig, tx0, ty0, tx1, ty1, tiles_x, [&](int tile, int src) {
-        bins[tile_off[tile] + tile_cnt[tile] + atomicAdd(tile_cur + tile, 1u)] = (uint32_t)(first + src);
+        bins[tile_off[tile] + tile_cnt[tile] + atomicAdd(tile_cur + tile, 1u)] = (uint32_t)((first + src) >> spread);
     });
 }
 
@@ -826,10 +838,11 @@ cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const Shad
                               int tiles_x, int tiles_y, int reverse, cudaStream_t s)
 {
     (void)tiles_y;
-    k_face_setup<<<grid_for(m.n_faces, 256), 256, 0, s>>>(m.fverts, m.fedges, m.fbound, m.fstat.get(), m.elevel,
+    const int spread = spread_for(m.n_faces);
+    k_face_setup<<<grid_for(m.n_faces << spread, 256), 256, 0, s>>>(m.fverts, m.fedges, m.fbound, m.fstat.get(), m.elevel,
                                                            m.eattr, fb.vproj, fb.ved, m.n_faces, sp, cam.W, cam.H,
                                                            tiles_x, reverse, fb.fframe, fb.tzsum, fb.trange, fb.slots, fb.fextra,
-                                                           fb.tile_cnt, fb.tile_big, fb.tile_skip);
+                                                           fb.tile_cnt, fb.tile_big, fb.tile_skip, spread);
     return cudaGetLastError();
 }
 
@@ -845,8 +858,9 @@ cudaError_t launch_tile_scan(FrameBufs& fb, int64_t n_tiles, bool* ordered, cuda
 
 cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, cudaStream_t s)
 {
-    k_bin_fill<<<grid_for(2 * m.n_faces, 256), 256, 0, s>>>(fb.fframe, fb.trange, fb.slots, 2 * m.n_faces, W, H,
-                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins);
+    const int spread = spread_for(2 * m.n_faces);
+    k_bin_fill<<<grid_for((2 * m.n_faces) << spread, 256), 256, 0, s>>>(fb.fframe, fb.trange, fb.slots, 2 * m.n_faces, W, H,
+                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins, spread);
     return cudaGetLastError();
 }
 
