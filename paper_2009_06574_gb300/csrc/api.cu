@@ -626,7 +626,8 @@ hexfc_status job_read1(FrameJob& j)
 {
     FrameBufs& fb = *j.fb;
     hexfc_status st;
-    j.n_bins = fb.h_scal[8];   // padded to whole chunks per tile
+    j.n_bins = fb.bins_seen = fb.h_scal[8];   // padded to whole chunks per tile
+    fb.bin_limit = ~0ull;
     if (!fb.bins || fb.bin_cap < (int64_t)j.n_bins) {
         int64_t c1 = 0;
         dfree(fb.bins_tmp);
@@ -636,6 +637,13 @@ hexfc_status job_read1(FrameJob& j)
     if ((st = ensure(&fb.masks, &fb.mask_cap, (int64_t)j.n_bins * (kTilePix / kChunk))) != HEXFC_OK) return st;
     if ((st = ensure(&fb.zsuf, &fb.zsuf_cap, (int64_t)(j.n_bins / kChunk))) != HEXFC_OK) return st;
     return HEXFC_OK;
+}
+
+// Bins that the frame's buffers have room for.
+uint64_t bin_room(const FrameBufs& fb)
+{
+    if (!fb.bins) return 0;
+    return (uint64_t)std::min(fb.bin_cap, std::min(fb.mask_cap / (kTilePix / kChunk), fb.zsuf_cap * kChunk));
 }
 
 // Whether the frame's buffers, now that the bins are known, exceed its budget
@@ -749,7 +757,7 @@ hexfc_status job_silhouette(FrameJob& j, float* out, cudaStream_t s)
 {
     if (j.sil_alpha <= 0.f) return HEXFC_OK;
     CK(launch_silhouette(j.fb->zsil, j.tiles_x, j.cam.ox, j.cam.oy, j.frame_w, j.frame_h, j.sil_alpha,
-                         j.sil_threshold, out, j.win, s));
+                         j.sil_threshold, j.fb->scal + 8, j.fb->bin_limit, out, j.win, s));
     j.launches += 1;
     return HEXFC_OK;
 }
@@ -777,6 +785,7 @@ DrawItem draw_item(const FrameJob& j, uint64_t limit)
     it.scal = scal;
     it.err = scal + 5;
     it.limit = limit;
+    it.bin_limit = fb.bin_limit;
     it.sp = j.sp;
     it.win = j.win;
     it.tiles_x = j.tiles_x;
@@ -864,6 +873,7 @@ void keep_frame(hexfc_ctx* ctx, const FrameJob& j)
 hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_stats* stats, cudaStream_t s)
 {
     FrameJob j = make_job(ctx, &ctx->fb, m, out);
+    FrameBufs& fb = ctx->fb;
     hexfc_status st;
     ctx->have_frame = false;   // the frame buffers are this frame's from here on
     if ((st = job_alloc(j)) != HEXFC_OK) return st;
@@ -875,7 +885,24 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
     if (!ctx->ev_p1) CK(cudaEventCreateWithFlags(&ctx->ev_p1, cudaEventDisableTiming));
     j.p1_done = ctx->ev_p1;
     if ((st = job_phase1(j, s)) != HEXFC_OK) return st;
-    if ((st = job_wait1(ctx, j, s)) != HEXFC_OK) return st;
+    if (!ctx->ev_p2) CK(cudaEventCreateWithFlags(&ctx->ev_p2, cudaEventDisableTiming));
+    // With room for a frame's bins and no budget to check them against, the rest
+    // of the frame is launched without waiting for their number; if there turns
+    // out to be too little room, those launches have done nothing and follow
+    // again below. (The number of the last frame only picks the launches' shapes.)
+    // The wait was 15-17 us of an idle GPU a frame (4^3 at 256x256: XX -> XX us).
+    bool drawn = false;
+    if (!j.budget && !ctx->pend.active && bin_room(fb) > 0) {
+        fb.bin_limit = bin_room(fb);
+        j.n_bins = fb.bins_seen;
+        if ((st = job_phase2(j, s)) != HEXFC_OK) return st;
+        CK(cudaEventRecord(ctx->ev_p2, s));
+        if ((st = job_phase3(j, s)) != HEXFC_OK) return st;
+        CK(cudaEventSynchronize(ctx->ev_p2));
+        drawn = fb.h_scal[8] <= fb.bin_limit;
+        j.n_bins = fb.bins_seen = fb.h_scal[8];
+    }
+    if (!drawn && (st = job_wait1(ctx, j, s)) != HEXFC_OK) return st;
     collect(ctx);
     if (ctx->pend.active) {   // the previous frame (chosen capacities) has completed: verify it
         bool redrawn = false;
@@ -885,16 +912,17 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
             if ((st = job_wait1(ctx, j, s)) != HEXFC_OK) return st;
         }
     }
-    if ((st = job_read1(j)) != HEXFC_OK) return st;
-    if (drop_slots(j)) {
-        if ((st = job_phase1(j, s)) != HEXFC_OK) return st;
-        if ((st = job_wait1(ctx, j, s)) != HEXFC_OK) return st;
+    if (!drawn) {
+        if ((st = job_read1(j)) != HEXFC_OK) return st;
+        if (drop_slots(j)) {
+            if ((st = job_phase1(j, s)) != HEXFC_OK) return st;
+            if ((st = job_wait1(ctx, j, s)) != HEXFC_OK) return st;
+        }
+        if ((st = job_phase2(j, s)) != HEXFC_OK) return st;
+        CK(cudaEventRecord(ctx->ev_p2, s));
+        if ((st = job_phase3(j, s)) != HEXFC_OK) return st;
+        CK(cudaEventSynchronize(ctx->ev_p2));   // the totals, while the frame is drawn
     }
-    if ((st = job_phase2(j, s)) != HEXFC_OK) return st;
-    if (!ctx->ev_p2) CK(cudaEventCreateWithFlags(&ctx->ev_p2, cudaEventDisableTiming));
-    CK(cudaEventRecord(ctx->ev_p2, s));
-    if ((st = job_phase3(j, s)) != HEXFC_OK) return st;
-    CK(cudaEventSynchronize(ctx->ev_p2));   // the totals, while the frame is drawn
     st = job_read2(j, s);
     j.fs.frame = ++ctx->frame_seq;
     ctx->last = j.fs;
@@ -2089,28 +2117,58 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     CK(launch_face_setup(*m, ctx->cam, make_shade(ctx), fb, tiles_x, tiles_y, ctx->reverse_bins, s));
     bool ordered = false;
     CK(launch_tile_scan(fb, n_tiles, &ordered, s));
+    // The rest up to the counts is launched without waiting for the number of
+    // bins, laid out for as many as the array has room for (the passes do nothing
+    // if there are more), and the host waits once; the shapes of the launches are
+    // those of triangles in one tile each. What is refused is decided below, as if
+    // the bins had been laid out for their number.
+    const Arena laid = a;
+    const size_t per32 = kChunk * 2 * sizeof(uint32_t) + kTilePix * sizeof(uint32_t) + sizeof(uint32_t);
+    const size_t left = a.cap - a.used, room = left > 2048 ? (left - 2048) / per32 : 0;   // chunks
+    auto bins_in = [&](size_t n) {
+        fb.bins = a.take<uint32_t>(n);
+        fb.bins_tmp = a.take<uint32_t>(n);
+        fb.masks = a.take<uint32_t>(n * (kTilePix / kChunk));
+        fb.zsuf = a.take<uint32_t>(n / kChunk);
+        return fb.bins && fb.bins_tmp && fb.masks && fb.zsuf;
+    };
+    auto to_counts = [&](int64_t about) -> hexfc_status {
+        CK(launch_bin_fill(*m, fb, tiles_x, W, H, s));
+        CK(launch_bin_sort(fb, n_tiles, about, ctx->depth_buckets, CapFeatures{}, s));
+        CK(launch_count(fb, tiles_x, tiles_y, W, H, about, s));
+        return HEXFC_OK;
+    };
+    if (!ordered) CK(launch_tile_order(fb, n_tiles, s));
     uint64_t h[16] = {};  // pageable host copy of the totals (no pinned allocation)
-    CK(cudaMemcpyAsync(h + 8, fb.scal + 8, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    hexfc_status st;
+    fb.bin_limit = room * kChunk;
+    const bool ahead = room > 0 && bins_in(fb.bin_limit);
+    if (ahead && (st = to_counts(2 * m->n_faces)) != HEXFC_OK) return st;
+    CK(cudaMemcpyAsync(h, fb.scal, 9 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     const uint64_t n_bins = h[8];
-    fb.bins = a.take<uint32_t>((size_t)n_bins);
-    fb.bins_tmp = a.take<uint32_t>((size_t)n_bins);
-    fb.masks = a.take<uint32_t>((size_t)n_bins * (kTilePix / kChunk));
-    fb.zsuf = a.take<uint32_t>((size_t)(n_bins / kChunk));
     hexfc_frame_stats fs{};
     fs.bin_entries = n_bins;
     fs.width = (uint32_t)win.w;
     fs.height = (uint32_t)win.h;
-    if (!fb.bins || !fb.bins_tmp || !fb.masks || !fb.zsuf) {
+    const bool counted = ahead && n_bins <= fb.bin_limit;
+    const FrameBufs big = fb;
+    a = laid;
+    if (!bins_in((size_t)n_bins)) {
         if (stats) *stats = fs;
         return HEXFC_ERR_OVERFLOW;
     }
-    CK(launch_bin_fill(*m, fb, tiles_x, W, H, s));
-    CK(launch_bin_sort(fb, n_tiles, (int64_t)n_bins, ctx->depth_buckets, CapFeatures{}, s));
-    if (!ordered) CK(launch_tile_order(fb, n_tiles, s));
-    CK(launch_count(fb, tiles_x, tiles_y, W, H, (int64_t)n_bins, s));
-    CK(cudaMemcpyAsync(h, fb.scal, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    if (counted) {   // where they are
+        fb.bins = big.bins;
+        fb.bins_tmp = big.bins_tmp;
+        fb.masks = big.masks;
+        fb.zsuf = big.zsuf;
+    } else {         // within a few chunks of the array's size
+        fb.bin_limit = ~0ull;
+        if ((st = to_counts((int64_t)n_bins)) != HEXFC_OK) return st;
+        CK(cudaMemcpyAsync(h, fb.scal, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+    }
     if (h[5] != 0) {   // this call's count pass, or the previous call's fill or composite
         CK(cudaMemsetAsync(fb.scal + 5, 0, sizeof(uint64_t), s));
         CK(cudaStreamSynchronize(s));
@@ -2133,7 +2191,7 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     CK(launch_draw_tail(it, s));
     if (sil)
         CK(launch_silhouette(fb.zsil, tiles_x, ctx->cam.ox, ctx->cam.oy, ctx->view.width, ctx->view.height,
-                             ctx->style.sil_alpha, ctx->style.sil_threshold, out, win, s));
+                             ctx->style.sil_alpha, ctx->style.sil_threshold, fb.scal + 8, fb.bin_limit, out, win, s));
     return inject_error_bits(ctx, fb.scal, s);
 }
 

@@ -163,6 +163,8 @@ struct FrameBufs {
     uint32_t* bins = nullptr;       // face2tri ids grouped by tile, each tile padded to whole chunks
     uint32_t* bins_tmp = nullptr;   // scratch of the depth order of long tile lists (same layout)
     bool scal_fresh = false;        // scal just allocated (undefined contents)
+    uint64_t bin_limit = ~0ull;     // bins that there is room for: with more (scal[8]) the later passes do nothing
+    uint64_t bins_seen = 0;         // bins of the last frame
     int64_t bin_cap = 0;
     uint32_t* masks = nullptr;      // per chunk of a tile list: 256 per-pixel coverage masks
     uint32_t* zsuf = nullptr;       // per chunk: a lower bound of the depths of its tile's triangles from it on
@@ -205,6 +207,7 @@ struct CountItem {
     uint32_t* masks;
     uint32_t* tile_frag;
     unsigned long long* scal;
+    uint64_t bin_limit;   // see FrameBufs
     int tiles_x, W, H, n_tiles;
 };
 struct CountBatch {
@@ -230,7 +233,8 @@ struct DrawItem {
     unsigned long long* redo_cursor;
     const unsigned long long* scal;
     unsigned long long* err;
-    uint64_t limit;   // most fragments the frame may have (memory budget)
+    uint64_t limit;       // most fragments the frame may have (memory budget)
+    uint64_t bin_limit;   // see FrameBufs
     ShadeParams sp;
     OutWin win;
     int tiles_x, W, H;
@@ -304,7 +308,8 @@ cudaError_t launch_cap_to_half(CapNet& net, cudaStream_t s);
 // from the boundary surface's depths zsil of the drawn rectangle, which sits
 // at (fx0, fy0) of a frame_w x frame_h frame.
 cudaError_t launch_silhouette(const uint32_t* zsil, int tiles_x, int fx0, int fy0, int frame_w, int frame_h,
-                              float alpha, float threshold, float* out, OutWin win, cudaStream_t s);
+                              float alpha, float threshold, const uint64_t* n_bins, uint64_t bin_limit, float* out,
+                              OutWin win, cudaStream_t s);
 // The sorted lists of n pixels of a frame drawn as `a` (or their lengths, if d_counts).
 cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const int32_t* d_py, int64_t n,
                                 const uint64_t* d_dst_off, uint64_t* d_keys, float4* d_rgba, uint32_t* d_counts,

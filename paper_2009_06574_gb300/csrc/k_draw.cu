@@ -72,9 +72,10 @@ __device__ __forceinline__ bool out_index(const OutWin& w, int x, int y, int64_t
 // Whether the frame may be drawn: no error reported and not yet cleared, its
 // longest list within what the sort takes, its lists within the budget
 // (scal: see kScal).
-__device__ __forceinline__ bool frame_allowed(const unsigned long long* scal, uint64_t limit)
+__device__ __forceinline__ bool frame_allowed(const DrawItem& a)
 {
-    return scal[5] == 0 && scal[1] <= (unsigned long long)HEXFC_MAX_LIST && scal[0] <= limit;
+    const unsigned long long* scal = a.scal;
+    return scal[5] == 0 && scal[1] <= (unsigned long long)HEXFC_MAX_LIST && scal[0] <= a.limit && scal[8] <= a.bin_limit;
 }
 
 // ------------------------------------------------------------------ staging
@@ -318,7 +319,7 @@ __device__ __noinline__ CT block_list(const DrawItem& a, const PixelRef& r, uint
 __global__ void __launch_bounds__(kTilePix, 3) k_draw_tail(const __grid_constant__ DrawItem a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    if (!__syncthreads_and(frame_allowed(a.scal, a.limit))) return;
+    if (!__syncthreads_and(frame_allowed(a))) return;
     bool bad = false;
     const uint64_t n_redo = *a.redo_cursor;
     for (uint64_t i = blockIdx.x; i < n_redo; i += gridDim.x) {
@@ -365,7 +366,7 @@ __device__ __forceinline__ uint32_t load_acquire(const uint32_t* p)
 template <int KW, bool kSil>
 __device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, int tile)
 {
-    const bool allowed = frame_allowed(a.scal, a.limit);
+    const bool allowed = frame_allowed(a);
     const int px0 = (tile % a.tiles_x) * kTileW, py0 = (tile / a.tiles_x) * kTileH;
     const uint64_t beg = a.tile_off[tile];   // a multiple of kChunk
     const uint32_t n_chunks = a.tile_chunks[tile];
@@ -561,10 +562,11 @@ __device__ __forceinline__ uint32_t zsil_at(const uint32_t* __restrict__ zsil, i
 
 __global__ void __launch_bounds__(256) k_silhouette(const uint32_t* __restrict__ zsil, int tiles_x, int fx0, int fy0,
                                                     int frame_w, int frame_h, float alpha, int64_t T,
+                                                    const uint64_t* __restrict__ n_bins, uint64_t bin_limit,
                                                     float4* __restrict__ out, OutWin win)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)win.w * win.h) return;
+    if (i >= (int64_t)win.w * win.h || *n_bins > bin_limit) return;
     const int x = win.x0 + (int)(i % win.w), y = win.y0 + (int)(i / win.w);
     const uint32_t zp = zsil_at(zsil, tiles_x, x, y);
     if (zp == kNoDepth) return;
@@ -697,12 +699,14 @@ cudaError_t launch_draw_tail(const DrawItem& a, cudaStream_t s)
 }
 
 cudaError_t launch_silhouette(const uint32_t* zsil, int tiles_x, int fx0, int fy0, int frame_w, int frame_h,
-                              float alpha, float threshold, float* out, OutWin win, cudaStream_t s)
+                              float alpha, float threshold, const uint64_t* n_bins, uint64_t bin_limit, float* out,
+                              OutWin win, cudaStream_t s)
 {
     const int64_t n = (int64_t)win.w * win.h;
     if (n == 0) return cudaSuccess;
     k_silhouette<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(zsil, tiles_x, fx0, fy0, frame_w, frame_h, alpha,
-                                                             (int64_t)threshold, reinterpret_cast<float4*>(out), win);
+                                                             (int64_t)threshold, n_bins, bin_limit,
+                                                             reinterpret_cast<float4*>(out), win);
     return cudaGetLastError();
 }
 

@@ -305,8 +305,10 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
                                                   int64_t n_tris, int W, int H, int tiles_x,
                                                   const uint64_t* __restrict__ tile_off,
                                                   const uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_cur,
-                                                  uint32_t* __restrict__ bins, int spread)
+                                                  uint32_t* __restrict__ bins, int spread,
+                                                  const uint64_t* __restrict__ n_bins, uint64_t bin_limit)
 {
+    if (*n_bins > bin_limit) return;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, t = g >> spread;
     uint32_t range = 0;
     if (t < n_tris && t << spread == g)
@@ -459,8 +461,10 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
                                                  uint32_t* __restrict__ tile_chunks, uint32_t* __restrict__ bins,
                                                  const uint32_t* __restrict__ tzsum, int nb,
                                                  uint32_t* __restrict__ tmp, uint32_t* __restrict__ zsuf,
+                                                 const uint64_t* __restrict__ n_bins, uint64_t bin_limit,
                                                  const CapFeatures cf)
 {
+    if (*n_bins > bin_limit) return;
     constexpr uint32_t kMax = kT * kItems, kLow = kMax / kChunk;
     extern __shared__ uint32_t sort_sm[];
     uint32_t* s_out = sort_sm;                 // [kMax]
@@ -729,6 +733,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint64_t* __restrict_
 // kConsumerWarps chunks, the first sums the pixels' counts.
 __device__ __forceinline__ void count_tile(int tile, const CountItem& a, uint32_t slice, uint32_t slices)
 {
+    if (a.scal[8] > a.bin_limit) return;   // (all blocks alike)
     extern __shared__ __align__(16) unsigned char count_smem[];
     CountWarp* s_w = reinterpret_cast<CountWarp*>(count_smem);   // [kConsumerWarps]
     const int px0 = (tile % a.tiles_x) * kTileW, py0 = (tile / a.tiles_x) * kTileH;
@@ -860,7 +865,8 @@ cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W,
 {
     const int spread = spread_for(2 * m.n_faces);
     k_bin_fill<<<grid_for((2 * m.n_faces) << spread, 256), 256, 0, s>>>(fb.fframe, fb.trange, fb.slots, 2 * m.n_faces, W, H,
-                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins, spread);
+                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins, spread, fb.scal + 8,
+                                                             fb.bin_limit);
     return cudaGetLastError();
 }
 
@@ -869,7 +875,8 @@ cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int 
 {
     auto go = [&](auto kernel, int threads, int items) {
         kernel<<<(unsigned)n_tiles, threads, sort_smem(threads, items, buckets), s>>>(
-            fb.tile_off, fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, fb.tile_cur, fb.bins, fb.tzsum, buckets, fb.bins_tmp, fb.zsuf, cf);
+            fb.tile_off, fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, fb.tile_cur, fb.bins, fb.tzsum, buckets, fb.bins_tmp, fb.zsuf, fb.scal + 8,
+            fb.bin_limit, cf);
     };
     // Many tiles: several blocks an SM, to go on with others while one waits at its
     // barriers; 16 entries a thread where lists of more than 8 x 256 are common
@@ -892,7 +899,7 @@ cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s)
 CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H)
 {
     return CountItem{fb.tile_off, fb.tile_cur, fb.bins, fb.fframe, fb.tile_order, fb.cnt, fb.masks, fb.tile_frag,
-                     reinterpret_cast<unsigned long long*>(fb.scal), tiles_x, W, H, tiles_x * tiles_y};
+                     reinterpret_cast<unsigned long long*>(fb.scal), fb.bin_limit, tiles_x, W, H, tiles_x * tiles_y};
 }
 
 cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s)

@@ -150,3 +150,34 @@ def test_triangles_between_samples(hx, n, w, h, radius):
         assert torch.equal(img, imgs[0])
         assert st == stats[0]
     np.testing.assert_allclose(weights[1], weights[0], rtol=1e-5, atol=1e-7)
+
+
+def test_frames_whose_bins_outgrow_their_room(hx):
+    """Launches go ahead with the last frame's room for bins: views that need less, more and far more of
+    it, and meshes of other sizes in between, give what a fresh context gives."""
+    meshes = [synth.hex_grid(n, jitter=0.1, warp_amp=0.2, seed=n) for n in (6, 20)]
+    r = hx.Renderer(0)
+    mids = [r.upload_mesh(m.verts, m.cells, m.cell_scalar, m.edge_level) for m in meshes]
+    for k, (w, h, radius) in [(0, (64, 48, 3.0)), (0, (512, 400, 1.2)), (1, (64, 48, 3.0)), (1, (640, 480, 1.2)), (0, (33, 21, 2.0)),
+                              (1, (900, 700, 1.1))]:
+        view, lens, style = synth.orbit_view(7, 120, w, h, radius=radius), synth.lissajous_lens(7, 120), synth.Style(sil_alpha=0.5)
+        imgs, stats = [], []
+        for q, mid in ((r, mids[k]), (hx.Renderer(0), 0)):
+            if q is not r:
+                mid = q.upload_mesh(meshes[k].verts, meshes[k].cells, meshes[k].cell_scalar, meshes[k].edge_level)
+            q.set_view(view)
+            q.set_lens(lens)
+            q.set_style(style)
+            out = torch.full((h, w, 4), -1.0, device="cuda")
+            q.render(mid, out)
+            stats.append({n: q.last_stats[n] for n in ("fragments", "bin_entries", "max_list", "covered_pixels")})
+            imgs.append(out)
+            if q is not r:
+                if k == 0:   # (fits the fixed scratch array)
+                    imgs.append(torch.full((h, w, 4), -1.0, device="cuda"))
+                    q.render_noalloc(mid, imgs[-1])
+                q.close()
+        assert stats[0] == stats[1]
+        for img in imgs[1:]:
+            assert torch.equal(img, imgs[0])
+    r.close()
