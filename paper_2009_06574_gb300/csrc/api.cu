@@ -599,7 +599,8 @@ hexfc_status job_phase1(FrameJob& j, cudaStream_t s)
     CK(launch_tile_scan(fb, j.n_tiles, &j.order_done, s));
     job_mark(j, 3, s);
     j.launches = j.order_done ? 3 : 5;
-    CK(cudaMemcpyAsync(fb.h_scal + 8, fb.scal + 8, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    if (!j.order_done)   // (else the tile scan has written it there)
+        CK(cudaMemcpyAsync(fb.h_scal + 8, fb.scal + 8, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     if (j.p1_done) {
         CK(cudaEventRecord(j.p1_done, s));
         if (!j.order_done) {
@@ -682,23 +683,15 @@ hexfc_status job_phase2_bins(FrameJob& j, cudaStream_t s)
     return HEXFC_OK;
 }
 
-// Phase 2 after the count: its totals to the host.
-hexfc_status job_phase2_totals(FrameJob& j, cudaStream_t s)
-{
-    FrameBufs& fb = *j.fb;
-    job_mark(j, 6, s);
-    job_mark(j, 7, s);
-    j.launches += 1;   // the count
-    CK(cudaMemcpyAsync(fb.h_scal, fb.scal, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    return HEXFC_OK;
-}
-
 hexfc_status job_phase2(FrameJob& j, cudaStream_t s)
 {
     hexfc_status st;
     if ((st = job_phase2_bins(j, s)) != HEXFC_OK) return st;
     CK(launch_count(*j.fb, j.tiles_x, j.tiles_y, j.W, j.H, (int64_t)j.n_bins, s));
-    return job_phase2_totals(j, s);
+    job_mark(j, 6, s);
+    job_mark(j, 7, s);
+    j.launches += 1;   // (the count writes its totals to the host itself)
+    return HEXFC_OK;
 }
 
 // The most fragments the frame may have (what job_read2 refuses, the drawing
@@ -890,7 +883,8 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
     // of the frame is launched without waiting for their number; if there turns
     // out to be too little room, those launches have done nothing and follow
     // again below. (The number of the last frame only picks the launches' shapes.)
-    // The wait was 15-17 us of an idle GPU a frame (4^3 at 256x256: XX -> XX us).
+    // The wait left the GPU idle for 5-15 us a frame (8^3 at 250x190 without
+    // allocation 100 -> 85 us, 4^3 at 256x256 82 -> 78 us).
     bool drawn = false;
     if (!j.budget && !ctx->pend.active && bin_room(fb) > 0) {
         fb.bin_limit = bin_room(fb);
@@ -1016,7 +1010,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     }
     CK(scan_u32_to_u64(fb.tile_cap, fb.cap_off, j.n_tiles, fb.part, fb.part_max, fb.scal + 11, 0xFFFFFFFFu, s));
     job_mark(j, 5, s);
-    CK(launch_count(fb, j.tiles_x, j.tiles_y, j.W, j.H, (int64_t)j.n_bins, s));
+    CK(launch_count(fb, j.tiles_x, j.tiles_y, j.W, j.H, (int64_t)j.n_bins, s, false));
     job_mark(j, 6, s);
     CK(launch_capacity_check(fb, j.n_tiles, s));
     job_mark(j, 7, s);
@@ -1186,7 +1180,7 @@ struct NormalStream {
 // `post` of every frame on its stream again; `mid` and `post` may be empty.
 template <typename Pre, typename Mid, typename Post>
 hexfc_status batch_graph(hexfc_ctx* ctx, int phase, const std::vector<int>& items, Pre&& pre, Mid&& mid,
-                         Post&& post, bool has_mid)
+                         Post&& post, bool has_mid, bool has_post = true)
 {
     cudaStream_t o = ctx->origin;
     if (const cudaError_t e = cudaStreamBeginCapture(o, cudaStreamCaptureModeThreadLocal); e != cudaSuccess) {
@@ -1208,7 +1202,7 @@ hexfc_status batch_graph(hexfc_ctx* ctx, int phase, const std::vector<int>& item
     branches(pre);
     if (has_mid) {
         if (ok && st == HEXFC_OK) st = mid(o);
-        branches(post);
+        if (has_post) branches(post);
     }
     cudaGraph_t g = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(o, &g);
@@ -1495,9 +1489,10 @@ hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_ite
     const bool one = ctx->batch_launch;
     if (one && (st = batch_graph(
                     ctx, 1, live, [&](int i, cudaStream_t si) { return job_phase2_bins(jobs[(size_t)i], si); },
-                    count_all, [&](int i, cudaStream_t si) { return job_phase2_totals(jobs[(size_t)i], si); }, true)) !=
-                   HEXFC_OK)
+                    count_all, none, true, false)) != HEXFC_OK)
         return st;
+    if (one)
+        for (int i : live) jobs[(size_t)i].launches += 1;   // the count
     if (!one && (st = batch_graph(
                      ctx, 1, live, [&](int i, cudaStream_t si) { return job_phase2(jobs[(size_t)i], si); }, no_mid,
                      none, false)) != HEXFC_OK)

@@ -207,6 +207,7 @@ struct CountItem {
     uint32_t* masks;
     uint32_t* tile_frag;
     unsigned long long* scal;
+    uint64_t* h_scal;     // pinned host copy of scal[0..2] and [5], nullptr: not wanted
     uint64_t bin_limit;   // see FrameBufs
     int tiles_x, W, H, n_tiles;
 };
@@ -285,7 +286,8 @@ cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int 
                             cudaStream_t s);
 cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s);
 CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H);
-cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s);
+cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s,
+                         bool to_host = true);
 // The count and the drawing pass of several frames, each one launch.
 cudaError_t launch_count_batch(const CountBatch& b, cudaStream_t s);
 cudaError_t launch_draw_batch(const DrawBatch& b, bool sil, int window, cudaStream_t s);

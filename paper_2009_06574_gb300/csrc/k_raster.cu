@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__
                                                     const uint32_t* __restrict__ tile_big,
                                                     const uint32_t* __restrict__ tile_skip, int n,
                                                     uint64_t* __restrict__ tile_off, uint32_t* __restrict__ order,
-                                                    uint64_t* __restrict__ total)
+                                                    uint64_t* __restrict__ total, uint64_t* __restrict__ h_total)
 {
     constexpr int kPer = kScanTiles / 1024;
     __shared__ uint32_t s_hist[1024], s_warp[32], s_max[32], s_empty;
@@ -418,6 +418,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__
     if (threadIdx.x == 1023) {
         tile_off[n] = at * kChunk;
         *total = at * kChunk;
+        if (h_total) *h_total = at * kChunk;
     }
     __syncthreads();
     const uint32_t h = s_hist[threadIdx.x];
@@ -727,7 +728,8 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint64_t* __restrict_
 // tile_frag, and into copy tile % kStatCopies of the frame's statistics (after
 // the device scalars scal): [0] += fragments, [1] = longest list, [2] += lists
 // longer than kLongList. The last of the frame's tiles sums the copies into
-// scal[0..2].
+// scal[0..2] and writes them to the host itself, as the tile scan does with the
+// bin total: a copy on the stream would hold up the kernel after it (5-7 us).
 // The count of one tile (the body of k_count and k_count_batch), by the blocks
 // of a cluster: block `slice` of `slices` takes every slices-th run of
 // kConsumerWarps chunks, the first sums the pixels' counts.
@@ -799,6 +801,12 @@ __device__ __forceinline__ void count_tile(int tile, const CountItem& a, uint32_
         a.scal[0] = v0;
         a.scal[1] = v1;
         a.scal[2] = v2;
+        if (a.h_scal) {
+            a.h_scal[0] = v0;
+            a.h_scal[1] = v1;
+            a.h_scal[2] = v2;
+            a.h_scal[5] = __ldcg(&a.scal[5]);
+        }
     }
 }
 
@@ -857,7 +865,8 @@ cudaError_t launch_tile_scan(FrameBufs& fb, int64_t n_tiles, bool* ordered, cuda
     if (!*ordered)
         return scan_u32_to_u64(fb.tile_cnt, fb.tile_off, n_tiles, fb.part, fb.part_max, fb.scal + 8, 0xFFFFFFFFu, s,
                                (uint32_t)kChunk, fb.tile_big, fb.slots ? fb.tile_skip : nullptr);
-    k_tile_scan<<<1, 1024, 0, s>>>(fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, (int)n_tiles, fb.tile_off, fb.tile_order, fb.scal + 8);
+    k_tile_scan<<<1, 1024, 0, s>>>(fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, (int)n_tiles, fb.tile_off,
+                                 fb.tile_order, fb.scal + 8, fb.h_scal ? fb.h_scal + 8 : nullptr);
     return cudaGetLastError();
 }
 
@@ -899,10 +908,11 @@ cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s)
 CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H)
 {
     return CountItem{fb.tile_off, fb.tile_cur, fb.bins, fb.fframe, fb.tile_order, fb.cnt, fb.masks, fb.tile_frag,
-                     reinterpret_cast<unsigned long long*>(fb.scal), fb.bin_limit, tiles_x, W, H, tiles_x * tiles_y};
+                     reinterpret_cast<unsigned long long*>(fb.scal), fb.h_scal, fb.bin_limit, tiles_x, W, H, tiles_x * tiles_y};
 }
 
-cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s)
+cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s,
+                         bool to_host)
 {
     // Few tiles with long lists: several blocks a tile, up to four times what the
     // chip holds at once, so that the longest list does not decide alone, and a
@@ -925,7 +935,9 @@ cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, 
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_count, count_item(fb, tiles_x, tiles_y, W, H));
+    CountItem it = count_item(fb, tiles_x, tiles_y, W, H);
+    if (!to_host) it.h_scal = nullptr;
+    return cudaLaunchKernelEx(&cfg, k_count, it);
 }
 
 cudaError_t launch_count_batch(const CountBatch& b, cudaStream_t s)
