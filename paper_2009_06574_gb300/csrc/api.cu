@@ -750,7 +750,7 @@ hexfc_status job_silhouette(FrameJob& j, float* out, cudaStream_t s)
 {
     if (j.sil_alpha <= 0.f) return HEXFC_OK;
     CK(launch_silhouette(j.fb->zsil, j.tiles_x, j.cam.ox, j.cam.oy, j.frame_w, j.frame_h, j.sil_alpha,
-                         j.sil_threshold, j.fb->scal + 8, j.fb->bin_limit, out, j.win, s));
+                         j.sil_threshold, j.fb->scal + 8, j.fb->bin_limit, out, j.win, j.fb->chained, s));
     j.launches += 1;
     return HEXFC_OK;
 }
@@ -779,6 +779,7 @@ DrawItem draw_item(const FrameJob& j, uint64_t limit)
     it.err = scal + 5;
     it.limit = limit;
     it.bin_limit = fb.bin_limit;
+    it.chained = fb.chained;
     it.sp = j.sp;
     it.win = j.win;
     it.tiles_x = j.tiles_x;
@@ -875,6 +876,7 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
             for (auto& e : set) CK(cudaEventCreate(&e));
     ctx->ev_cur ^= 1;
     j.timing = ctx;
+    j.fb->chained = true;
     if (!ctx->ev_p1) CK(cudaEventCreateWithFlags(&ctx->ev_p1, cudaEventDisableTiming));
     j.p1_done = ctx->ev_p1;
     if ((st = job_phase1(j, s)) != HEXFC_OK) return st;
@@ -969,6 +971,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
             for (auto& e : set) CK(cudaEventCreate(&e));
     ctx->ev_cur ^= 1;
     j.timing = ctx;
+    j.fb->chained = true;
     if (!ctx->ev_p1) CK(cudaEventCreateWithFlags(&ctx->ev_p1, cudaEventDisableTiming));
     j.p1_done = ctx->ev_p1;
     if ((st = job_phase1(j, s)) != HEXFC_OK) return st;
@@ -2081,6 +2084,7 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     const int64_t nparts = scan_partials_needed(n_tiles) + 1;
     Arena a{scratch, 0, (size_t)HEXFC_NOALLOC_SCRATCH_BYTES};
     FrameBufs fb;
+    fb.chained = true;
     // the device scalars first, at the same place in every call: slot 5, the
     // device error word, outlives the call (see below)
     fb.scal = a.take<uint64_t>(kScalAll);
@@ -2186,7 +2190,7 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     CK(launch_draw_tail(it, s));
     if (sil)
         CK(launch_silhouette(fb.zsil, tiles_x, ctx->cam.ox, ctx->cam.oy, ctx->view.width, ctx->view.height,
-                             ctx->style.sil_alpha, ctx->style.sil_threshold, fb.scal + 8, fb.bin_limit, out, win, s));
+                             ctx->style.sil_alpha, ctx->style.sil_threshold, fb.scal + 8, fb.bin_limit, out, win, fb.chained, s));
     return inject_error_bits(ctx, fb.scal, s);
 }
 

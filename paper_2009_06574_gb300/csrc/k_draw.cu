@@ -318,6 +318,7 @@ __device__ __noinline__ CT block_list(const DrawItem& a, const PixelRef& r, uint
 // the 20 pixels of the 64^3 frame at 1920x1080).
 __global__ void __launch_bounds__(kTilePix, 3) k_draw_tail(const __grid_constant__ DrawItem a)
 {
+    chain_begin();
     extern __shared__ __align__(128) unsigned char smem[];
     if (!__syncthreads_and(frame_allowed(a))) return;
     bool bad = false;
@@ -525,6 +526,7 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, in
 template <int KW, bool kSil>
 __global__ void __launch_bounds__(kTilePix, 3) k_draw(const __grid_constant__ DrawItem a)
 {
+    chain_wait();
     extern __shared__ __align__(128) unsigned char smem[];
     draw_tile<KW, kSil>(*reinterpret_cast<DrawRing<KW>*>(smem), a, (int)a.order[blockIdx.x]);
 }
@@ -565,6 +567,7 @@ __global__ void __launch_bounds__(256) k_silhouette(const uint32_t* __restrict__
                                                     const uint64_t* __restrict__ n_bins, uint64_t bin_limit,
                                                     float4* __restrict__ out, OutWin win)
 {
+    chain_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)win.w * win.h || *n_bins > bin_limit) return;
     const int x = win.x0 + (int)(i % win.w), y = win.y0 + (int)(i / win.w);
@@ -678,8 +681,7 @@ cudaError_t prepare_draw_kernels()
 cudaError_t launch_draw(const DrawItem& a, int64_t n_tiles, int window, cudaStream_t s)
 {
     return for_variant<DrawKernel>(window, a.zsil != nullptr, [&](auto k) {
-        k.fn<<<(unsigned)n_tiles, kTilePix, k.smem, s>>>(a);
-        return cudaGetLastError();
+        return launch_chained(k.fn, (unsigned)n_tiles, kTilePix, k.smem, s, a.chained, a);
     });
 }
 
@@ -694,20 +696,17 @@ cudaError_t launch_draw_batch(const DrawBatch& b, bool sil, int window, cudaStre
 
 cudaError_t launch_draw_tail(const DrawItem& a, cudaStream_t s)
 {
-    k_draw_tail<<<kTailBlocks, kTilePix, sizeof(PixelList), s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(k_draw_tail, kTailBlocks, kTilePix, sizeof(PixelList), s, a.chained, a);
 }
 
 cudaError_t launch_silhouette(const uint32_t* zsil, int tiles_x, int fx0, int fy0, int frame_w, int frame_h,
                               float alpha, float threshold, const uint64_t* n_bins, uint64_t bin_limit, float* out,
-                              OutWin win, cudaStream_t s)
+                              OutWin win, bool chained, cudaStream_t s)
 {
     const int64_t n = (int64_t)win.w * win.h;
     if (n == 0) return cudaSuccess;
-    k_silhouette<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(zsil, tiles_x, fx0, fy0, frame_w, frame_h, alpha,
-                                                             (int64_t)threshold, n_bins, bin_limit,
-                                                             reinterpret_cast<float4*>(out), win);
-    return cudaGetLastError();
+    return launch_chained(k_silhouette, (unsigned)((n + 255) / 256), 256, 0, s, chained, zsil, tiles_x, fx0, fy0, frame_w,
+                          frame_h, alpha, (int64_t)threshold, n_bins, bin_limit, reinterpret_cast<float4*>(out), win);
 }
 
 cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const int32_t* d_py, int64_t n,

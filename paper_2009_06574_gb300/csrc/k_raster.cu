@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ 
                                                       uint32_t* __restrict__ tile_cur, int64_t n_tiles,
                                                       uint64_t* __restrict__ scal)
 {
+    chain_begin();
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t i = v; i < n_tiles; i += (int64_t)gridDim.x * blockDim.x) {
         tile_cnt[i] = 0;
@@ -213,6 +214,7 @@ __global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fve
                                                     uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_big,
                                                     uint32_t* __restrict__ tile_skip, int spread)
 {
+    chain_begin();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = g >> spread;
     const bool in = i < n_faces && i << spread == g;
     const int64_t f = !in ? 0 : reverse ? n_faces - 1 - i : i;
@@ -308,6 +310,7 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
                                                   uint32_t* __restrict__ bins, int spread,
                                                   const uint64_t* __restrict__ n_bins, uint64_t bin_limit)
 {
+    chain_begin();
     if (*n_bins > bin_limit) return;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, t = g >> spread;
     uint32_t range = 0;
@@ -356,6 +359,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__
                                                     uint64_t* __restrict__ tile_off, uint32_t* __restrict__ order,
                                                     uint64_t* __restrict__ total, uint64_t* __restrict__ h_total)
 {
+    chain_begin();
     constexpr int kPer = kScanTiles / 1024;
     __shared__ uint32_t s_hist[1024], s_warp[32], s_max[32], s_empty;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -465,6 +469,7 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
                                                  const uint64_t* __restrict__ n_bins, uint64_t bin_limit,
                                                  const CapFeatures cf)
 {
+    chain_begin();
     if (*n_bins > bin_limit) return;
     constexpr uint32_t kMax = kT * kItems, kLow = kMax / kChunk;
     extern __shared__ uint32_t sort_sm[];
@@ -812,6 +817,7 @@ __device__ __forceinline__ void count_tile(int tile, const CountItem& a, uint32_
 
 __global__ void __launch_bounds__(kTilePix, kCountBlocks) k_count(const __grid_constant__ CountItem a)
 {
+    chain_wait();
     const uint32_t slices = cooperative_groups::this_cluster().num_blocks();
     count_tile((int)a.order[blockIdx.x / slices], a, blockIdx.x % slices, slices);
 }
@@ -841,10 +847,9 @@ cudaError_t prepare_raster_kernels()
 cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, int64_t n_tiles, cudaStream_t s)
 {
     const unsigned tiles = std::min(grid_for(n_tiles, 256), 1216u);   // (two blocks' worth of clears an SM at most)
-    k_vertex_setup<<<std::max(grid_for(m.n_verts, 256), tiles), 256, 0, s>>>(m.verts, m.n_verts, cam, cam_pairs(cam),
-                                                                             fb.vproj, fb.ved, fb.tile_cnt, fb.tile_big,
-                                                                             fb.tile_skip, fb.tile_cur, n_tiles, fb.scal);
-    return cudaGetLastError();
+    return launch_chained(k_vertex_setup, std::max(grid_for(m.n_verts, 256), tiles), 256, 0, s, false, m.verts, m.n_verts,
+                          cam, cam_pairs(cam), fb.vproj, fb.ved, fb.tile_cnt, fb.tile_big, fb.tile_skip, fb.tile_cur,
+                          n_tiles, fb.scal);
 }
 
 cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const ShadeParams& sp, FrameBufs& fb,
@@ -852,11 +857,10 @@ cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const Shad
 {
     (void)tiles_y;
     const int spread = spread_for(m.n_faces);
-    k_face_setup<<<grid_for(m.n_faces << spread, 256), 256, 0, s>>>(m.fverts, m.fedges, m.fbound, m.fstat.get(), m.elevel,
-                                                           m.eattr, fb.vproj, fb.ved, m.n_faces, sp, cam.W, cam.H,
-                                                           tiles_x, reverse, fb.fframe, fb.tzsum, fb.trange, fb.slots, fb.fextra,
-                                                           fb.tile_cnt, fb.tile_big, fb.tile_skip, spread);
-    return cudaGetLastError();
+    return launch_chained(k_face_setup, grid_for(m.n_faces << spread, 256), 256, 0, s, fb.chained, m.fverts, m.fedges,
+                          m.fbound, m.fstat.get(), m.elevel, m.eattr, fb.vproj, fb.ved, m.n_faces, sp, cam.W, cam.H,
+                          tiles_x, reverse, fb.fframe, fb.tzsum, fb.trange, fb.slots, fb.fextra, fb.tile_cnt, fb.tile_big,
+                          fb.tile_skip, spread);
 }
 
 cudaError_t launch_tile_scan(FrameBufs& fb, int64_t n_tiles, bool* ordered, cudaStream_t s)
@@ -865,27 +869,26 @@ cudaError_t launch_tile_scan(FrameBufs& fb, int64_t n_tiles, bool* ordered, cuda
     if (!*ordered)
         return scan_u32_to_u64(fb.tile_cnt, fb.tile_off, n_tiles, fb.part, fb.part_max, fb.scal + 8, 0xFFFFFFFFu, s,
                                (uint32_t)kChunk, fb.tile_big, fb.slots ? fb.tile_skip : nullptr);
-    k_tile_scan<<<1, 1024, 0, s>>>(fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, (int)n_tiles, fb.tile_off,
-                                 fb.tile_order, fb.scal + 8, fb.h_scal ? fb.h_scal + 8 : nullptr);
-    return cudaGetLastError();
+    return launch_chained(k_tile_scan, 1, 1024, 0, s, fb.chained, fb.tile_cnt, fb.tile_big,
+                          fb.slots ? fb.tile_skip : nullptr, (int)n_tiles, fb.tile_off, fb.tile_order, fb.scal + 8,
+                          fb.h_scal ? fb.h_scal + 8 : nullptr);
 }
 
 cudaError_t launch_bin_fill(const DevMesh& m, FrameBufs& fb, int tiles_x, int W, int H, cudaStream_t s)
 {
     const int spread = spread_for(2 * m.n_faces);
-    k_bin_fill<<<grid_for((2 * m.n_faces) << spread, 256), 256, 0, s>>>(fb.fframe, fb.trange, fb.slots, 2 * m.n_faces, W, H,
-                                                             tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins, spread, fb.scal + 8,
-                                                             fb.bin_limit);
-    return cudaGetLastError();
+    return launch_chained(k_bin_fill, grid_for((2 * m.n_faces) << spread, 256), 256, 0, s, fb.chained, fb.fframe, fb.trange,
+                          fb.slots, 2 * m.n_faces, W, H, tiles_x, fb.tile_off, fb.tile_cnt, fb.tile_cur, fb.bins, spread,
+                          fb.scal + 8, fb.bin_limit);
 }
 
 cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int buckets, const CapFeatures& cf,
                             cudaStream_t s)
 {
     auto go = [&](auto kernel, int threads, int items) {
-        kernel<<<(unsigned)n_tiles, threads, sort_smem(threads, items, buckets), s>>>(
-            fb.tile_off, fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, fb.tile_cur, fb.bins, fb.tzsum, buckets, fb.bins_tmp, fb.zsuf, fb.scal + 8,
-            fb.bin_limit, cf);
+        return launch_chained(kernel, (unsigned)n_tiles, threads, sort_smem(threads, items, buckets), s, fb.chained,
+                              fb.tile_off, fb.tile_cnt, fb.tile_big, fb.slots ? fb.tile_skip : nullptr, fb.tile_cur,
+                              fb.bins, fb.tzsum, buckets, fb.bins_tmp, fb.zsuf, fb.scal + 8, fb.bin_limit, cf);
     };
     // Many tiles: several blocks an SM, to go on with others while one waits at its
     // barriers; 16 entries a thread where lists of more than 8 x 256 are common
@@ -893,10 +896,9 @@ cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int 
     // 1920x1080, 500 a tile: 8 entries 0.061 ms, 16 entries 0.076). Few tiles with
     // long lists (a large mesh drawn small): most of an SM for each (96^3 at
     // 320x180: 0.51 ms with 256 threads, 0.07 with 1024).
-    if (n_bins <= 768 * n_tiles) go(k_bin_sort<256, 8>, 256, 8);
-    else if (n_tiles > 1024) go(k_bin_sort<256, 16>, 256, 16);
-    else go(k_bin_sort<1024, 16>, 1024, 16);
-    return cudaGetLastError();
+    if (n_bins <= 768 * n_tiles) return go(k_bin_sort<256, 8>, 256, 8);
+    if (n_tiles > 1024) return go(k_bin_sort<256, 16>, 256, 16);
+    return go(k_bin_sort<1024, 16>, 1024, 16);
 }
 
 cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s)
@@ -929,12 +931,14 @@ cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, 
     cfg.blockDim = dim3(kTilePix);
     cfg.dynamicSmemBytes = kConsumerWarps * sizeof(CountWarp);
     cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = slices;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = slices;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = fb.chained ? 2 : 1;
     CountItem it = count_item(fb, tiles_x, tiles_y, W, H);
     if (!to_host) it.h_scal = nullptr;
     return cudaLaunchKernelEx(&cfg, k_count, it);
