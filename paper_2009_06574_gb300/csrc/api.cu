@@ -795,7 +795,7 @@ hexfc_status job_phase3(FrameJob& j, cudaStream_t s)
     uint64_t limit;
     if (job_limit(j, limit)) {
         const DrawItem it = draw_item(j, limit);
-        CK(launch_draw(it, j.n_tiles, j.window, s));
+        CK(launch_draw(it, j.n_tiles, j.n_bins, j.window, s));
         job_mark(j, 9, s);
         CK(launch_draw_tail(it, s));
         j.launches += 2;
@@ -1019,7 +1019,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     job_mark(j, 7, s);
     job_mark(j, 8, s);
     const DrawItem it = draw_item(j, ~0ull);
-    CK(launch_draw(it, j.n_tiles, j.window, s));
+    CK(launch_draw(it, j.n_tiles, j.n_bins, j.window, s));
     job_mark(j, 9, s);
     CK(launch_draw_tail(it, s));
     if ((st = job_silhouette(j, out, s)) != HEXFC_OK) return st;
@@ -2186,7 +2186,7 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     if (!a.take<uint64_t>((size_t)total) || !a.take<float4>((size_t)total)) return HEXFC_ERR_OVERFLOW;
     FrameJob j = make_job(ctx, &fb, m, out);
     const DrawItem it = draw_item(j, ~0ull);
-    CK(launch_draw(it, n_tiles, ctx->window, s));
+    CK(launch_draw(it, n_tiles, n_bins, ctx->window, s));
     CK(launch_draw_tail(it, s));
     if (sil)
         CK(launch_silhouette(fb.zsil, tiles_x, ctx->cam.ox, ctx->cam.oy, ctx->view.width, ctx->view.height,

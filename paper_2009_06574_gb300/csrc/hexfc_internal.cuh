@@ -329,7 +329,8 @@ cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, 
 cudaError_t launch_count_batch(const CountBatch& b, cudaStream_t s);
 cudaError_t launch_draw_batch(const DrawBatch& b, bool sil, int window, cudaStream_t s);
 // The drawing pass of a frame, and its second pass (pixels out of order).
-cudaError_t launch_draw(const DrawItem& a, int64_t n_tiles, int window, cudaStream_t s);
+// n_bins: the frame's bins, about (they pick the form of the pass)
+cudaError_t launch_draw(const DrawItem& a, int64_t n_tiles, uint64_t n_bins, int window, cudaStream_t s);
 cudaError_t launch_draw_tail(const DrawItem& a, cudaStream_t s);
 // Tile capacities from the previous frame's exact counts, or `uniform` (> 0) per tile.
 cudaError_t launch_capacity_from_previous(FrameBufs& fb, int64_t n_tiles, float margin, uint32_t pad,

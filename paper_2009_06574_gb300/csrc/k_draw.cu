@@ -33,8 +33,11 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarps = kTilePix / 32;          // a warp per group of 32 pixels
 constexpr uint32_t kService = 8;               // steps between two looks at the ring (a power of two)
-constexpr int kRing = kWarps;                  // chunks staged ahead: a slot for each warp to stage
-static_assert((kRing & (kRing - 1)) == 0, "slots by the low bits");
+// Chunks staged ahead, and warps that only stage (none: the eight that draw stage too, a slot each).
+__host__ __device__ constexpr int ring_of(bool wide) { return wide ? 16 : kWarps; }
+__host__ __device__ constexpr int stagers_of(bool wide) { return wide ? 8 : 0; }
+static_assert((ring_of(false) & (ring_of(false) - 1)) == 0 && (ring_of(true) & (ring_of(true) - 1)) == 0,
+              "slots by the low bits");
 constexpr uint32_t kGone = 0xffffffffu;        // progress of a warp that needs no more chunks
 constexpr unsigned long long kErrWait = 4ull;  // error bits
 constexpr unsigned long long kErrDepth = 1ull;
@@ -87,8 +90,9 @@ struct DrawSlot {
     uint32_t mask[kTilePix];
 };
 
-template <int KW>
+template <int KW, bool kWide>
 struct DrawRing {
+    static constexpr int kRing = ring_of(kWide);
     DrawSlot ring[kRing];
     ShadeRec none;                      // what a lane without a triangle reads
     float4 window[KW][kTilePix];
@@ -364,9 +368,10 @@ __device__ __forceinline__ uint32_t load_acquire(const uint32_t* p)
 // behind the last blended one (zsuf: the least depth from a chunk on) the
 // pixel is finished; a warp whose pixels are all finished only stages, and the
 // block ends when all have.
-template <int KW, bool kSil>
-__device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, int tile)
+template <int KW, bool kSil, bool kWide>
+__device__ __forceinline__ void draw_tile(DrawRing<KW, kWide>& S, const DrawItem& a, int tile)
 {
+    constexpr int kRing = ring_of(kWide), kStagers = stagers_of(kWide), kStep = kWide ? kStagers : kWarps;
     const bool allowed = frame_allowed(a);
     const int px0 = (tile % a.tiles_x) * kTileW, py0 = (tile / a.tiles_x) * kTileH;
     const uint64_t beg = a.tile_off[tile];   // a multiple of kChunk
@@ -378,10 +383,10 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, in
     mbar_init_fence();
     if (!__syncthreads_and(allowed)) return;   // (one answer for the block: another may set an error bit meanwhile)
     // staging: this warp's next chunk and its triangles
-    uint32_t mine = (uint32_t)warp;
+    uint32_t mine = (uint32_t)(kWide ? warp - kWarps : warp);   // (the wide form's consumers: not used)
     uint32_t f2t_m = mine < n_chunks ? a.bins[beg + (uint64_t)mine * kChunk + lane] : kPadBin;
     auto stage = [&]() {
-        DrawSlot& D = S.ring[warp];
+        DrawSlot& D = S.ring[kWide ? mine & (kRing - 1) : warp];
         // the masks: eight pixels of a row a lane
         const uint4* mp = reinterpret_cast<const uint4*>(a.masks + (beg / kChunk + mine) * kTilePix) + 2 * lane;
         const int mx = (8 * lane) % kTileW, my = (8 * lane) / kTileW;
@@ -392,13 +397,35 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, in
                         py0, a.sp, D.sh[lane]);
         md[0] = ma;
         md[1] = mb;
-        mbar_arrive(&S.full[warp]);
-        mine += kWarps;
+        mbar_arrive(&S.full[kWide ? mine & (kRing - 1) : warp]);
+        mine += kStep;
         f2t_m = mine < n_chunks ? a.bins[beg + (uint64_t)mine * kChunk + lane] : kPadBin;
     };
     // the least progress of the block's warps (kGone: all are finished)
     auto slowest = [&]() { return __reduce_min_sync(kFull, lane < kWarps ? load_acquire(&S.rel[lane]) : kGone); };
-    if (mine < n_chunks) stage();
+    // what is left to stage, as slots become free
+    auto stage_rest = [&]() {
+        long long t0 = clock64();
+        while (mine < n_chunks) {
+            const uint32_t r = slowest();
+            if (r == kGone) break;
+            if (mine < r + kRing) {
+                stage();
+                if (kWide) t0 = clock64();
+            } else {
+                if (__any_sync(kFull, clock64() - t0 > kWaitCycles)) {
+                    if (lane == 0) atomicOr(a.err, kErrWait);
+                    break;
+                }
+                __nanosleep(kWide ? 40 : 200);
+            }
+        }
+    };
+    if (kWide && warp >= kWarps) {
+        stage_rest();
+        return;
+    }
+    if (!kWide && mine < n_chunks) stage();
     // consumers
     const int p = draw_pixel(threadIdx.x), lx = p % kTileW, ly = p / kTileW;
     const int x = px0 + lx, y = py0 + ly;
@@ -445,7 +472,7 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, in
                 if (lane == 0) store_release(&S.rel[warp], rel);
             }
             __syncwarp();
-            if (mine < n_chunks && mine < min(slowest(), kGone - kRing) + kRing) stage();
+            if (!kWide && mine < n_chunks && mine < min(slowest(), kGone - kRing) + kRing) stage();
             bool got = false;
             while (hi < n_chunks && hi < rel + kRing &&
                    __all_sync(kFull, mbar_test(&S.full[hi & (kRing - 1)], (hi / kRing) & 1u))) {
@@ -507,20 +534,7 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW>& S, const DrawItem& a, in
     }
     // this warp's chunks are still to be staged for the others
     __syncwarp();
-    const long long t0 = clock64();
-    while (mine < n_chunks) {
-        const uint32_t r = slowest();
-        if (r == kGone) break;
-        if (mine < r + kRing) {
-            stage();
-        } else {
-            if (__any_sync(kFull, clock64() - t0 > kWaitCycles)) {
-                if (lane == 0) atomicOr(a.err, kErrWait);
-                break;
-            }
-            __nanosleep(200);
-        }
-    }
+    if (!kWide) stage_rest();
 }
 
 template <int KW, bool kSil>
@@ -528,7 +542,20 @@ __global__ void __launch_bounds__(kTilePix, 3) k_draw(const __grid_constant__ Dr
 {
     chain_wait();
     extern __shared__ __align__(128) unsigned char smem[];
-    draw_tile<KW, kSil>(*reinterpret_cast<DrawRing<KW>*>(smem), a, (int)a.order[blockIdx.x]);
+    draw_tile<KW, kSil, false>(*reinterpret_cast<DrawRing<KW, false>*>(smem), a, (int)a.order[blockIdx.x]);
+}
+
+// Few tiles with long lists (a large mesh drawn small): what a tile takes decides,
+// not what the chip can issue, and most triangles of a chunk are not a warp's
+// own. Eight warps draw, eight others stage, and 16 chunks ahead give the lanes
+// more to go on with (96^3 at 320x180, 240 tiles: 0.95 ms with the form above, with
+// 8 slots and 8 stagers 0.75, 16 and 16 0.67, 16 and 4 0.57, 16 and 8 0.53).
+template <int KW, bool kSil>
+__global__ void __launch_bounds__(kTilePix + 32 * stagers_of(true), 1) k_draw_wide(const __grid_constant__ DrawItem a)
+{
+    chain_wait();
+    extern __shared__ __align__(128) unsigned char smem[];
+    draw_tile<KW, kSil, true>(*reinterpret_cast<DrawRing<KW, true>*>(smem), a, (int)a.order[blockIdx.x]);
 }
 
 // The drawing pass of several frames in one grid (a batch).
@@ -540,7 +567,8 @@ __global__ void __launch_bounds__(kTilePix, 3) k_draw_batch(const __grid_constan
     const int i = batch_item(b.tile_begin, b.n, blockIdx.x);
     if (threadIdx.x == 0) s_it = b.it[i];
     __syncthreads();
-    draw_tile<KW, kSil>(*reinterpret_cast<DrawRing<KW>*>(smem), s_it, (int)s_it.order[blockIdx.x - b.tile_begin[i]]);
+    draw_tile<KW, kSil, false>(*reinterpret_cast<DrawRing<KW, false>*>(smem), s_it,
+                               (int)s_it.order[blockIdx.x - b.tile_begin[i]]);
 }
 
 // ---------------------------------------------------------------- silhouettes
@@ -651,12 +679,17 @@ cudaError_t for_variant(int window, bool sil, F&& f)
 template <int KW, bool kSil>
 struct DrawKernel {
     static constexpr auto fn = &k_draw<KW, kSil>;
-    static constexpr int smem = sizeof(DrawRing<KW>);
+    static constexpr int smem = sizeof(DrawRing<KW, false>);
+};
+template <int KW, bool kSil>
+struct DrawWideKernel {
+    static constexpr auto fn = &k_draw_wide<KW, kSil>;
+    static constexpr int smem = sizeof(DrawRing<KW, true>);
 };
 template <int KW, bool kSil>
 struct DrawBatchKernel {
     static constexpr auto fn = &k_draw_batch<KW, kSil>;
-    static constexpr int smem = sizeof(DrawRing<KW>);
+    static constexpr int smem = sizeof(DrawRing<KW, false>);
 };
 
 }  // namespace
@@ -670,6 +703,7 @@ cudaError_t prepare_draw_kernels()
             };
             cudaError_t e = for_variant<DrawKernel>(window, sil, set);
             if (e == cudaSuccess) e = for_variant<DrawBatchKernel>(window, sil, set);
+            if (e == cudaSuccess) e = for_variant<DrawWideKernel>(window, sil, set);
             if (e != cudaSuccess) return e;
         }
     const cudaError_t e = cudaFuncSetAttribute(k_draw_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -678,8 +712,21 @@ cudaError_t prepare_draw_kernels()
     return cudaFuncSetAttribute(k_debug_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PixelList));
 }
 
-cudaError_t launch_draw(const DrawItem& a, int64_t n_tiles, int window, cudaStream_t s)
+cudaError_t launch_draw(const DrawItem& a, int64_t n_tiles, uint64_t n_bins, int window, cudaStream_t s)
 {
+    // The wide form, one block an SM, for a frame that has the chip to itself, lists
+    // of some length, and no more tiles than the other form holds at once, or not
+    // many more and long lists (sides measured, wide / other, ms a frame: 96^3 at
+    // 240 tiles 0.71 / 0.94, 2040 tiles 0.67 / 0.71; 64^3 at 920 tiles 0.30 / 0.32,
+    // 2040 tiles equal; 16^3 at 240 tiles 0.076 / 0.080, 920 tiles 0.114 / 0.102; 4^3
+    // and 8^3 at 200 tiles, 26 and 78 entries a list: 2-3% slower). In a batch frames
+    // fill each other's gaps: 48 thumbnails 16.1 / 14.4 ms.
+    const uint64_t t = (uint64_t)n_tiles;
+    const bool few = n_bins >= 96 * t && (t <= 2 * 152 || (t < 10000 && t * t * t <= 3200 * n_bins));
+    if (a.chained && few)
+        return for_variant<DrawWideKernel>(window, a.zsil != nullptr, [&](auto k) {
+            return launch_chained(k.fn, (unsigned)n_tiles, kTilePix + 32 * stagers_of(true), k.smem, s, a.chained, a);
+        });
     return for_variant<DrawKernel>(window, a.zsil != nullptr, [&](auto k) {
         return launch_chained(k.fn, (unsigned)n_tiles, kTilePix, k.smem, s, a.chained, a);
     });
