@@ -498,7 +498,7 @@ FrameJob make_job(hexfc_ctx* ctx, FrameBufs* fb, DevMesh* m, float* out)
 // places of the binning and the faces' extras are not counted: a frame does
 // without them if need be.
 constexpr uint64_t kFragBytes = sizeof(uint64_t) + sizeof(float4);
-constexpr uint64_t kSlotBytes = 2 * (sizeof(uint32_t) + sizeof(uint4)) + sizeof(FaceExtra);   // a face's places, extras
+constexpr uint64_t kSlotBytes = 2 * (sizeof(uint2) + sizeof(uint4)) + sizeof(FaceExtra);   // a face's places, extras
 uint64_t frame_bytes(const FrameBufs& f, int64_t frags)
 {
     uint64_t b = 0;

@@ -69,7 +69,11 @@ __device__ __forceinline__ void count_chunks(CountWarp& me, int lane, const uint
     uint32_t f2t = first < n_chunks ? bins[beg + (uint64_t)first * kChunk + lane] : kPadBin;
     for (uint32_t c = first; c < n_chunks; c += step) {
         int4 a = make_int4(0, 0, 0, 0), b = a;
-        if (f2t != kPadBin) { a = fframe[f2t >> 1].X; b = fframe[f2t >> 1].Y; }
+        if (f2t != kPadBin) {
+            const Pair16 v = load32(&fframe[f2t >> 1].X);
+            a = as_int4(v.a);
+            b = as_int4(v.b);
+        }
         const uint32_t f2t_next =
             c + step < n_chunks ? bins[beg + (uint64_t)(c + step) * kChunk + lane] : kPadBin;
 #pragma unroll

@@ -143,8 +143,8 @@ struct FrameBufs {
     int64_t f_cap = 0;
     // binning of triangles that touch at most 2x2 tiles: each pair's place in its tile's list is found
     // with its count (nullptr: all places are found in a second pass)
-    uint32_t* trange = nullptr;     // [2F] the triangle's tiles (kRange...)
-    uint4* slots = nullptr;         // [2F] places in the lists of its 2x2 tiles
+    uint2* trange = nullptr;        // [2F] the triangle's tiles (kRange...), its place in the first one's list
+    uint4* slots = nullptr;         // [2F] places in the lists of its 2x2 tiles, if more than one
     FaceExtra* fextra = nullptr;    // [F]
     int64_t slot_cap = 0;           // faces of these three
     uint64_t slots_refused = 0;     // the budget that had no room for them

@@ -134,7 +134,7 @@ __device__ __forceinline__ bool outside_lens(const float (&o)[3][3], const float
 // touches a second column and row (kRangeSmall) and that it covers no sample
 // (kRangeSkip), or that there are more than 2x2 (kRangeBig: found again in the
 // second pass).
-constexpr uint32_t kRangeSmall = 1u << 24, kRangeBig = 1u << 25, kRangeSkip = 1u << 26;
+constexpr uint32_t kRangeMore = 3u << 22, kRangeSmall = 1u << 24, kRangeBig = 1u << 25, kRangeSkip = 1u << 26;
 __device__ __forceinline__ uint32_t pack_range(int tx0, int ty0, int tx1, int ty1)
 {
     return (uint32_t)tx0 | ((uint32_t)ty0 << 11) | ((uint32_t)(tx1 - tx0) << 22) | ((uint32_t)(ty1 - ty0) << 23) |
@@ -155,8 +155,10 @@ __device__ __forceinline__ uint4 count_places(uint32_t* ctr, uint32_t* ctr_skip,
     uint32_t base[4], place[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        peers[k] = __match_any_sync(0xffffffffu, tile[k] | apart);
         base[k] = 0;
+        peers[k] = 0xffffffffu;
+        if (!__any_sync(0xffffffffu, tile[k] >= 0)) continue;
+        peers[k] = __match_any_sync(0xffffffffu, tile[k] | apart);
         if (tile[k] >= 0 && lane == __ffs(peers[k]) - 1) base[k] = atomicAdd(c + tile[k], (uint32_t)__popc(peers[k]));
     }
 #pragma unroll
@@ -194,22 +196,26 @@ __device__ __forceinline__ bool covers(const TriGeom& t, int px, int py)
 }
 
 // Thread per face: its record of the frame, its triangles' depths, and the
-// counts of the tiles they touch. Bound by the latency of its gathers and
-// atomics (39% of the issue slots). A triangle of at most 2x2 tiles keeps the
-// places its counts gave it, so that the binning needs no second round of
-// atomics: that pass 64 -> 36 us at 64^3 and 1920x1080, of which the scattered
-// 4-byte writes into 8160 lists remain. Triangles of more tiles are counted by
-// their whole warp (a 4^3 grid at 256x256, one block: 25 + 31 us for both passes
-// with a loop per thread, 12 + 8 us now).
-__global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fverts, const int4* __restrict__ fedges,
+// counts of the tiles they touch. Bound by the latency of its gathers (41% of the
+// issue slots; five blocks an SM for that, the atomics issued before the rest did
+// not help). A triangle of at most 2x2 tiles keeps the places its counts gave it,
+// the first beside its range, so that the binning needs no second round of atomics:
+// that pass 64 -> 36 us at 64^3 and 1920x1080, of which the scattered 4-byte writes
+// into 8160 lists remain. A face of which nothing is drawn gets no record, records
+// are written a sector at a time, and the lens test reads the vertices, which the
+// caches hold, instead of the faces' 64-byte static records (96^3 at 320x180: 153
+// -> 131 us; 128^3 at 3840x2160: 400 -> 372 us; 64^3 at 1920x1080: 71 -> 70 us).
+// Triangles of more tiles are counted by their whole warp (a 4^3 grid at 256x256,
+// one block: 25 + 31 us for both passes with a loop per thread, 12 + 8 us with).
+__global__ void __launch_bounds__(256, 5) k_face_setup(const int4* __restrict__ fverts, const int4* __restrict__ fedges,
                                                     const uint8_t* __restrict__ fbound,
-                                                    const FaceStatic* __restrict__ fstat,
+                                                    const float* __restrict__ verts,
                                                     const uint8_t* __restrict__ elevel,
                                                     const float* __restrict__ eattr, const int4* __restrict__ vproj,
                                                     const float* __restrict__ ved, int64_t n_faces,
                                                     const __grid_constant__ ShadeParams sp, int W, int H, int tiles_x,
                                                     int reverse, FaceFrame* __restrict__ fframe,
-                                                    uint32_t* __restrict__ tzsum, uint32_t* __restrict__ trange,
+                                                    uint32_t* __restrict__ tzsum, uint2* __restrict__ trange,
                                                     uint4* __restrict__ slots, FaceExtra* __restrict__ fextra,
                                                     uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_big,
                                                     uint32_t* __restrict__ tile_skip, int spread)
@@ -248,7 +254,6 @@ __global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fve
         const bool drawn = vok && t.valid;
         int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
         if (drawn) {
-            flags |= kFaceDrawn << tri;
             if (t.vi[1] != 1 + tri) flags |= kFaceSwapped << tri;
             area[tri] = t.area < (1ll << 26) ? (uint32_t)t.area : 0u;
             tile_range(t, tx0, ty0, tx1, ty1);
@@ -260,6 +265,7 @@ __global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fve
         // (96^3 at 320x180: 4.2 -> 2.8 million, 2.01 -> 1.35 ms a frame), none at
         // 64^3 and 1920x1080; boxes of up to four samples would be 1% more.
         const bool skip = small && t.bx1 - t.bx0 + t.by1 - t.by0 <= 1 && !covers(t, t.bx0, t.by0) && !covers(t, t.bx1, t.by1);
+        if (drawn && !skip) flags |= kFaceDrawn << tri;
         if (small) range[tri] = pack_range(tx0, ty0, tx1, ty1) | (skip ? kRangeSkip : 0u);
         else if (drawn) range[tri] = kRangeBig;
         const int t0 = ty0 * tiles_x + tx0;
@@ -270,11 +276,11 @@ __global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fve
     }
     if (!in) return;
     if (sp.lens_mode == HEXFC_LENS_SPHERE && sp.bounded && (flags & (3u * kFaceDrawn))) {
-        const float4 px = fstat[f].px, py = fstat[f].py, pz = fstat[f].pz;
-        const float o[4][3] = {{px.x - sp.lens_c[0], py.x - sp.lens_c[1], pz.x - sp.lens_c[2]},
-                               {px.y - sp.lens_c[0], py.y - sp.lens_c[1], pz.y - sp.lens_c[2]},
-                               {px.z - sp.lens_c[0], py.z - sp.lens_c[1], pz.z - sp.lens_c[2]},
-                               {px.w - sp.lens_c[0], py.w - sp.lens_c[1], pz.w - sp.lens_c[2]}};
+        float o[4][3];   // (from the vertices, which neighbours share in the caches)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) o[k][d] = __ldg(verts + 3 * (int64_t)id[k] + d) - sp.lens_c[d];
 #pragma unroll
         for (int tri = 0; tri < 2; ++tri) {
             const float v[3][3] = {{o[0][0], o[0][1], o[0][2]},
@@ -284,26 +290,28 @@ __global__ void __launch_bounds__(256) k_face_setup(const int4* __restrict__ fve
             if (outside_lens(v, d, sp.ortho != 0, sp.lens_inv_r)) flags |= kFaceOut << tri;
         }
     }
-    FaceFrame& r = fframe[f];
-    r.X = make_int4(X[0], X[1], X[2], X[3]);
-    r.Y = make_int4(Y[0], Y[1], Y[2], Y[3]);
-    r.Z = make_uint4(Z[0] | (edges << 24), Z[1] | (flags << 24), Z[2], Z[3]);
-    r.q = sp.ortho ? make_float4(1.f, 1.f, 1.f, 1.f)
-                   : make_float4(__frcp_rn(E[0]), __frcp_rn(E[1]), __frcp_rn(E[2]), __frcp_rn(E[3]));
     reinterpret_cast<uint2*>(tzsum)[f] = make_uint2(pack_depths(Z[0], Z[1], Z[2]), pack_depths(Z[0], Z[2], Z[3]));
     if (slots) {
-        reinterpret_cast<uint2*>(trange)[f] = make_uint2(range[0], range[1]);
-        fextra[f].nl = edge_scales(r.X, r.Y);
-        fextra[f].area = make_uint4(area[0], area[1], __float_as_uint(__frcp_rn((float)area[0])),
-                                    __float_as_uint(__frcp_rn((float)area[1])));
-        if (range[0] & kRangeSmall) slots[2 * f] = place[0];
-        if (range[1] & kRangeSmall) slots[2 * f + 1] = place[1];
+        reinterpret_cast<uint4*>(trange)[f] = make_uint4(range[0], place[0].x, range[1], place[1].x);
+        if (range[0] & kRangeMore) slots[2 * f] = place[0];
+        if (range[1] & kRangeMore) slots[2 * f + 1] = place[1];
+        if (!(flags & (3u * kFaceDrawn))) return;   // in no list that is drawn
     }
+    const int4 fx = make_int4(X[0], X[1], X[2], X[3]), fy = make_int4(Y[0], Y[1], Y[2], Y[3]);
+    FaceFrame& r = fframe[f];
+    store32(&r.X, make_uint4(fx.x, fx.y, fx.z, fx.w), make_uint4(fy.x, fy.y, fy.z, fy.w));
+    store32(&r.Z, make_uint4(Z[0] | (edges << 24), Z[1] | (flags << 24), Z[2], Z[3]),
+            as_uint4(sp.ortho ? make_float4(1.f, 1.f, 1.f, 1.f)
+                              : make_float4(__frcp_rn(E[0]), __frcp_rn(E[1]), __frcp_rn(E[2]), __frcp_rn(E[3]))));
+    if (slots)
+        store32(&fextra[f], as_uint4(edge_scales(fx, fy)),
+                make_uint4(area[0], area[1], __float_as_uint(__frcp_rn((float)area[0])),
+                           __float_as_uint(__frcp_rn((float)area[1]))));
 }
 
 // Thread per triangle (2 face + triangle): into the lists of its tiles.
 __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ fframe,
-                                                  const uint32_t* __restrict__ trange, const uint4* __restrict__ slots,
+                                                  const uint2* __restrict__ trange, const uint4* __restrict__ slots,
                                                   int64_t n_tris, int W, int H, int tiles_x,
                                                   const uint64_t* __restrict__ tile_off,
                                                   const uint32_t* __restrict__ tile_cnt, uint32_t* __restrict__ tile_cur,
@@ -313,21 +321,30 @@ __global__ void __launch_bounds__(256) k_bin_fill(const FaceFrame* __restrict__ 
     chain_begin();
     if (*n_bins > bin_limit) return;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, t = g >> spread;
-    uint32_t range = 0;
-    if (t < n_tris && t << spread == g)
-        range = trange ? trange[t] : (face_tris(fframe[t >> 1].Z) >> (t & 1)) & 1u ? kRangeBig : 0u;
+    uint32_t range = 0, place = 0;
+    if (t < n_tris && t << spread == g) {
+        if (trange) {
+            const uint2 v = trange[t];
+            range = v.x;
+            place = v.y;
+        } else if ((face_tris(fframe[t >> 1].Z) >> (t & 1)) & 1u) {
+            range = kRangeBig;
+        }
+    }
     if (range & kRangeSmall) {
-        const uint4 p = slots[t];
         const int tile = (int)((range >> 11) & 2047u) * tiles_x + (int)(range & 2047u);
         const bool c2 = (range >> 22) & 1u, r2 = (range >> 23) & 1u;
         // set aside: from the end of the tile's list down
         const uint64_t* off = range & kRangeSkip ? tile_off + 1 : tile_off;
         const uint32_t down = range & kRangeSkip ? ~0u : 0u;   // (~place is -1 - place)
-        auto put = [&](int at, uint32_t place) { bins[(int64_t)off[at] + (int32_t)(place ^ down)] = (uint32_t)t; };
-        put(tile, p.x);
-        if (c2) put(tile + 1, p.y);
-        if (r2) put(tile + tiles_x, p.z);
-        if (c2 && r2) put(tile + tiles_x + 1, p.w);
+        auto put = [&](int at, uint32_t k) { bins[(int64_t)off[at] + (int32_t)(k ^ down)] = (uint32_t)t; };
+        put(tile, place);
+        if (c2 || r2) {
+            const uint4 p = slots[t];
+            if (c2) put(tile + 1, p.y);
+            if (r2) put(tile + tiles_x, p.z);
+            if (c2 && r2) put(tile + tiles_x + 1, p.w);
+        }
     }
     int tx0 = 0, ty0 = 0, tx1 = 0, ty1 = 0;
     if (range & kRangeBig) {
@@ -858,7 +875,7 @@ cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const Shad
     (void)tiles_y;
     const int spread = spread_for(m.n_faces);
     return launch_chained(k_face_setup, grid_for(m.n_faces << spread, 256), 256, 0, s, fb.chained, m.fverts, m.fedges,
-                          m.fbound, m.fstat.get(), m.elevel, m.eattr, fb.vproj, fb.ved, m.n_faces, sp, cam.W, cam.H,
+                          m.fbound, m.verts, m.elevel, m.eattr, fb.vproj, fb.ved, m.n_faces, sp, cam.W, cam.H,
                           tiles_x, reverse, fb.fframe, fb.tzsum, fb.trange, fb.slots, fb.fextra, fb.tile_cnt, fb.tile_big,
                           fb.tile_skip, spread);
 }

@@ -6,6 +6,36 @@
 
 namespace hexfc {
 
+// A whole sector at once (32-byte accesses; as two of 16 bytes, each of them
+// takes a sector of its own on the way to L2).
+struct Pair16 {
+    uint4 a, b;
+};
+__device__ __forceinline__ Pair16 load32(const void* p)   // (not written by the kernel)
+{
+    unsigned long long q0, q1, q2, q3;
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(q0), "=l"(q1), "=l"(q2), "=l"(q3) : "l"(p));
+    Pair16 v;
+    v.a = make_uint4((uint32_t)q0, (uint32_t)(q0 >> 32), (uint32_t)q1, (uint32_t)(q1 >> 32));
+    v.b = make_uint4((uint32_t)q2, (uint32_t)(q2 >> 32), (uint32_t)q3, (uint32_t)(q3 >> 32));
+    return v;
+}
+__device__ __forceinline__ void store32(void* p, const uint4& a, const uint4& b)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+                 "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+__device__ __forceinline__ int4 as_int4(const uint4& v) { return make_int4((int)v.x, (int)v.y, (int)v.z, (int)v.w); }
+__device__ __forceinline__ float4 as_float4(const uint4& v)
+{
+    return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+__device__ __forceinline__ uint4 as_uint4(const float4& v)
+{
+    return make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w));
+}
+
 // 2x the signed area of (a, b, p): (b - a) x (p - a), exact in int64.
 __device__ __forceinline__ int64_t edge_fn(int32_t xa, int32_t ya, int32_t xb, int32_t yb, int32_t px,
                                            int32_t py)
@@ -65,16 +95,11 @@ __device__ __forceinline__ void tri_setup(const int32_t FX[4], const int32_t FY[
     int32_t xmin = min(t.X[0], min(t.X[1], t.X[2])), xmax = max(t.X[0], max(t.X[1], t.X[2]));
     int32_t ymin = min(t.Y[0], min(t.Y[1], t.Y[2])), ymax = max(t.Y[0], max(t.Y[1], t.Y[2]));
     // pixel p has its centre at 256 p + 128
-    int64_t bx0 = -floor_div_i64(-((int64_t)xmin - 128), 256);
-    int64_t by0 = -floor_div_i64(-((int64_t)ymin - 128), 256);
-    int64_t bx1 = floor_div_i64((int64_t)xmax - 128, 256);
-    int64_t by1 = floor_div_i64((int64_t)ymax - 128, 256);
-    bx0 = max(bx0, (int64_t)0);
-    by0 = max(by0, (int64_t)0);
-    bx1 = min(bx1, (int64_t)W - 1);
-    by1 = min(by1, (int64_t)H - 1);
-    t.bx0 = (int32_t)bx0; t.by0 = (int32_t)by0; t.bx1 = (int32_t)bx1; t.by1 = (int32_t)by1;
-    t.valid = (t.area != 0) && bx0 <= bx1 && by0 <= by1;
+    t.bx0 = max((xmin + 127) >> 8, 0);
+    t.by0 = max((ymin + 127) >> 8, 0);
+    t.bx1 = min((xmax - 128) >> 8, W - 1);
+    t.by1 = min((ymax - 128) >> 8, H - 1);
+    t.valid = (t.area != 0) && t.bx0 <= t.bx1 && t.by0 <= t.by1;
 }
 
 // Exact floor(n / a) for a > 0 and |n / a| < 2^25, with |n| < 2^63:

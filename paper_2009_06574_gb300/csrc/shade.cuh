@@ -58,15 +58,18 @@ __device__ __forceinline__ float4 edge_scales(const int4& X, const int4& Y)
 __device__ __forceinline__ void make_record(const FaceFrame& F, const FaceStatic& S, const FaceExtra* E, uint32_t f2t,
                                             int px0, int py0, const ShadeParams& sp, ShadeRec& R)
 {
-    const int4 X = F.X, Y = F.Y;
-    const uint4 Z = F.Z;
-    const float4 fq = F.q, imp = S.imp;
+    const Pair16 fa = load32(&F.X), fb = load32(&F.Z);
+    const int4 X = as_int4(fa.a), Y = as_int4(fa.b);
+    const uint4 Z = fb.a;
+    const float4 fq = as_float4(fb.b), imp = S.imp;
+    Pair16 ex{};
+    if (E) ex = load32(E);
     const bool second = f2t & 1u;
     const uint32_t flags = face_flags(Z) >> (f2t & 1u);   // this triangle's bits in triangle 0's places
     // |coordinate| <= 2^22: exact in float
     R.nx = make_float4(-(float)X.x, -(float)X.y, -(float)X.z, -(float)X.w);
     R.ny = make_float4(-(float)Y.x, -(float)Y.y, -(float)Y.z, -(float)Y.w);
-    R.nl = E ? E->nl : edge_scales(X, Y);
+    R.nl = E ? as_float4(ex.a) : edge_scales(X, Y);
     // vertices 1 and 2: corners (1, 2) or (2, 3), swapped if the triangle winds the other way
     const bool sw = flags & kFaceSwapped;
     auto pick = [&](auto b, auto c, auto d, auto& v1, auto& v2) {
@@ -99,7 +102,7 @@ __device__ __forceinline__ void make_record(const FaceFrame& F, const FaceStatic
     const bool lens = !(flags & kFaceOut) && sp.lens_mode == HEXFC_LENS_SPHERE;
     uint32_t area, iw;
     if (E) {
-        const uint4 A = E->area;
+        const uint4 A = ex.b;
         area = second ? A.y : A.x;
         iw = second ? A.w : A.z;
     } else {
