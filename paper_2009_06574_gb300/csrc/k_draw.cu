@@ -93,8 +93,8 @@ struct DrawSlot {
 template <int KW, bool kWide>
 struct DrawRing {
     static constexpr int kRing = ring_of(kWide);
+    ShadeRec none;                      // what a lane without a triangle reads (kWide), or reads past slot 0
     DrawSlot ring[kRing];
-    ShadeRec none;                      // what a lane without a triangle reads
     float4 window[KW][kTilePix];
     uint64_t full[kRing];               // a slot is staged (the 32 lanes of the warp that staged it arrive)
     uint32_t rel[kWarps];               // chunks that a warp is past (kGone: it needs no more)
@@ -497,7 +497,10 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW, kWide>& S, const DrawItem
             }
         }
         const bool live = m != 0;   // (a lane without a triangle goes along)
-        const ShadeRec& R = live ? S.ring[ch & (kRing - 1)].sh[__ffs(m) - 1] : S.none;
+        // (a lane without a triangle: triangle -1 of its slot, whatever memory of the
+        // ring that is; its results go nowhere. Where there are many such lanes they
+        // read one record instead)
+        const ShadeRec& R = !kWide || live ? S.ring[ch & (kRing - 1)].sh[__ffs(m) - 1] : S.none;
         m &= m - 1;   // (0 stays 0)
         const uint4 zf = R.zf, ha = R.ha;
         const Sample q = sample_of(R, zf, ha, (uint32_t)lx << 8, (uint32_t)ly << 8, live, bad);
