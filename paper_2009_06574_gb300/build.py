@@ -30,7 +30,8 @@ def out_dir() -> str:
 def lib_file() -> str:
     return os.path.join(out_dir(), "libhexfc.so")
 
-SOURCES = ["api.cu", "k_quality.cu", "k_raster.cu", "k_draw.cu", "k_scan.cu", "k_capacity.cu", "mesh_host.cpp"]
+SOURCES = ["api.cu", "k_quality.cu", "k_raster.cu", "k_draw.cu", "k_scan.cu", "k_capacity.cu", "k_mesh.cu",
+           "mesh_host.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-ffp-contract=off,-O2",
          "-I", INCLUDE, "-I", CSRC]

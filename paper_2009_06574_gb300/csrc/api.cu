@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "hexfc_internal.cuh"
+#include "mesh_device.h"
 #include "mesh_host.h"
 
 using namespace hexfc;
@@ -1343,46 +1344,87 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
     if (n_cells <= 0) return HEXFC_ERR_MESH;
     if (n_verts >= (1ll << 31) || n_cells >= (1ll << 27)) return HEXFC_ERR_ARG;
     DeviceGuard g(ctx->device);
-    HostTables t;
-    if (build_host_tables(verts, n_verts, cells, n_cells, cell_edge_level, t) != 0) return HEXFC_ERR_MESH;
-    if (2 * t.n_faces >= (1ll << 32)) return HEXFC_ERR_ARG;
+    if (!valid_mesh(verts, n_verts, cells, n_cells)) return HEXFC_ERR_MESH;
     DevMesh* m = new (std::nothrow) DevMesh();
     if (!m) return HEXFC_ERR_OOM;
     m->n_verts = n_verts;
     m->n_cells = n_cells;
-    m->n_faces = t.n_faces;
-    m->n_edges = t.n_edges;
     hexfc_status st = HEXFC_OK;
+    cudaError_t e = cudaSuccess;
     auto A = [&](hexfc_status s2) { if (st == HEXFC_OK) st = s2; };
+    auto H2D = [&](void* d, const void* h, size_t bytes) {
+        if (e == cudaSuccess) e = cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice);
+    };
     A(dalloc(&m->verts, 3 * (size_t)n_verts));
     A(dalloc(&m->cells, 8 * (size_t)n_cells));
     A(dalloc(&m->cell_edges, 12 * (size_t)n_cells));
-    A(dalloc(&m->cell_imp, (size_t)n_cells));
-    A(dalloc(&m->vkey, (size_t)n_verts));
-    A(dalloc(&m->ekey, (size_t)t.n_edges));
-    A(dalloc(&m->vimp, (size_t)n_verts));
-    A(dalloc(&m->eattr, (size_t)t.n_edges));
-    A(dalloc(&m->elevel, (size_t)t.n_edges));
-    A(dalloc(&m->fverts, (size_t)t.n_faces));
-    A(dalloc(&m->fedges, (size_t)t.n_faces));
-    bool fresh = false;
-    A(own_fstat(*m, &fresh));
-    A(dalloc(&m->fbound, (size_t)t.n_faces));
+    if (st == HEXFC_OK) {
+        H2D(m->verts, verts, sizeof(float) * 3 * (size_t)n_verts);
+        H2D(m->cells, cells, sizeof(int32_t) * 8 * (size_t)n_cells);
+    }
+    // Faces and edges: on the device, or on the host if that has no memory for it or
+    // the mesh is not for it.
+    MeshScratch tables;
+    HostTables t;
+    uint64_t n_faces = 0, n_edges = 0;
+    bool host = false;
+    if (st == HEXFC_OK && e == cudaSuccess) {
+        e = tables.number(m->cells, n_cells, n_verts, &n_faces, &n_edges, &host);
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            e = cudaSuccess;
+            host = true;
+        }
+    }
+    auto on_host = [&]() -> hexfc_status {
+        try {
+            if (build_host_tables(cells, n_cells, cell_edge_level, t) != 0) return HEXFC_ERR_MESH;
+        } catch (...) {
+            return HEXFC_ERR_OOM;
+        }
+        n_faces = (uint64_t)t.n_faces;
+        n_edges = (uint64_t)t.n_edges;
+        return HEXFC_OK;
+    };
+    if (host) A(on_host());
+    if (st == HEXFC_OK && 2 * n_faces >= (1ull << 32)) st = HEXFC_ERR_ARG;
+    if (st == HEXFC_OK && e == cudaSuccess) {
+        m->n_faces = (int64_t)n_faces;
+        m->n_edges = (int64_t)n_edges;
+        bool fresh = false;
+        A(dalloc(&m->cell_imp, (size_t)n_cells));
+        A(dalloc(&m->vkey, (size_t)n_verts));
+        A(dalloc(&m->ekey, (size_t)n_edges));
+        A(dalloc(&m->vimp, (size_t)n_verts));
+        A(dalloc(&m->eattr, (size_t)n_edges));
+        A(dalloc(&m->elevel, (size_t)n_edges));
+        A(dalloc(&m->fverts, (size_t)n_faces));
+        A(dalloc(&m->fedges, (size_t)n_faces));
+        A(own_fstat(*m, &fresh));
+        A(dalloc(&m->fbound, (size_t)n_faces));
+    }
+    if (st == HEXFC_OK && e == cudaSuccess && !host) {
+        uint8_t* level = nullptr;
+        if (cell_edge_level) {
+            A(dalloc(&level, 12 * (size_t)n_cells));
+            if (st == HEXFC_OK) H2D(level, cell_edge_level, 12 * (size_t)n_cells);
+        }
+        if (st == HEXFC_OK && e == cudaSuccess)
+            e = tables.write(m->cells, n_cells, level, m->cell_edges, m->elevel, m->fverts, m->fedges, m->fbound, &host);
+        dfree(level);
+        if (host) A(on_host());   // (as many of both)
+    }
     if (st != HEXFC_OK) {
         free_mesh(m);
         return st;
     }
-    cudaError_t e = cudaSuccess;
-    auto H2D = [&](void* d, const void* h, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice);
-    };
-    H2D(m->verts, verts, sizeof(float) * 3 * (size_t)n_verts);
-    H2D(m->cells, cells, sizeof(int32_t) * 8 * (size_t)n_cells);
-    H2D(m->cell_edges, t.cell_edges.data(), sizeof(int32_t) * t.cell_edges.size());
-    H2D(m->elevel, t.elevel.data(), t.elevel.size());
-    H2D(m->fverts, t.fverts.data(), sizeof(int32_t) * t.fverts.size());
-    H2D(m->fedges, t.fedges.data(), sizeof(int32_t) * t.fedges.size());
-    H2D(m->fbound, t.fbound.data(), t.fbound.size());
+    if (host) {
+        H2D(m->cell_edges, t.cell_edges.data(), sizeof(int32_t) * t.cell_edges.size());
+        H2D(m->elevel, t.elevel.data(), t.elevel.size());
+        H2D(m->fverts, t.fverts.data(), sizeof(int32_t) * t.fverts.size());
+        H2D(m->fedges, t.fedges.data(), sizeof(int32_t) * t.fedges.size());
+        H2D(m->fbound, t.fbound.data(), t.fbound.size());
+    }
     if (cell_scalar) H2D(m->cell_imp, cell_scalar, sizeof(float) * (size_t)n_cells);
     if (e == cudaSuccess && !cell_scalar) e = launch_cell_quality(*m, HEXFC_METRIC_IMPORTANCE, m->cell_imp, 0);
     if (e == cudaSuccess) e = launch_importance(*m, true, 0);

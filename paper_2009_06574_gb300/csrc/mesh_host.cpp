@@ -1,4 +1,5 @@
-// Unique faces and edges of a hexahedral mesh (host precomputation).
+// Unique faces and edges of a hexahedral mesh (host precomputation; k_mesh.cu finds
+// the same tables on the device).
 //
 // Every geometric face is drawn once as a quad of two triangles (Section
 // "Method Overview"; Section "GPU Implementation"). A face is identified by
@@ -34,14 +35,17 @@ inline uint64_t pack(int32_t a, int32_t b) { return ((uint64_t)(uint32_t)a << 32
 
 }  // namespace
 
-int build_host_tables(const float* verts, int64_t n_verts, const int32_t* cells, int64_t n_cells,
-                      const uint8_t* cell_edge_level, HostTables& out)
+bool valid_mesh(const float* verts, int64_t n_verts, const int32_t* cells, int64_t n_cells)
 {
     for (int64_t i = 0; i < 3 * n_verts; ++i)
-        if (!std::isfinite(verts[i])) return -1;
+        if (!std::isfinite(verts[i])) return false;
     for (int64_t i = 0; i < 8 * n_cells; ++i)
-        if (cells[i] < 0 || cells[i] >= n_verts) return -1;
+        if (cells[i] < 0 || cells[i] >= n_verts) return false;
+    return true;
+}
 
+int build_host_tables(const int32_t* cells, int64_t n_cells, const uint8_t* cell_edge_level, HostTables& out)
+{
     // ---- faces
     std::vector<FaceRec> fr((size_t)(6 * n_cells));
     for (int64_t c = 0; c < n_cells; ++c) {

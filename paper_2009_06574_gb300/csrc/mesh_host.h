@@ -15,8 +15,10 @@ struct HostTables {
     int64_t n_faces = 0, n_edges = 0;
 };
 
-// Returns 0 on success, -1 on an invalid mesh (index out of range, non-finite vertex).
-int build_host_tables(const float* verts, int64_t n_verts, const int32_t* cells, int64_t n_cells,
-                      const uint8_t* cell_edge_level, HostTables& out);
+// Finite vertices, and cells of vertices that there are?
+bool valid_mesh(const float* verts, int64_t n_verts, const int32_t* cells, int64_t n_cells);
+
+// Of a valid mesh. Returns 0 on success, -1 on cells whose faces have other edges than theirs.
+int build_host_tables(const int32_t* cells, int64_t n_cells, const uint8_t* cell_edge_level, HostTables& out);
 
 }  // namespace hexfc
