@@ -1647,7 +1647,7 @@ hexfc_status hexfc_capacity_grad(hexfc_ctx* ctx, const float* x, const uint32_t*
     if ((st = cap_inputs(c, n)) != HEXFC_OK) return st;
     CK(cudaMemcpy(c.x, x, sizeof(float) * 4 * (size_t)n, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c.t, counts, sizeof(uint32_t) * (size_t)n, cudaMemcpyHostToDevice));
-    CK(launch_cap_grad(c, c.x, c.t, n, 0.f, 0));
+    CK(launch_cap_grad(c, c.x, c.t, n, 0.f, false, 0));
     CK(cudaMemcpy(grad, c.grad, sizeof(float) * kCapParams, cudaMemcpyDeviceToHost));
     if (loss) CK(cudaMemcpy(loss, c.grad + kCapParams, sizeof(float), cudaMemcpyDeviceToHost));
     return HEXFC_OK;
@@ -1661,9 +1661,13 @@ hexfc_status hexfc_capacity_train(hexfc_ctx* ctx, int32_t steps, float lr, float
     CapNet& c = ctx->cap;
     const cudaStream_t s = (cudaStream_t)stream;
     const int64_t n = ctx->feat_tiles;
-    for (int32_t k = 0; k < steps; ++k) CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, lr, s));
+    cudaStreamCaptureStatus captured = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(s, &captured));
+    const bool chain = captured == cudaStreamCaptureStatusNone;
+    for (int32_t k = 0; k < steps; ++k)
+        CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, lr, chain && k > 0, s));
     if (loss) {
-        if (steps == 0) CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, 0.f, s));
+        if (steps == 0) CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, 0.f, false, s));
         CK(cudaMemcpyAsync(loss, c.grad + kCapParams, sizeof(float), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
     }

@@ -342,7 +342,9 @@ cudaError_t launch_cap_forward(const CapNet& net, FrameBufs& fb, int64_t n_tiles
 cudaError_t prepare_capacity_kernels();
 int64_t cap_partials();   // floats of CapNet::part
 // Loss and gradient into net.grad, and (lr > 0) an Adam step.
-cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, float lr, cudaStream_t s);
+// chained: after another step on the same stream
+cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, float lr, bool chained,
+                            cudaStream_t s);
 cudaError_t launch_cap_to_half(CapNet& net, cudaStream_t s);
 // White silhouettes over the output (Section "Blending Focus and Context"):
 // from the boundary surface's depths zsil of the drawn rectangle, which sits

@@ -39,21 +39,27 @@ inline unsigned grid_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b);
 // products (layer 2, its gradient, the error back through it) are register tiles
 // over operands in shared memory, the gradient's sums stay in registers over the
 // block's groups, and what leaves the block is its share of the gradient, summed
-// in a fixed order (so a training step gives the same bits every time). 8 Adam
-// steps at 1920x1080: 0.90 -> XX ms.
+// in a fixed order (so a training step gives the same bits every time). Then the
+// weights' loads were a third of a step and the transposed stores went into one
+// bank: all loads at once, rows apart. Backward 75 + 32 us -> 15 + 4.4; 8 Adam steps
+// at 1920x1080, weights set and read: 0.93 -> 0.30 -> 0.19 ms. Bound by shared-memory
+// reads (9 of the 15 us) and the phases' barriers.
 constexpr int kGroup = 32;
 constexpr int kCapThreads = 256;
 constexpr int kCapBlocks = 304;   // two blocks an SM at most; more tiles than kGroup * 304: several groups each
 
+constexpr int kPartStride = (kCapParams + 1 + 3) / 4 * 4;   // a block's share: the gradient, the loss
+static_assert(oW2 % 4 == 0, "16-byte stores");
+
 struct NetSmem {
     float w1[kHid * kIn], b1[kHid], b2[kHid], w3[kHid];
-    float w2[kHid][kHid];       // [j][i]
-    float w2t[kHid][kHid];      // [i][j]
+    float w2[kHid][kHid + 16];  // [j][i] (rows apart for the stores of net_load)
+    float w2t[kHid][kHid + 4];  // [i][j]
     float x[kGroup][kIn];
     float h1[kGroup][kHid];     // [t][i]
-    float h1t[kHid][kGroup];    // [i][t]
+    float h1t[kHid][kGroup + 2];   // [i][t] (written along i: without the 2, all into one bank)
     float da[kGroup][kHid];     // [t][j]: errors of layer 2, then [t][i]: of layer 1
-    float dat[kHid][kGroup];    // [j][t]
+    float dat[kHid][kGroup + 2];   // [j][t]
     float red[2][16][kHid];     // sums over the groups of tiles at the end
     float dy[16][2];
     float b3;
@@ -65,20 +71,34 @@ static_assert(offsetof(NetSmem, b2) % 16 == 0 && offsetof(NetSmem, w3) % 16 == 0
                   offsetof(NetSmem, dat) % 8 == 0,
               "alignment of the vector reads");
 
+// The weights into shared memory: all of a thread's loads in flight at once (one
+// after another they were a third of a training step).
 __device__ __forceinline__ void net_load(NetSmem& S, const __half* __restrict__ w16)
 {
-    for (int p = threadIdx.x; p < kCapParams; p += kCapThreads) {
-        const float v = __half2float(w16[p]);
-        if (p < oB1) S.w1[p] = v;
-        else if (p < oW2) S.b1[p - oB1] = v;
-        else if (p < oB2) {
-            const int j = (p - oW2) / kHid, i = (p - oW2) % kHid;
-            S.w2[j][i] = v;
-            S.w2t[i][j] = v;
-        }
-        else if (p < oW3) S.b2[p - oB2] = v;
-        else if (p < oB3) S.w3[p - oW3] = v;
-        else S.b3 = v;
+    static_assert(kCapThreads == 4 * kHid && kHid == 64 && oW2 % 8 == 0, "a quarter of a row of W2 each");
+    const int tid = threadIdx.x, j = tid >> 2, c = (tid & 3) * 4;
+    uint2 r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r[k] = *reinterpret_cast<const uint2*>(w16 + oW2 + j * kHid + 16 * k + c);
+    const __half w1 = w16[oW1 + tid];
+    const int at = tid < kHid ? oB1 + tid : tid < 2 * kHid ? oB2 + tid - kHid : tid < 3 * kHid ? oW3 + tid - 2 * kHid : oB3;
+    const __half rest = w16[at];
+    S.w1[tid] = __half2float(w1);
+    const float v = __half2float(rest);
+    if (tid < kHid) S.b1[tid] = v;
+    else if (tid < 2 * kHid) S.b2[tid - kHid] = v;
+    else if (tid < 3 * kHid) S.w3[tid - 2 * kHid] = v;
+    else if (tid == 3 * kHid) S.b3 = v;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&r[k].x)),
+                     hi = __half22float2(*reinterpret_cast<const __half2*>(&r[k].y));
+        const int i = 16 * k + c;
+        *reinterpret_cast<float4*>(&S.w2[j][i]) = make_float4(lo.x, lo.y, hi.x, hi.y);
+        S.w2t[i][j] = lo.x;
+        S.w2t[i + 1][j] = lo.y;
+        S.w2t[i + 2][j] = hi.x;
+        S.w2t[i + 3][j] = hi.y;
     }
 }
 
@@ -154,7 +174,7 @@ __global__ void __launch_bounds__(kCapThreads) k_cap_forward(const float* __rest
 }
 
 // Loss (mean over the n tiles of (y - log1p(count))^2) and gradient: block b's
-// shares into part[b][kCapParams + 1].
+// shares into part[b][kPartStride].
 __global__ void __launch_bounds__(kCapThreads) k_cap_backward(const float* __restrict__ X,
                                                               const uint32_t* __restrict__ counts, int64_t n,
                                                               const __half* __restrict__ w16,
@@ -162,6 +182,7 @@ __global__ void __launch_bounds__(kCapThreads) k_cap_backward(const float* __res
 {
     extern __shared__ __align__(16) unsigned char net_smem[];
     NetSmem& S = *reinterpret_cast<NetSmem*>(net_smem);
+    chain_begin();
     net_load(S, w16);
     const int tid = threadIdx.x, q = tid & 15, g = tid >> 4;
     float gw2[4][4] = {}, gw3[4] = {}, gb2[4] = {}, gw1 = 0.f, gb1 = 0.f, gb3 = 0.f, loss = 0.f;
@@ -230,11 +251,10 @@ __global__ void __launch_bounds__(kCapThreads) k_cap_backward(const float* __res
             gb1 += d;
         }
     }
-    float* P = part + (int64_t)blockIdx.x * (kCapParams + 1);
+    float* P = part + (int64_t)blockIdx.x * kPartStride;
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) P[oW2 + (4 * g + u) * kHid + 4 * q + v] = gw2[u][v];
+        *reinterpret_cast<float4*>(P + oW2 + (4 * g + u) * kHid + 4 * q) = make_float4(gw2[u][0], gw2[u][1], gw2[u][2], gw2[u][3]);
     P[oW1 + tid] = gw1;
     if ((tid & 3) == 0) P[oB1 + (tid >> 2)] = gb1;
     __syncthreads();
@@ -261,33 +281,45 @@ __global__ void __launch_bounds__(kCapThreads) k_cap_backward(const float* __res
     }
 }
 
-// The blocks' shares summed, 8 threads a parameter; with `adam`, an Adam step on
-// the master copy and its FP16 copy.
-__global__ void __launch_bounds__(256) k_cap_sum(const float* __restrict__ part, int blocks, float* __restrict__ grad,
-                                                 bool adam, float* __restrict__ w, __half* __restrict__ w16,
-                                                 float* __restrict__ m, float* __restrict__ v, float lr, float b1,
-                                                 float b2, float eps, float c1, float c2)
+// The blocks' shares summed, 16 threads a parameter; with `adam`, an Adam step on
+// the master copy and its FP16 copy. Bound by the latency of its loads, so all
+// that can be are in flight together.
+constexpr int kSumWarps = 16;
+__global__ void __launch_bounds__(32 * kSumWarps) k_cap_sum(const float* __restrict__ part, int blocks, float* __restrict__ grad,
+                                                            bool adam, float* __restrict__ w, __half* __restrict__ w16,
+                                                            float* __restrict__ m, float* __restrict__ v, float lr, float b1,
+                                                            float b2, float eps, float c1, float c2)
 {
-    __shared__ float s[8][32];
+    __shared__ float s[kSumWarps][32];
     const int lane = threadIdx.x & 31, k = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
+    const bool step = adam && k == 0 && p < kCapParams;
+    const float m0 = step ? m[p] : 0.f, v0 = step ? v[p] : 0.f, w0 = step ? w[p] : 0.f;   // (the last step's: complete)
+    chain_begin();
     float sum = 0.f;
     if (p <= kCapParams) {
-#pragma unroll 8
-        for (int b = k; b < blocks; b += 8) sum += part[(int64_t)b * (kCapParams + 1) + p];
+        constexpr int kMost = (kCapBlocks + kSumWarps - 1) / kSumWarps;
+        float x[kMost];
+#pragma unroll
+        for (int i = 0; i < kMost; ++i) {
+            const int b = k + i * kSumWarps;
+            x[i] = b < blocks ? part[(int64_t)b * kPartStride + p] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < kMost; ++i) sum += x[i];
     }
     s[k][lane] = sum;
     __syncthreads();
     if (k != 0 || p > kCapParams) return;
     float g = 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) g += s[i][lane];
+    for (int i = 0; i < kSumWarps; ++i) g += s[i][lane];
     grad[p] = g;
-    if (!adam || p == kCapParams) return;
-    const float mm = fmaf(b1, m[p], (1.f - b1) * g);
-    const float vv = fmaf(b2, v[p], (1.f - b2) * g * g);
+    if (!step) return;
+    const float mm = fmaf(b1, m0, (1.f - b1) * g);
+    const float vv = fmaf(b2, v0, (1.f - b2) * g * g);
     m[p] = mm;
     v[p] = vv;
-    const float wn = w[p] - lr * (mm * c1) / (sqrtf(vv * c2) + eps);
+    const float wn = w0 - lr * (mm * c1) / (sqrtf(vv * c2) + eps);
     w[p] = wn;
     w16[p] = __float2half_rn(wn);
 }
@@ -351,7 +383,7 @@ cudaError_t prepare_capacity_kernels()
     return cudaFuncSetAttribute(k_cap_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(NetSmem));
 }
 
-int64_t cap_partials() { return (int64_t)kCapBlocks * (kCapParams + 1); }
+int64_t cap_partials() { return (int64_t)kCapBlocks * kPartStride; }
 
 static unsigned cap_grid(int64_t n) { return (unsigned)std::min<int64_t>((n + kGroup - 1) / kGroup, kCapBlocks); }
 
@@ -363,17 +395,19 @@ cudaError_t launch_cap_forward(const CapNet& net, FrameBufs& fb, int64_t n_tiles
     return cudaGetLastError();
 }
 
-cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, float lr, cudaStream_t s)
+cudaError_t launch_cap_grad(CapNet& net, const float* X, const uint32_t* counts, int64_t n, float lr, bool chained,
+                            cudaStream_t s)
 {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const bool adam = lr > 0.f;
     if (adam) net.step += 1;
     const float c1 = 1.f / (1.f - std::pow(b1, (float)net.step)), c2 = 1.f / (1.f - std::pow(b2, (float)net.step));
     const unsigned blocks = cap_grid(n);
-    k_cap_backward<<<blocks, kCapThreads, sizeof(NetSmem), s>>>(X, counts, n, net.w16, net.part);
-    k_cap_sum<<<grid_for(kCapParams + 1, 32), 256, 0, s>>>(net.part, (int)blocks, net.grad, adam, net.w, net.w16, net.m,
-                                                           net.v, lr, b1, b2, eps, c1, c2);
-    return cudaGetLastError();
+    cudaError_t e = launch_chained(k_cap_backward, blocks, kCapThreads, sizeof(NetSmem), s, chained, X, counts, n, net.w16,
+                                   net.part);
+    if (e != cudaSuccess) return e;
+    return launch_chained(k_cap_sum, grid_for(kCapParams + 1, 32), 32 * kSumWarps, 0, s, chained, net.part, (int)blocks,
+                          net.grad, adam, net.w, net.w16, net.m, net.v, lr, b1, b2, eps, c1, c2);
 }
 
 cudaError_t launch_cap_to_half(CapNet& net, cudaStream_t s)
