@@ -181,7 +181,7 @@ void free_mesh(DevMesh* m)
 {
     if (!m) return;
     dfree(m->verts); dfree(m->cells); dfree(m->cell_edges); dfree(m->cell_imp);
-    dfree(m->vkey); dfree(m->ekey); dfree(m->vimp); dfree(m->eattr); dfree(m->elevel);
+    dfree(m->vkey); dfree(m->ekey); dfree(m->eattr); dfree(m->elevel);
     dfree(m->fverts); dfree(m->fedges); dfree(m->fbound);
     delete m;
 }
@@ -1395,7 +1395,6 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
         A(dalloc(&m->cell_imp, (size_t)n_cells));
         A(dalloc(&m->vkey, (size_t)n_verts));
         A(dalloc(&m->ekey, (size_t)n_edges));
-        A(dalloc(&m->vimp, (size_t)n_verts));
         A(dalloc(&m->eattr, (size_t)n_edges));
         A(dalloc(&m->elevel, (size_t)n_edges));
         A(dalloc(&m->fverts, (size_t)n_faces));
@@ -1427,7 +1426,7 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
     }
     if (cell_scalar) H2D(m->cell_imp, cell_scalar, sizeof(float) * (size_t)n_cells);
     if (e == cudaSuccess && !cell_scalar) e = launch_cell_quality(*m, HEXFC_METRIC_IMPORTANCE, m->cell_imp, 0);
-    if (e == cudaSuccess) e = launch_importance(*m, true, 0);
+    if (e == cudaSuccess) e = launch_importance(*m, true, true, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         note_cuda(e);
@@ -1754,7 +1753,7 @@ hexfc_status hexfc_set_cell_importance(hexfc_ctx* ctx, int32_t mesh, const float
     if (cap == cudaStreamCaptureStatusNone)
         if (const hexfc_status st = own_fstat(*m, &fresh); st != HEXFC_OK) return st;
     CK(cudaMemcpyAsync(m->cell_imp, cell_importance, sizeof(float) * (size_t)m->n_cells, cudaMemcpyDeviceToDevice, s));
-    CK(launch_importance(*m, fresh, s));   // positions unchanged since the upload
+    CK(launch_importance(*m, fresh, cap == cudaStreamCaptureStatusNone, s));   // positions unchanged since the upload
     return HEXFC_OK;
 }
 

@@ -100,7 +100,6 @@ struct DevMesh {
     float* cell_imp = nullptr;     // [C]
     int32_t* vkey = nullptr;       // [V] ordered-int max of incident importance
     int32_t* ekey = nullptr;       // [E]
-    float* vimp = nullptr;         // [V]
     float* eattr = nullptr;        // [E]
     uint8_t* elevel = nullptr;     // [E]
     int4* fverts = nullptr;        // [F] canonical corners
@@ -300,7 +299,8 @@ static_assert(sizeof(DrawBatch) < 30000 && sizeof(CountBatch) < 30000,
 cudaError_t launch_cell_quality(const DevMesh& m, int metric, float* out, cudaStream_t s);
 // Vertex and edge importance (max over cells) and the faces' static records;
 // positions: also the corners' world positions (once, at the upload).
-cudaError_t launch_importance(const DevMesh& m, bool positions, cudaStream_t s);
+// From m.cell_imp; chained: see launch_chained.
+cudaError_t launch_importance(const DevMesh& m, bool positions, bool chained, cudaStream_t s);
 
 cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, int64_t n_tiles, cudaStream_t s);
 cudaError_t launch_face_setup(const DevMesh& m, const CamParams& cam, const ShadeParams& sp, FrameBufs& fb,
