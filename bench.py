@@ -30,16 +30,20 @@ import time
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# Algorithmic bytes of the kernels: what the method must move, counted once
-# (a fragment record written by the fill and read by the composite, a face
-# record read once per frame), independent of how the kernels tile the work.
+# Algorithmic bytes of the kernels: what the method must move, counted once (a
+# face and a vertex read once per frame, a pixel written once), independent of
+# how the kernels tile the work.
 # DRAM traffic of one k_draw launch (ncu dram__bytes_read.sum + dram__bytes_write.sum,
 # one pass, on the 1920x1080 bench frame), per fragment of the frame, and the drawing
 # kernel's sources it was taken on: reported only while those sources are unchanged.
-DRAW_DRAM = {"bytes_per_fragment": None, "sha256": None, "profile": None}
+DRAW_DRAM = {"bytes_per_fragment": 3.746,
+             "sha256": "be0cf5861f9c1564a68fe6ebd7accae0edce446955a7ab600c6c4ad493c6054b",
+             "profile": "profiles/dram_k_draw_grid64_orbit_1080p.md"}
 # Warp instructions it executes per fragment (ncu smsp__inst_executed.sum on the same
 # frame and sources): its issue roofline, beside the HBM one.
-DRAW_ISSUE = {"warp_instructions_per_fragment": None, "sha256": None, "profile": None}
+DRAW_ISSUE = {"warp_instructions_per_fragment": 8.936,
+              "sha256": "be0cf5861f9c1564a68fe6ebd7accae0edce446955a7ab600c6c4ad493c6054b",
+              "profile": "profiles/issue_k_draw_grid64_orbit_1080p.md"}
 SCHEDULERS_PER_SM = 4    # warp schedulers (issue slots per cycle) of a Blackwell SM
 DRAW_SOURCES = ("csrc/k_draw.cu", "csrc/shade.cuh", "csrc/raster_common.cuh", "csrc/pipeline.cuh",
                 "csrc/hexfc_internal.cuh")
@@ -72,7 +76,7 @@ def parse_args():
     ap.add_argument("--no-secondary", action="store_true",
                     help="skip the learned-capacity, batch and serving measurements after the main line")
     ap.add_argument("--predicted", type=int, default=0,
-                    help="tile capacities: 0 count-then-fill, 1 previous frame's counts, 2 capacity network")
+                    help="tile capacities: 0 none, 1 previous frame's counts, 2 capacity network")
     # serving mode (--workload serving): Poisson request stream over resident meshes
     ap.add_argument("--rate", type=float, default=200.0, help="serving: mean requests per second")
     ap.add_argument("--requests", type=int, default=600, help="serving: requests in the timed stream")
@@ -426,7 +430,7 @@ def run_ours(args, rank, world, local_rank):
         except Exception as e:   # the main line stands on its own
             sec = {"workload": "grid128_orbit_4k", "failed": str(e)}
     # the metric's other parts, each measured after the main line with its own
-    # clock record: learned capacity against count-then-fill (128^3, 3840x2160),
+    # clock record: learned capacity against frames without it (128^3, 3840x2160),
     # batched views against one by one, the serving loop (rank 0 at N = 1)
     secondaries = {}
     if not args.no_secondary and rank == 0 and world == 1 and args.workload == "grid64_orbit_1080p":
@@ -676,9 +680,9 @@ def run_batch(args, rank, world, steps=None, warmup=None):
 
 def run_learned(args, rank, world):
     """Learned tile capacities: a warped 128^3 grid at 3840x2160 along a
-    500-frame camera and lens path. Frames 0-399 are drawn by count-then-fill
+    500-frame camera and lens path. Frames 0-399 are drawn without capacities
     and the capacity network trains on each frame's exact tile counts; frames
-    400-499 are then drawn (timed) by count-then-fill and with chosen tile
+    400-499 are then drawn (timed) without and with chosen tile
     capacities (no pixel scan, no host wait after the count, each frame
     verified by the next call and drawn again exactly if they ran out): the
     network's, the previous frame's counts, and the previous total spread

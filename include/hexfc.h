@@ -43,7 +43,7 @@ enum {
                                  confirmed) */
 };
 
-/* Longest per-pixel fragment list the sort/composite pass accepts. */
+/* Longest per-pixel fragment list a frame may have. */
 #define HEXFC_MAX_LIST 8192
 
 typedef struct hexfc_ctx hexfc_ctx;

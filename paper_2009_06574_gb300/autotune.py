@@ -5,7 +5,7 @@ number of depth buckets of the per-tile triangle order
 (HEXFC_OPT_DEPTH_BUCKETS: more buckets give per-pixel lists closer to sorted,
 at a larger histogram per tile) and the sorted window of the per-pixel resolve
 (HEXFC_OPT_COMPOSITE_WINDOW: a wider window leaves fewer lists to the
-warp-sort pass, at more registers and moves per element). `tune` times every candidate on
+sorting pass, at more registers and moves per element). `tune` times every candidate on
 a few frames of the caller's own workload with CUDA events, keeps the
 fastest, applies it to the renderer, and caches the choice in a JSON file
 keyed by the GPU, the mesh size and the resolution, so that a workload is

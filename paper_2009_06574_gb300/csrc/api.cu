@@ -944,7 +944,7 @@ constexpr uint64_t kErrPoolBit = 16;     // device error bit: no room for a tile
 // the count. The frame is verified by the next call on the
 // context, at that call's first host wait (it has completed by then), or by
 // hexfc_finish: if its capacities ran out, it is drawn again exactly by
-// count-then-fill into its own output, before anything else.
+// the exact path into its own output, before anything else.
 hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_stats* stats,
                                     cudaStream_t s)
 {
@@ -1060,7 +1060,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
 // Verify the pending frame (drawn with chosen capacities), which must have
 // completed or be about to (its stream is waited for): its device scalars give
 // its statistics; device error bits are reported; if its pool ran out or a list
-// is too long for the resolve, it is drawn again exactly (count-then-fill) into
+// is too long for the resolve, it is drawn again exactly into
 // its output with its own camera, lens and style. s: the stream of the caller's
 // frame, on which the consumed error bits are cleared.
 hexfc_status settle_pending(hexfc_ctx* ctx, cudaStream_t s, bool* redrawn)
@@ -2213,7 +2213,7 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
         CK(cudaMemcpyAsync(h, fb.scal, 6 * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
     }
-    if (h[5] != 0) {   // this call's count pass, or the previous call's fill or composite
+    if (h[5] != 0) {   // this call's count pass, or the previous call's drawing passes
         CK(cudaMemsetAsync(fb.scal + 5, 0, sizeof(uint64_t), s));
         CK(cudaStreamSynchronize(s));
         if (stats) *stats = fs;

@@ -26,9 +26,10 @@ __device__ __forceinline__ float len3(float3 a) { return sqrtf(a.x * a.x + a.y *
 // One thread a cell, the metric at compile time (the ratio needs no lengths), all
 // indices too (the corners stay in registers). The 12 edges' lengths are taken
 // once: the two corners of an edge see it with the same length, bit for bit.
-// 262,144 cells, caches cold: 17 -> 15 us (scaled Jacobian), 17 -> 11 us (ratio).
-// Bound by the gathers' latency, then by the 9 divisions and 15 square roots a
-// cell; cells, vertices and results are 13 MB, 2 us at the copy rate.
+// 262,144 cells: 11.0 -> 7.1 us (scaled Jacobian), 11.0 -> 4.3 us (ratio); with caches
+// cold 17 -> 15 and 17 -> 11. Bound by the gathers' latency, then by the 9 divisions
+// and 15 square roots a cell; cells, vertices and results are 13 MB, 2 us at the copy
+// rate. (64 registers, 8 blocks an SM: 8.8 us.)
 template <int kMetric>
 __global__ void __launch_bounds__(128) k_cell_quality(const float* __restrict__ verts, const int32_t* __restrict__ cells,
                                                       int64_t n_cells, float* __restrict__ out)

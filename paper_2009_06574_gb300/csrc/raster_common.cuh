@@ -52,13 +52,6 @@ __device__ __forceinline__ bool top_left(int32_t xa, int32_t ya, int32_t xb, int
     return (dy < 0) || (dy == 0 && dx > 0);
 }
 
-__device__ __forceinline__ int64_t floor_div_i64(int64_t a, int64_t b)  // b > 0
-{
-    int64_t q = a / b;
-    if ((a % b != 0) && (a < 0)) --q;
-    return q;
-}
-
 // Triangle of a face: tri 0 = corners (0,1,2), tri 1 = (0,2,3), wound to positive area.
 struct TriGeom {
     int32_t X[3], Y[3];
@@ -124,13 +117,6 @@ __device__ __forceinline__ int64_t floor_div_est(int64_t n, int64_t a, bool& bad
 __device__ __forceinline__ float u64_to_f32(uint64_t v)
 {
     return fmaf((float)(uint32_t)(v >> 32), 4294967296.f, (float)(uint32_t)v);
-}
-
-// |v| < 2^55 to float by sign and magnitude (u64_to_f32): within 0.75 ulp.
-__device__ __forceinline__ float i64_to_f32(int64_t v)
-{
-    const float m = u64_to_f32((uint64_t)(v < 0 ? -v : v));
-    return v < 0 ? -m : m;
 }
 
 // Per-sample depth: z0 + floor((l1 d1 + l2 d2) / area), exact, with d1, d2 the
