@@ -475,6 +475,9 @@ __host__ __device__ constexpr size_t sort_smem(int threads, int items, int nb)
 // A block of kT threads holds up to kT * kItems entries in registers (read
 // once); longer lists go through global scratch. The block also leaves the tile's
 // features of the capacity network (cf).
+// Bound by the latency of its steps and barriers (40% of the issue slots): short
+// lists take fewer buckets, those of a chunk one warp without any (29^3 at 1280x720,
+// 160 entries a tile: binning 48 -> 41 us, 4^3 at 256x256, 26 a tile: 12.5 -> 10.6).
 template <int kT, int kItems>
 __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bin_sort(const uint64_t* __restrict__ tile_off,
                                                             const uint32_t* __restrict__ tile_cnt,
@@ -489,6 +492,7 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
     chain_begin();
     if (*n_bins > bin_limit) return;
     constexpr uint32_t kMax = kT * kItems, kLow = kMax / kChunk;
+    constexpr bool kShort = kItems == 8;   // the form for short lists: they are common in it
     extern __shared__ uint32_t sort_sm[];
     uint32_t* s_out = sort_sm;                 // [kMax]
     uint32_t* s_low = s_out + kMax;            // [kLow] least depth of each chunk
@@ -508,7 +512,31 @@ __global__ void __launch_bounds__(kT, kT == 1024 ? 1 : kItems == 8 ? 6 : 5) k_bi
         pad();
         for (uint32_t i = threadIdx.x; i < n_chunks; i += kT) zsuf[beg / kChunk + i] = 0u;
         zmin = 0;
+    } else if (kShort && n <= 32) {   // one warp, each entry's rank counted
+        if (warp != 0) return;
+        const uint32_t* aside = bins + tile_off[tile + 1] - n_skip;
+        for (uint32_t i = lane; i < n_skip; i += 32) {
+            const uint32_t z = tzsum[aside[i]] & kZSum;
+            zmin = min(zmin, z);
+            zmax = max(zmax, z);
+        }
+        const bool in = (uint32_t)lane < n;
+        const uint32_t f = in ? bins[beg + lane] : kPadBin;
+        const uint32_t zs = in ? tzsum[f] : 0u, z = zs & kZSum;
+        uint32_t rank = 0;
+        for (uint32_t j = 0; j < n; ++j) {
+            const uint32_t o = __shfl_sync(0xffffffffu, z, j);
+            rank += o < z || (o == z && j < (uint32_t)lane) ? 1u : 0u;
+        }
+        __syncwarp();   // (the list and what was set aside have been read)
+        if (n > 0) bins[beg + (in ? rank : (uint32_t)lane)] = f;
+        const uint32_t low = __reduce_min_sync(0xffffffffu, in ? packed_least(zs) : 0xFFFFFFFFu);
+        if (n > 0 && lane == 0) zsuf[beg / kChunk] = low;
+        zmin = __reduce_min_sync(0xffffffffu, in ? min(zmin, z) : zmin);
+        zmax = __reduce_max_sync(0xffffffffu, in ? max(zmax, z) : zmax);
     } else {
+        if (kShort)
+            while (nb > 256 && (uint32_t)nb >= 8 * n) nb >>= 1;   // as many buckets an entry as long lists have
         // triangles that cover no sample count for the tile's depth range only
         if (n_skip) {
             const uint32_t* aside = bins + tile_off[tile + 1] - n_skip;

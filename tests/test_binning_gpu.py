@@ -124,7 +124,8 @@ def test_counts_with_and_without_clusters(hx, n, w, h):
 
 
 # meshes drawn so small that triangles lie between samples: set aside when binned, where places are kept
-@pytest.mark.parametrize("n,w,h,radius", [(24, 33, 21, 2.0), (40, 64, 48, 2.6), (40, 16, 16, 8.0), (12, 1, 1, 2.0)])
+@pytest.mark.parametrize("n,w,h,radius", [(24, 33, 21, 2.0), (40, 64, 48, 2.6), (40, 16, 16, 8.0), (12, 1, 1, 2.0),
+                                            (4, 16, 16, 40.0), (3, 40, 16, 25.0), (2, 33, 17, 8.0)])
 def test_triangles_between_samples(hx, n, w, h, radius):
     mesh = synth.hex_grid(n, jitter=0.1, warp_amp=0.2, seed=13)
     view, lens, style = synth.orbit_view(17, 120, w, h, radius=radius), synth.lissajous_lens(17, 120), synth.Style()
