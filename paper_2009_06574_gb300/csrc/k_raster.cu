@@ -391,6 +391,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__
     }
     s_hist[threadIdx.x] = 0;
     if (threadIdx.x == 0) s_empty = 0;
+    uint32_t all = 0;   // the scan's total
     auto block_scan = [&](uint32_t v) -> uint32_t {   // exclusive, over the block's threads
         uint32_t incl = v;
 #pragma unroll
@@ -408,11 +409,26 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__
             if (lane >= o) w += y;
         }
         const uint32_t before = __shfl_sync(0xffffffffu, w, warp - 1);
+        all = __shfl_sync(0xffffffffu, w, 31);
         return incl - v + (warp > 0 ? before : 0u);
     };
     mx = __reduce_max_sync(0xffffffffu, mx);
     if (lane == 0) s_max[warp] = mx;
     uint64_t at = block_scan(sum);   // (fewer than 2^32 chunks: its barriers publish s_max, s_hist, s_empty too)
+    if (threadIdx.x == 1023) {
+        tile_off[n] = (uint64_t)all * kChunk;
+        *total = (uint64_t)all * kChunk;
+        if (h_total) *h_total = (uint64_t)all * kChunk;
+    }
+    // Three drawing blocks an SM hold all tiles of a small frame at once: any order
+    // does (but not for long lists, whose form has one, launch_draw).
+    if (n <= 3 * 152 && all < 3u * (uint32_t)n) {
+        if ((int)threadIdx.x < n) {   // (a tile a thread)
+            tile_off[threadIdx.x] = at * kChunk;
+            order[threadIdx.x] = threadIdx.x;
+        }
+        return;
+    }
     mx = __reduce_max_sync(0xffffffffu, s_max[lane]);
     int shift = 0;
     while ((mx >> shift) >= 1024u) ++shift;
@@ -435,11 +451,6 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const uint32_t* __restrict__
                 else rank[k] = atomicAdd(&s_hist[1023u - (nc[k] >> shift)], 1u);
             }
         }
-    }
-    if (threadIdx.x == 1023) {
-        tile_off[n] = at * kChunk;
-        *total = at * kChunk;
-        if (h_total) *h_total = at * kChunk;
     }
     __syncthreads();
     const uint32_t h = s_hist[threadIdx.x];
