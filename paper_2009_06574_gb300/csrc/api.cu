@@ -747,11 +747,10 @@ hexfc_status job_read2(FrameJob& j, cudaStream_t s)
 }
 
 // After the drawing pass: the white silhouettes over the output window.
-hexfc_status job_silhouette(FrameJob& j, float* out, cudaStream_t s)
+hexfc_status job_silhouette(FrameJob& j, const DrawItem& it, cudaStream_t s)
 {
     if (j.sil_alpha <= 0.f) return HEXFC_OK;
-    CK(launch_silhouette(j.fb->zsil, j.tiles_x, j.cam.ox, j.cam.oy, j.frame_w, j.frame_h, j.sil_alpha,
-                         j.sil_threshold, j.fb->scal + 8, j.fb->bin_limit, out, j.win, j.fb->chained, s));
+    CK(launch_silhouette(it, j.cam.ox, j.cam.oy, j.frame_w, j.frame_h, j.sil_alpha, j.sil_threshold, s));
     j.launches += 1;
     return HEXFC_OK;
 }
@@ -800,7 +799,7 @@ hexfc_status job_phase3(FrameJob& j, cudaStream_t s)
         job_mark(j, 9, s);
         CK(launch_draw_tail(it, s));
         j.launches += 2;
-        if ((st = job_silhouette(j, j.out, s)) != HEXFC_OK) return st;
+        if ((st = job_silhouette(j, it, s)) != HEXFC_OK) return st;
     } else {
         job_mark(j, 9, s);
     }
@@ -1023,7 +1022,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     CK(launch_draw(it, j.n_tiles, j.n_bins, j.window, s));
     job_mark(j, 9, s);
     CK(launch_draw_tail(it, s));
-    if ((st = job_silhouette(j, out, s)) != HEXFC_OK) return st;
+    if ((st = job_silhouette(j, it, s)) != HEXFC_OK) return st;
     job_mark(j, 10, s);
     j.launches += 1 + 3 + 1 + 1 + 2;   // capacities, their scan, count, check, drawing passes
     // the frame's scalars for its verification; no wait here
@@ -1569,9 +1568,10 @@ hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_ite
     };
     auto tail = [&](int i, cudaStream_t si) -> hexfc_status {   // pixels out of order, silhouettes
         FrameJob& j = jobs[(size_t)i];
-        CK(launch_draw_tail(draw_item(j, limits[(size_t)i]), si));
+        const DrawItem it = draw_item(j, limits[(size_t)i]);
+        CK(launch_draw_tail(it, si));
         j.launches += 2;
-        return job_silhouette(j, j.out, si);
+        return job_silhouette(j, it, si);
     };
     if (one && !draw.empty() && (st = batch_graph(ctx, 2, draw, none, draw_all, tail, true)) != HEXFC_OK) return st;
     if (!one && !draw.empty() &&
@@ -2234,8 +2234,8 @@ hexfc_status render_frame_noalloc(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_
     CK(launch_draw(it, n_tiles, n_bins, ctx->window, s));
     CK(launch_draw_tail(it, s));
     if (sil)
-        CK(launch_silhouette(fb.zsil, tiles_x, ctx->cam.ox, ctx->cam.oy, ctx->view.width, ctx->view.height,
-                             ctx->style.sil_alpha, ctx->style.sil_threshold, fb.scal + 8, fb.bin_limit, out, win, fb.chained, s));
+        CK(launch_silhouette(it, ctx->cam.ox, ctx->cam.oy, ctx->view.width, ctx->view.height, ctx->style.sil_alpha,
+                             ctx->style.sil_threshold, s));
     return inject_error_bits(ctx, fb.scal, s);
 }
 

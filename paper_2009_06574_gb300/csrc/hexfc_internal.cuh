@@ -349,9 +349,8 @@ cudaError_t launch_cap_to_half(CapNet& net, cudaStream_t s);
 // White silhouettes over the output (Section "Blending Focus and Context"):
 // from the boundary surface's depths zsil of the drawn rectangle, which sits
 // at (fx0, fy0) of a frame_w x frame_h frame.
-cudaError_t launch_silhouette(const uint32_t* zsil, int tiles_x, int fx0, int fy0, int frame_w, int frame_h,
-                              float alpha, float threshold, const uint64_t* n_bins, uint64_t bin_limit, float* out,
-                              OutWin win, bool chained, cudaStream_t s);
+cudaError_t launch_silhouette(const DrawItem& a, int fx0, int fy0, int frame_w, int frame_h, float alpha, float threshold,
+                              cudaStream_t s);
 // The sorted lists of n pixels of a frame drawn as `a` (or their lengths, if d_counts).
 cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const int32_t* d_py, int64_t n,
                                 const uint64_t* d_dst_off, uint64_t* d_keys, float4* d_rgba, uint32_t* d_counts,

@@ -602,14 +602,16 @@ __device__ __forceinline__ uint32_t zsil_at(const uint32_t* __restrict__ zsil, i
     return zsil[t * kTilePix + (y % kTileH) * kTileW + (x % kTileW)];
 }
 
-__global__ void __launch_bounds__(256) k_silhouette(const uint32_t* __restrict__ zsil, int tiles_x, int fx0, int fy0,
-                                                    int frame_w, int frame_h, float alpha, int64_t T,
-                                                    const uint64_t* __restrict__ n_bins, uint64_t bin_limit,
-                                                    float4* __restrict__ out, OutWin win)
+__global__ void __launch_bounds__(256) k_silhouette(const __grid_constant__ DrawItem a, int fx0, int fy0, int frame_w,
+                                                    int frame_h, float alpha, int64_t T)
 {
     chain_begin();
+    const OutWin& win = a.win;
+    const uint32_t* zsil = a.zsil;
+    const int tiles_x = a.tiles_x;
+    float4* out = a.out;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)win.w * win.h || *n_bins > bin_limit) return;
+    if (i >= (int64_t)win.w * win.h || !frame_allowed(a)) return;   // (a refused frame leaves its output alone)
     const int x = win.x0 + (int)(i % win.w), y = win.y0 + (int)(i / win.w);
     const uint32_t zp = zsil_at(zsil, tiles_x, x, y);
     if (zp == kNoDepth) return;
@@ -758,14 +760,13 @@ cudaError_t launch_draw_tail(const DrawItem& a, cudaStream_t s)
     return launch_chained(k_draw_tail, kTailBlocks, kTilePix, sizeof(PixelList), s, a.chained, a);
 }
 
-cudaError_t launch_silhouette(const uint32_t* zsil, int tiles_x, int fx0, int fy0, int frame_w, int frame_h,
-                              float alpha, float threshold, const uint64_t* n_bins, uint64_t bin_limit, float* out,
-                              OutWin win, bool chained, cudaStream_t s)
+cudaError_t launch_silhouette(const DrawItem& a, int fx0, int fy0, int frame_w, int frame_h, float alpha, float threshold,
+                              cudaStream_t s)
 {
-    const int64_t n = (int64_t)win.w * win.h;
+    const int64_t n = (int64_t)a.win.w * a.win.h;
     if (n == 0) return cudaSuccess;
-    return launch_chained(k_silhouette, (unsigned)((n + 255) / 256), 256, 0, s, chained, zsil, tiles_x, fx0, fy0, frame_w,
-                          frame_h, alpha, (int64_t)threshold, n_bins, bin_limit, reinterpret_cast<float4*>(out), win);
+    return launch_chained(k_silhouette, (unsigned)((n + 255) / 256), 256, 0, s, a.chained, a, fx0, fy0, frame_w, frame_h, alpha,
+                          (int64_t)threshold);
 }
 
 cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const int32_t* d_py, int64_t n,

@@ -182,3 +182,25 @@ def test_frames_whose_bins_outgrow_their_room(hx):
         for img in imgs[1:]:
             assert torch.equal(img, imgs[0])
     r.close()
+
+
+def test_refused_frames_leave_their_output_alone(hx):
+    """A frame refused for its budget, silhouettes and all, after one of another view that was drawn."""
+    mesh = synth.hex_grid(16, jitter=0.1, warp_amp=0.2, seed=15)
+    r = hx.Renderer(0, frag_budget_bytes=24 << 20)
+    mid = r.upload_mesh(mesh.verts, mesh.cells, mesh.cell_scalar, mesh.edge_level)
+    r.set_lens(synth.lissajous_lens(3, 120))
+    r.set_style(synth.Style(sil_alpha=0.7))
+    small = torch.full((48, 64, 4), -1.0, device="cuda")
+    r.set_view(synth.orbit_view(3, 120, 64, 48))
+    r.render(mid, small)
+    large = torch.full((480, 640, 4), -1.0, device="cuda")
+    r.set_view(synth.orbit_view(3, 120, 640, 480))
+    assert r.render(mid, large, check=False) != 0
+    torch.cuda.synchronize()
+    assert (large == -1.0).all()
+    r.set_view(synth.orbit_view(3, 120, 64, 48))
+    again = torch.full((48, 64, 4), -1.0, device="cuda")
+    r.render(mid, again)
+    assert torch.equal(again, small)
+    r.close()
