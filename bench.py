@@ -37,12 +37,12 @@ sys.path.insert(0, ROOT)
 # one pass, on the 1920x1080 bench frame), per fragment of the frame, and the drawing
 # kernel's sources it was taken on: reported only while those sources are unchanged.
 DRAW_DRAM = {"bytes_per_fragment": 3.746,
-             "sha256": "be0cf5861f9c1564a68fe6ebd7accae0edce446955a7ab600c6c4ad493c6054b",
+             "sha256": "07c7e546cf8e66ddaa759137f77dd5700ea2344364c17bf139c877d0e156b1d6",
              "profile": "profiles/dram_k_draw_grid64_orbit_1080p.md"}
 # Warp instructions it executes per fragment (ncu smsp__inst_executed.sum on the same
 # frame and sources): its issue roofline, beside the HBM one.
-DRAW_ISSUE = {"warp_instructions_per_fragment": 8.936,
-              "sha256": "be0cf5861f9c1564a68fe6ebd7accae0edce446955a7ab600c6c4ad493c6054b",
+DRAW_ISSUE = {"warp_instructions_per_fragment": 8.937,
+              "sha256": "07c7e546cf8e66ddaa759137f77dd5700ea2344364c17bf139c877d0e156b1d6",
               "profile": "profiles/issue_k_draw_grid64_orbit_1080p.md"}
 SCHEDULERS_PER_SM = 4    # warp schedulers (issue slots per cycle) of a Blackwell SM
 DRAW_SOURCES = ("csrc/k_draw.cu", "csrc/shade.cuh", "csrc/raster_common.cuh", "csrc/pipeline.cuh",

@@ -134,7 +134,8 @@ typedef struct hexfc_frame_stats {
 } hexfc_frame_stats;
 
 /* Stages timed by HEXFC_OPT_STAGE_TIMING (CUDA events on the render stream).
- * GAP stages are the host round trips that read the bin and fragment totals. */
+ * GAP1 is the host's wait for the bin total, where a frame has to make room for
+ * its bins; GAP2 and SCAN are kept for callers that read all stages. */
 enum {
     HEXFC_STAGE_VERTEX = 0,   /* vertex projection */
     HEXFC_STAGE_FACE = 1,     /* face setup and tile counts */
