@@ -1661,7 +1661,10 @@ hexfc_status hexfc_capacity_train(hexfc_ctx* ctx, int32_t steps, float lr, float
     const cudaStream_t s = (cudaStream_t)stream;
     const int64_t n = ctx->feat_tiles;
     cudaStreamCaptureStatus captured = cudaStreamCaptureStatusNone;
-    CK(cudaStreamIsCapturing(s, &captured));
+    if (cudaStreamIsCapturing(s, &captured) != cudaSuccess) {   // (the launches answer for it, as in an importance update)
+        (void)cudaGetLastError();
+        captured = cudaStreamCaptureStatusActive;
+    }
     const bool chain = captured == cudaStreamCaptureStatusNone;
     for (int32_t k = 0; k < steps; ++k)
         CK(launch_cap_grad(c, ctx->fb.cap_x, ctx->fb.tile_frag, n, lr, chain && k > 0, s));
