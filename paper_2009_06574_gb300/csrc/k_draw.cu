@@ -25,6 +25,7 @@
 // pixel, so the order is unique, and every path blends a list one element
 // after the other in that order with the same operations: the image does not
 // depend on which path resolved a pixel, nor on the window's size, bit for bit.
+#include "draw_slot.h"
 #include "pipeline.cuh"
 #include "shade.cuh"
 
@@ -84,17 +85,16 @@ __device__ __forceinline__ bool frame_allowed(const DrawItem& a)
 
 // ------------------------------------------------------------------ staging
 
-// A ring slot: the records of one chunk, and its masks in the consumers' order
-// (the 32 pixels of a warp's group one after the other).
+// A ring slot: the records of one chunk (draw_slot.h), and its masks in the
+// consumers' order (the 32 pixels of a warp's group one after the other).
 struct DrawSlot {
-    ShadeRec sh[kChunk];
+    ShadeRec sh[slot_records(kChunk)];
     uint32_t mask[kTilePix];
 };
 
 template <int KW, bool kWide>
 struct DrawRing {
     static constexpr int kRing = ring_of(kWide);
-    ShadeRec none;                      // what a lane without a triangle reads (kWide), or reads past slot 0
     DrawSlot ring[kRing];
     float4 window[KW][kTilePix];
     uint64_t full[kRing];               // a slot is staged (the 32 lanes of the warp that staged it arrive)
@@ -388,7 +388,9 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW, kWide>& S, const DrawItem
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < kRing) mbar_init(&S.full[threadIdx.x], 32);
     if (threadIdx.x < kWarps) S.rel[threadIdx.x] = 0;
-    if (threadIdx.x < sizeof(ShadeRec) / sizeof(uint32_t)) reinterpret_cast<uint32_t*>(&S.none)[threadIdx.x] = 0u;
+    constexpr int kWords = sizeof(ShadeRec) / sizeof(uint32_t);   // the slots' blank records
+    for (int i = threadIdx.x; i < kRing * kWords; i += blockDim.x)
+        reinterpret_cast<uint32_t*>(&S.ring[i / kWords].sh[kSlotBlank])[i % kWords] = 0u;
     mbar_init_fence();
     if (!__syncthreads_and(allowed)) return;   // (one answer for the block: another may set an error bit meanwhile)
     // staging: this warp's next chunk and its triangles
@@ -403,7 +405,7 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW, kWide>& S, const DrawItem
         const uint4 ma = mp[0], mb = mp[1];
         if (f2t_m != kPadBin)
             make_record(a.fframe[f2t_m >> 1], a.fstat[f2t_m >> 1], a.fextra ? a.fextra + (f2t_m >> 1) : nullptr, f2t_m, px0,
-                        py0, a.sp, D.sh[lane]);
+                        py0, a.sp, D.sh[slot_place(lane)]);
         md[0] = ma;
         md[1] = mb;
         mbar_arrive(&S.full[kWide ? mine & (kRing - 1) : warp]);
@@ -506,10 +508,9 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW, kWide>& S, const DrawItem
             }
         }
         const bool live = m != 0;   // (a lane without a triangle goes along)
-        // (a lane without a triangle: triangle -1 of its slot, whatever memory of the
-        // ring that is; its results go nowhere. Where there are many such lanes they
-        // read one record instead)
-        const ShadeRec& R = !kWide || live ? S.ring[ch & (kRing - 1)].sh[__ffs(m) - 1] : S.none;
+        // (a lane without a triangle: the blank record of its slot; its results go
+        // nowhere. Where there are many such lanes they read one of them)
+        const ShadeRec& R = S.ring[!kWide || live ? ch & (kRing - 1) : 0].sh[next_place(m)];
         m &= m - 1;   // (0 stays 0)
         const uint4 zf = R.zf, ha = R.ha;
         const Sample q = sample_of(R, zf, ha, (uint32_t)lx << 8, (uint32_t)ly << 8, live, bad);
