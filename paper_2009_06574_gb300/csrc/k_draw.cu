@@ -412,8 +412,14 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW, kWide>& S, const DrawItem
         mine += kStep;
         f2t_m = mine < n_chunks ? a.bins[beg + (uint64_t)mine * kChunk + lane] : kPadBin;
     };
-    // the least progress of the block's warps (kGone: all are finished)
-    auto slowest = [&]() { return __reduce_min_sync(kFull, lane < kWarps ? load_acquire(&S.rel[lane]) : kGone); };
+    // the least progress of the block's warps (kGone: all are finished). What those
+    // warps read before it comes before what any lane of this one writes after it: a
+    // lane's acquire is the warp's by the __syncwarp (the reduction orders no memory).
+    auto slowest = [&]() {
+        const uint32_t r = __reduce_min_sync(kFull, lane < kWarps ? load_acquire(&S.rel[lane]) : kGone);
+        __syncwarp();
+        return r;
+    };
     // what is left to stage, as slots become free
     auto stage_rest = [&]() {
         long long t0 = clock64();
@@ -478,11 +484,11 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW, kWide>& S, const DrawItem
         if (!act || (step++ & (kService - 1)) == 0) {
             // release the chunks every lane is past, stage the next one if its slot is free, take what is staged
             const uint32_t lo = __reduce_min_sync(kFull, done ? hi : (uint32_t)(m != 0 ? ch : ch + 1));
+            __syncwarp();   // what the lanes read of those chunks comes before lane 0's release
             if (lo > rel) {
                 rel = lo;
                 if (lane == 0) store_release(&S.rel[warp], rel);
             }
-            __syncwarp();
             if (!kWide && mine < n_chunks && mine < min(slowest(), kGone - kRing) + kRing) stage();
             bool got = false;
             while (hi < n_chunks && hi < rel + kRing &&
