@@ -420,15 +420,20 @@ __device__ __forceinline__ void draw_tile(DrawRing<KW, kWide>& S, const DrawItem
         __syncwarp();
         return r;
     };
-    // what is left to stage, as slots become free
+    // what is left to stage, as slots become free. The wait is bounded from the last
+    // progress of the slowest warp: a tile may take longer than a wait.
     auto stage_rest = [&]() {
         long long t0 = clock64();
+        uint32_t seen = 0;
         while (mine < n_chunks) {
             const uint32_t r = slowest();
             if (r == kGone) break;
+            if (r != seen) {
+                seen = r;
+                t0 = clock64();
+            }
             if (mine < r + kRing) {
                 stage();
-                if (kWide) t0 = clock64();
             } else {
                 if (__any_sync(kFull, clock64() - t0 > kWaitCycles)) {
                     if (lane == 0) atomicOr(a.err, kErrWait);

@@ -5,7 +5,10 @@
 
 namespace hexfc {
 
-constexpr long long kWaitCycles = 1ll << 30;       // about half a second of SM clock
+#ifndef HEXFC_WAIT_CYCLES
+#define HEXFC_WAIT_CYCLES (1ll << 30)
+#endif
+constexpr long long kWaitCycles = HEXFC_WAIT_CYCLES;   // about half a second of SM clock (a build-time choice, for tests)
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
