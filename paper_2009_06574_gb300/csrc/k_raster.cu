@@ -23,6 +23,7 @@
 #include <cooperative_groups.h>
 
 #include "count_tiles.cuh"
+#include "lens_test.h"
 #include "shade.cuh"
 
 namespace hexfc {
@@ -105,29 +106,6 @@ __device__ __forceinline__ uint32_t packed_least(uint32_t v)
 {
     const uint32_t mean = (v & kZSum) / 3u, s = depth_spread(v >> 26);
     return mean > s ? mean - s : 0u;
-}
-
-// Whether the triangle of corners with offsets o[k] from the sphere lens' centre
-// and eye depths e[k] lies wholly outside the lens. The offsets, projected on
-// the direction of their sum, are all above the radius, so every point of the
-// triangle is. The margin covers the rounding of a sample's distance (affine
-// sums of offset / w and 1 / w in float: below 12 * 2^-24 of the largest
-// offset, times the ratio of the eye depths), so that the computed distance is
-// at least 1 too, and the sample's focus exactly 0.
-__device__ __forceinline__ bool outside_lens(const float (&o)[3][3], const float (&e)[3], bool ortho, float inv_r)
-{
-    const float mx = o[0][0] + o[1][0] + o[2][0], my = o[0][1] + o[1][1] + o[2][1],
-                mz = o[0][2] + o[1][2] + o[2][2];
-    const float im = rsqrtf(mx * mx + my * my + mz * mz);
-    float lo = INFINITY, far = 0.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        lo = fminf(lo, (o[k][0] * mx + o[k][1] * my + o[k][2] * mz) * im);
-        far = fmaxf(far, fabsf(o[k][0]) + fabsf(o[k][1]) + fabsf(o[k][2]));
-    }
-    const float e_lo = fminf(e[0], fminf(e[1], e[2])), e_hi = fmaxf(e[0], fmaxf(e[1], e[2]));
-    const float ratio = ortho ? 1.f : __fdividef(e_hi, e_lo);
-    return (ortho || e_lo > 0.f) && lo * inv_r >= 1.0001f + 8e-6f * far * inv_r * ratio;
 }
 
 // A triangle's tiles in one word: the first one's column and row, whether it
