@@ -335,8 +335,7 @@ hexfc_status hexfc_render_host(hexfc_ctx* ctx, int32_t mesh, float* out_rgba_hos
 /*
  * Parity hook: the fragment lists of the last render for `n` listed pixels
  * (px[i], py[i], host), built from what that frame was drawn from (an importance
- * update after it changes nothing, unless it was captured into a CUDA graph:
- * such an update rewrites the mesh's records in place). counts (host, n) receives each list length; keys
+ * update after it changes nothing). counts (host, n) receives each list length; keys
  * (host, cap) and rgba (host, cap*4 float) receive the lists concatenated in
  * the order of the pixel list, each sorted ascending by key =
  * (z24 << 32) | (2*face_id + triangle), rgba premultiplied (Eq. 4).

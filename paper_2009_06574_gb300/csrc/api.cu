@@ -67,7 +67,7 @@ struct hexfc_ctx {
     bool have_frame = false;
     DrawItem last_draw{};
     std::shared_ptr<DevMesh> last_mesh;
-    std::shared_ptr<FaceStatic> last_fstat;   // the mesh's records it was drawn with
+    DrawnCorners last_corners{};
     hexfc_frame_stats last{};
     float* d_out = nullptr;   // image buffer of hexfc_render_host
     int64_t d_out_cap = 0;
@@ -182,7 +182,7 @@ void free_mesh(DevMesh* m)
     if (!m) return;
     dfree(m->verts); dfree(m->cells); dfree(m->cell_edges); dfree(m->cell_imp);
     dfree(m->vkey); dfree(m->ekey); dfree(m->eattr); dfree(m->elevel);
-    dfree(m->fverts); dfree(m->fedges); dfree(m->fbound);
+    dfree(m->fverts); dfree(m->fedges); dfree(m->fbound); dfree(m->fstat);
     delete m;
 }
 
@@ -194,31 +194,6 @@ void free_frame(FrameBufs& f)
     dfree(f.part); dfree(f.part_max); dfree(f.redo); dfree(f.scal);
     if (f.h_scal) cudaFreeHost(f.h_scal);
     f = FrameBufs{};
-}
-
-// A set of static face records that no frame keeps becomes the mesh's own;
-// *fresh: it is new (no positions in it yet).
-hexfc_status own_fstat(DevMesh& m, bool* fresh)
-{
-    *fresh = false;
-    if (m.fstat && m.fstat.use_count() == 2) return HEXFC_OK;   // fstat and fstat_sets
-    for (const auto& f : m.fstat_sets)
-        if (f.use_count() == 1) {
-            m.fstat = f;
-            return HEXFC_OK;
-        }
-    FaceStatic* p = nullptr;
-    const hexfc_status st = dalloc(&p, (size_t)m.n_faces);
-    if (st != HEXFC_OK) return st;
-    try {
-        std::shared_ptr<FaceStatic> f(p, [](FaceStatic* q) { cudaFree(q); });   // (frees p if it throws)
-        m.fstat_sets.push_back(f);
-        m.fstat = std::move(f);
-    } catch (...) {
-        return HEXFC_ERR_OOM;
-    }
-    *fresh = true;
-    return HEXFC_OK;
 }
 
 void free_slots(FrameBufs& f)
@@ -766,7 +741,7 @@ DrawItem draw_item(const FrameJob& j, uint64_t limit)
     it.masks = fb.masks;
     it.zsuf = fb.zsuf;
     it.fframe = fb.fframe;
-    it.fstat = j.m->fstat.get();
+    it.fstat = j.m->fstat;
     it.fextra = fb.fextra;
     it.order = fb.tile_order;
     it.cnt = fb.cnt;
@@ -855,7 +830,7 @@ void keep_frame(hexfc_ctx* ctx, const FrameJob& j)
     ctx->last_draw = draw_item(j, ~0ull);
     for (const auto& m : ctx->meshes)
         if (m.get() == j.m) ctx->last_mesh = m;
-    ctx->last_fstat = j.m->fstat;
+    ctx->last_corners = DrawnCorners{j.m->fverts, j.fb->vproj};
     ctx->last_win = j.win;
     ctx->counts_W = j.W;
     ctx->counts_H = j.H;
@@ -1307,7 +1282,6 @@ void hexfc_destroy(hexfc_ctx* ctx)
     ctx->pend.mesh.reset();
     if (ctx->h_pend) cudaFreeHost(ctx->h_pend);
     ctx->h_pend = nullptr;
-    ctx->last_fstat.reset();
     ctx->last_mesh.reset();
     ctx->meshes.clear();   // a mesh is freed with its last holder
     free_frame(ctx->fb);
@@ -1390,7 +1364,6 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
     if (st == HEXFC_OK && e == cudaSuccess) {
         m->n_faces = (int64_t)n_faces;
         m->n_edges = (int64_t)n_edges;
-        bool fresh = false;
         A(dalloc(&m->cell_imp, (size_t)n_cells));
         A(dalloc(&m->vkey, (size_t)n_verts));
         A(dalloc(&m->ekey, (size_t)n_edges));
@@ -1398,7 +1371,7 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
         A(dalloc(&m->elevel, (size_t)n_edges));
         A(dalloc(&m->fverts, (size_t)n_faces));
         A(dalloc(&m->fedges, (size_t)n_faces));
-        A(own_fstat(*m, &fresh));
+        A(dalloc(&m->fstat, (size_t)n_faces));
         A(dalloc(&m->fbound, (size_t)n_faces));
     }
     if (st == HEXFC_OK && e == cudaSuccess && !host) {
@@ -1710,7 +1683,6 @@ hexfc_status hexfc_trim(hexfc_ctx* ctx)
     dfree(ctx->d_out);
     ctx->d_out_cap = 0;
     ctx->have_frame = false;
-    ctx->last_fstat.reset();
     ctx->last_mesh.reset();
     return HEXFC_OK;
 }
@@ -1745,18 +1717,14 @@ hexfc_status hexfc_set_cell_importance(hexfc_ctx* ctx, int32_t mesh, const float
     if (!m) return HEXFC_ERR_STATE;
     DeviceGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    // (a captured update writes the current records in place: nothing may be
-    // allocated, and every replay has to write what the renders read)
+    // (all in place: nothing is allocated, and every replay of a captured update writes what the renders read)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
         (void)cudaGetLastError();
         cap = cudaStreamCaptureStatusActive;
     }
-    bool fresh = false;
-    if (cap == cudaStreamCaptureStatusNone)
-        if (const hexfc_status st = own_fstat(*m, &fresh); st != HEXFC_OK) return st;
     CK(cudaMemcpyAsync(m->cell_imp, cell_importance, sizeof(float) * (size_t)m->n_cells, cudaMemcpyDeviceToDevice, s));
-    CK(launch_importance(*m, fresh, cap == cudaStreamCaptureStatusNone, s));   // positions unchanged since the upload
+    CK(launch_importance(*m, false, cap == cudaStreamCaptureStatusNone, s));   // positions unchanged since the upload
     return HEXFC_OK;
 }
 
@@ -1931,7 +1899,7 @@ hexfc_status hexfc_debug_pixels(hexfc_ctx* ctx, const int32_t* px, const int32_t
     cudaError_t e = cudaMemcpy(d_px, px, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(d_py, py, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = launch_debug_gather(ctx->last_draw, d_px, d_py, n, nullptr, nullptr, nullptr, d_cnt, 0);
+        e = launch_debug_gather(ctx->last_draw, ctx->last_corners, d_px, d_py, n, nullptr, nullptr, nullptr, d_cnt, 0);
     if (e == cudaSuccess) e = cudaMemcpy(counts, d_cnt, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) {
         note_cuda(e);
@@ -1958,7 +1926,7 @@ hexfc_status hexfc_debug_pixels(hexfc_ctx* ctx, const int32_t* px, const int32_t
     }
     e = cudaMemcpy(d_off, hoff.data(), sizeof(uint64_t) * (size_t)n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = launch_debug_gather(ctx->last_draw, d_px, d_py, n, d_off, d_keys, d_rgba, nullptr, 0);
+        e = launch_debug_gather(ctx->last_draw, ctx->last_corners, d_px, d_py, n, d_off, d_keys, d_rgba, nullptr, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess && keys) e = cudaMemcpy(keys, d_keys, sizeof(uint64_t) * total, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess && rgba) e = cudaMemcpy(rgba, d_rgba, sizeof(float4) * total, cudaMemcpyDeviceToHost);

@@ -4,10 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <memory>
 #include <type_traits>
 #include <utility>
-#include <vector>
 
 #include "hexfc.h"
 #include "vertex_stage.h"
@@ -49,8 +47,8 @@ struct ShadeParams {
 // A face as two 64-byte records: the per-frame one (window corners, depths,
 // flags, eye depths), written by the face stage of every frame into the
 // rendering context's buffers, and the static one (corner importance and world
-// position), owned by the mesh and rewritten only when importance changes, so
-// that contexts can render one resident mesh at the same time.
+// position), owned by the mesh and rewritten in place only when importance
+// changes, so that contexts can render one resident mesh at the same time.
 struct __align__(64) FaceFrame {
     int4 X, Y;            // corner window position, 16.8 fixed point
     uint4 Z;              // bits 0-23: corner window depth (z24). Bits 24-31 of Z.x: edge flags (bits 0-3
@@ -69,6 +67,7 @@ struct __align__(64) FaceStatic {
 };
 static_assert(sizeof(FaceFrame) == 64 && sizeof(FaceStatic) == 64, "two sectors each");
 constexpr uint32_t kZ24 = 0xFFFFFFu;
+constexpr int32_t kVertexValid = 1 << 24;   // of a projected vertex' depth word
 // Face flags, bit t for triangle t where shifted by it.
 constexpr uint32_t kFaceDrawn = 1u;      // << t: triangle drawn
 constexpr uint32_t kFaceBoundary = 4u;   // a face of one cell
@@ -105,12 +104,20 @@ struct DevMesh {
     int4* fverts = nullptr;        // [F] canonical corners
     int4* fedges = nullptr;        // [F] unique edge id of local edge k = (c_k, c_k+1)
     uint8_t* fbound = nullptr;     // [F] 1: a boundary face (one cell)
-    // [F] static face records. A frame keeps the records it was drawn with (its
-    // lists are rebuilt from them on request), so an importance update writes
-    // records that no frame keeps: at most one set per context and one more.
-    std::shared_ptr<FaceStatic> fstat;
-    std::vector<std::shared_ptr<FaceStatic>> fstat_sets;   // all sets, fstat among them
+    FaceStatic* fstat = nullptr;   // [F] static face records
 };
+
+// An importance as an int of the same order (vkey, ekey), so that atomicMax on
+// int is a float max; an unreferenced vertex or edge (INT32_MIN) has 0.
+__device__ __forceinline__ int32_t importance_key(float f)
+{
+    const int32_t i = __float_as_int(f);
+    return i >= 0 ? i : (i ^ 0x7FFFFFFF);
+}
+__device__ __forceinline__ float importance_of(int32_t k)
+{
+    return k == INT32_MIN ? 0.f : __int_as_float(k >= 0 ? k : (k ^ 0x7FFFFFFF));
+}
 
 // Tile-capacity network (4 -> 64 -> 64 -> 1): FP32 master weights, the FP16
 // copy the kernels use, Adam moments, and per-tile training values.
@@ -133,7 +140,9 @@ struct CapNet {
 // Per-frame buffers owned by the context.
 struct FrameBufs {
     // vertex stage
-    int4* vproj = nullptr;   // {X, Y, z24, valid}
+    // {X, Y, z24 | kVertexValid, importance key}: the key is the frame's own copy, so that its fragments can
+    // be found again (hexfc_debug_pixels) after the mesh's importance has changed
+    int4* vproj = nullptr;
     float* ved = nullptr;    // eye depth
     int64_t v_cap = 0;
     // faces
@@ -351,8 +360,13 @@ cudaError_t launch_cap_to_half(CapNet& net, cudaStream_t s);
 // at (fx0, fy0) of a frame_w x frame_h frame.
 cudaError_t launch_silhouette(const DrawItem& a, int fx0, int fy0, int frame_w, int frame_h, float alpha, float threshold,
                               cudaStream_t s);
-// The sorted lists of n pixels of a frame drawn as `a` (or their lengths, if d_counts).
-cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const int32_t* d_py, int64_t n,
+// What a frame keeps of its faces' corners: their vertices, and the vertices as it projected them.
+struct DrawnCorners {
+    const int4* fverts;
+    const int4* vproj;
+};
+// The sorted lists of n pixels of a frame drawn as `a` with corners dc (or their lengths, if d_counts).
+cudaError_t launch_debug_gather(const DrawItem& a, const DrawnCorners& dc, const int32_t* d_px, const int32_t* d_py, int64_t n,
                                 const uint64_t* d_dst_off, uint64_t* d_keys, float4* d_rgba, uint32_t* d_counts,
                                 cudaStream_t s);
 

@@ -238,10 +238,21 @@ __device__ __forceinline__ uint64_t fragment_key(const DrawItem& a, const PixelR
     return ((uint64_t)zv << 32) | f2t;
 }
 
-__device__ __noinline__ float4 fragment_colour(const DrawItem& a, const PixelRef& r, uint32_t f2t, bool& bad)
+// kKept: with the importances that the frame has kept itself (dc), not the mesh's.
+template <bool kKept>
+__device__ __noinline__ float4 fragment_colour(const DrawItem& a, const DrawnCorners& dc, const PixelRef& r, uint32_t f2t,
+                                               bool& bad)
 {
     ShadeRec R;
-    make_record(a.fframe[f2t >> 1], a.fstat[f2t >> 1], nullptr, f2t, r.px0, r.py0, a.sp, R);
+    if constexpr (kKept) {
+        FaceStatic S = a.fstat[f2t >> 1];
+        const int4 v = dc.fverts[f2t >> 1];
+        S.imp = make_float4(importance_of(dc.vproj[v.x].w), importance_of(dc.vproj[v.y].w), importance_of(dc.vproj[v.z].w),
+                            importance_of(dc.vproj[v.w].w));
+        make_record(a.fframe[f2t >> 1], S, nullptr, f2t, r.px0, r.py0, a.sp, R);
+    } else {
+        make_record(a.fframe[f2t >> 1], a.fstat[f2t >> 1], nullptr, f2t, r.px0, r.py0, a.sp, R);
+    }
     const Sample s = sample_of(R, R.zf, R.ha, (uint32_t)r.lx << 8, (uint32_t)r.ly << 8, true, bad);
     const int x = r.px0 + r.lx, y = r.py0 + r.ly;
     const float dist = a.sp.lens_mode == HEXFC_LENS_SCREEN ? screen_lens_dist(x, y, a.sp) : 0.f;
@@ -258,8 +269,9 @@ struct PixelList {   // the list of one pixel in a block's shared memory
 // sorted list is written. A fragment a thread: up to kTilePix of them each
 // thread finds the rank of its own key, beyond that a bitonic sort; then they
 // are shaded kTilePix at a time, and blended by thread 0.
-__device__ __noinline__ CT block_list(const DrawItem& a, const PixelRef& r, uint32_t n, PixelList& L, uint64_t* out_key,
-                                      float4* out_rgba, bool& bad)
+template <bool kKept>
+__device__ __noinline__ CT block_list(const DrawItem& a, const DrawnCorners& dc, const PixelRef& r, uint32_t n, PixelList& L,
+                                      uint64_t* out_key, float4* out_rgba, bool& bad)
 {
     if (threadIdx.x < 32)
         list_walk(a, r, (int)threadIdx.x, n, [&](uint32_t i, uint32_t f2t) { L.k[i] = f2t; });
@@ -299,7 +311,7 @@ __device__ __noinline__ CT block_list(const DrawItem& a, const PixelRef& r, uint
         const uint32_t i = b + threadIdx.x;
         if (i < n) {
             const uint64_t key = L.k[i];
-            const float4 f = fragment_colour(a, r, (uint32_t)key, bad);
+            const float4 f = fragment_colour<kKept>(a, dc, r, (uint32_t)key, bad);
             L.c[threadIdx.x] = f;
             if (out_key) {
                 out_key[i] = key;
@@ -331,8 +343,8 @@ __global__ void __launch_bounds__(kTilePix, 3) k_draw_tail(const __grid_constant
     for (uint64_t i = blockIdx.x; i < n_redo; i += gridDim.x) {
         const uint32_t q = a.redo[i];
         const PixelRef r = pixel_ref(q, a.tiles_x);
-        const CT c = block_list(a, r, min(a.cnt[q], (uint32_t)HEXFC_MAX_LIST), *reinterpret_cast<PixelList*>(smem),
-                                nullptr, nullptr, bad);
+        const CT c = block_list<false>(a, DrawnCorners{}, r, min(a.cnt[q], (uint32_t)HEXFC_MAX_LIST),
+                                       *reinterpret_cast<PixelList*>(smem), nullptr, nullptr, bad);
         int64_t o;
         if (threadIdx.x == 0 && out_index(a.win, r.px0 + r.lx, r.py0 + r.ly, o)) a.out[o] = finish(c, a.sp);
         __syncthreads();   // the list is the next pixel's
@@ -666,7 +678,7 @@ __device__ __forceinline__ int64_t pixel_index(int x, int y, int tiles_x)
     return ((int64_t)(y / kTileH) * tiles_x + x / kTileW) * kTilePix + (y % kTileH) * kTileW + (x % kTileW);
 }
 
-__global__ void __launch_bounds__(kTilePix) k_debug_lists(const __grid_constant__ DrawItem a,
+__global__ void __launch_bounds__(kTilePix) k_debug_lists(const __grid_constant__ DrawItem a, const DrawnCorners dc,
                                                           const int32_t* __restrict__ px,
                                                           const int32_t* __restrict__ py,
                                                           const uint64_t* __restrict__ dst_off,
@@ -679,8 +691,8 @@ __global__ void __launch_bounds__(kTilePix) k_debug_lists(const __grid_constant_
     const uint32_t n = a.cnt[q];
     if (n == 0 || n > (uint32_t)HEXFC_MAX_LIST) return;
     bool bad = false;
-    (void)block_list(a, pixel_ref(q, a.tiles_x), n, *reinterpret_cast<PixelList*>(smem), out_key + dst_off[i],
-                     out_rgba + dst_off[i], bad);
+    (void)block_list<true>(a, dc, pixel_ref(q, a.tiles_x), n, *reinterpret_cast<PixelList*>(smem), out_key + dst_off[i],
+                           out_rgba + dst_off[i], bad);
     if (bad) atomicOr(a.err, kErrDepth);
 }
 
@@ -781,7 +793,7 @@ cudaError_t launch_silhouette(const DrawItem& a, int fx0, int fy0, int frame_w, 
                           (int64_t)threshold);
 }
 
-cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const int32_t* d_py, int64_t n,
+cudaError_t launch_debug_gather(const DrawItem& a, const DrawnCorners& dc, const int32_t* d_px, const int32_t* d_py, int64_t n,
                                 const uint64_t* d_dst_off, uint64_t* d_keys, float4* d_rgba, uint32_t* d_counts,
                                 cudaStream_t s)
 {
@@ -790,7 +802,7 @@ cudaError_t launch_debug_gather(const DrawItem& a, const int32_t* d_px, const in
         k_debug_counts<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a.cnt, d_px, d_py, n, a.tiles_x, d_counts);
         return cudaGetLastError();
     }
-    k_debug_lists<<<(unsigned)n, kTilePix, sizeof(PixelList), s>>>(a, d_px, d_py, d_dst_off, d_keys, d_rgba);
+    k_debug_lists<<<(unsigned)n, kTilePix, sizeof(PixelList), s>>>(a, dc, d_px, d_py, d_dst_off, d_keys, d_rgba);
     return cudaGetLastError();
 }
 

@@ -92,14 +92,6 @@ __global__ void __launch_bounds__(128) k_cell_quality(const float* __restrict__ 
     out[c] = v;
 }
 
-// float <-> int order-preserving map, so that atomicMax on int is a float max
-__device__ __forceinline__ int32_t f2key(float f)
-{
-    int32_t i = __float_as_int(f);
-    return i >= 0 ? i : (i ^ 0x7FFFFFFF);
-}
-__device__ __forceinline__ float key2f(int32_t k) { return __int_as_float(k >= 0 ? k : (k ^ 0x7FFFFFFF)); }
-
 // Importance of every vertex and edge, the largest of its cells': keys cleared,
 // scattered with an atomic each (bound by them: 20 a cell), and written where the
 // frames read them. Three launches, each behind the one before, instead of
@@ -129,7 +121,7 @@ __global__ void __launch_bounds__(256) k_importance_scatter(const int32_t* __res
     const int4* p = reinterpret_cast<const int4*>(cells) + 2 * c;
     const int4* q = reinterpret_cast<const int4*>(cell_edges) + 3 * c;
     const int4 a[2] = {p[0], p[1]}, b[3] = {q[0], q[1], q[2]};
-    const int32_t k = f2key(v);
+    const int32_t k = importance_key(v);
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         atomicMax(vkey + a[j].x, k);
@@ -145,9 +137,6 @@ __global__ void __launch_bounds__(256) k_importance_scatter(const int32_t* __res
         atomicMax(ekey + b[j].w, k);
     }
 }
-
-// A key's importance; an unreferenced vertex or edge has 0.
-__device__ __forceinline__ float importance_of(int32_t k) { return k == INT32_MIN ? 0.f : key2f(k); }
 
 // Thread per face: the importances of its corners in its static record, and with
 // `positions` (a new record) their world positions; then a thread per edge.
@@ -204,7 +193,7 @@ cudaError_t launch_importance(const DevMesh& m, bool positions, bool chained, cu
                            m.n_cells, m.vkey, m.ekey);
     if (e == cudaSuccess)
         e = launch_chained(k_face_static, grid_for(m.n_faces + m.n_edges, 256), 256, 0, s, chained, m.fverts, m.vkey, m.verts,
-                           m.n_faces, positions, m.fstat.get(), m.ekey, m.n_edges, m.eattr);
+                           m.n_faces, positions, m.fstat, m.ekey, m.n_edges, m.eattr);
     return e;
 }
 

@@ -45,10 +45,12 @@ inline int spread_for(int64_t n)
 
 // ------------------------------------------------------------------ vertex stage
 
-// Thread per vertex: window position on 1/256 pixel, 24-bit depth, eye depth.
+// Thread per vertex: window position on 1/256 pixel, 24-bit depth, eye depth, and
+// the importance that the frame is drawn with.
 // It also clears the frame's counters (tile_cnt, tile_big, tile_skip, tile_cur, and the
 // device scalars but the error word), which every frame starts from zero.
-__global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ verts, int64_t n,
+__global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ verts,
+                                                      const int32_t* __restrict__ vkey, int64_t n,
                                                       const __grid_constant__ CamParams cam,
                                                       const __grid_constant__ CamPairs pairs,
                                                       int4* __restrict__ vproj, float* __restrict__ ved,
@@ -71,7 +73,7 @@ __global__ void __launch_bounds__(256) k_vertex_setup(const float* __restrict__ 
     const float x = verts[3 * v], y = verts[3 * v + 1], z = verts[3 * v + 2];
     ProjVertex o;
     if (!pairs.usable || !vertex_pairs(x, y, z, pairs, cam, o)) vertex_double(x, y, z, cam, o);
-    vproj[v] = make_int4(o.x, o.y, o.z, o.valid);
+    vproj[v] = make_int4(o.x, o.y, o.z | (o.valid ? kVertexValid : 0), vkey[v]);
     ved[v] = o.depth;
 }
 
@@ -211,7 +213,7 @@ __global__ void __launch_bounds__(256, 5) k_face_setup(const int4* __restrict__ 
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int4 p = vproj[id[k]];
-        X[k] = p.x; Y[k] = p.y; Z[k] = (uint32_t)p.z & kZ24; ok[k] = in && p.w != 0;
+        X[k] = p.x; Y[k] = p.y; Z[k] = (uint32_t)p.z & kZ24; ok[k] = in && (p.z & kVertexValid) != 0;
         E[k] = ved[id[k]];
     }
     uint32_t edges = 0, flags = fbound[f] ? kFaceBoundary : 0u;
@@ -881,8 +883,8 @@ cudaError_t prepare_raster_kernels()
 cudaError_t launch_vertex_setup(const DevMesh& m, const CamParams& cam, FrameBufs& fb, int64_t n_tiles, cudaStream_t s)
 {
     const unsigned tiles = std::min(grid_for(n_tiles, 256), 1216u);   // (two blocks' worth of clears an SM at most)
-    return launch_chained(k_vertex_setup, std::max(grid_for(m.n_verts, 256), tiles), 256, 0, s, false, m.verts, m.n_verts,
-                          cam, cam_pairs(cam), fb.vproj, fb.ved, fb.tile_cnt, fb.tile_big, fb.tile_skip, fb.tile_cur,
+    return launch_chained(k_vertex_setup, std::max(grid_for(m.n_verts, 256), tiles), 256, 0, s, false, m.verts, m.vkey,
+                          m.n_verts, cam, cam_pairs(cam), fb.vproj, fb.ved, fb.tile_cnt, fb.tile_big, fb.tile_skip, fb.tile_cur,
                           n_tiles, fb.scal);
 }
 
