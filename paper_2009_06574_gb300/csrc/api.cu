@@ -877,7 +877,9 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
     collect(ctx);
     if (ctx->pend.active) {   // the previous frame (chosen capacities) has completed: verify it
         bool redrawn = false;
-        if ((st = settle_pending(ctx, s, &redrawn)) != HEXFC_OK) return st;
+        st = settle_pending(ctx, s, &redrawn);
+        ctx->have_frame = false;   // (a frame drawn again was kept: the buffers are this one's again)
+        if (st != HEXFC_OK) return st;
         if (redrawn) {   // it was drawn again in these buffers: this frame's first passes once more
             if ((st = job_phase1(j, s)) != HEXFC_OK) return st;
             if ((st = job_wait1(ctx, j, s)) != HEXFC_OK) return st;
@@ -954,7 +956,9 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     collect(ctx);
     if (ctx->pend.active) {   // the previous frame has completed: verify it
         bool redrawn = false;
-        if ((st = settle_pending(ctx, s, &redrawn)) != HEXFC_OK) return st;
+        st = settle_pending(ctx, s, &redrawn);
+        ctx->have_frame = false;   // (a frame drawn again was kept: the buffers are this one's again)
+        if (st != HEXFC_OK) return st;
         if (redrawn) {   // its exact redraw reused these buffers: this frame's first passes once more
             if (ctx->predicted == 1 && (ctx->counts_W != j.W || ctx->counts_H != j.H))
                 return render_frame(ctx, m, out, stats, s);

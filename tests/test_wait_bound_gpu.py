@@ -18,13 +18,13 @@ ROOT = os.path.dirname(TESTS)
 LAYERS = 8000
 
 
-def column():
-    """2 x 2 x LAYERS cells along the view direction, wider than the frame: every
+def column(layers=LAYERS):
+    """2 x 2 x layers cells along the view direction, wider than the frame: every
     pixel's list has a fragment of every layer."""
-    x, z = np.array([-2.0, 0.0, 2.0]), np.linspace(-1.0, 1.0, LAYERS + 1)
+    x, z = np.array([-2.0, 0.0, 2.0]), np.linspace(-1.0, 1.0, layers + 1)
     zz, yy, xx = np.meshgrid(z, x, x, indexing="ij")
     verts = np.stack([xx.ravel(), yy.ravel(), zz.ravel()], axis=1).astype(np.float32)
-    k, j, i = np.meshgrid(np.arange(LAYERS), np.arange(2), np.arange(2), indexing="ij")
+    k, j, i = np.meshgrid(np.arange(layers), np.arange(2), np.arange(2), indexing="ij")
     at = lambda a, b, c: ((i + a) + 3 * ((j + b) + 3 * (k + c))).ravel()
     corners = [(0, 0, 0), (1, 0, 0), (1, 1, 0), (0, 1, 0), (0, 0, 1), (1, 0, 1), (1, 1, 1), (0, 1, 1)]
     return verts, np.stack([at(*c) for c in corners], axis=1).astype(np.int32)
