@@ -366,6 +366,9 @@ enum {
     HEXFC_OPT_FRAG_BUDGET = 7,       /* bytes: the cap of hexfc_create's frag_budget_bytes, per frame
                                         (0: none); a serving loop sets it to what the other frames in
                                         flight leave */
+    HEXFC_OPT_DEBUG_FAIL_ALLOC = 9,  /* test hook, n > 0: the n-th memory allocation that the library makes
+                                        on the calling host thread from here on fails as if there were no
+                                        memory (0: none does) */
     HEXFC_OPT_BATCH_LAUNCH = 8       /* hexfc_render_batch: 0 (default): every item its own launches,
                                         the items as parallel branches of each phase's graph; 1: the
                                         coverage count and the drawing pass of all items each one kernel

@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <initializer_list>
 #include <memory>
 #include <new>
 #include <vector>
@@ -96,6 +97,33 @@ struct hexfc_ctx {
 
 namespace {
 
+// Test hook (HEXFC_OPT_DEBUG_FAIL_ALLOC): allocations from here to the one that
+// fails on this host thread, 0: none does.
+thread_local int64_t t_fail_alloc = 0;
+bool alloc_refused() { return t_fail_alloc > 0 && --t_fail_alloc == 0; }
+
+}  // namespace
+
+cudaError_t hexfc::device_alloc(void** p, size_t bytes)
+{
+    *p = nullptr;
+    if (alloc_refused()) return cudaErrorMemoryAllocation;
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) *p = nullptr;
+    return e;
+}
+
+namespace {
+
+cudaError_t pinned_alloc(void** p, size_t bytes)
+{
+    *p = nullptr;
+    if (alloc_refused()) return cudaErrorMemoryAllocation;
+    const cudaError_t e = cudaMallocHost(p, bytes);
+    if (e != cudaSuccess) *p = nullptr;
+    return e;
+}
+
 // The CUDA error of the last failed runtime call or launch made by the library
 // on this host thread (hexfc_last_cuda_error).
 thread_local int32_t t_last_cuda = 0;
@@ -144,18 +172,17 @@ struct DeviceGuard {
     }
 };
 
+hexfc_status alloc_status(cudaError_t e)
+{
+    if (e == cudaSuccess) return HEXFC_OK;
+    note_cuda(e);
+    return e == cudaErrorMemoryAllocation ? HEXFC_ERR_OOM : HEXFC_ERR_CUDA;
+}
+
 template <typename T>
 hexfc_status dalloc(T** p, size_t n)
 {
-    *p = nullptr;
-    if (n == 0) n = 1;
-    cudaError_t e = cudaMalloc((void**)p, n * sizeof(T));
-    if (e != cudaSuccess) {
-        note_cuda(e);
-        *p = nullptr;
-        return e == cudaErrorMemoryAllocation ? HEXFC_ERR_OOM : HEXFC_ERR_CUDA;
-    }
-    return HEXFC_OK;
+    return alloc_status(device_alloc((void**)p, (n == 0 ? 1 : n) * sizeof(T)));
 }
 
 template <typename T>
@@ -165,16 +192,51 @@ void dfree(T*& p)
     p = nullptr;
 }
 
-// Grow a device array to hold at least n elements (contents are not kept).
+// Device arrays that belong together: each has `per` elements for every one of
+// the group's. They are all there or none is: a group of which some allocation
+// failed is given back whole, so that a pointer that is there says that all are.
+struct Part {
+    void** p;
+    size_t bytes;
+};
+template <typename T>
+Part part(T** p, size_t per = 1)
+{
+    return Part{(void**)p, per * sizeof(T)};
+}
+
+void free_all(std::initializer_list<Part> parts)
+{
+    for (const Part& a : parts) dfree(*a.p);
+}
+
+hexfc_status alloc_all(int64_t n, std::initializer_list<Part> parts)
+{
+    free_all(parts);
+    for (const Part& a : parts)
+        if (const hexfc_status st = alloc_status(device_alloc(a.p, (size_t)(n > 0 ? n : 1) * a.bytes)); st != HEXFC_OK) {
+            free_all(parts);
+            return st;
+        }
+    return HEXFC_OK;
+}
+
+// Grow a group to hold at least n (contents are not kept); *cap: what it holds.
+hexfc_status ensure_all(int64_t* cap, int64_t n, std::initializer_list<Part> parts)
+{
+    if (*parts.begin()->p && *cap >= n) return HEXFC_OK;
+    const int64_t want = n + n / 4 + 1024;
+    *cap = 0;
+    const hexfc_status st = alloc_all(want, parts);
+    if (st == HEXFC_OK) *cap = want;
+    return st;
+}
+
+// The same for one array.
 template <typename T>
 hexfc_status ensure(T** p, int64_t* cap, int64_t n)
 {
-    if (*p && *cap >= n) return HEXFC_OK;
-    dfree(*p);
-    int64_t want = n + n / 4 + 1024;
-    hexfc_status st = dalloc(p, (size_t)want);
-    *cap = st == HEXFC_OK ? want : 0;
-    return st;
+    return ensure_all(cap, n, {part(p)});
 }
 
 void free_mesh(DevMesh* m)
@@ -495,65 +557,29 @@ hexfc_status job_alloc(FrameJob& j)
     FrameBufs& fb = *j.fb;
     const DevMesh* m = j.m;
     hexfc_status st;
-    if (!fb.vproj || fb.v_cap < m->n_verts) {
-        int64_t c1 = 0;
-        dfree(fb.ved);
-        if ((st = ensure(&fb.vproj, &fb.v_cap, m->n_verts)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.ved, &c1, fb.v_cap)) != HEXFC_OK) return st;
-    }
-    if (!fb.fframe || fb.f_cap < m->n_faces) {
-        int64_t c1 = 0;
-        dfree(fb.tzsum);
-        if ((st = ensure(&fb.fframe, &fb.f_cap, m->n_faces)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.tzsum, &c1, 2 * fb.f_cap)) != HEXFC_OK) return st;
-        free_slots(fb);
-    }
-    if (!fb.tile_cnt || fb.t_cap < j.n_tiles + 1) {
-        int64_t c1 = 0, c2 = 0, c3 = 0, c4 = 0, c5 = 0, c6 = 0, c7 = 0;
-        dfree(fb.tile_off); dfree(fb.tile_cur); dfree(fb.tile_order); dfree(fb.tile_frag); dfree(fb.tile_big);
-        dfree(fb.tile_skip);
-        dfree(fb.cap_x);
-        if ((st = ensure(&fb.tile_cnt, &fb.t_cap, j.n_tiles + 1)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.tile_off, &c1, fb.t_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.tile_cur, &c2, fb.t_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.tile_order, &c3, fb.t_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.tile_frag, &c4, fb.t_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.tile_big, &c5, fb.t_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.cap_x, &c6, 4 * fb.t_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.tile_skip, &c7, fb.t_cap)) != HEXFC_OK) return st;
-    }
-    if (!fb.cnt || fb.p_cap < j.n_pix + 1) {
-        int64_t c1 = 0, c2 = 0;
-        dfree(fb.zsil); dfree(fb.redo);
-        if ((st = ensure(&fb.cnt, &fb.p_cap, j.n_pix + 1)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.zsil, &c1, fb.p_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.redo, &c2, fb.p_cap)) != HEXFC_OK) return st;
-    }
+    if ((st = ensure_all(&fb.v_cap, m->n_verts, {part(&fb.vproj), part(&fb.ved)})) != HEXFC_OK) return st;
+    if ((st = ensure_all(&fb.f_cap, m->n_faces, {part(&fb.fframe), part(&fb.tzsum, 2)})) != HEXFC_OK) return st;
+    if (fb.slot_cap != fb.f_cap) free_slots(fb);
+    if ((st = ensure_all(&fb.t_cap, j.n_tiles + 1,
+                         {part(&fb.tile_cnt), part(&fb.tile_off), part(&fb.tile_cur), part(&fb.tile_order),
+                          part(&fb.tile_frag), part(&fb.tile_big), part(&fb.cap_x, 4), part(&fb.tile_skip)})) != HEXFC_OK)
+        return st;
+    if ((st = ensure_all(&fb.p_cap, j.n_pix + 1, {part(&fb.cnt), part(&fb.zsil), part(&fb.redo)})) != HEXFC_OK) return st;
     const int64_t nparts = scan_partials_needed(j.n_tiles) + 1;
-    if (!fb.part || fb.part_cap < 2 * nparts) {
-        int64_t c1 = 0;
-        dfree(fb.part_max);
-        if ((st = ensure(&fb.part, &fb.part_cap, 2 * nparts)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.part_max, &c1, fb.part_cap)) != HEXFC_OK) return st;
-    }
-    // places of the binning and the faces' extras: faster, not needed (72 bytes a
+    if ((st = ensure_all(&fb.part_cap, 2 * nparts, {part(&fb.part), part(&fb.part_max)})) != HEXFC_OK) return st;
+    // places of the binning and the faces' extras: faster, not needed (kSlotBytes a
     // face): only in what a budget leaves
     const bool room = !j.budget || (j.may_drop_slots && fb.slots_refused != j.budget &&
                                     frame_bytes(fb, 0) + (uint64_t)fb.f_cap * kSlotBytes <= j.budget);
     if (fb.slots && !room) free_slots(fb);
-    if (!fb.slots && room) {
-        int64_t c1 = 0, c2 = 0, c3 = 0;
-        if (ensure(&fb.trange, &c1, 2 * fb.f_cap) == HEXFC_OK && ensure(&fb.slots, &c2, 2 * fb.f_cap) == HEXFC_OK &&
-            ensure(&fb.fextra, &c3, fb.f_cap) == HEXFC_OK)
-            fb.slot_cap = fb.f_cap;
-        else
-            free_slots(fb);
-    }
+    if (!fb.slots && room &&
+        alloc_all(fb.f_cap, {part(&fb.trange, 2), part(&fb.slots, 2), part(&fb.fextra)}) == HEXFC_OK)
+        fb.slot_cap = fb.f_cap;
     if (!fb.scal) {
         if ((st = dalloc(&fb.scal, kScalAll)) != HEXFC_OK) return st;
-        CK(cudaMallocHost((void**)&fb.h_scal, kScal * sizeof(uint64_t)));
         fb.scal_fresh = true;   // contents undefined: phase 1 clears all of it
     }
+    if (!fb.h_scal) CK(pinned_alloc((void**)&fb.h_scal, kScal * sizeof(uint64_t)));   // (hexfc_trim keeps it)
     return HEXFC_OK;
 }
 
@@ -605,12 +631,7 @@ hexfc_status job_read1(FrameJob& j)
     hexfc_status st;
     j.n_bins = fb.bins_seen = fb.h_scal[8];   // padded to whole chunks per tile
     fb.bin_limit = ~0ull;
-    if (!fb.bins || fb.bin_cap < (int64_t)j.n_bins) {
-        int64_t c1 = 0;
-        dfree(fb.bins_tmp);
-        if ((st = ensure(&fb.bins, &fb.bin_cap, (int64_t)j.n_bins)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.bins_tmp, &c1, fb.bin_cap)) != HEXFC_OK) return st;
-    }
+    if ((st = ensure_all(&fb.bin_cap, (int64_t)j.n_bins, {part(&fb.bins), part(&fb.bins_tmp)})) != HEXFC_OK) return st;
     if ((st = ensure(&fb.masks, &fb.mask_cap, (int64_t)j.n_bins * (kTilePix / kChunk))) != HEXFC_OK) return st;
     if ((st = ensure(&fb.zsuf, &fb.zsuf_cap, (int64_t)(j.n_bins / kChunk))) != HEXFC_OK) return st;
     return HEXFC_OK;
@@ -936,13 +957,9 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     hexfc_status st;
     ctx->have_frame = false;
     if ((st = job_alloc(j)) != HEXFC_OK) return st;
-    if (!fb.tile_cap || fb.cap_cap < fb.t_cap) {   // capacity arrays follow the tile arrays
-        int64_t c1 = 0;
-        dfree(fb.cap_off);
-        if ((st = ensure(&fb.tile_cap, &fb.cap_cap, fb.t_cap)) != HEXFC_OK) return st;
-        if ((st = ensure(&fb.cap_off, &c1, fb.cap_cap)) != HEXFC_OK) return st;
-    }
-    if (!ctx->h_pend) CK(cudaMallocHost((void**)&ctx->h_pend, kScal * sizeof(uint64_t)));
+    // capacity arrays follow the tile arrays
+    if ((st = ensure_all(&fb.cap_cap, fb.t_cap, {part(&fb.tile_cap), part(&fb.cap_off)})) != HEXFC_OK) return st;
+    if (!ctx->h_pend) CK(pinned_alloc((void**)&ctx->h_pend, kScal * sizeof(uint64_t)));
     if (ctx->timing && !ctx->ev[0][0])
         for (auto& set : ctx->ev)
             for (auto& e : set) CK(cudaEventCreate(&e));
@@ -1972,6 +1989,10 @@ hexfc_status hexfc_set_option(hexfc_ctx* ctx, int32_t option, int64_t value)
     case HEXFC_OPT_BATCH_LAUNCH:
         if (value != 0 && value != 1) return HEXFC_ERR_ARG;
         ctx->batch_launch = value != 0;
+        return HEXFC_OK;
+    case HEXFC_OPT_DEBUG_FAIL_ALLOC:
+        if (value < 0) return HEXFC_ERR_ARG;
+        t_fail_alloc = value;
         return HEXFC_OK;
     case HEXFC_OPT_DEBUG_ERROR_BITS:
         if (value < 0 || value > 7) return HEXFC_ERR_ARG;

@@ -304,6 +304,9 @@ __device__ __forceinline__ int batch_item(const uint32_t* begin, int n, uint32_t
 static_assert(sizeof(DrawBatch) < 30000 && sizeof(CountBatch) < 30000,
               "a batch's parameters fit a kernel's parameter space");
 
+// cudaMalloc of the library (api.cu; HEXFC_OPT_DEBUG_FAIL_ALLOC); *p is null if it fails.
+cudaError_t device_alloc(void** p, size_t bytes);
+
 // ---- launches (each returns cudaGetLastError()) -----------------------------------------
 cudaError_t launch_cell_quality(const DevMesh& m, int metric, float* out, cudaStream_t s);
 // Vertex and edge importance (max over cells) and the faces' static records;

@@ -231,7 +231,7 @@ cudaError_t MeshScratch::number(const int32_t* cells, int64_t n_cells, int64_t n
     const size_t o_foff = room((V + 1) * 8), o_eoff = room((V + 1) * 8), o_frec = room(F * 16), o_fsort = room(F * 16),
                  o_erec = room(E * 8), o_esort = room(E * 8), o_fnum = room(F * 4), o_enum = room(E * 4),
                  o_part = room(2 * (size_t)parts * 8), o_max = room(2 * (size_t)parts * 4);
-    cudaError_t e = cudaMalloc(&block, used);
+    cudaError_t e = device_alloc(&block, used);
     if (e != cudaSuccess) return e;
     auto at = [&](size_t o) { return static_cast<unsigned char*>(block) + o; };
     scal = (uint64_t*)at(o_scal);

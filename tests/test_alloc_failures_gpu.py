@@ -1,0 +1,117 @@
+"""A frame whose memory cannot be had is refused, and the context goes on: each
+allocation of a frame made to fail in turn (HEXFC_OPT_DEBUG_FAIL_ALLOC), frames
+small and large after it are the same bit for bit as without; through every call
+that draws."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2009_06574_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+STYLE = synth.Style(w_base=1.5, lod=2)
+LENS = synth.lissajous_lens(5, 120)
+SMALL = (synth.hex_grid(5, jitter=0.1, seed=2), synth.orbit_view(5, 120, 64, 48))
+LARGE = (synth.hex_grid(12, jitter=0.1, seed=3), synth.orbit_view(5, 120, 656, 500))   # (more tiles than the small frame leaves room for)
+
+
+@pytest.fixture(scope="module")
+def hx():
+    from paper_2009_06574_gb300 import hexfc
+    hexfc.load()
+    return hexfc
+
+
+class Context:
+    def __init__(self, hx, kind):
+        self.hx, self.kind = hx, kind
+        self.r = hx.Renderer(0)
+        self.ids = [self.r.upload_mesh(m.verts, m.cells, m.cell_scalar, m.edge_level) for m, _ in (SMALL, LARGE)]
+        self.r.set_lens(LENS)
+        self.r.set_style(STYLE)
+        if kind == "predicted":
+            self.r.set_option(hx.HEXFC_OPT_PREDICTED_CAPACITY, 3)   # (capacities for any size after the first frame)
+
+    def draw(self, which):
+        """Status and image (None if refused) of the small (0) or large (1) frame."""
+        view = (SMALL, LARGE)[which][1]
+        out = torch.full((view.height, view.width, 4), -1.0, device="cuda")
+        if self.kind == "batch":
+            st = self.r.render_batch([(self.ids[which], view, LENS, STYLE, out)] * 2, check=False)[0]
+        else:
+            self.r.set_view(view)
+            if self.kind == "host":
+                img = np.empty((view.height, view.width, 4), np.float32)
+                st = self.r.render_host(self.ids[which], img, check=False)
+                return st, img if st == 0 else None
+            st = self.r.render(self.ids[which], out, check=False)
+            if st == 0:
+                self.r.finish()
+        torch.cuda.synchronize()
+        return st, out.cpu().numpy() if st == 0 else None
+
+    def fail(self, k):
+        self.r.set_option(self.hx.HEXFC_OPT_DEBUG_FAIL_ALLOC, k)
+
+
+@pytest.fixture(scope="module")
+def images(hx):
+    c = Context(hx, "render")
+    imgs = [c.draw(w)[1] for w in (0, 1)]
+    c.r.close()
+    return imgs
+
+
+@pytest.mark.parametrize("kind", ["render", "host", "batch", "predicted"])
+@pytest.mark.parametrize("first", [True, False])
+def test_each_allocation_of_a_frame(hx, images, kind, first):
+    refused = 0
+    for k in range(1, 60):
+        c = Context(hx, kind)
+        if not first:   # (buffers of the small frame are there)
+            st, img = c.draw(0)
+            assert st == 0
+        c.fail(k)
+        st, _ = c.draw(1)
+        c.fail(0)
+        if st != 0:
+            assert st in (hx.HEXFC_ERR_OOM, hx.HEXFC_ERR_CUDA)
+            refused += 1
+        for which in (0, 1, 0):
+            st, img = c.draw(which)
+            assert st == 0
+            np.testing.assert_array_equal(img, images[which])
+        c.r.close()
+    assert refused >= 15
+
+
+def _allocations(hx, draw):
+    """The most that a frame's k-th allocation can be for the frame to be refused."""
+    most = 0
+    for k in range(1, 50):
+        if draw(k) != 0:
+            most = k
+    return most
+
+
+def test_trim_keeps_the_pinned_copy(hx):
+    def fresh(k):
+        c = Context(hx, "render")
+        c.fail(k)
+        st, _ = c.draw(1)
+        c.fail(0)
+        c.r.close()
+        return st
+
+    def trimmed(k):
+        c = Context(hx, "render")
+        c.draw(1)
+        c.r.trim()
+        c.fail(k)
+        st, _ = c.draw(1)
+        c.fail(0)
+        c.r.close()
+        return st
+
+    assert _allocations(hx, trimmed) == _allocations(hx, fresh) - 1
