@@ -1123,22 +1123,12 @@ hexfc_status finish_pending(hexfc_ctx* ctx)
     return settle_pending(ctx, ctx->pend.stream, &redrawn);
 }
 
-// Capture `body(i, stream_i)` for the listed items, each on its own stream
-// forked from the context's origin stream and joined back, as one graph;
-// reuse the phase's executable graph when only parameters changed.
 // Weights, moments and gradient of the capacity network (once).
 hexfc_status cap_alloc(CapNet& n)
 {
-    hexfc_status st = HEXFC_OK;
-    if (!n.w) {
-        if ((st = dalloc(&n.w, kCapParams)) != HEXFC_OK) return st;
-        if ((st = dalloc(&n.w16, kCapParams)) != HEXFC_OK) return st;
-        if ((st = dalloc(&n.m, kCapParams)) != HEXFC_OK) return st;
-        if ((st = dalloc(&n.v, kCapParams)) != HEXFC_OK) return st;
-        if ((st = dalloc(&n.grad, kCapParams + 1)) != HEXFC_OK) return st;
-        if ((st = dalloc(&n.part, (size_t)cap_partials())) != HEXFC_OK) return st;
-    }
-    return st;
+    if (n.w) return HEXFC_OK;
+    return alloc_all(1, {part(&n.w, kCapParams), part(&n.w16, kCapParams), part(&n.m, kCapParams), part(&n.v, kCapParams),
+                         part(&n.grad, kCapParams + 1), part(&n.part, (size_t)cap_partials())});
 }
 
 // Features and counts of n tiles handed in by the caller.

@@ -115,3 +115,35 @@ def test_trim_keeps_the_pinned_copy(hx):
         return st
 
     assert _allocations(hx, trimmed) == _allocations(hx, fresh) - 1
+
+
+def test_each_allocation_of_the_network(hx):
+    """Weights whose memory cannot be had are refused; set again, they train as ever."""
+    def train(k):
+        c = Context(hx, "render")
+        c.draw(0)
+        c.fail(k)
+        try:
+            c.r.capacity_reset(3)
+            refused = False
+        except hx.HexfcError as e:
+            assert e.status == hx.HEXFC_ERR_OOM
+            refused = True
+        c.fail(0)
+        if refused:
+            with pytest.raises(hx.HexfcError) as e:
+                c.r.capacity_train(1)
+            assert e.value.status == hx.HEXFC_ERR_STATE
+            c.r.capacity_reset(3)
+        c.r.capacity_train(2)
+        w = c.r.capacity_get_weights()
+        c.r.close()
+        return refused, w
+
+    _, want = train(0)
+    refused = 0
+    for k in range(1, 10):
+        r, w = train(k)
+        refused += r
+        np.testing.assert_array_equal(w, want)
+    assert refused == 6
