@@ -56,14 +56,14 @@ struct hexfc_ctx {
     hexfc_frame_stats completed{};     // final statistics of the last verified frame
     hexfc_frame_stats history[16]{};   // final statistics of recent frames, at frame % 16
     uint64_t frame_seq = 0;            // frames drawn by this context
-    // exact tile counts of the last frame (fb.tile_frag) are valid for this size
+    // size and fragments of the last counted frame; with feat_tiles, its exact tile counts are in fb.tile_frag
     int counts_W = 0, counts_H = 0;
     uint64_t counts_total = 0;
     // tile-capacity network and the camera of the previous frame (its motion is a feature)
     CapNet cap;
     bool have_prev_cam = false;
     double prev_eye[3] = {0, 0, 0}, prev_F[3] = {0, 0, 1};
-    int64_t feat_tiles = 0;   // tiles whose features and exact counts the last frame left for training
+    int64_t feat_tiles = 0;   // tiles whose features and exact counts that frame left, 0: they are gone
     // last render: what its fragment lists can be rebuilt from (hexfc_debug_pixels)
     bool have_frame = false;
     DrawItem last_draw{};
@@ -525,7 +525,7 @@ FrameJob make_job(hexfc_ctx* ctx, FrameBufs* fb, DevMesh* m, float* out)
     j.budget = ctx->budget;
     j.out = out;
     feature_constants(ctx, ctx->view, ctx->lens, ctx->cam, ctx->zref, j);
-    j.prev_counts = fb == &ctx->fb && ctx->counts_W == j.W && ctx->counts_H == j.H;
+    j.prev_counts = fb == &ctx->fb && ctx->feat_tiles != 0 && ctx->counts_W == j.W && ctx->counts_H == j.H;
     return j;
 }
 
@@ -843,8 +843,31 @@ hexfc_status inject_error_bits(hexfc_ctx* ctx, uint64_t* scal, cudaStream_t s)
     return HEXFC_OK;
 }
 
-// What the context keeps of the frame just drawn: its lists' inputs, the exact
-// tile counts that k_count left in fb.tile_frag, its features and camera.
+// The tile counts and features in fb.tile_frag and fb.cap_x (the next frame's
+// capacities and features, training) are frame j's: its count has run, whether it
+// is drawn or refused.
+void keep_counts(hexfc_ctx* ctx, const FrameJob& j)
+{
+    ctx->counts_W = j.W;
+    ctx->counts_H = j.H;
+    ctx->feat_tiles = j.n_tiles;
+}
+// There are none: their arrays are gone, or new. (The last frame's size and total still say what to expect.)
+void forget_counts(hexfc_ctx* ctx) { ctx->feat_tiles = 0; }
+
+// job_alloc of a frame in the context's own buffers.
+hexfc_status own_alloc(hexfc_ctx* ctx, FrameJob& j)
+{
+    const int64_t had = ctx->fb.t_cap;
+    const hexfc_status st = job_alloc(j);
+    if (ctx->fb.t_cap != had) {   // (other tile arrays: larger, or none)
+        forget_counts(ctx);
+        j.prev_counts = false;
+    }
+    return st;
+}
+
+// What the context keeps of the frame just drawn: its lists' inputs and camera.
 void keep_frame(hexfc_ctx* ctx, const FrameJob& j)
 {
     ctx->have_frame = true;
@@ -853,9 +876,6 @@ void keep_frame(hexfc_ctx* ctx, const FrameJob& j)
         if (m.get() == j.m) ctx->last_mesh = m;
     ctx->last_corners = DrawnCorners{j.m->fverts, j.fb->vproj};
     ctx->last_win = j.win;
-    ctx->counts_W = j.W;
-    ctx->counts_H = j.H;
-    ctx->feat_tiles = j.n_tiles;
     remember_camera(ctx, j.cam);
 }
 
@@ -866,7 +886,7 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
     FrameBufs& fb = ctx->fb;
     hexfc_status st;
     ctx->have_frame = false;   // the frame buffers are this frame's from here on
-    if ((st = job_alloc(j)) != HEXFC_OK) return st;
+    if ((st = own_alloc(ctx, j)) != HEXFC_OK) return st;
     if (ctx->timing && !ctx->ev[0][0])
         for (auto& set : ctx->ev)
             for (auto& e : set) CK(cudaEventCreate(&e));
@@ -917,6 +937,8 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
         if ((st = job_phase3(j, s)) != HEXFC_OK) return st;
         CK(cudaEventSynchronize(ctx->ev_p2));   // the totals, while the frame is drawn
     }
+    keep_counts(ctx, j);
+    ctx->counts_total = fb.h_scal[0];
     st = job_read2(j, s);
     j.fs.frame = ++ctx->frame_seq;
     ctx->last = j.fs;
@@ -926,7 +948,6 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
     if ((st = inject_error_bits(ctx, fb_of(j), s)) != HEXFC_OK) return st;
     ctx->ev_pending[ctx->ev_cur] = ctx->timing;
     keep_frame(ctx, j);
-    ctx->counts_total = j.total;
     return HEXFC_OK;
 }
 
@@ -949,14 +970,15 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     // previous-frame capacities need the tile counts of a frame of this size; the
     // network (that feature is then 0) and the uniform capacity need only some
     // earlier frame, for the size of the pool
-    const bool same_size = ctx->counts_W == draw_w(ctx) && ctx->counts_H == draw_h(ctx);
+    const bool same_size =
+        ctx->feat_tiles != 0 && ctx->counts_W == draw_w(ctx) && ctx->counts_H == draw_h(ctx);
     if (ctx->counts_W == 0 || (ctx->predicted == 1 && !same_size))
         return render_frame(ctx, m, out, stats, s);
     FrameJob j = make_job(ctx, &ctx->fb, m, out);
     FrameBufs& fb = ctx->fb;
     hexfc_status st;
     ctx->have_frame = false;
-    if ((st = job_alloc(j)) != HEXFC_OK) return st;
+    if ((st = own_alloc(ctx, j)) != HEXFC_OK) return st;
     // capacity arrays follow the tile arrays
     if ((st = ensure_all(&fb.cap_cap, fb.t_cap, {part(&fb.tile_cap), part(&fb.cap_off)})) != HEXFC_OK) return st;
     if (!ctx->h_pend) CK(pinned_alloc((void**)&ctx->h_pend, kScal * sizeof(uint64_t)));
@@ -1048,6 +1070,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     p.fs = fs;
     ctx->last = fs;
     if (stats) *stats = fs;
+    keep_counts(ctx, j);   // (their total once it is verified)
     keep_frame(ctx, j);
     return HEXFC_OK;
 }
@@ -1694,6 +1717,7 @@ hexfc_status hexfc_trim(hexfc_ctx* ctx)
     dfree(ctx->d_out);
     ctx->d_out_cap = 0;
     ctx->have_frame = false;
+    forget_counts(ctx);
     ctx->last_mesh.reset();
     return HEXFC_OK;
 }
