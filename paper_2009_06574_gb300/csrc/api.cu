@@ -239,12 +239,16 @@ hexfc_status ensure(T** p, int64_t* cap, int64_t n)
     return ensure_all(cap, n, {part(p)});
 }
 
+void free_tables(DevMesh& m)
+{
+    dfree(m.cell_edges); dfree(m.elevel); dfree(m.fverts); dfree(m.fedges); dfree(m.fbound);
+}
+
 void free_mesh(DevMesh* m)
 {
     if (!m) return;
-    dfree(m->verts); dfree(m->cells); dfree(m->cell_edges); dfree(m->cell_imp);
-    dfree(m->vkey); dfree(m->ekey); dfree(m->eattr); dfree(m->elevel);
-    dfree(m->fverts); dfree(m->fedges); dfree(m->fbound); dfree(m->fstat);
+    dfree(m->verts); dfree(m->cells); dfree(m->cell_imp); dfree(m->vkey); dfree(m->ekey); dfree(m->eattr); dfree(m->fstat);
+    free_tables(*m);
     delete m;
 }
 
@@ -264,6 +268,45 @@ void free_slots(FrameBufs& f)
     dfree(f.slots);
     dfree(f.fextra);
     f.slot_cap = 0;
+}
+
+// The arrays of the mesh's tables, for its n_faces and n_edges: all or none.
+hexfc_status alloc_tables(DevMesh& m)
+{
+    return alloc_all(1, {part(&m.cell_edges, 12 * (size_t)m.n_cells), part(&m.elevel, (size_t)m.n_edges),
+                         part(&m.fverts, (size_t)m.n_faces), part(&m.fedges, (size_t)m.n_faces),
+                         part(&m.fbound, (size_t)m.n_faces)});
+}
+
+// The mesh's tables found on the device; *host: there was no memory for it, or the
+// mesh is not for it, and nothing of the tables is there.
+hexfc_status device_tables(DevMesh& m, const uint8_t* cell_edge_level, bool* host)
+{
+    MeshScratch scratch;   // (given back at the end)
+    uint8_t* level = nullptr;
+    uint64_t n_faces = 0, n_edges = 0;
+    *host = false;
+    hexfc_status st = alloc_status(scratch.number(m.cells, m.n_cells, m.n_verts, &n_faces, &n_edges, host));
+    if (st == HEXFC_OK && !*host && 2 * n_faces >= (1ull << 32)) return HEXFC_ERR_ARG;
+    if (st == HEXFC_OK && !*host) {
+        m.n_faces = (int64_t)n_faces;
+        m.n_edges = (int64_t)n_edges;
+        st = alloc_tables(m);
+        if (st == HEXFC_OK && cell_edge_level) {
+            const size_t n = 12 * (size_t)m.n_cells;
+            if ((st = dalloc(&level, n)) == HEXFC_OK)
+                st = alloc_status(cudaMemcpy(level, cell_edge_level, n, cudaMemcpyHostToDevice));
+        }
+        if (st == HEXFC_OK)
+            st = alloc_status(scratch.write(m.cells, m.n_cells, level, m.cell_edges, m.elevel, m.fverts, m.fedges, m.fbound, host));
+        dfree(level);
+    }
+    if (st == HEXFC_ERR_OOM) {
+        *host = true;
+        st = HEXFC_OK;
+    }
+    if (*host || st != HEXFC_OK) free_tables(m);
+    return st;
 }
 
 DevMesh* get_mesh(hexfc_ctx* ctx, int32_t id)
@@ -1364,71 +1407,45 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
     };
     A(dalloc(&m->verts, 3 * (size_t)n_verts));
     A(dalloc(&m->cells, 8 * (size_t)n_cells));
-    A(dalloc(&m->cell_edges, 12 * (size_t)n_cells));
     if (st == HEXFC_OK) {
         H2D(m->verts, verts, sizeof(float) * 3 * (size_t)n_verts);
         H2D(m->cells, cells, sizeof(int32_t) * 8 * (size_t)n_cells);
     }
     // Faces and edges: on the device, or on the host if that has no memory for it or
-    // the mesh is not for it.
-    MeshScratch tables;
-    HostTables t;
-    uint64_t n_faces = 0, n_edges = 0;
+    // the mesh is not for it. What the device sorts in takes about 500 bytes a cell,
+    // more than the mesh: it is given back before the rest of the mesh is allocated,
+    // and whatever cannot be had beside it is asked for again without it.
     bool host = false;
-    if (st == HEXFC_OK && e == cudaSuccess) {
-        e = tables.number(m->cells, n_cells, n_verts, &n_faces, &n_edges, &host);
-        if (e == cudaErrorMemoryAllocation) {
-            (void)cudaGetLastError();
-            e = cudaSuccess;
-            host = true;
-        }
-    }
-    auto on_host = [&]() -> hexfc_status {
+    if (st == HEXFC_OK && e == cudaSuccess) st = device_tables(*m, cell_edge_level, &host);
+    if (st == HEXFC_OK && e == cudaSuccess && host) {
+        HostTables t;
+        st = HEXFC_ERR_OOM;
         try {
-            if (build_host_tables(cells, n_cells, cell_edge_level, t) != 0) return HEXFC_ERR_MESH;
+            st = build_host_tables(cells, n_cells, cell_edge_level, t) == 0 ? HEXFC_OK : HEXFC_ERR_MESH;
         } catch (...) {
-            return HEXFC_ERR_OOM;
         }
-        n_faces = (uint64_t)t.n_faces;
-        n_edges = (uint64_t)t.n_edges;
-        return HEXFC_OK;
-    };
-    if (host) A(on_host());
-    if (st == HEXFC_OK && 2 * n_faces >= (1ull << 32)) st = HEXFC_ERR_ARG;
-    if (st == HEXFC_OK && e == cudaSuccess) {
-        m->n_faces = (int64_t)n_faces;
-        m->n_edges = (int64_t)n_edges;
-        A(dalloc(&m->cell_imp, (size_t)n_cells));
-        A(dalloc(&m->vkey, (size_t)n_verts));
-        A(dalloc(&m->ekey, (size_t)n_edges));
-        A(dalloc(&m->eattr, (size_t)n_edges));
-        A(dalloc(&m->elevel, (size_t)n_edges));
-        A(dalloc(&m->fverts, (size_t)n_faces));
-        A(dalloc(&m->fedges, (size_t)n_faces));
-        A(dalloc(&m->fstat, (size_t)n_faces));
-        A(dalloc(&m->fbound, (size_t)n_faces));
-    }
-    if (st == HEXFC_OK && e == cudaSuccess && !host) {
-        uint8_t* level = nullptr;
-        if (cell_edge_level) {
-            A(dalloc(&level, 12 * (size_t)n_cells));
-            if (st == HEXFC_OK) H2D(level, cell_edge_level, 12 * (size_t)n_cells);
+        if (st == HEXFC_OK && 2 * t.n_faces >= (1ll << 32)) st = HEXFC_ERR_ARG;
+        if (st == HEXFC_OK) {
+            m->n_faces = t.n_faces;
+            m->n_edges = t.n_edges;
+            st = alloc_tables(*m);
         }
-        if (st == HEXFC_OK && e == cudaSuccess)
-            e = tables.write(m->cells, n_cells, level, m->cell_edges, m->elevel, m->fverts, m->fedges, m->fbound, &host);
-        dfree(level);
-        if (host) A(on_host());   // (as many of both)
+        if (st == HEXFC_OK) {
+            H2D(m->cell_edges, t.cell_edges.data(), sizeof(int32_t) * t.cell_edges.size());
+            H2D(m->elevel, t.elevel.data(), t.elevel.size());
+            H2D(m->fverts, t.fverts.data(), sizeof(int32_t) * t.fverts.size());
+            H2D(m->fedges, t.fedges.data(), sizeof(int32_t) * t.fedges.size());
+            H2D(m->fbound, t.fbound.data(), t.fbound.size());
+        }
     }
+    A(dalloc(&m->cell_imp, (size_t)n_cells));
+    A(dalloc(&m->vkey, (size_t)n_verts));
+    A(dalloc(&m->ekey, (size_t)m->n_edges));
+    A(dalloc(&m->eattr, (size_t)m->n_edges));
+    A(dalloc(&m->fstat, (size_t)m->n_faces));
     if (st != HEXFC_OK) {
         free_mesh(m);
         return st;
-    }
-    if (host) {
-        H2D(m->cell_edges, t.cell_edges.data(), sizeof(int32_t) * t.cell_edges.size());
-        H2D(m->elevel, t.elevel.data(), t.elevel.size());
-        H2D(m->fverts, t.fverts.data(), sizeof(int32_t) * t.fverts.size());
-        H2D(m->fedges, t.fedges.data(), sizeof(int32_t) * t.fedges.size());
-        H2D(m->fbound, t.fbound.data(), t.fbound.size());
     }
     if (cell_scalar) H2D(m->cell_imp, cell_scalar, sizeof(float) * (size_t)n_cells);
     if (e == cudaSuccess && !cell_scalar) e = launch_cell_quality(*m, HEXFC_METRIC_IMPORTANCE, m->cell_imp, 0);

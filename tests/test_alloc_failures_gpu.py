@@ -147,3 +147,39 @@ def test_each_allocation_of_the_network(hx):
         refused += r
         np.testing.assert_array_equal(w, want)
     assert refused == 6
+
+
+def test_each_allocation_of_an_upload(hx):
+    """A mesh is refused only for its own memory: what is allocated beside the sorting of its faces and edges is asked for
+    again without that, and the same frame is drawn."""
+    mesh, view = synth.hex_grid(20, jitter=0.1, seed=7), synth.orbit_view(5, 120, 150, 110)
+    view_img = []
+
+    def upload(k):
+        r = hx.Renderer(0)
+        r.set_option(hx.HEXFC_OPT_DEBUG_FAIL_ALLOC, k)
+        try:
+            mid = r.upload_mesh(mesh.verts, mesh.cells, mesh.cell_scalar, mesh.edge_level)
+        except hx.HexfcError as e:
+            assert e.status == hx.HEXFC_ERR_OOM
+            mid = None
+        r.set_option(hx.HEXFC_OPT_DEBUG_FAIL_ALLOC, 0)
+        if mid is not None:
+            r.set_view(view)
+            r.set_lens(LENS)
+            r.set_style(STYLE)
+            out = torch.empty((view.height, view.width, 4), device="cuda")
+            r.render(mid, out)
+            view_img.append((out.cpu().numpy(), r.mesh_info(mid)))
+        torch.cuda.synchronize()
+        r.close()
+        return mid is not None
+
+    assert upload(0)
+    free = torch.cuda.mem_get_info()[0]
+    # vertices, cells | scratch, cell edges, levels, corners, sides, boundary, given levels | five arrays of values
+    assert [upload(k) for k in range(1, 17)] == [False] * 2 + [True] * 7 + [False] * 5 + [True] * 2
+    assert torch.cuda.mem_get_info()[0] == free
+    for img, info in view_img[1:]:
+        assert info == view_img[0][1]
+        np.testing.assert_array_equal(img, view_img[0][0])
