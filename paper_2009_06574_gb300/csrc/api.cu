@@ -865,7 +865,7 @@ hexfc_status batched(B& b, const std::vector<int>& items, Add&& add, Go&& go)
 
 inline uint64_t* fb_of(FrameJob& j) { return j.fb->scal; }
 
-hexfc_status settle_pending(hexfc_ctx* ctx, cudaStream_t s, bool* redrawn);
+hexfc_status settle_pending(hexfc_ctx* ctx, bool* redrawn);
 
 // A frame's final statistics: the latest verified, and kept by sequence number.
 inline void record_final(hexfc_ctx* ctx, const hexfc_frame_stats& fs)
@@ -961,7 +961,7 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
     collect(ctx);
     if (ctx->pend.active) {   // the previous frame (chosen capacities) has completed: verify it
         bool redrawn = false;
-        st = settle_pending(ctx, s, &redrawn);
+        st = settle_pending(ctx, &redrawn);
         ctx->have_frame = false;   // (a frame drawn again was kept: the buffers are this one's again)
         if (st != HEXFC_OK) return st;
         if (redrawn) {   // it was drawn again in these buffers: this frame's first passes once more
@@ -1038,7 +1038,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     collect(ctx);
     if (ctx->pend.active) {   // the previous frame has completed: verify it
         bool redrawn = false;
-        st = settle_pending(ctx, s, &redrawn);
+        st = settle_pending(ctx, &redrawn);
         ctx->have_frame = false;   // (a frame drawn again was kept: the buffers are this one's again)
         if (st != HEXFC_OK) return st;
         if (redrawn) {   // its exact redraw reused these buffers: this frame's first passes once more
@@ -1122,9 +1122,9 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
 // completed or be about to (its stream is waited for): its device scalars give
 // its statistics; device error bits are reported; if its pool ran out or a list
 // is too long for the resolve, it is drawn again exactly into
-// its output with its own camera, lens and style. s: the stream of the caller's
-// frame, on which the consumed error bits are cleared.
-hexfc_status settle_pending(hexfc_ctx* ctx, cudaStream_t s, bool* redrawn)
+// its output with its own camera, lens and style. All of it is on the frame's own
+// stream, and done when this returns.
+hexfc_status settle_pending(hexfc_ctx* ctx, bool* redrawn)
 {
     *redrawn = false;
     if (!ctx->pend.active) return HEXFC_OK;
@@ -1141,7 +1141,10 @@ hexfc_status settle_pending(hexfc_ctx* ctx, cudaStream_t s, bool* redrawn)
     fs.fragments = h[0];
     fs.max_list = (uint32_t)h[1];
     fs.long_lists = (uint32_t)h[2];
-    if (bits) CK(cudaMemsetAsync(ctx->fb.scal + 5, 0, sizeof(uint64_t), s));
+    if (bits) {   // (before a redraw asks for them)
+        CK(cudaMemsetAsync(ctx->fb.scal + 5, 0, sizeof(uint64_t), p.stream));
+        CK(cudaStreamSynchronize(p.stream));
+    }
     if (bits & ~kErrPoolBit) {   // a bounded wait ran out or a check failed
         record_final(ctx, fs);
         return device_error_status(bits);
@@ -1186,7 +1189,7 @@ hexfc_status finish_pending(hexfc_ctx* ctx)
 {
     if (!ctx->pend.active) return HEXFC_OK;
     bool redrawn = false;
-    return settle_pending(ctx, ctx->pend.stream, &redrawn);
+    return settle_pending(ctx, &redrawn);
 }
 
 // Weights, moments and gradient of the capacity network (once).
