@@ -91,6 +91,8 @@ struct hexfc_ctx {
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     cudaEvent_t ev_p1 = nullptr;   // a single frame's phase 1: bin total copied (FrameJob::p1_done)
     cudaEvent_t ev_p2 = nullptr;   // its phase 2: totals copied; the drawing pass runs after it
+    cudaEvent_t ev_drawn = nullptr;       // the last frame's last kernel,
+    cudaStream_t drawn_on = nullptr;      // on this stream
     cudaGraphExec_t graph_exec[3] = {nullptr, nullptr, nullptr};
     uint64_t graph_instantiations = 0, graph_updates = 0;
 };
@@ -754,6 +756,7 @@ hexfc_status job_read2(FrameJob& j, cudaStream_t s)
     if (fb.h_scal[5] != 0) {  // a bounded device wait ran out, or an exactness check failed
         const uint64_t bits = fb.h_scal[5];
         CK(cudaMemsetAsync(fb.scal + 5, 0, sizeof(uint64_t), s));
+        CK(cudaStreamSynchronize(s));   // (whatever stream the next frame is on)
         return device_error_status(bits);
     }
     j.total = fb.h_scal[0];
@@ -910,6 +913,21 @@ hexfc_status own_alloc(hexfc_ctx* ctx, FrameJob& j)
     return st;
 }
 
+// A frame's buffers are the context's: on another stream than the last frame's,
+// it waits for that frame's last kernels.
+hexfc_status follow_last(hexfc_ctx* ctx, cudaStream_t s)
+{
+    if (ctx->ev_drawn && ctx->drawn_on != s) CK(cudaStreamWaitEvent(s, ctx->ev_drawn, 0));
+    return HEXFC_OK;
+}
+hexfc_status note_last(hexfc_ctx* ctx, cudaStream_t s)
+{
+    if (!ctx->ev_drawn) CK(cudaEventCreateWithFlags(&ctx->ev_drawn, cudaEventDisableTiming));
+    CK(cudaEventRecord(ctx->ev_drawn, s));
+    ctx->drawn_on = s;
+    return HEXFC_OK;
+}
+
 // What the context keeps of the frame just drawn: its lists' inputs and camera.
 void keep_frame(hexfc_ctx* ctx, const FrameJob& j)
 {
@@ -930,6 +948,7 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
     hexfc_status st;
     ctx->have_frame = false;   // the frame buffers are this frame's from here on
     if ((st = own_alloc(ctx, j)) != HEXFC_OK) return st;
+    if ((st = follow_last(ctx, s)) != HEXFC_OK) return st;
     if (ctx->timing && !ctx->ev[0][0])
         for (auto& set : ctx->ev)
             for (auto& e : set) CK(cudaEventCreate(&e));
@@ -953,6 +972,7 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
         if ((st = job_phase2(j, s)) != HEXFC_OK) return st;
         CK(cudaEventRecord(ctx->ev_p2, s));
         if ((st = job_phase3(j, s)) != HEXFC_OK) return st;
+        if ((st = note_last(ctx, s)) != HEXFC_OK) return st;
         CK(cudaEventSynchronize(ctx->ev_p2));
         drawn = fb.h_scal[8] <= fb.bin_limit;
         j.n_bins = fb.bins_seen = fb.h_scal[8];
@@ -978,6 +998,7 @@ hexfc_status render_frame(hexfc_ctx* ctx, DevMesh* m, float* out, hexfc_frame_st
         if ((st = job_phase2(j, s)) != HEXFC_OK) return st;
         CK(cudaEventRecord(ctx->ev_p2, s));
         if ((st = job_phase3(j, s)) != HEXFC_OK) return st;
+        if ((st = note_last(ctx, s)) != HEXFC_OK) return st;
         CK(cudaEventSynchronize(ctx->ev_p2));   // the totals, while the frame is drawn
     }
     keep_counts(ctx, j);
@@ -1022,6 +1043,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     hexfc_status st;
     ctx->have_frame = false;
     if ((st = own_alloc(ctx, j)) != HEXFC_OK) return st;
+    if ((st = follow_last(ctx, s)) != HEXFC_OK) return st;
     // capacity arrays follow the tile arrays
     if ((st = ensure_all(&fb.cap_cap, fb.t_cap, {part(&fb.tile_cap), part(&fb.cap_off)})) != HEXFC_OK) return st;
     if (!ctx->h_pend) CK(pinned_alloc((void**)&ctx->h_pend, kScal * sizeof(uint64_t)));
@@ -1088,6 +1110,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
     j.launches += 1 + 3 + 1 + 1 + 2;   // capacities, their scan, count, check, drawing passes
     // the frame's scalars for its verification; no wait here
     CK(cudaMemcpyAsync(ctx->h_pend, fb.scal, kScal * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    if ((st = note_last(ctx, s)) != HEXFC_OK) return st;
     ctx->ev_pending[ctx->ev_cur] = ctx->timing;
     hexfc_frame_stats& fs = j.fs;
     fs = hexfc_frame_stats{};
@@ -1382,6 +1405,7 @@ void hexfc_destroy(hexfc_ctx* ctx)
     if (ctx->ev_out) cudaEventDestroy(ctx->ev_out);
     if (ctx->ev_p1) cudaEventDestroy(ctx->ev_p1);
     if (ctx->ev_p2) cudaEventDestroy(ctx->ev_p2);
+    if (ctx->ev_drawn) cudaEventDestroy(ctx->ev_drawn);
     dfree(ctx->d_out);
     for (auto& set : ctx->ev)
         for (auto& e : set)

@@ -51,7 +51,6 @@ def test_a_frame_on_another_stream_finds_the_pool_run_out(hx):
             r.set_view(VIEWS[k])
             r.render(mid, o, stream=a)
         jumped = r.last_stats["frame"]
-        torch.cuda.synchronize()
         r.render(mid, outs[3], stream=b)
         assert r.completed_stats(jumped)["redrawn"] == 1
         assert r.finish()["redrawn"] == 0
@@ -59,3 +58,28 @@ def test_a_frame_on_another_stream_finds_the_pool_run_out(hx):
         for o, k in zip(outs, (0, 0, 1, 1)):
             np.testing.assert_array_equal(o.cpu().numpy(), want[k])
         r.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1, 3])
+def test_frames_in_turn_on_two_streams(hx, mode):
+    """Back to back, of two meshes and sizes, without a wait in between: a frame waits for the last one's kernels, whose
+    buffers it writes."""
+    meshes = [synth.hex_grid(24, jitter=0.1, warp_amp=0.3, seed=6), synth.hex_grid(7, jitter=0.1, seed=2)]
+    views = [synth.orbit_view(3, 120, 640, 360, radius=1.4), synth.orbit_view(9, 120, 200, 150, radius=1.4)]
+    want = [_exact(hx, m, v) for m, v in zip(meshes, views)]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    r, big = _context(hx, meshes[0])
+    small = r.upload_mesh(meshes[1].verts, meshes[1].cells, meshes[1].cell_scalar, meshes[1].edge_level)
+    r.set_option(hx.HEXFC_OPT_PREDICTED_CAPACITY, mode)
+    outs = [[torch.empty((v.height, v.width, 4), device="cuda") for v in views] for _ in range(12)]
+    torch.cuda.synchronize()
+    for pair in outs:
+        for k in (0, 1):
+            r.set_view(views[k])
+            r.render((big, small)[k], pair[k], stream=streams[k])
+    r.finish()
+    torch.cuda.synchronize()
+    for pair in outs:
+        for k in (0, 1):
+            np.testing.assert_array_equal(pair[k].cpu().numpy(), want[k])
+    r.close()
