@@ -94,6 +94,7 @@ struct hexfc_ctx {
     cudaEvent_t ev_drawn = nullptr;       // the last frame's last kernel,
     cudaStream_t drawn_on = nullptr;      // on this stream
     cudaGraphExec_t graph_exec[3] = {nullptr, nullptr, nullptr};
+    std::vector<unsigned> graph_slices;   // count_slices of the items of graph_exec[1]
     uint64_t graph_instantiations = 0, graph_updates = 0;
 };
 
@@ -1581,6 +1582,17 @@ hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_ite
             [&](CountBatch& cb) { return launch_count_batch(cb, o); });
     };
     const bool one = ctx->batch_launch;
+    // The update of an executable graph takes over a kernel's grid but not its
+    // cluster size, and answers success: with other cluster sizes than it was
+    // instantiated with, the graph is built anew.
+    std::vector<unsigned> slices;
+    if (!one)
+        for (int i : live) slices.push_back(count_slices(jobs[(size_t)i].n_tiles, (int64_t)jobs[(size_t)i].n_bins));
+    if (slices != ctx->graph_slices && ctx->graph_exec[1]) {
+        cudaGraphExecDestroy(ctx->graph_exec[1]);
+        ctx->graph_exec[1] = nullptr;
+    }
+    ctx->graph_slices = std::move(slices);
     if (one && (st = batch_graph(
                     ctx, 1, live, [&](int i, cudaStream_t si) { return job_phase2_bins(jobs[(size_t)i], si); },
                     count_all, none, true, false)) != HEXFC_OK)

@@ -335,6 +335,8 @@ cudaError_t launch_bin_sort(FrameBufs& fb, int64_t n_tiles, int64_t n_bins, int 
                             cudaStream_t s);
 cudaError_t launch_tile_order(FrameBufs& fb, int n_tiles, cudaStream_t s);
 CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H);
+// Blocks a tile (the cluster size) of a frame's count.
+unsigned count_slices(int64_t n_tiles, int64_t n_bins);
 cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s,
                          bool to_host = true);
 // The count and the drawing pass of several frames, each one launch.

@@ -855,6 +855,7 @@ __global__ void __launch_bounds__(kTilePix, kCountBlocks) k_count(const __grid_c
 {
     chain_wait();
     const uint32_t slices = cooperative_groups::this_cluster().num_blocks();
+    if (blockIdx.x / slices >= (uint32_t)a.n_tiles) return;   // (not reached while grid and clusters belong together)
     count_tile((int)a.order[blockIdx.x / slices], a, blockIdx.x % slices, slices);
 }
 
@@ -949,19 +950,25 @@ CountItem count_item(const FrameBufs& fb, int tiles_x, int tiles_y, int W, int H
                      reinterpret_cast<unsigned long long*>(fb.scal), fb.h_scal, fb.bin_limit, tiles_x, W, H, tiles_x * tiles_y};
 }
 
-cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s,
-                         bool to_host)
+unsigned count_slices(int64_t n_tiles, int64_t n_bins)
 {
     // Few tiles with long lists: several blocks a tile, up to four times what the
     // chip holds at once, so that the longest list does not decide alone, and a
     // run of chunks for every warp (96^3 at 320x180, 240 tiles of up to 1500
     // chunks: one block 0.48 ms, as many as fit at once 0.26, twice 0.15, four
     // times 0.11). The blocks of a tile are a cluster.
-    const int64_t n_tiles = (int64_t)tiles_x * tiles_y;
     unsigned slices = 1;
     while (slices < kCountSlices && 2 * slices * n_tiles <= 4 * 152 * kCountBlocks &&
            slices * n_tiles * 2 * kConsumerWarps * kChunk < n_bins)
         slices *= 2;
+    return slices;
+}
+
+cudaError_t launch_count(FrameBufs& fb, int tiles_x, int tiles_y, int W, int H, int64_t n_bins, cudaStream_t s,
+                         bool to_host)
+{
+    const int64_t n_tiles = (int64_t)tiles_x * tiles_y;
+    const unsigned slices = count_slices(n_tiles, n_bins);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)n_tiles * slices);
     cfg.blockDim = dim3(kTilePix);
