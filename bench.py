@@ -45,7 +45,7 @@ DRAW_ISSUE = {"warp_instructions_per_fragment": 8.937,
               "sha256": "07c7e546cf8e66ddaa759137f77dd5700ea2344364c17bf139c877d0e156b1d6",
               "profile": "profiles/issue_k_draw_grid64_orbit_1080p.md"}
 SCHEDULERS_PER_SM = 4    # warp schedulers (issue slots per cycle) of a Blackwell SM
-DRAW_SOURCES = ("csrc/k_draw.cu", "csrc/shade.cuh", "csrc/raster_common.cuh", "csrc/pipeline.cuh",
+DRAW_SOURCES = ("csrc/k_draw.cu", "csrc/draw_slot.h", "csrc/shade.cuh", "csrc/raster_common.cuh", "csrc/pipeline.cuh",
                 "csrc/hexfc_internal.cuh")
 
 
@@ -683,7 +683,7 @@ def run_learned(args, rank, world):
     500-frame camera and lens path. Frames 0-399 are drawn without capacities
     and the capacity network trains on each frame's exact tile counts; frames
     400-499 are then drawn (timed) without and with chosen tile
-    capacities (no pixel scan, no host wait after the count, each frame
+    capacities (no host wait after the count, each frame
     verified by the next call and drawn again exactly if they ran out): the
     network's, the previous frame's counts, and the previous total spread
     evenly over the tiles."""

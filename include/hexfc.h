@@ -1,9 +1,9 @@
 /*
  * hexfc.h -- C ABI of the GB300 focus+context hex-mesh renderer.
  *
- * The library renders every face of a hexahedral mesh into per-pixel fragment
- * lists, shades each fragment in the focus+context edge/face style, sorts
- * each list by depth and blends it front to back ("Interactive Focus+Context
+ * The library renders every face of a hexahedral mesh: each pixel's fragments
+ * are shaded in the focus+context edge/face style, ordered by depth and
+ * blended front to back ("Interactive Focus+Context
  * Rendering for Hexahedral Mesh Inspection", Neuhauser, Wang, Westermann:
  * Section "Method Overview", Section "Focus+Context" Eqs. 1-4, Section
  * "GPU Implementation").
@@ -17,6 +17,7 @@
  *     live until hexfc_destroy.
  *   - No C++ exception crosses this boundary; every failure is a status < 0.
  *   - A context is not thread-safe: calls on one context must be serialised.
+ *     Its frames may be on different streams: each waits for the last one.
  */
 #ifndef HEXFC_H
 #define HEXFC_H
@@ -185,9 +186,11 @@ void hexfc_destroy(hexfc_ctx* ctx);
  *                    Detail Structure": each edge carries the highest level
  *                    at which it still exists), or NULL for level 0
  * Builds the unique faces (each geometric face once, canonical corner order,
- * face id = rank of its sorted vertex ids) and unique edges on the host, and
- * the per-vertex / per-edge importance (max over incident cells, Section
- * "Method Overview") on the device. *mesh_id_out receives the mesh handle.
+ * face id = rank of its sorted vertex ids) and unique edges, on the device or,
+ * where that has no memory to sort them in or a mesh is not for it, on the
+ * host, and the per-vertex / per-edge importance (max over incident cells,
+ * Section "Method Overview") on the device. *mesh_id_out receives the mesh
+ * handle.
  * Errors: ARG, MESH (index out of range, non-finite vertex, n_cells == 0),
  * OOM, CUDA. Synchronous.
  */
@@ -269,7 +272,9 @@ hexfc_status hexfc_cell_quality(hexfc_ctx* ctx, int32_t mesh, int32_t metric, fl
 /*
  * Replace the mesh's per-cell importance with `cell_importance` (device,
  * n_cells float) and recompute the per-vertex and per-edge maxima on the
- * device (Section "Method Overview"). Errors: ARG, STATE, CUDA.
+ * device (Section "Method Overview"), in place: nothing is allocated, the call
+ * can be captured into a CUDA graph, and each replay is what the next frame
+ * reads. Errors: ARG, STATE, CUDA.
  */
 hexfc_status hexfc_set_cell_importance(hexfc_ctx* ctx, int32_t mesh, const float* cell_importance,
                                        void* stream);
@@ -309,9 +314,11 @@ hexfc_status hexfc_set_style(hexfc_ctx* ctx, const hexfc_style* style);
  * Steps, all on `stream`: vertex projection to 16.8 fixed point and 24-bit
  * depth; triangle setup and tile binning in depth order; per-pixel fragment
  * count; then every fragment shaded with Eqs. 1-4 and blended front to back in
- * order of depth. The call waits for the bin total (to size the buffers) and,
- * while the frame is drawn, for the fragment total (statistics, limits); the
- * image is complete when `stream` reaches the end of the call.
+ * order of depth. The call waits once, while the frame is drawn, for the bin
+ * and fragment totals (statistics, limits); it waits for the bin total before
+ * that if its buffers may have no room for the bins (a first frame, a memory
+ * budget, more bins than ever). The image is complete when `stream` reaches the
+ * end of the call.
  * stats (host, nullable) receives the frame statistics.
  * Errors: ARG, STATE (no view), OOM (the frame's buffers would exceed the
  * budget; stats still filled: fragments tells how far), OVERFLOW (a list longer than HEXFC_MAX_LIST), CUDA, and TIMEOUT or
@@ -387,8 +394,9 @@ hexfc_status hexfc_set_option(hexfc_ctx* ctx, int32_t option, int64_t value);
  * A predicted frame's image is final once the next hexfc_render* call or
  * hexfc_finish on its context has returned (and the stream work it issued has
  * run); its output buffer must stay valid until then. Waits for the last
- * frame's stream. stats (host, nullable): the final statistics of the last
- * frame (pending = 0; redrawn = 1 if it was drawn again). Errors: ARG,
+ * frame's stream. A frame drawn again reads the mesh's importance as it then is:
+ * call this before hexfc_set_cell_importance where that must be the frame's own.
+ * stats (host, nullable): the final statistics of the last frame (pending = 0; redrawn = 1 if it was drawn again). Errors: ARG,
  * TIMEOUT/CHECK (device error bits of the verified frame), CUDA. Not in the
  * paper, which sizes its fragment buffer once (Section "GPU Implementation").
  */
@@ -423,8 +431,8 @@ hexfc_status hexfc_completed_stats(const hexfc_ctx* ctx, uint64_t frame, hexfc_f
  * distance to the lens and the camera's motion since the previous frame;
  * the capacity is expm1(y) * 1.15 + 256. Weights are used in FP16 with FP32
  * sums; training keeps FP32 master weights and Adam moments on the device.
- * Every frame leaves its features and exact tile counts (from the count pass
- * or the fused pass) for training. Parameters: HEXFC_CAPACITY_PARAMS floats,
+ * Every frame, drawn or refused after its count, leaves its features and exact
+ * tile counts for training. Parameters: HEXFC_CAPACITY_PARAMS floats,
  * in the order W1 (64 x 4, row-major), b1 (64), W2 (64 x 64, row-major,
  * W2[j][i] from hidden unit i of the first layer to unit j of the second),
  * b2 (64), w3 (64), b3 (1).
@@ -441,7 +449,8 @@ hexfc_status hexfc_completed_stats(const hexfc_ctx* ctx, uint64_t frame, hexfc_f
  * hexfc_capacity_train: `steps` Adam steps (rate lr) on the last frame's
  *   features and exact tile counts, on `stream`; *loss (nullable) receives
  *   the loss before the last step (the host waits when loss != NULL).
- *   Errors: ARG, STATE (no weights or no frame yet), OOM, CUDA.
+ *   Errors: ARG, STATE (no weights, no frame yet, or none since hexfc_trim),
+ *   OOM, CUDA.
  */
 #define HEXFC_CAPACITY_PARAMS 4545
 hexfc_status hexfc_capacity_reset(hexfc_ctx* ctx, uint64_t seed);
@@ -508,8 +517,9 @@ void hexfc_raster_tile(int32_t* width, int32_t* height);
  *   counters that must start at zero are cleared on the stream). Calls whose
  *   work overlaps on the GPU (other streams, other threads, other contexts of
  *   the same process on the same device) race on it: serialise them.
- * - It waits on `stream` twice, like hexfc_render, and returns with the drawing
- *   passes still running. Their device error bits (a bounded wait
+ * - It waits on `stream` once for the totals (again only for a frame within a
+ *   few chunks of the array's size) and returns with the drawing passes still
+ *   running. Their device error bits (a bounded wait
  *   that ran out, a failed exactness check) stay in the array and are
  *   reported, as TIMEOUT or CHECK, by the next hexfc_render_noalloc call on
  *   the same device, as hexfc_render reports its previous frame's.

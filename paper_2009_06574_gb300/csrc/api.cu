@@ -1145,7 +1145,7 @@ hexfc_status render_frame_predicted(hexfc_ctx* ctx, DevMesh* m, float* out, hexf
 // Verify the pending frame (drawn with chosen capacities), which must have
 // completed or be about to (its stream is waited for): its device scalars give
 // its statistics; device error bits are reported; if its pool ran out or a list
-// is too long for the resolve, it is drawn again exactly into
+// is too long to be sorted, it is drawn again exactly into
 // its output with its own camera, lens and style. All of it is on the frame's own
 // stream, and done when this returns.
 hexfc_status settle_pending(hexfc_ctx* ctx, bool* redrawn)
@@ -1909,7 +1909,7 @@ hexfc_status hexfc_render_host(hexfc_ctx* ctx, int32_t mesh, float* out_rgba_hos
     cudaStream_t s = (cudaStream_t)stream;
     size_t bytes = sizeof(float) * 4 * (size_t)draw_w(ctx) * (size_t)draw_h(ctx);
     // A page-locked buffer of this device, 16-byte aligned, is written by the
-    // resolve kernels through its device mapping: the image crosses to the
+    // drawing kernels through its device mapping: the image crosses to the
     // host while they run rather than in a copy after them.
     float* d_out = nullptr;
     cudaPointerAttributes pa{};

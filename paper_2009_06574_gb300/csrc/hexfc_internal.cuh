@@ -163,7 +163,7 @@ struct FrameBufs {
     uint64_t* tile_off = nullptr;   // [T+1]
     uint32_t* tile_cur = nullptr;   // [T] the binning's places without counts, then the tiles' chunks
     uint32_t* tile_order = nullptr; // [T] tiles by decreasing chunk count
-    uint32_t* tile_frag = nullptr;  // [T] exact fragments per tile (the count's or the fused pass's)
+    uint32_t* tile_frag = nullptr;  // [T] exact fragments per tile (the count's)
     float* cap_x = nullptr;         // [4T] capacity-network features of the frame
     uint32_t* tile_cap = nullptr;   // [T+1] chosen fragment capacity per tile (predicted frames)
     uint64_t* cap_off = nullptr;    // [T+1] its exclusive prefix

@@ -1,7 +1,9 @@
 // Geometry and fragment stages of the renderer.
 //
-//   k_vertex_setup  per vertex: camera transform in double (no FMA), window
-//                   position snapped to 16.8 fixed point, 24-bit window depth.
+//   k_vertex_setup  per vertex: camera transform (in double by definition, no
+//                   FMA; from pairs of floats where those decide the result),
+//                   window position snapped to 16.8 fixed point, 24-bit window
+//                   depth.
 //   k_face_setup    per unique face: gather the 4 projected corners, edge
 //                   visibility masks of Eq. 1, triangle validity, and the
 //                   number of raster tiles each triangle's box touches.
@@ -14,10 +16,9 @@
 // The drawing pass is in k_draw.cu.
 //
 // Each face is drawn as two triangles (Section "Method Overview"; Section "GPU
-// Implementation"), all covered samples are kept (per-pixel fragment lists,
-// Section "GPU Implementation"), and the fragment shader computes focus from
-// the lens, the edge distance to the four face edges ignoring invisible ones,
-// and Eqs. 1-4 (Section "Focus+Context").
+// Implementation"), and all covered samples take part (the paper keeps them in
+// per-pixel fragment lists, Section "GPU Implementation"; here they are bits of
+// the coverage masks, in the tile's depth order).
 #include <algorithm>
 
 #include <cooperative_groups.h>

@@ -1,5 +1,5 @@
 // Fragment shading of the focus+context renderer (Section "Focus+Context",
-// Eqs. 1-4), used by the fill kernel of this library.
+// Eqs. 1-4), used by the drawing kernels of this library.
 #pragma once
 #include "raster_common.cuh"
 
