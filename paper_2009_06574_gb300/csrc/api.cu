@@ -1500,7 +1500,7 @@ hexfc_status hexfc_upload_mesh(hexfc_ctx* ctx, const float* verts, int64_t n_ver
 
 hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_item* items,
                                 hexfc_frame_stats* stats, hexfc_status* item_status, void* stream)
-{
+try {
     if (!ctx || n < 0 || (n > 0 && !items)) return HEXFC_ERR_ARG;
     std::vector<CamParams> cams((size_t)n);
     std::vector<double> zrefs((size_t)n, 1.0);
@@ -1654,6 +1654,8 @@ hexfc_status hexfc_render_batch(hexfc_ctx* ctx, int32_t n, const hexfc_batch_ite
         if (first == HEXFC_OK) first = res[(size_t)i];
     }
     return first;
+} catch (...) {   // (host memory)
+    return HEXFC_ERR_OOM;
 }
 
 hexfc_status hexfc_capacity_set_weights(hexfc_ctx* ctx, const float* w, int64_t n)
@@ -1676,7 +1678,7 @@ hexfc_status hexfc_capacity_set_weights(hexfc_ctx* ctx, const float* w, int64_t 
 }
 
 hexfc_status hexfc_capacity_reset(hexfc_ctx* ctx, uint64_t seed)
-{
+try {
     if (!ctx) return HEXFC_ERR_ARG;
     std::vector<float> w((size_t)kCapParams, 0.f);
     NormalStream rs{seed};
@@ -1687,6 +1689,8 @@ hexfc_status hexfc_capacity_reset(hexfc_ctx* ctx, uint64_t seed)
     for (int i = oW3; i < oB3; ++i) w[(size_t)i] = (float)(rs.next() * std::sqrt(1.0 / kCapHid));
     w[(size_t)oB3] = 5.f;   // log(1 + count) of a few hundred fragments
     return hexfc_capacity_set_weights(ctx, w.data(), kCapParams);
+} catch (...) {   // (host memory)
+    return HEXFC_ERR_OOM;
 }
 
 hexfc_status hexfc_capacity_get_weights(hexfc_ctx* ctx, float* w, int64_t n)
@@ -1952,7 +1956,7 @@ hexfc_status hexfc_render_host(hexfc_ctx* ctx, int32_t mesh, float* out_rgba_hos
 
 hexfc_status hexfc_debug_pixels(hexfc_ctx* ctx, const int32_t* px, const int32_t* py, int64_t n, uint32_t* counts,
                                 uint64_t* keys, float* rgba, uint64_t cap)
-{
+try {
     if (!ctx || !px || !py || !counts || n < 0) return HEXFC_ERR_ARG;
     if (!ctx->have_frame) return HEXFC_ERR_STATE;
     if (ctx->pend.active) {
@@ -1965,6 +1969,7 @@ hexfc_status hexfc_debug_pixels(hexfc_ctx* ctx, const int32_t* px, const int32_t
         if (px[i] < 0 || py[i] < 0 || px[i] >= win.w || py[i] >= win.h) return HEXFC_ERR_ARG;
     if (n == 0) return HEXFC_OK;
     std::vector<int32_t> qx((size_t)n), qy((size_t)n);
+    std::vector<uint64_t> hoff((size_t)n);
     for (int64_t i = 0; i < n; ++i) {
         qx[(size_t)i] = px[i] + win.x0;
         qy[(size_t)i] = py[i] + win.y0;
@@ -1997,7 +2002,6 @@ hexfc_status hexfc_debug_pixels(hexfc_ctx* ctx, const int32_t* px, const int32_t
         cleanup();
         return HEXFC_ERR_CUDA;
     }
-    std::vector<uint64_t> hoff((size_t)n);
     uint64_t total = 0;
     for (int64_t i = 0; i < n; ++i) {
         hoff[(size_t)i] = total;
@@ -2032,6 +2036,8 @@ hexfc_status hexfc_debug_pixels(hexfc_ctx* ctx, const int32_t* px, const int32_t
         return HEXFC_ERR_CUDA;
     }
     return st;
+} catch (...) {   // (host memory)
+    return HEXFC_ERR_OOM;
 }
 
 hexfc_status hexfc_set_option(hexfc_ctx* ctx, int32_t option, int64_t value)
