@@ -36,13 +36,13 @@ sys.path.insert(0, ROOT)
 # DRAM traffic of one k_draw launch (ncu dram__bytes_read.sum + dram__bytes_write.sum,
 # one pass, on the 1920x1080 bench frame), per fragment of the frame, and the drawing
 # kernel's sources it was taken on: reported only while those sources are unchanged.
-DRAW_DRAM = {"bytes_per_fragment": 3.746,
-             "sha256": "07c7e546cf8e66ddaa759137f77dd5700ea2344364c17bf139c877d0e156b1d6",
+DRAW_DRAM = {"bytes_per_fragment": 3.742,
+             "sha256": "5cf807ba17105ef4c9ae1ad06cd5e8e352655952b681bf567ef4e82421475028",
              "profile": "profiles/dram_k_draw_grid64_orbit_1080p.md"}
 # Warp instructions it executes per fragment (ncu smsp__inst_executed.sum on the same
 # frame and sources): its issue roofline, beside the HBM one.
-DRAW_ISSUE = {"warp_instructions_per_fragment": 8.937,
-              "sha256": "07c7e546cf8e66ddaa759137f77dd5700ea2344364c17bf139c877d0e156b1d6",
+DRAW_ISSUE = {"warp_instructions_per_fragment": 8.783,
+              "sha256": "5cf807ba17105ef4c9ae1ad06cd5e8e352655952b681bf567ef4e82421475028",
               "profile": "profiles/issue_k_draw_grid64_orbit_1080p.md"}
 SCHEDULERS_PER_SM = 4    # warp schedulers (issue slots per cycle) of a Blackwell SM
 DRAW_SOURCES = ("csrc/k_draw.cu", "csrc/draw_slot.h", "csrc/shade.cuh", "csrc/raster_common.cuh", "csrc/pipeline.cuh",
@@ -598,7 +598,7 @@ def run_batch(args, rank, world, steps=None, warmup=None):
     96) x 16 orbit views each at 1280x720, drawn as one batch per step (each
     frame phase of all 48 views captured as one CUDA graph, every view its own
     launches on parallel branches), with the tuning options chosen by the
-    autotuner; against the same batch with the count, fill and resolve of all
+    autotuner; against the same batch with the count and the drawing pass of all
     views each one launch, and against the 48 frames drawn one by one. The
     same three ways are timed again on 320x180 thumbnails of the same views."""
     import numpy as np

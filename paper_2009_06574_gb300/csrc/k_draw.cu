@@ -383,10 +383,11 @@ __device__ __forceinline__ uint32_t load_acquire(const uint32_t* p)
 // pixel is finished; a warp whose pixels are all finished only stages, and the
 // block ends when all have.
 //
-// Bound by instruction issue: 64^3 at 1920x1080, 75.6 M fragments in 0.733 ms (the
-// pass that stored 24-byte fragments and the one that read and blended them:
-// 0.91 + 0.39 ms, 4.2 GB of DRAM), at 9 warp instructions a fragment, of which the
-// edge distances of Eq. 1 are about 3; 128^3 at 3840x2160 5.46 ms. Three blocks an SM
+// Bound by instruction issue: 64^3 at 1920x1080, 77.6 M fragments (mean of an
+// orbit) in 0.724 ms (the pass that stored 24-byte fragments and the one that read
+// and blended them: 0.91 + 0.39 ms, 4.2 GB of DRAM), at 8.8 warp instructions a
+// fragment, of which the edge distances of Eq. 1 are about 3; 128^3 at 3840x2160,
+// 604 M fragments, 4.98 ms. Three blocks an SM
 // of 80 registers (two or four: 6% and 10% slower); kService steps between looks at
 // the ring 8 (4, 16, 32: 1-2% slower).
 template <int KW, bool kSil, bool kWide>
